@@ -96,6 +96,10 @@ struct LoraArgs {
   int nseg;
   LoraSeg seg[3];
   float* T;                       // dev fp32 [M][nseg][rank], already multiplied by the adapter scale
+  // the same for the tcgen05 projection (nullptr: T is used): fp16 [M][nseg][2][ke], T as value + rounding remainder in
+  // the columns slot * rank + j of the row's own slot, zeros elsewhere; ke = k_slots * rank rounded up to 64
+  __half* text;
+  int ke, k_slots, slot_is_adapter;   // slots: streams of the pass, or (1) the adapters themselves
 };
 
 struct GemmArgs {
@@ -112,6 +116,13 @@ struct GemmArgs {
   size_t partial_capacity;        // floats
   unsigned* counters;             // zeroed, >= n_blocks * m_blocks entries
   LoraArgs lora;
+  // tcgen05 path only
+  int late_wait;                  // the kernel ahead produces only the adapters' T: the activations are complete already
+  const unsigned long long* ssq_in;   // the rows of h still lack 1/rms: their sums of squares [M] (fixed point), or nullptr
+  float eps;
+  unsigned long long* ssq_out;    // EPI_RESID: sums of squares of the new residual rows are added here (nullptr: not wanted)
+  __half* xg_out;                 // EPI_RESID: new residual x gain_next as fp16 (nullptr: not wanted)
+  const __half* gain_next;
 };
 
 struct ShrinkArgs {
@@ -122,6 +133,7 @@ struct ShrinkArgs {
   __half* h_out;                  // NORM mode: normalised fp16 rows written here
   int M, K;
   LoraArgs lora;                  // adapter_idx == nullptr: only the norm is done
+  int pdl;                        // launch_shrink_rows: programmatic launch behind the kernel that writes h_in
 };
 
 struct AttnArgs {
@@ -302,14 +314,19 @@ cudaError_t launch_dequant(const unsigned char* w, int K, int N, int G, int tile
                            __half* out, cudaStream_t st);
 int gemm_pick_split(int K, int N, int M, size_t partial_capacity);
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t st);
-// tcgen05 path for passes with 32 rows or more: partial sums on the tensor cores, then an epilogue kernel
+// tcgen05 path for passes with TC_MIN_ROWS rows or more
+constexpr int TC_MIN_ROWS = 9;
 cudaError_t init_gemm_tc();
 bool gemm_tc_eligible(const GemmArgs& a);
 cudaError_t launch_gemm_tc(const GemmArgs& a, int sm_count, int* status, cudaStream_t st);
 cudaError_t launch_shrink(const ShrinkArgs& a, cudaStream_t st);
+// T of a pass whose rows are grouped by stream (rows_per_stream each), from fp16 rows, on mma.sync
+cudaError_t launch_shrink_rows(const ShrinkArgs& a, cudaStream_t st);
+bool tensor_maps_available();
 cudaError_t launch_embed(const int32_t* tokens, const __half* embed, const __half* hidden_in, float* X, int M,
                          int d, int vocab, int* status, cudaStream_t st, const __half* forecast = nullptr,
-                         int n_forecast = 0);
+                         int n_forecast = 0, const __half* gain = nullptr, __half* xg = nullptr,
+                         unsigned long long* ssq = nullptr);
 cudaError_t launch_draft(const float* logits, int V, int n, int R, int m, int wmax, const int32_t* widths,
                          const int32_t* level, const int32_t* rank, const int32_t* forecast_of, const int32_t* acc_len,
                          const int32_t* acc_idx, const int32_t* next, int32_t* cand, int32_t* out_tokens, int* status,

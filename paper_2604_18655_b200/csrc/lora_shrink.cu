@@ -6,6 +6,22 @@
 
 namespace mlora {
 
+// one entry of T for the tcgen05 projection: value and rounding remainder (LoraArgs::text)
+__device__ __forceinline__ void text_store(const LoraArgs& l, int m, int seg, int k, float v) {
+  __half* row = l.text + ((size_t)m * l.nseg + seg) * 2 * l.ke + k;
+  const __half h = __float2half_rn(v);
+  row[0] = h;
+  row[l.ke] = __float2half_rn(v - __half2float(h));
+}
+// zeros everywhere outside the columns [k0, k1) of the row
+__device__ __forceinline__ void text_clear(const LoraArgs& l, int m, int seg, int k0, int k1, int tid, int nthreads) {
+  __half* row = l.text + ((size_t)m * l.nseg + seg) * 2 * l.ke;
+  for (int k = tid; k < 2 * l.ke; k += nthreads) {
+    const int kk = k < l.ke ? k : k - l.ke;
+    if (kk < k0 || kk >= k1) row[k] = __float2half_rn(0.f);
+  }
+}
+
 constexpr int SHRINK_THREADS = 256;
 constexpr int SHRINK_JCHUNK = 8;   // rank indices per CTA
 
@@ -59,8 +75,11 @@ __global__ void __launch_bounds__(SHRINK_THREADS) norm_shrink_kernel(const Shrin
   float* T = p.lora.T + ((size_t)m * p.lora.nseg + seg) * r;
   const __half* A = nullptr;
   if (a >= 0 && a < p.lora.n_slots) A = p.lora.tabA[(size_t)a * p.lora.tab_stride + p.lora.seg[seg].proj_index];
+  const int slot = p.lora.slot_is_adapter ? a : m / p.lora.rows_per_stream;
+  if (p.lora.text != nullptr && jc == 0) text_clear(p.lora, m, seg, A ? slot * r : 0, A ? slot * r + r : 0, threadIdx.x, SHRINK_THREADS);
   if (A == nullptr) {
-    for (int j = j0 + threadIdx.x; j < j1; j += SHRINK_THREADS) T[j] = 0.f;
+    if (p.lora.text == nullptr)
+      for (int j = j0 + threadIdx.x; j < j1; j += SHRINK_THREADS) T[j] = 0.f;
     return;
   }
   const float s = p.lora.scale[a];
@@ -80,41 +99,51 @@ __global__ void __launch_bounds__(SHRINK_THREADS) norm_shrink_kernel(const Shrin
       }
     }
     acc = warp_sum(acc);
-    if (lane == 0) T[j] = s * acc;
+    if (lane == 0) {
+      if (p.lora.text != nullptr) text_store(p.lora, m, seg, slot * r + j, s * acc);
+      else T[j] = s * acc;
+    }
   }
 }
 
-// LoRA shrink on mma.sync for passes whose rows come in runs of 16 that share an adapter (rows_per_stream a multiple
-// of 16: DS2D trees of 16 or 32 nodes).  One CTA per (16 rows, segment, 8 rank indices); its sixteen warps split K in
-// contiguous ranges and the partial fragments are added in warp order.  Per 16 features a thread loads 8 consecutive
+// LoRA shrink on mma.sync for passes whose rows are grouped by stream (one adapter per rows_per_stream rows: DS2D trees,
+// decode steps of many streams).  One CTA per (up to 16 rows of a stream, segment, 8 rank indices); its sixteen warps split
+// K in contiguous ranges and the partial fragments are added in warp order.  Per 16 features a thread loads 8 consecutive
 // features of an activation row (rows g and g+8 of the tile) and of an A row (rank index j0 + g): the two k16 steps
 // use features {0,1 | 2,3} and {4,5 | 6,7} of that piece for the fragment's (k 2t.. | k 2t+8..) slots -- any pairing of
 // slots with features is valid as long as both operands use the same one.  The activations are the fp16 rows the
-// GEMM reads (written by the norm pass before), so the A matrix of a stream is fetched once per 16 rows.
+// GEMM reads, so the A matrix of a stream is fetched once per 16 rows.  Programmatic launch: the A rows (immutable) are
+// asked for ahead of the wait; the projection behind this kernel is let go behind it, so that it finds the activations
+// complete and only has to wait for T.
 constexpr int SHRINK_MMA_WARPS = 16;
-__global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_mma_kernel(const ShrinkArgs p, const __half* __restrict__ h) {
-  // (the tensor-core projection launched after this kernel may start streaming its weights now)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+__global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_mma_kernel(const ShrinkArgs p, const int tiles_per_stream) {
   __shared__ float red[SHRINK_MMA_WARPS][32][4];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int m0 = blockIdx.x * 16, r = p.lora.rank, K = p.K;
+  const int T = p.lora.rows_per_stream, stream = blockIdx.x / tiles_per_stream;
+  const int m0 = stream * T + (blockIdx.x - stream * tiles_per_stream) * 16, m_end = min(p.M, (stream + 1) * T);
+  const int r = p.lora.rank, K = p.K;
   const int jtiles = (r + 7) / 8;
   const int seg = blockIdx.y / jtiles, j0 = (blockIdx.y % jtiles) * 8;
   const int mA = m0 + g, mB = mA + 8;
-  const int a = p.lora.adapter_idx[m0 / p.lora.rows_per_stream];
+  const int a = p.lora.adapter_idx[stream];
   const __half* A = nullptr;
   if (a >= 0 && a < p.lora.n_slots) A = p.lora.tabA[(size_t)a * p.lora.tab_stride + p.lora.seg[seg].proj_index];
+  const float s = A != nullptr ? p.lora.scale[a] : 0.f;
+  // a warp takes a contiguous range of 64-feature blocks; per block a thread reads 32 contiguous bytes of each of
+  // its three rows, so a warp fetches whole 128-byte lines
+  const int nblk = K / 64, per = (nblk + SHRINK_MMA_WARPS - 1) / SHRINK_MMA_WARPS;
+  const int b0 = warp * per, b1 = min(nblk, b0 + per);
+  const uint4* Ar = A != nullptr ? reinterpret_cast<const uint4*>(A + (size_t)min(j0 + g, r - 1) * K) + 2 * t : nullptr;
+  if (A != nullptr && t == 0)
+    for (int b = b0; b < b1; ++b) asm volatile("prefetch.global.L1 [%0];" ::"l"(Ar + b * 8) : "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   float acc[4] = {0.f, 0.f, 0.f, 0.f};
   if (A != nullptr) {
     const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-    // a warp takes a contiguous range of 64-feature blocks; per block a thread reads 32 contiguous bytes of each of
-    // its three rows, so a warp fetches whole 128-byte lines
-    const int nblk = K / 64, per = (nblk + SHRINK_MMA_WARPS - 1) / SHRINK_MMA_WARPS;
-    const int b0 = warp * per, b1 = min(nblk, b0 + per);
-    const uint4* hA = reinterpret_cast<const uint4*>(h + (size_t)min(mA, p.M - 1) * K) + 2 * t;
-    const uint4* hB = reinterpret_cast<const uint4*>(h + (size_t)min(mB, p.M - 1) * K) + 2 * t;
-    const uint4* Ar = reinterpret_cast<const uint4*>(A + (size_t)min(j0 + g, r - 1) * K) + 2 * t;
-    const bool okA = mA < p.M, okB = mB < p.M, okJ = j0 + g < r;
+    const uint4* hA = reinterpret_cast<const uint4*>(p.h_in + (size_t)min(mA, p.M - 1) * K) + 2 * t;
+    const uint4* hB = reinterpret_cast<const uint4*>(p.h_in + (size_t)min(mB, p.M - 1) * K) + 2 * t;
+    const bool okA = mA < m_end, okB = mB < m_end, okJ = j0 + g < r;
     auto block = [&](const uint4 (&va)[2], const uint4 (&vb)[2], const uint4 (&vw)[2]) {
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
@@ -131,7 +160,7 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_mma_kernel(const
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const int o = (b + u) * 8 + q;
-          va[u][q] = okA ? __ldg(hA + o) : zero; vb[u][q] = okB ? __ldg(hB + o) : zero; vw[u][q] = okJ ? __ldg(Ar + o) : zero;
+          va[u][q] = okA ? __ldcg(hA + o) : zero; vb[u][q] = okB ? __ldcg(hB + o) : zero; vw[u][q] = okJ ? __ldg(Ar + o) : zero;
         }
       block(va[0], vb[0], vw[0]);
       block(va[1], vb[1], vw[1]);
@@ -141,28 +170,41 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_mma_kernel(const
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         const int o = b * 8 + q;
-        va[q] = okA ? __ldg(hA + o) : zero; vb[q] = okB ? __ldg(hB + o) : zero; vw[q] = okJ ? __ldg(Ar + o) : zero;
+        va[q] = okA ? __ldcg(hA + o) : zero; vb[q] = okB ? __ldcg(hB + o) : zero; vw[q] = okJ ? __ldg(Ar + o) : zero;
       }
       block(va, vb, vw);
     }
   }
-#pragma unroll
-  for (int e = 0; e < 4; ++e) red[warp][lane][e] = acc[e];
+  *reinterpret_cast<float4*>(red[warp][lane]) = make_float4(acc[0], acc[1], acc[2], acc[3]);
   __syncthreads();
-  if (warp == 0) {
-    const float s = (A != nullptr) ? p.lora.scale[a] : 0.f;
-    float tot[4] = {0.f, 0.f, 0.f, 0.f};
+  if (warp < 4) {
+    // accumulator element e = warp of every lane's fragment: [0],[1] = row mA, rank j0 + 2t, +1;  [2],[3] = row mB
+    const int e = warp;
+    float tot = 0.f;
 #pragma unroll
-    for (int w = 0; w < SHRINK_MMA_WARPS; ++w)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) tot[e] += red[w][lane][e];
-    // fragment: [0],[1] = row mA, rank j0 + 2t, +1;  [2],[3] = row mB
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int m = (e < 2) ? mA : mB, j = j0 + 2 * t + (e & 1);
-      if (m < p.M && j < r) p.lora.T[((size_t)m * p.lora.nseg + seg) * r + j] = s * tot[e];
+    for (int w = 0; w < SHRINK_MMA_WARPS; ++w) tot += red[w][lane][e];
+    const int m = (e < 2) ? mA : mB, j = j0 + 2 * t + (e & 1);
+    if (m < m_end && j < r) {
+      if (p.lora.text != nullptr) text_store(p.lora, m, seg, stream * r + j, s * tot);
+      else p.lora.T[((size_t)m * p.lora.nseg + seg) * r + j] = s * tot;
     }
+  } else if (p.lora.text != nullptr && j0 == 0) {
+    for (int m = m0 + warp - 4; m < min(m0 + 16, m_end); m += 12) text_clear(p.lora, m, seg, stream * r, stream * r + r, lane, 32);
   }
+}
+
+cudaError_t launch_shrink_rows(const ShrinkArgs& a, cudaStream_t st) {
+  const int T = a.lora.rows_per_stream, tps = (T + 15) / 16;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)((a.M + T - 1) / T * tps), (unsigned)(a.lora.nseg * ((a.lora.rank + 7) / 8)));
+  cfg.blockDim = dim3(SHRINK_MMA_WARPS * 32);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = a.pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, shrink_mma_kernel, a, tps);
 }
 
 cudaError_t init_shrink() {
@@ -173,8 +215,8 @@ cudaError_t launch_shrink(const ShrinkArgs& a, cudaStream_t st) {
   // Runs of 16 rows share an adapter: the norm (if any) as its own pass, the shrink on mma.sync from the fp16 rows.
   // With a norm this costs a second launch, which pays only when the shrink is large.
   const bool big = (long long)a.lora.rank * a.lora.nseg * a.K >= 150000;
-  if (a.lora.adapter_idx != nullptr && a.lora.rows_per_stream % 16 == 0 && a.M >= 32 && (a.x_f32 == nullptr || big)) {
-    const __half* h = a.h_in;
+  if (a.lora.adapter_idx != nullptr && !a.lora.slot_is_adapter && a.lora.rows_per_stream % 16 == 0 && a.M >= 32 && (a.x_f32 == nullptr || big)) {
+    ShrinkArgs r = a;
     if (a.x_f32 != nullptr) {
       ShrinkArgs n = a;
       n.lora.adapter_idx = nullptr;
@@ -182,11 +224,9 @@ cudaError_t launch_shrink(const ShrinkArgs& a, cudaStream_t st) {
       norm_shrink_kernel<<<grid, SHRINK_THREADS, (size_t)a.K * sizeof(__half), st>>>(n, 1);
       const cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
-      h = a.h_out;
+      r.h_in = a.h_out;
     }
-    dim3 grid((a.M + 15) / 16, a.lora.nseg * ((a.lora.rank + 7) / 8));
-    shrink_mma_kernel<<<grid, SHRINK_MMA_WARPS * 32, 0, st>>>(a, h);
-    return cudaGetLastError();
+    return launch_shrink_rows(r, st);
   }
   int jchunks = 1, gy = 1;
   if (a.lora.adapter_idx != nullptr) {

@@ -75,7 +75,10 @@ struct mlora_ctx {
   size_t prefix_layer_stride = 0, prefix_head_stride = 0;
   size_t own_layer_stride = 0, own_stream_stride = 0, own_head_stride = 0;
   // scratch
+  __half* text = nullptr;            // adapters' T of a pass as the tcgen05 projection reads it (LoraArgs::text)
   float *X = nullptr, *qkv = nullptr, *logits = nullptr, *T = nullptr, *partial = nullptr, *att_ws = nullptr;
+  __half* h_ffn = nullptr;           // passes of many rows: residual rows times the gain of the norm ahead of gate/up (h: ahead of q,k,v)
+  unsigned long long* row_ssq = nullptr;   // ... and the residual rows' sums of squares, [2 L + 1][Mmax], fixed point
   __half *h = nullptr, *attn16 = nullptr, *act16 = nullptr;
   size_t partial_floats = 0, att_ws_floats = 0;
   unsigned* counters = nullptr;
@@ -199,6 +202,7 @@ struct PassIO {
   bool fused_done = false;
   bool last_row_logits = false;            // prefill: only the pass's last row goes through the final norm and lm_head
                                            // (io.logits receives that one row)
+  bool tc = false;                         // the projections run on the tcgen05 path
   bool rows_resolved = false;              // the rows' adapter pointers were looked up earlier in this call (same adapter_idx)
   AttnArgs plan;                           // chunking, filled by plan_pass
 };
@@ -219,6 +223,7 @@ LoraArgs lora_args(mlora_ctx* c, const PassIO& io, int l, int nseg, const int* p
   la.nseg = nseg;
   for (int i = 0; i < nseg; ++i) { la.seg[i].proj_index = l * 7 + projs[i]; la.seg[i].n = widths[i]; }
   la.T = c->T;
+  if (io.tc) { la.text = c->text; la.k_slots = io.n; la.ke = (io.n * la.rank + 63) & ~63; }
   return la;
 }
 
@@ -369,12 +374,6 @@ int forward_chain(mlora_ctx* c, const PassIO& io) {
   return MLORA_OK;
 }
 
-// one projection of a pass with more than 8 rows: tensor-core path from 32 rows up, split-K mma.sync below
-cudaError_t launch_projection(mlora_ctx* c, const GemmArgs& g, cudaStream_t st) {
-  if (!c->dbg_no_tc && gemm_tc_eligible(g)) return launch_gemm_tc(g, c->sm_count, c->status, st);
-  return launch_gemm(g, st);
-}
-
 // the launch sequence of one pass over M = n*T rows (Sec. 3.1 decoder, Eq. 1-4 projections)
 // decode-sized pass as one small kernel per projection group (decode_lean.cu), attention between them
 bool lean_eligible(const mlora_ctx* c, const PassIO& io) {
@@ -448,9 +447,91 @@ int forward_lean(mlora_ctx* c, PassIO& io) {
   return MLORA_OK;
 }
 
+// A pass of TC_MIN_ROWS rows and more: four tcgen05 projections and the attention a layer, the adapters' shrink between
+// them.  No normalisation pass: whatever writes the residual also writes its fp16 copy times the gain of the norm that
+// follows and the rows' sums of squares, and the projection behind scales its finished sums (the shrink of unnormalised
+// rows gives a T that the same factor completes).
+int forward_rows(mlora_ctx* c, PassIO& io) {
+  const mlora_model_desc& d = c->d;
+  cudaStream_t st = c->stream;
+  const int M = io.n * io.T, dm = d.d_model, F = d.d_ffn;
+  const size_t ld_ssq = (size_t)c->Mmax;
+  io.tc = true;
+  CK(cudaMemsetAsync(c->row_ssq, 0, (size_t)(2 * c->L + 1) * ld_ssq * sizeof(unsigned long long), st));
+  CK(run(c, MLORA_PROF_MISC, [&] { return launch_tree_prep(io.parent, io.n, io.T, c->anc, c->depth, c->status, st); }));
+  CK(run(c, MLORA_PROF_MISC, [&] {
+    return launch_embed(io.tokens, (const __half*)d.embed, io.hidden_in, c->X, M, dm, d.vocab, c->status, st, c->forecast,
+                        c->n_forecast, c->rms_attn[0], c->h, c->row_ssq);
+  }));
+  // one projection group: the shrink of its input rows (if it has adapters), then the projection
+  auto project = [&](GemmArgs& g, const PackedWeight& w, const __half* in, int l, int nseg, const int* projs, const int* widths) -> int {
+    g.w = w.data; g.K = w.K; g.N = w.N; g.G = w.G; g.h = in; g.M = M; g.eps = d.rms_eps;
+    if (nseg > 0) g.lora = lora_args(c, io, l, nseg, projs, widths);
+    if (g.lora.adapter_idx != nullptr) {
+      ShrinkArgs s{};
+      s.h_in = in; s.M = M; s.K = w.K; s.lora = g.lora; s.pdl = 1;
+      CK(run(c, MLORA_PROF_SHRINK, [&] { return launch_shrink_rows(s, st); }));
+      g.late_wait = 1;
+    }
+    CK(run(c, MLORA_PROF_GEMM, [&] { return launch_gemm_tc(g, c->sm_count, c->status, st); }));
+    return MLORA_OK;
+  };
+  int rc;
+  for (int l = 0; l < c->L; ++l) {
+    {
+      const int projs[3] = {0, 1, 2}, widths[3] = {c->Nq, c->Nkv, c->Nkv};
+      GemmArgs g{};
+      g.mode = MODE_QKV; g.epi = EPI_F32; g.seg_n0 = c->Nq; g.seg_n1 = c->Nkv; g.out_f32 = c->qkv; g.ldo = c->Nqkv;
+      g.ssq_in = c->row_ssq + (size_t)(2 * l) * ld_ssq;
+      if ((rc = project(g, c->w_qkv[l], c->h, l, 3, projs, widths)) != MLORA_OK) return rc;
+    }
+    if ((rc = launch_attention_block(c, io, l)) != MLORA_OK) return rc;
+    {
+      const int projs[1] = {3}, widths[1] = {dm};
+      GemmArgs g{};
+      g.mode = MODE_PLAIN; g.epi = EPI_RESID; g.resid = c->X;
+      g.xg_out = c->h_ffn; g.gain_next = c->rms_ffn[l]; g.ssq_out = c->row_ssq + (size_t)(2 * l + 1) * ld_ssq;
+      if ((rc = project(g, c->w_o[l], c->attn16, l, 1, projs, widths)) != MLORA_OK) return rc;
+    }
+    {
+      const int projs[2] = {4, 5}, widths[2] = {F, F};
+      GemmArgs g{};
+      g.mode = MODE_GATEUP; g.epi = EPI_SWIGLU; g.out_f16 = c->act16;
+      g.ssq_in = c->row_ssq + (size_t)(2 * l + 1) * ld_ssq;
+      if ((rc = project(g, c->w_gateup[l], c->h_ffn, l, 2, projs, widths)) != MLORA_OK) return rc;
+    }
+    {
+      const int projs[1] = {6}, widths[1] = {dm};
+      GemmArgs g{};
+      g.mode = MODE_PLAIN; g.epi = EPI_RESID; g.resid = c->X;
+      const __half* gain = l + 1 < c->L ? c->rms_attn[l + 1] : (const __half*)d.rms_final;
+      if (gain != nullptr) { g.xg_out = c->h; g.gain_next = gain; g.ssq_out = c->row_ssq + (size_t)(2 * l + 2) * ld_ssq; }
+      if ((rc = project(g, c->w_down[l], c->act16, l, 1, projs, widths)) != MLORA_OK) return rc;
+    }
+  }
+  if (d.vocab > 0 && io.logits != nullptr) {
+    const unsigned long long* ssq = c->row_ssq + (size_t)(2 * c->L) * ld_ssq;
+    if (io.last_row_logits) {
+      // one row: the decode path's lm_head
+      LeanArgs a{};
+      a.M = 1; a.eps = d.rms_eps; a.logits = io.logits; a.ssq = const_cast<unsigned long long*>(ssq) + (M - 1);
+      StepPhase ph{};
+      ph.kind = SK_GEMM; ph.w = c->w_lm.data; ph.K = dm; ph.N = d.vocab; ph.G = c->w_lm.G; ph.mode = MODE_PLAIN; ph.epi = EPI_F32;
+      ph.in16 = c->h + (size_t)(M - 1) * dm; ph.norm_in = 0; ph.ldo = d.vocab; ph.ssq_out = -1;
+      CK(run(c, MLORA_PROF_GEMM, [&] { return launch_lean_gemm(a, ph, st); }));
+    } else {
+      GemmArgs g{};
+      g.mode = MODE_PLAIN; g.epi = EPI_F32; g.out_f32 = io.logits; g.ldo = d.vocab; g.ssq_in = ssq;
+      if ((rc = project(g, c->w_lm, c->h, 0, 0, nullptr, nullptr)) != MLORA_OK) return rc;
+    }
+  }
+  return MLORA_OK;
+}
+
 int forward(mlora_ctx* c, PassIO& io) {
   if (lean_eligible(c, io)) return forward_lean(c, io);
   if (chain_eligible(c, io)) return forward_chain(c, io);
+  if (!c->dbg_no_tc && io.n * io.T >= TC_MIN_ROWS && tensor_maps_available()) return forward_rows(c, io);
   const mlora_model_desc& d = c->d;
   cudaStream_t st = c->stream;
   const int M = io.n * io.T;
@@ -472,7 +553,7 @@ int forward(mlora_ctx* c, PassIO& io) {
       g.out_f32 = c->qkv; g.ldo = c->Nqkv;
       g.partial = c->partial; g.partial_capacity = c->partial_floats; g.counters = c->counters;
       g.lora = s.lora;
-      CK(run(c, MLORA_PROF_GEMM, [&] { return launch_projection(c, g, st); }));
+      CK(run(c, MLORA_PROF_GEMM, [&] { return launch_gemm(g, st); }));
     }
     {
       int rc = launch_attention_block(c, io, l);
@@ -492,7 +573,7 @@ int forward(mlora_ctx* c, PassIO& io) {
       g.mode = MODE_PLAIN; g.epi = EPI_RESID; g.resid = c->X;
       g.partial = c->partial; g.partial_capacity = c->partial_floats; g.counters = c->counters;
       g.lora = la;
-      CK(run(c, MLORA_PROF_GEMM, [&] { return launch_projection(c, g, st); }));
+      CK(run(c, MLORA_PROF_GEMM, [&] { return launch_gemm(g, st); }));
     }
     // MLP block
     {
@@ -507,7 +588,7 @@ int forward(mlora_ctx* c, PassIO& io) {
       g.mode = MODE_GATEUP; g.epi = EPI_SWIGLU; g.out_f16 = c->act16;
       g.partial = c->partial; g.partial_capacity = c->partial_floats; g.counters = c->counters;
       g.lora = s.lora;
-      CK(run(c, MLORA_PROF_GEMM, [&] { return launch_projection(c, g, st); }));
+      CK(run(c, MLORA_PROF_GEMM, [&] { return launch_gemm(g, st); }));
     }
     {
       const int projs[1] = {6}, widths[1] = {dm};
@@ -523,7 +604,7 @@ int forward(mlora_ctx* c, PassIO& io) {
       g.mode = MODE_PLAIN; g.epi = EPI_RESID; g.resid = c->X;
       g.partial = c->partial; g.partial_capacity = c->partial_floats; g.counters = c->counters;
       g.lora = la;
-      CK(run(c, MLORA_PROF_GEMM, [&] { return launch_projection(c, g, st); }));
+      CK(run(c, MLORA_PROF_GEMM, [&] { return launch_gemm(g, st); }));
     }
   }
   if (d.vocab > 0 && io.logits != nullptr) {
@@ -536,7 +617,7 @@ int forward(mlora_ctx* c, PassIO& io) {
     g.w = w.data; g.K = w.K; g.N = w.N; g.G = w.G; g.h = c->h; g.M = Ml;
     g.mode = MODE_PLAIN; g.epi = EPI_F32; g.out_f32 = io.logits; g.ldo = d.vocab;
     g.partial = c->partial; g.partial_capacity = c->partial_floats; g.counters = c->counters;
-    CK(run(c, MLORA_PROF_GEMM, [&] { return launch_projection(c, g, st); }));
+    CK(run(c, MLORA_PROF_GEMM, [&] { return launch_gemm(g, st); }));
   }
   return MLORA_OK;
 }
@@ -764,10 +845,14 @@ int mlora_create(const mlora_model_desc* desc, mlora_ctx** out) {
   CKC(cudaMalloc(&c->X, Mm * dm * sizeof(float)));
   CKC(cudaMalloc(&c->qkv, Mm * c->Nqkv * sizeof(float)));
   CKC(cudaMalloc(&c->h, Mm * maxK * sizeof(__half)));
+  CKC(cudaMalloc(&c->h_ffn, Mm * dm * sizeof(__half)));
+  CKC(cudaMalloc(&c->row_ssq, (size_t)(2 * L + 1) * Mm * sizeof(unsigned long long)));
   CKC(cudaMalloc(&c->attn16, Mm * Nq * sizeof(__half)));
   CKC(cudaMalloc(&c->act16, Mm * F * sizeof(__half)));
   if (d.vocab > 0) CKC(cudaMalloc(&c->logits, (size_t)d.max_streams * d.max_tree * d.vocab * sizeof(float)));   // (prefill: one row)
   CKC(cudaMalloc(&c->T, Mm * 3 * (d.lora_rank > 0 ? d.lora_rank : 1) * sizeof(float)));
+  if (d.lora_rank > 0)
+    CKC(cudaMalloc(&c->text, (size_t)d.max_streams * d.max_tree * 6 * (((size_t)d.max_streams * d.lora_rank + 63) / 64 * 64) * sizeof(__half)));
   c->partial_floats = (size_t)16 << 20;               // 64 MB of split-K scratch
   CKC(cudaMalloc(&c->partial, c->partial_floats * sizeof(float)));
   CKC(cudaMalloc(&c->counters, 4096 * sizeof(unsigned)));
@@ -1013,8 +1098,8 @@ int mlora_destroy(mlora_ctx* c) {
   for (auto& w : c->w_gateup) free_packed(w);
   for (auto& w : c->w_down) free_packed(w);
   free_packed(c->w_lm);
-  void* dev_ptrs[] = {c->prefix_k, c->prefix_v, c->own_k, c->own_v, c->X, c->qkv, c->logits, c->T, c->partial, c->att_ws,
-                      c->h, c->attn16, c->act16, c->counters, c->anc, c->depth, c->argmax, c->suffix_len,
+  void* dev_ptrs[] = {c->prefix_k, c->prefix_v, c->own_k, c->own_v, c->X, c->qkv, c->logits, c->T, c->text, c->partial, c->att_ws,
+                      c->h, c->h_ffn, c->row_ssq, c->attn16, c->act16, c->counters, c->anc, c->depth, c->argmax, c->suffix_len,
                       c->zero_len, c->chain_parent, c->root_parent, c->status, c->cs_table, (void*)c->tabA,
                       (void*)c->tabB, c->ad_scale, c->phases, c->chain_sync, c->host_io, c->step_phases, c->xg_attn, c->xg_ffn,
                       c->step_tacc, c->step_amax, c->step_trace, c->tmapA, c->tmapB, c->gen_tokens, c->draft_cand,
@@ -1657,6 +1742,12 @@ int mlora_linear(mlora_weight* w, const void* x, int32_t M, const int32_t* row_a
     la.tab_stride = 1; la.n_slots = n_adapters; la.rank = rank; la.nseg = 1;
     la.seg[0].proj_index = 0; la.seg[0].n = w->w.N;
     la.T = (float*)(ws + LIN_COUNTER_BYTES);
+    // the tcgen05 kernel takes T as a matrix over all adapters (in the room of the split-K partial sums, which it does
+    // not need), where that fits
+    const long long ke = ((long long)n_adapters * rank + 63) / 64 * 64;
+    if (M >= TC_MIN_ROWS && ke <= 4096 && (size_t)M * 2 * ke * sizeof(__half) + 256 <= workspace_bytes - fixed) {
+      la.text = (__half*)(ws + (fixed + 255) / 256 * 256); la.ke = (int)ke; la.k_slots = n_adapters; la.slot_is_adapter = 1;
+    }
     ShrinkArgs s{};
     s.h_in = (const __half*)x; s.M = M; s.K = w->w.K; s.lora = la;
     CK(launch_shrink(s, w->stream));
@@ -1667,7 +1758,8 @@ int mlora_linear(mlora_weight* w, const void* x, int32_t M, const int32_t* row_a
   g.partial = (float*)(ws + fixed); g.partial_capacity = (workspace_bytes - fixed) / sizeof(float);
   g.counters = (unsigned*)(ws + LIN_SYNC_BYTES);
   g.lora = la;
-  if (gemm_tc_eligible(g)) CK(launch_gemm_tc(g, w->sm_count, (int*)(ws + 32), w->stream));
+  g.late_wait = lora;                                      // (x is there already: the shrink kernel adds only T)
+  if (gemm_tc_eligible(g) && (!lora || la.text != nullptr)) CK(launch_gemm_tc(g, w->sm_count, (int*)(ws + 32), w->stream));
   else CK(launch_gemm(g, w->stream));
   return MLORA_OK;
 }

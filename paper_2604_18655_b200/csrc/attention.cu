@@ -1145,6 +1145,7 @@ static bool attn_stream_shape(const AttnArgs& a, int sm_count) {
 
 void attn_plan(AttnArgs& a, int sm_count) {
   a.stream_mode = 0;
+  a.tc_nq = 0;
   if (attn_stream_shape(a, sm_count)) {
     const int NT = (a.P + STR_KEYS - 1) / STR_KEYS;
     int chunks = sm_count / a.Hkv;
@@ -1271,6 +1272,7 @@ static cudaError_t launch_attention_stream(const AttnArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_attention(const AttnArgs& a, cudaStream_t st) {
+  if (a.tc_nq) return launch_attention_tc(a, st);
   if (a.stream_mode) return launch_attention_stream(a, st);
   if (attn_single_pass(a)) {
     const float scale_log2 = 1.4426950408889634f / sqrtf((float)a.hd);
@@ -1299,7 +1301,7 @@ cudaError_t launch_attention(const AttnArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_attention_merge(const AttnArgs& a, cudaStream_t st) {
-  if (attn_single_pass(a)) return cudaSuccess;             // nothing to merge
+  if (a.tc_nq ? a.causal : attn_single_pass(a)) return cudaSuccess;   // nothing to merge
   const int warps = a.n * a.T * a.Hq;
   attn_merge_kernel<<<(warps + 3) / 4, 128, 0, st>>>(a);
   return cudaGetLastError();

@@ -77,7 +77,7 @@ constexpr int GEMM_PF = 8;                     // weight tiles in flight per lan
 constexpr int GEMM_MAX_MT = 16;                // m-tiles of 8 rows per CTA (128 rows)
 
 enum GemmMode { MODE_PLAIN = 0, MODE_QKV = 1, MODE_GATEUP = 2 };
-enum GemmEpi { EPI_F32 = 0, EPI_RESID = 1, EPI_SWIGLU = 2 };
+enum GemmEpi { EPI_F32 = 0, EPI_RESID = 1, EPI_SWIGLU = 2, EPI_QKV = 3 /* tcgen05 path: rotated q, K/V into the cache */ };
 
 struct LoraSeg {
   int proj_index;   // index into the adapter pointer tables (layer*7 + proj), or the plain table index 0
@@ -123,6 +123,13 @@ struct GemmArgs {
   unsigned long long* ssq_out;    // EPI_RESID: sums of squares of the new residual rows are added here (nullptr: not wanted)
   __half* xg_out;                 // EPI_RESID: new residual x gain_next as fp16 (nullptr: not wanted)
   const __half* gain_next;
+  // EPI_QKV: row m = (stream m / T, node m % T) sits at position pos_base + suffix_len[stream] + depth[m]; its K/V go to row
+  // suffix_len[stream] + node of the stream's segment
+  __half *q_out, *k_out, *v_out;
+  const float2* cs_table;
+  const int32_t *suffix_len, *depth;
+  size_t kv_stream_stride, kv_head_stride;
+  int hd, pos_base, rows_per_stream;
 };
 
 struct ShrinkArgs {
@@ -155,6 +162,7 @@ struct AttnArgs {
   const float2* cs_table;         // cos/sin of pos * theta^(-2i/hd): [pos][hd/2]
   int pos_base;                   // position of a row = pos_base + suffix_len[s] + depth[row]
   const int32_t* depth;           // dev [rows]
+  int tc_nq;                      // set by attn_plan_tc: the tcgen05 kernel, with so many row blocks a CTA (0: another kernel)
   int stream_mode;                // set by attn_plan: the streaming kernel for one row per stream over a long prefix
   int* status;                    // dev status word for bounded waits that run out (may be null)
   // single-kernel decode attention only: partial LoRA shrink of the o projection over the (kv head, stream)'s output
@@ -334,6 +342,9 @@ cudaError_t launch_draft(const float* logits, int V, int n, int R, int m, int wm
 cudaError_t launch_tree_prep(const int32_t* parent, int n, int T, unsigned long long* anc, int32_t* depth,
                              int* status, cudaStream_t st);
 void attn_plan(AttnArgs& a, int sm_count);
+void attn_plan_tc(AttnArgs& a, int sm_count);
+cudaError_t init_attention_tc();
+cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t st);
 size_t attn_workspace_floats(const AttnArgs& a);
 bool attn_decode_o_slice_fits(int hd, int g_heads, int rank);
 bool attn_single_pass(const AttnArgs& a);          // one kernel does the whole softmax: no merge launch follows

@@ -77,6 +77,7 @@ struct mlora_ctx {
   // scratch
   __half* text = nullptr;            // adapters' T of a pass as the tcgen05 projection reads it (LoraArgs::text)
   float *X = nullptr, *qkv = nullptr, *logits = nullptr, *T = nullptr, *partial = nullptr, *att_ws = nullptr;
+  __half* q16 = nullptr;             // passes of many rows: rotated q, fp16 [Mmax][Nq]
   __half* h_ffn = nullptr;           // passes of many rows: residual rows times the gain of the norm ahead of gate/up (h: ahead of q,k,v)
   unsigned long long* row_ssq = nullptr;   // ... and the residual rows' sums of squares, [2 L + 1][Mmax], fixed point
   __half *h = nullptr, *attn16 = nullptr, *act16 = nullptr;
@@ -233,7 +234,10 @@ void plan_pass(mlora_ctx* c, PassIO& io) {
   a.P = io.pos_base;
   a.n = io.n; a.T = io.T; a.Hq = c->d.n_q_heads; a.Hkv = c->d.n_kv_heads; a.hd = c->d.head_dim;
   a.suffix_bound = (io.suffix_bound + 63) / 64 * 64;   // coarse, so the launch shape changes rarely
-  attn_plan(a, c->sm_count);
+  a.causal = io.prefill ? 1 : 0;
+  io.tc = !c->dbg_no_tc && io.n * io.T >= TC_MIN_ROWS && tensor_maps_available();
+  if (io.tc) { attn_plan_tc(a, c->sm_count); a.suffix_bound = 0; }     // (its launch shape does not depend on the bound)
+  else attn_plan(a, c->sm_count);
 }
 
 // where a pass writes the K/V of its rows
@@ -256,8 +260,11 @@ int launch_attention_block(mlora_ctx* c, const PassIO& io, int l) {
   size_t sstride, hstride;
   kv_destination(c, io, l, kd, vd, sstride, hstride);
   AttnArgs a = io.plan;
-  // q and the new k rows are rotated on load, the new K/V rows appended by the attention kernel itself
-  a.qkv_f32 = c->qkv; a.cs_table = c->cs_table; a.pos_base = io.pos_base; a.depth = c->depth;
+  // q and the new k rows are rotated on load, the new K/V rows appended by the attention kernel itself -- or by the
+  // epilogue of the tcgen05 q,k,v projection
+  if (io.tc) { a.q = c->q16; a.pdl = 1; }
+  else a.qkv_f32 = c->qkv;
+  a.cs_table = c->cs_table; a.pos_base = io.pos_base; a.depth = c->depth;
   a.prefix_k = c->prefix_k + (size_t)l * c->prefix_layer_stride;
   a.prefix_v = c->prefix_v + (size_t)l * c->prefix_layer_stride;
   a.prefix_head_stride = c->prefix_head_stride;
@@ -268,7 +275,7 @@ int launch_attention_block(mlora_ctx* c, const PassIO& io, int l) {
   a.part_o = c->att_ws;
   a.part_ml = c->att_ws + (attn_workspace_floats(a) / (a.hd + 2)) * a.hd;
   CK(run(c, MLORA_PROF_ATTN, [&] { return launch_attention(a, st); }));
-  if (!attn_single_pass(a)) CK(run(c, MLORA_PROF_ATTN_MERGE, [&] { return launch_attention_merge(a, st); }));
+  if (a.tc_nq ? !a.causal : !attn_single_pass(a)) CK(run(c, MLORA_PROF_ATTN_MERGE, [&] { return launch_attention_merge(a, st); }));
   return MLORA_OK;
 }
 
@@ -456,7 +463,6 @@ int forward_rows(mlora_ctx* c, PassIO& io) {
   cudaStream_t st = c->stream;
   const int M = io.n * io.T, dm = d.d_model, F = d.d_ffn;
   const size_t ld_ssq = (size_t)c->Mmax;
-  io.tc = true;
   CK(cudaMemsetAsync(c->row_ssq, 0, (size_t)(2 * c->L + 1) * ld_ssq * sizeof(unsigned long long), st));
   CK(run(c, MLORA_PROF_MISC, [&] { return launch_tree_prep(io.parent, io.n, io.T, c->anc, c->depth, c->status, st); }));
   CK(run(c, MLORA_PROF_MISC, [&] {
@@ -481,7 +487,10 @@ int forward_rows(mlora_ctx* c, PassIO& io) {
     {
       const int projs[3] = {0, 1, 2}, widths[3] = {c->Nq, c->Nkv, c->Nkv};
       GemmArgs g{};
-      g.mode = MODE_QKV; g.epi = EPI_F32; g.seg_n0 = c->Nq; g.seg_n1 = c->Nkv; g.out_f32 = c->qkv; g.ldo = c->Nqkv;
+      g.mode = MODE_QKV; g.epi = EPI_QKV; g.seg_n0 = c->Nq; g.seg_n1 = c->Nkv; g.q_out = c->q16;
+      kv_destination(c, io, l, g.k_out, g.v_out, g.kv_stream_stride, g.kv_head_stride);
+      g.cs_table = c->cs_table; g.suffix_len = io.suffix_len; g.depth = c->depth; g.hd = d.head_dim; g.pos_base = io.pos_base;
+      g.rows_per_stream = io.T;
       g.ssq_in = c->row_ssq + (size_t)(2 * l) * ld_ssq;
       if ((rc = project(g, c->w_qkv[l], c->h, l, 3, projs, widths)) != MLORA_OK) return rc;
     }
@@ -531,7 +540,7 @@ int forward_rows(mlora_ctx* c, PassIO& io) {
 int forward(mlora_ctx* c, PassIO& io) {
   if (lean_eligible(c, io)) return forward_lean(c, io);
   if (chain_eligible(c, io)) return forward_chain(c, io);
-  if (!c->dbg_no_tc && io.n * io.T >= TC_MIN_ROWS && tensor_maps_available()) return forward_rows(c, io);
+  if (io.tc) return forward_rows(c, io);
   const mlora_model_desc& d = c->d;
   cudaStream_t st = c->stream;
   const int M = io.n * io.T;
@@ -695,6 +704,7 @@ int init_kernels() {
   CK(init_chain());
   CK(init_step());
   CK(init_gemm_tc());
+  CK(init_attention_tc());
   done = true;
   return MLORA_OK;
 }
@@ -847,6 +857,7 @@ int mlora_create(const mlora_model_desc* desc, mlora_ctx** out) {
   CKC(cudaMalloc(&c->h, Mm * maxK * sizeof(__half)));
   CKC(cudaMalloc(&c->h_ffn, Mm * dm * sizeof(__half)));
   CKC(cudaMalloc(&c->row_ssq, (size_t)(2 * L + 1) * Mm * sizeof(unsigned long long)));
+  CKC(cudaMalloc(&c->q16, Mm * Nq * sizeof(__half)));
   CKC(cudaMalloc(&c->attn16, Mm * Nq * sizeof(__half)));
   CKC(cudaMalloc(&c->act16, Mm * F * sizeof(__half)));
   if (d.vocab > 0) CKC(cudaMalloc(&c->logits, (size_t)d.max_streams * d.max_tree * d.vocab * sizeof(float)));   // (prefill: one row)
@@ -1099,7 +1110,7 @@ int mlora_destroy(mlora_ctx* c) {
   for (auto& w : c->w_down) free_packed(w);
   free_packed(c->w_lm);
   void* dev_ptrs[] = {c->prefix_k, c->prefix_v, c->own_k, c->own_v, c->X, c->qkv, c->logits, c->T, c->text, c->partial, c->att_ws,
-                      c->h, c->h_ffn, c->row_ssq, c->attn16, c->act16, c->counters, c->anc, c->depth, c->argmax, c->suffix_len,
+                      c->h, c->q16, c->h_ffn, c->row_ssq, c->attn16, c->act16, c->counters, c->anc, c->depth, c->argmax, c->suffix_len,
                       c->zero_len, c->chain_parent, c->root_parent, c->status, c->cs_table, (void*)c->tabA,
                       (void*)c->tabB, c->ad_scale, c->phases, c->chain_sync, c->host_io, c->step_phases, c->xg_attn, c->xg_ffn,
                       c->step_tacc, c->step_amax, c->step_trace, c->tmapA, c->tmapB, c->gen_tokens, c->draft_cand,
@@ -1850,6 +1861,8 @@ static void attn_fill(AttnArgs& a, int n, int T, int Hq, int Hkv, int hd, int P,
   a.P = P; a.n = n; a.T = T; a.Hq = Hq; a.Hkv = Hkv; a.hd = hd;
   a.suffix_bound = suffix_bound;
   attn_plan(a, 148);
+  // (one row per stream: the decode kernels, where their shapes fit)
+  if (!attn_single_pass(a) && !a.stream_mode && Hq / Hkv <= 128 && tensor_maps_available()) attn_plan_tc(a, 148);
 }
 
 size_t mlora_attention_workspace_bytes(int32_t n, int32_t T, int32_t Hq, int32_t Hkv, int32_t hd, int32_t P,

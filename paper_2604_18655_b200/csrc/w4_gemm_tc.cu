@@ -24,15 +24,13 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
-#include "../../include/mlora.h"
-#include "common.cuh"
+#include "tc.cuh"
 
 namespace mlora {
 
 constexpr int TC_BM = 128;                 // output features per CTA (UMMA M)
 constexpr int TC_BK = 64;                  // input features per step: one 128-byte swizzle row of fp16
 constexpr int TC_WSLOT = 1024 + 64;        // ring slot of a warp: two tiles of nibbles, two scale entries
-constexpr long long TC_WAIT_CYCLES = 4000000000ll;
 constexpr float TC_FIX = 4294967296.f, TC_UNFIX = 1.f / 4294967296.f;   // fixed point of the rows' sums of squares
 
 // GR = groups of four dequantising warps: two where two CTAs share an SM (up to 128 rows), four where one has it alone.
@@ -46,74 +44,6 @@ template <int NR> struct TcCfg {
   static constexpr int THREADS = GR * 128 + 64;       // + one warp for the activation copies, one for the MMAs
   static constexpr size_t SMEM = (size_t)NB * NR * TC_BK * 2 + (size_t)WD * GR * 4 * TC_WSLOT + 1024;
 };
-
-__device__ __forceinline__ uint32_t tc_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ bool tc_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-// the same without waiting at all (try_wait may suspend the warp for some microseconds)
-__device__ __forceinline__ bool tc_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-// (the clock is read on the slow path only: a wait for a phase that is over already is on the MMA thread's critical path)
-static __device__ __noinline__ bool tc_wait_slow(uint32_t bar, uint32_t parity, int* status) {
-  const long long t0 = clock64();
-  for (int it = 0;; ++it) {
-    if (tc_try(bar, parity)) return true;
-    if ((it & 255) == 255 && clock64() - t0 > TC_WAIT_CYCLES) {
-      if (status != nullptr) atomicCAS(status, 0, MLORA_ERR_TIMEOUT);
-      return false;
-    }
-  }
-}
-__device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity, int* status) {
-  for (int it = 0; it < 8; ++it)
-    if (tc_try(bar, parity)) return true;
-  return tc_wait_slow(bar, parity, status);
-}
-__device__ __forceinline__ uint32_t tc_elect() {
-  uint32_t pred;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));
-  return pred;
-}
-// shared-memory matrix descriptor: K-major, 128B swizzle, 1024 bytes between 8-row groups (descriptor version 1)
-__device__ __forceinline__ uint64_t tc_desc(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
-         ((uint64_t)2 << 61);
-}
-// 16 lanes x 32 columns of tensor memory from the registers of a warp, in the fragment layout of an m16n8 accumulator:
-// registers 4j..4j+3 of lane (g, t) = (row g: columns 8j + 2t, + 1), (row g + 8: the same columns)
-__device__ __forceinline__ void tc_st_16x256b_x4(uint32_t addr, const uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-      ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
-}
-// 32 lanes x 16 columns: lane l of the warp = tensor-memory lane l, register j = column j
-__device__ __forceinline__ void tc_st_32x32b_x16(uint32_t addr, const uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-      ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
-}
-__device__ __forceinline__ void tc_ld_32x32b_x16(uint32_t addr, float (&f)[16]) {
-  uint32_t v[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
-        "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]) : "r"(addr) : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
-}
 
 template <int NR, int S>
 __global__ void __launch_bounds__(TcCfg<NR>::THREADS, TcCfg<NR>::OCC)
@@ -131,6 +61,8 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
   __shared__ uint32_t tmem_base_s;
   __shared__ float s_inv[CW];
   __shared__ unsigned long long s_ssq[CW];
+  __shared__ int s_pos[CW];                           // EPI_QKV: the rows' positions ...
+  __shared__ size_t s_dst[CW];                        // ... and their places in the cache
 
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int rank = S > 1 ? (int)blockIdx.x : 0;       // position in the K-splitting cluster
@@ -454,6 +386,11 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
     if (p.ssq_in != nullptr && row0 + tid < p.M)
       inv = rsqrtf(__ll2float_rn((long long)__ldcg(p.ssq_in + row0 + tid)) * TC_UNFIX / (float)p.K + p.eps);
     s_inv[tid] = inv;
+    if (p.epi == EPI_QKV && row0 + tid < p.M) {
+      const int m = row0 + tid, st = m / p.rows_per_stream, cached = p.suffix_len[st];
+      s_pos[tid] = p.pos_base + cached + p.depth[m];
+      s_dst[tid] = (size_t)st * p.kv_stream_stride + (size_t)(cached + m - st * p.rows_per_stream) * p.hd;
+    }
   }
   constexpr int HC = CW / NH;                              // columns of a warp
   constexpr int CH = HC < 16 ? HC : 16;                    // columns handled at a time
@@ -472,7 +409,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
   const bool done = tc_wait(tc_smem_u32(&done_bar), 0u, status);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  __syncthreads();
+  const bool fine = __syncthreads_and(done && alive);      // (one answer for the CTA: there are barriers below)
   float* const xch = reinterpret_cast<float*>(base);       // [S][CW][128] partial sums for the rows this CTA finishes
   if constexpr (S > 1) {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -493,7 +430,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
     }
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
-  if (done && alive && ep_warp) {
+  if (fine && ep_warp) {
 #pragma unroll 1
     for (int c0 = c_lo; c0 < c_lo + HC; c0 += CH) {
       float v[16];
@@ -515,6 +452,32 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
 #pragma unroll
         for (int j = 0; j < CH; ++j)
           if (n_ok && row0 + c0 + j < p.M) p.out_f32[(size_t)(row0 + c0 + j) * p.ldo + n] = v[j];
+      } else if (p.epi == EPI_QKV) {
+        // RoPE on q and k (pairs (i, i + hd/2): the partner feature is two warps (hd 128) or one warp (hd 64) on, its values
+        // come through shared memory), fp16, q to its matrix, k and v into the stream's cache
+        int seg = 0, col = 0;
+        if (n_ok) map_col(p.mode, n, p.seg_n0, p.seg_n1, seg, col);
+        float* const x = reinterpret_cast<float*>(wring) + (size_t)((c0 / CH & 1) * NH + half) * (4 * CH * 32);
+#pragma unroll
+        for (int j = 0; j < CH; ++j) x[(lq * CH + j) * 32 + lane] = v[j];
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
+        const int hh = p.hd >> 1, i = col & (hh - 1), d = col & (p.hd - 1);
+        const bool lo = d < hh;
+        __half* const kv = (seg == 1 ? p.k_out : p.v_out) + (size_t)(col / p.hd) * p.kv_head_stride + d;
+#pragma unroll
+        for (int j = 0; j < CH; ++j) {
+          const int m = row0 + c0 + j;
+          if (n_ok && m < p.M) {
+            float y = v[j];
+            if (seg < 2) {
+              const float2 cs = __ldg(p.cs_table + (size_t)s_pos[c0 + j] * hh + i);
+              const float o = x[((lq ^ (hh >> 5)) * CH + j) * 32 + lane];
+              y = lo ? y * cs.x - o * cs.y : y * cs.x + o * cs.y;
+            }
+            if (seg == 0) p.q_out[(size_t)m * p.seg_n0 + col] = __float2half_rn(y);
+            else kv[s_dst[c0 + j]] = __float2half_rn(y);
+          }
+        }
       } else if (p.epi == EPI_SWIGLU) {
         // lanes 0-15 hold a gate tile's features, lanes 16-31 the up tile's: of every two rows the lower half takes the
         // first, the upper half the second
@@ -577,8 +540,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)C::COLS) : "memory");
 }
 
-// cuTensorMapEncodeTiled through the runtime's driver entry point lookup (the library does not link libcuda)
-static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
     void* sym = nullptr;
     cudaDriverEntryPointQueryResult q;

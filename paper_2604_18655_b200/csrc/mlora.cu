@@ -33,7 +33,7 @@ void free_packed(PackedWeight& w) {
   w.data = nullptr;
 }
 
-constexpr int PREFILL_ROWS = 1024;                 // rows of one causal prefill pass
+constexpr int PREFILL_ROWS = 2048;                 // rows of one causal prefill pass
 constexpr int MAX_FORECAST = 8, MAX_DRAFT_WIDTH = 32;
 
 struct GraphKey {

@@ -57,7 +57,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
   // 1024-byte aligned activation tiles (the swizzle pattern is tied to address bits 7..9), then the warps' weight rings
   unsigned char* const base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
   unsigned char* const wring = base + (size_t)NB * B_BYTES;
-  __shared__ __align__(8) uint64_t b_full[NB], b_empty[NB], a_full[NA], a_empty[NA], done_bar;
+  __shared__ __align__(8) uint64_t b_full[NB], b_empty[NB], a_full[NA], a_empty[NA], done_bar, acc_free;
   __shared__ uint32_t tmem_base_s;
   __shared__ float s_inv[CW];
   __shared__ unsigned long long s_ssq[CW];
@@ -66,26 +66,37 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
 
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int rank = S > 1 ? (int)blockIdx.x : 0;       // position in the K-splitting cluster
-  const int slab = blockIdx.y, m0 = blockIdx.z * NR;
   const WLayout L = make_wlayout(p.K, p.N, p.G);
+  const int slabs = (p.N + TC_BM - 1) / TC_BM, tiles = slabs * ((p.M + NR - 1) / NR);
 
-  // ---- steps: KT k-tiles of the weights, then the expand's blocks of 64 (slot, rank index) pairs, per segment that the
-  // slab touches; a CTA of the cluster takes a contiguous share
-  int seg0 = 0, nE = 0, kb0 = 0, nseg_in = 0;
-  if (p.lora.text != nullptr) {
-    int s_lo = 0, s_hi = p.lora.k_slots - 1;
-    if (!p.lora.slot_is_adapter) { s_lo = m0 / p.lora.rows_per_stream; s_hi = min(s_hi, (min(p.M, m0 + NR) - 1) / p.lora.rows_per_stream); }
-    kb0 = (s_lo * p.lora.rank) & ~63;
-    nE = ((s_hi + 1) * p.lora.rank - kb0 + 63) >> 6;
-    int c, seg1;
-    map_col(p.mode, slab * TC_BM, p.seg_n0, p.seg_n1, seg0, c);
-    map_col(p.mode, min(p.N, slab * TC_BM + TC_BM) - 1, p.seg_n0, p.seg_n1, seg1, c);
-    if (p.mode == MODE_GATEUP) { seg0 = 0; seg1 = 1; }
-    nseg_in = seg1 - seg0 + 1;
-  }
-  const int total = L.KT + nE * nseg_in;
-  const int u0 = (total * rank) / S, u1 = (total * (rank + 1)) / S;
-  const int nsteps = u1 - u0;
+  // ---- a tile = 128 output features x NR rows.  Its steps: KT k-tiles of the weights, then the expand's blocks of 64
+  // (slot, rank index) pairs, per segment that the features touch; a CTA of a cluster takes a contiguous share of them.
+  struct Tile { int slab, m0, seg0, nE, kb0, u0, u1; };
+  auto tile_of = [&](int t) {
+    Tile x;
+    const int mb = t / slabs;
+    x.slab = t - mb * slabs; x.m0 = mb * NR;
+    x.seg0 = 0; x.nE = 0; x.kb0 = 0;
+    int nseg_in = 0;
+    if (p.lora.text != nullptr) {
+      int s_lo = 0, s_hi = p.lora.k_slots - 1;
+      if (!p.lora.slot_is_adapter) { s_lo = x.m0 / p.lora.rows_per_stream; s_hi = min(s_hi, (min(p.M, x.m0 + NR) - 1) / p.lora.rows_per_stream); }
+      x.kb0 = (s_lo * p.lora.rank) & ~63;
+      x.nE = ((s_hi + 1) * p.lora.rank - x.kb0 + 63) >> 6;
+      int c, seg1;
+      map_col(p.mode, x.slab * TC_BM, p.seg_n0, p.seg_n1, x.seg0, c);
+      map_col(p.mode, min(p.N, x.slab * TC_BM + TC_BM) - 1, p.seg_n0, p.seg_n1, seg1, c);
+      if (p.mode == MODE_GATEUP) { x.seg0 = 0; seg1 = 1; }
+      nseg_in = seg1 - x.seg0 + 1;
+    }
+    const int total = L.KT + x.nE * nseg_in;
+    x.u0 = (total * rank) / S; x.u1 = (total * (rank + 1)) / S;
+    return x;
+  };
+  // n-tile (16 features) of the slab that lanes 16 h .. 16 h + 15 of accumulator quarter q hold: consecutive ones; with
+  // RoPE in the epilogue a pair of tiles half a head apart, so that a feature's partner sits 16 lanes on
+  const int rope_gap = p.epi == EPI_QKV ? p.hd >> 5 : 0;   // 2 (hd 64) or 4 (hd 128) tiles
+  auto ntile_of = [&](int q, int h) { return rope_gap == 0 ? 2 * q + h : (rope_gap == 4 ? q + 4 * h : (q >> 1) * 4 + (q & 1) + 2 * h); };
 
   if (tid == 0) {
     for (int s = 0; s < NB; ++s) {
@@ -97,9 +108,9 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_smem_u32(a_empty + s)) : "memory");
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_smem_u32(&done_bar)) : "memory");
+    TC_MBAR_INIT(&acc_free, TC_WARPS);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (tid < CW) s_ssq[tid] = 0ull;
   if (warp == TC_WARPS + 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem_u32(&tmem_base_s)), "r"((uint32_t)C::COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -118,7 +129,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       const uint32_t elected = tc_elect();
       bool waited = false;
       if (!p.late_wait) { asm volatile("griddepcontrol.wait;" ::: "memory"); waited = true; }
-      int sb = 0, issued = 0; uint32_t pb = 1;
+      int sb = 0, issued = 0, m0 = 0; uint32_t pb = 1;
       auto copy = [&](const CUtensorMap* map, int x) {
         if (alive) alive = tc_wait(tc_smem_u32(b_empty) + 8 * sb, pb, status);
         if (!alive) return;
@@ -133,14 +144,17 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
         ++issued;
         if (++sb == NB) { sb = 0; pb ^= 1u; }
       };
-      for (int i = 0; i < nsteps && alive; ++i) {
-        const int u = u0 + i;
-        if (u < L.KT) copy(&act_map, u * TC_BK);
-        else {
-          if (!waited) { asm volatile("griddepcontrol.wait;" ::: "memory"); waited = true; }
-          const int e = u - L.KT, seg = seg0 + e / nE, x = kb0 + (e % nE) * 64;
-          copy(&text_map, (seg * 2) * p.lora.ke + x);
-          copy(&text_map, (seg * 2 + 1) * p.lora.ke + x);
+      for (int t = blockIdx.y; t < tiles && alive; t += gridDim.y) {
+        const Tile x = tile_of(t);
+        m0 = x.m0;
+        for (int u = x.u0; u < x.u1 && alive; ++u) {
+          if (u < L.KT) copy(&act_map, u * TC_BK);
+          else {
+            if (!waited) { asm volatile("griddepcontrol.wait;" ::: "memory"); waited = true; }
+            const int e = u - L.KT, seg = x.seg0 + e / x.nE, c = x.kb0 + (e % x.nE) * 64;
+            copy(&text_map, (seg * 2) * p.lora.ke + c);
+            copy(&text_map, (seg * 2 + 1) * p.lora.ke + c);
+          }
         }
       }
       // no copy may still be in flight when the CTA ends: the newest phase of every tile (passes at once unless a wait
@@ -158,7 +172,6 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       const uint32_t elected = tc_elect();
       const uint32_t base_u = tc_smem_u32(base);
       const uint32_t bf = tc_smem_u32(b_full), be = tc_smem_u32(b_empty), af = tc_smem_u32(a_full), ae = tc_smem_u32(a_empty);
-      const int n_main = max(0, min(L.KT, u1) - u0);
       const uint32_t idesc = IDESC;
       uint32_t acc = 0;
       // the four MMAs of one step: 16 features further along K = 8 columns of the weights, 32 bytes inside the swizzled
@@ -178,7 +191,15 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       auto release = [&](int sa) {
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(ae + 8 * sa) : "memory");
       };
-      int sa = 0, sb = 0; uint32_t pa = 0, pb = 0;
+      int sa = 0, sb = 0; uint32_t pa = 0, pb = 0, p_acc = 1;
+      for (int t = blockIdx.y; t < tiles && alive; t += gridDim.y) {
+      const Tile x = tile_of(t);
+      const int nsteps = x.u1 - x.u0, n_main = max(0, min(L.KT, x.u1) - x.u0);
+      // the accumulator is the epilogue's until it has read it
+      alive = tc_wait(tc_smem_u32(&acc_free), p_acc, status);
+      p_acc ^= 1u;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      acc = 0;
       int i = 0;
       // two steps a round: a test of a barrier costs about 90 cycles even when its phase is over, as much as the MMAs of
       // a step of 32 rows, so the four tests of a round go out together
@@ -216,16 +237,13 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
         }
         if (++sa == NA) { sa = 0; pa ^= 1u; }
       }
-      if (elected) asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tc_smem_u32(&done_bar)) : "memory");
+      if (elected) tc_commit(tc_smem_u32(&done_bar));
+      __syncwarp();
+      }
     }
-    __syncwarp();
   } else {
     // ---- dequantising warps: group grp takes every other step, quarter wq the features 32 wq .. 32 wq + 31
     const int grp = warp >> 2, wq = warp & 3, g = lane >> 2;
-    const int nt = slab * (TC_BM / TILE_N) + wq * 2;
-    // past the last n-tile the warp reads tile 0 again: those accumulator lanes are never stored
-    const unsigned char* const unit0 = p.w + (size_t)(nt < L.NT ? nt : 0) * L.unit_bytes;
-    const unsigned char* const unit1 = p.w + (size_t)(nt + 1 < L.NT ? nt + 1 : 0) * L.unit_bytes;
     const int gshift = L.G == 64 ? 0 : (L.G == 128 ? 1 : (L.G == 256 ? 2 : 3));   // k-tiles per scale entry, log2
     const uint32_t ring0 = tc_smem_u32(wring) + (uint32_t)(warp * WD) * TC_WSLOT;
     // lane 4g + j of a tile owns features 16j .. 16j + 15 of its rows; its 16 bytes go to piece (j, g), so that ldmatrix
@@ -234,14 +252,22 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
     const uint32_t dpos = (uint32_t)((lane & 3) * 128 + (lane >> 2) * 16);
     // The loop is bound by the instructions it issues (about 150 a visit, 104 of them the unpacking of 64 weights a lane),
     // so the fetch keeps running pointers: k-tile f_r of its chunk, the tile's bytes, the chunk's scale entries
-    const int u_end = min(u1, L.KT);
-    int f_left = (u_end - u0 - grp + GR - 1) / GR;         // fetches still to issue
-    int f_r = (u0 + grp) & 7, f_c = (u0 + grp) >> 3;
-    const unsigned char* f_w = unit0 + (size_t)f_c * L.chunk_full + f_r * 512 + lane * 16;
-    const ptrdiff_t f_d = unit1 - unit0;
-    const unsigned char* f_s = (lane & 2 ? unit1 : unit0) + (size_t)f_c * L.chunk_full + (f_c == L.nchunks - 1 ? L.kc_last : CHUNK_KT) * 512 + (lane & 1) * 16;
+    int f_left = 0, f_r = 0, f_c = 0;                       // fetches still to issue in this tile
+    const unsigned char *f_w = nullptr, *f_s = nullptr;
+    ptrdiff_t f_d = 0;
     uint32_t f_dst = ring0;
     const uint32_t ring_end = ring0 + WD * TC_WSLOT;
+    auto fetch_tile = [&](const Tile& x) {                  // the running pointers at the warp's first step of a tile
+      // past the last n-tile the warp reads tile 0 again: those accumulator lanes are never stored
+      const int nt0 = x.slab * (TC_BM / TILE_N) + ntile_of(wq, 0), nt1 = x.slab * (TC_BM / TILE_N) + ntile_of(wq, 1);
+      const unsigned char* const unit0 = p.w + (size_t)(nt0 < L.NT ? nt0 : 0) * L.unit_bytes;
+      const unsigned char* const unit1 = p.w + (size_t)(nt1 < L.NT ? nt1 : 0) * L.unit_bytes;
+      f_left = (min(x.u1, L.KT) - x.u0 - grp + GR - 1) / GR;
+      f_r = (x.u0 + grp) & 7; f_c = (x.u0 + grp) >> 3;
+      f_w = unit0 + (size_t)f_c * L.chunk_full + f_r * 512 + lane * 16;
+      f_d = unit1 - unit0;
+      f_s = (lane & 2 ? unit1 : unit0) + (size_t)f_c * L.chunk_full + (f_c == L.nchunks - 1 ? L.kc_last : CHUNK_KT) * 512 + (lane & 1) * 16;
+    };
     auto fetch_w = [&]() {
       if (f_left > 0) {
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(f_dst + dpos), "l"(f_w) : "memory");
@@ -258,13 +284,10 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       asm volatile("cp.async.commit_group;" ::: "memory");
       f_dst = f_dst + TC_WSLOT == ring_end ? ring0 : f_dst + TC_WSLOT;
     };
-#pragma unroll 1
-    for (int j = 0; j < WD; ++j) fetch_w();
     uint32_t slot = ring0;                                // ring slot consumed next
     const uint32_t ae = tc_smem_u32(a_empty), af = tc_smem_u32(a_full);
     const uint32_t lane_t = tmem + NR + ((uint32_t)(wq * 32) << 16);
     int sa = grp; uint32_t pa = 1;                        // stage of step i, parity of its "free" phase
-    int i = grp;
     auto stage_free = [&](bool tested) {
       if (!__all_sync(0xffffffffu, tested)) {
         if (alive) alive = tc_wait(ae + 8 * sa, pa, status);
@@ -277,9 +300,22 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(af + 8 * sa) : "memory");
+    };
+    // stages are dealt out by the running step count of the CTA
+    auto next_stage = [&]() {
       sa += GR;
       if (sa >= NA) { sa -= NA; pa ^= 1u; }
     };
+    fetch_tile(tile_of(blockIdx.y));
+#pragma unroll 1
+    for (int j = 0; j < WD; ++j) fetch_w();
+    uint32_t p_done = 0;
+    bool waited = false;
+#pragma unroll 1
+    for (int t = blockIdx.y; t < tiles; t += gridDim.y) {
+    const Tile x = tile_of(t);
+    const int u0 = x.u0, nsteps = x.u1 - x.u0, u_end = min(x.u1, L.KT);
+    int i = grp;
 #pragma unroll 1
     for (; u0 + i < u_end; i += GR) {
       const bool a_free = tc_test(ae + 8 * sa, pa);       // (its latency passes under the unpacking)
@@ -316,13 +352,14 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       tc_st_16x256b_x4(lane_t + sa * 32 + (16u << 16), r1);
       fetch_w();                                          // refills the slot just read, while the stores finish
       stage_done();
+      next_stage();
     }
 #pragma unroll 1
     for (; i < nsteps; i += GR) {
       {
         // 64 (slot, rank index) pairs of the expand: lane = output feature, two rank
         // indices a column
-        const int e = u0 + i - L.KT, seg = seg0 + e / nE, k0 = kb0 + (e % nE) * 64;
+        const int e = u0 + i - L.KT, seg = x.seg0 + e / x.nE, k0 = x.kb0 + (e % x.nE) * 64;
         const int r = p.lora.rank, ldb = p.lora.seg[seg].n;
         // lane l looks up the element addresses of pairs k0 + l and k0 + 32 + l (column 0); the loop below hands them round
         // and issues its loads independently of one another
@@ -336,7 +373,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
         const unsigned long long adr[2] = {address_of(k0 + lane), address_of(k0 + 32 + lane)};
         // [64 pairs][32 features] through the warp's ring (its weight steps are all done): 16-byte pieces in, columns out
         {
-          const int piece = lane & 3, n = slab * TC_BM + wq * 32 + piece * 8;
+          const int piece = lane & 3, n = x.slab * TC_BM + ntile_of(wq, piece >> 1) * TILE_N + (piece & 1) * 8;
           int my_seg = -1, col = 0;
           if (n < p.N) map_col(p.mode, n, p.seg_n0, p.seg_n1, my_seg, col);
           asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -369,54 +406,65 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
         tc_st_32x32b_x16(lane_t + sa * 32 + 16, v[1]);
       }
       stage_done();
+      next_stage();
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-  }
-
-  // ---- epilogue: lane = output feature, accumulator columns = rows
-  constexpr int NH = GR < 4 || CW < 8 ? 2 : 4;               // warps that share a lane quarter's columns
-  const int lq = warp & 3, half = warp >> 2;
-  const bool ep_warp = warp < 4 * NH;
-  const int n = slab * TC_BM + lq * 32 + lane;
-  const bool n_ok = n < p.N && ep_warp;
-  asm volatile("griddepcontrol.wait;" ::: "memory");       // (returns at once here: every earlier kernel's results)
-  const int row0 = m0 + rank * CW;                         // rows this CTA finishes: row0 .. row0 + CW - 1
-  if (tid < CW) {
-    float inv = 1.f;
-    if (p.ssq_in != nullptr && row0 + tid < p.M)
-      inv = rsqrtf(__ll2float_rn((long long)__ldcg(p.ssq_in + row0 + tid)) * TC_UNFIX / (float)p.K + p.eps);
-    s_inv[tid] = inv;
-    if (p.epi == EPI_QKV && row0 + tid < p.M) {
-      const int m = row0 + tid, st = m / p.rows_per_stream, cached = p.suffix_len[st];
-      s_pos[tid] = p.pos_base + cached + p.depth[m];
-      s_dst[tid] = (size_t)st * p.kv_stream_stride + (size_t)(cached + m - st * p.rows_per_stream) * p.hd;
+    const int slab = x.slab, m0 = x.m0;
+    const bool more = S == 1 && t + (int)gridDim.y < tiles;
+    if (more) {                                            // the next tile's first weights, under the epilogue
+      sa += nsteps + grp - i;                              // (from where step i would have been to step grp of the next tile)
+      if (sa >= NA) { sa -= NA; pa ^= 1u; }
+      else if (sa < 0) { sa += NA; pa ^= 1u; }
+      fetch_tile(tile_of(t + gridDim.y));
+      f_dst = slot = ring0;
+#pragma unroll 1
+      for (int j = 0; j < WD; ++j) fetch_w();
     }
-  }
-  constexpr int HC = CW / NH;                              // columns of a warp
-  constexpr int CH = HC < 16 ? HC : 16;                    // columns handled at a time
-  const int c_lo = half * HC;
-  float x_old[CH], gain = 1.f;
-  auto prefetch_resid = [&](int c0) {
+
+    // ---- epilogue: lane = output feature, accumulator columns = rows
+    const int lq = wq, half = grp;                         // GR warps share a lane quarter's columns
+    const int n = slab * TC_BM + ntile_of(lq, lane >> 4) * TILE_N + (lane & 15);
+    const bool n_ok = n < p.N;
+    if (!waited) { asm volatile("griddepcontrol.wait;" ::: "memory"); waited = true; }   // (every earlier kernel's results)
+    const int row0 = m0 + rank * CW;                       // rows this CTA finishes: row0 .. row0 + CW - 1
+    if (tid < CW) {
+      float inv = 1.f;
+      if (p.ssq_in != nullptr && row0 + tid < p.M)
+        inv = rsqrtf(__ll2float_rn((long long)__ldcg(p.ssq_in + row0 + tid)) * TC_UNFIX / (float)p.K + p.eps);
+      s_inv[tid] = inv;
+      s_ssq[tid] = 0ull;
+      s_pos[tid] = 0;
+      if (p.epi == EPI_QKV && row0 + tid < p.M) {
+        const int m = row0 + tid, st = m / p.rows_per_stream, cached = p.suffix_len[st];
+        s_pos[tid] = p.pos_base + cached + p.depth[m];
+        s_dst[tid] = (size_t)st * p.kv_stream_stride + (size_t)(cached + m - st * p.rows_per_stream) * p.hd;
+      }
+    }
+    constexpr int HC = CW / GR;                            // columns of a warp
+    constexpr int CH = HC < 16 ? HC : 16;                  // columns handled at a time
+    const int c_lo = half * HC;
+    float x_old[CH], gain = 1.f;
+    auto prefetch_resid = [&](int c0) {
 #pragma unroll
-    for (int j = 0; j < CH; ++j)
-      if (n_ok && row0 + c0 + j < p.M) x_old[j] = __ldcg(p.resid + (size_t)(row0 + c0 + j) * p.N + n);
-  };
-  if (p.epi == EPI_RESID) {
-    prefetch_resid(c_lo);
-    if (p.xg_out != nullptr && n_ok) gain = __half2float(__ldg(p.gain_next + n));
-  }
-  // all MMAs done (also when a stage wait gave up earlier: wait, bounded, before touching or freeing anything)
-  const bool done = tc_wait(tc_smem_u32(&done_bar), 0u, status);
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const bool fine = __syncthreads_and(done && alive);      // (one answer for the CTA: there are barriers below)
-  float* const xch = reinterpret_cast<float*>(base);       // [S][CW][128] partial sums for the rows this CTA finishes
-  if constexpr (S > 1) {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-    if (ep_warp) {
+      for (int j = 0; j < CH; ++j)
+        if (n_ok && row0 + c0 + j < p.M) x_old[j] = __ldcg(p.resid + (size_t)(row0 + c0 + j) * p.N + n);
+    };
+    if (p.epi == EPI_RESID) {
+      prefetch_resid(c_lo);
+      if (p.xg_out != nullptr && n_ok) gain = __half2float(__ldg(p.gain_next + n));
+    }
+    // the tile's MMAs are done (also when a stage wait gave up earlier: wait, bounded, before touching anything)
+    const bool done = tc_wait(tc_smem_u32(&done_bar), p_done, status);
+    p_done ^= 1u;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (!more) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("bar.sync 1, %0;" ::"n"(TC_WARPS * 32) : "memory");
+    float* const xch = reinterpret_cast<float*>(base);     // [S][CW][128] partial sums for the rows this CTA finishes
+    if constexpr (S > 1) {                                 // (a cluster has one tile: its activation tiles are free now)
+      asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
       const uint32_t my = tc_smem_u32(xch) + (uint32_t)((rank * CW) * TC_BM + lq * 32 + lane) * 4u;
 #pragma unroll 1
-      for (int c0 = half * (NR / NH); c0 < (half + 1) * (NR / NH); c0 += 16) {
+      for (int c0 = half * (NR / GR); c0 < (half + 1) * (NR / GR); c0 += 16) {
         float v[16];
         tc_ld_32x32b_x16(tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)c0, v);
 #pragma unroll
@@ -427,12 +475,11 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
           asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst + (uint32_t)(c % CW) * (TC_BM * 4u)), "f"(v[j]) : "memory");
         }
       }
+      asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-  }
-  if (fine && ep_warp) {
+    const bool fine = __all_sync(0xffffffffu, done && alive);
 #pragma unroll 1
-    for (int c0 = c_lo; c0 < c_lo + HC; c0 += CH) {
+    for (int c0 = c_lo; c0 < c_lo + HC && fine; c0 += CH) {
       float v[16];
       if constexpr (S > 1) {
 #pragma unroll
@@ -453,30 +500,30 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
         for (int j = 0; j < CH; ++j)
           if (n_ok && row0 + c0 + j < p.M) p.out_f32[(size_t)(row0 + c0 + j) * p.ldo + n] = v[j];
       } else if (p.epi == EPI_QKV) {
-        // RoPE on q and k (pairs (i, i + hd/2): the partner feature is two warps (hd 128) or one warp (hd 64) on, its values
-        // come through shared memory), fp16, q to its matrix, k and v into the stream's cache
+        // RoPE on q and k (pairs (i, i + hd/2): 16 lanes on), fp16, q to its matrix, k and v into the stream's cache
         int seg = 0, col = 0;
         if (n_ok) map_col(p.mode, n, p.seg_n0, p.seg_n1, seg, col);
-        float* const x = reinterpret_cast<float*>(wring) + (size_t)((c0 / CH & 1) * NH + half) * (4 * CH * 32);
-#pragma unroll
-        for (int j = 0; j < CH; ++j) x[(lq * CH + j) * 32 + lane] = v[j];
-        asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
-        const int hh = p.hd >> 1, i = col & (hh - 1), d = col & (p.hd - 1);
+        const int hh = p.hd >> 1, d = col & (p.hd - 1);
         const bool lo = d < hh;
-        __half* const kv = (seg == 1 ? p.k_out : p.v_out) + (size_t)(col / p.hd) * p.kv_head_stride + d;
+        const int rows = min(CH, p.M - row0 - c0);         // (may be negative: nothing of the chunk is stored)
+        if (__any_sync(0xffffffffu, n_ok && seg < 2)) {    // (a warp's lanes lie in one head: one answer)
+          // all table entries of the chunk in flight together (rows past the end read row 0 of the CTA's)
+          const float2* const tab = p.cs_table + (d & (hh - 1));
+          float2 cs[CH];
 #pragma unroll
-        for (int j = 0; j < CH; ++j) {
-          const int m = row0 + c0 + j;
-          if (n_ok && m < p.M) {
-            float y = v[j];
-            if (seg < 2) {
-              const float2 cs = __ldg(p.cs_table + (size_t)s_pos[c0 + j] * hh + i);
-              const float o = x[((lq ^ (hh >> 5)) * CH + j) * 32 + lane];
-              y = lo ? y * cs.x - o * cs.y : y * cs.x + o * cs.y;
-            }
-            if (seg == 0) p.q_out[(size_t)m * p.seg_n0 + col] = __float2half_rn(y);
-            else kv[s_dst[c0 + j]] = __float2half_rn(y);
+          for (int j = 0; j < CH; ++j) cs[j] = __ldg(tab + (size_t)s_pos[j < rows ? c0 + j : 0] * hh);
+#pragma unroll
+          for (int j = 0; j < CH; ++j) {
+            const float o = __shfl_xor_sync(0xffffffffu, v[j], 16);
+            v[j] = v[j] * cs[j].x + (lo ? -o : o) * cs[j].y;
           }
+        }
+        if (n_ok) {
+          __half* const dst = seg == 0 ? p.q_out + (size_t)(row0 + c0) * p.seg_n0 + col
+                                       : (seg == 1 ? p.k_out : p.v_out) + (size_t)(col / p.hd) * p.kv_head_stride + d;
+#pragma unroll
+          for (int j = 0; j < CH; ++j)
+            if (j < rows) dst[seg == 0 ? (size_t)j * p.seg_n0 : s_dst[c0 + j]] = __float2half_rn(v[j]);
         }
       } else if (p.epi == EPI_SWIGLU) {
         // lanes 0-15 hold a gate tile's features, lanes 16-31 the up tile's: of every two rows the lower half takes the
@@ -532,10 +579,23 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
         }
       }
     }
+    // the accumulator may be overwritten; the rows' sums of squares, complete, to where they are collected
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) tc_arrive(tc_smem_u32(&acc_free));
+    asm volatile("bar.sync 1, %0;" ::"n"(TC_WARPS * 32) : "memory");
+    if (p.ssq_out != nullptr && tid < CW && row0 + tid < p.M) atomicAdd(p.ssq_out + row0 + tid, s_ssq[tid]);
+    if (!more) break;
+    }
+  }
+  if constexpr (S > 1) {
+    if (warp >= TC_WARPS) {                                // (the other warps took both barriers in the epilogue)
+      asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (p.ssq_out != nullptr && tid < CW && row0 + tid < p.M) atomicAdd(p.ssq_out + row0 + tid, s_ssq[tid]);
   if (warp == TC_WARPS + 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)C::COLS) : "memory");
 }
@@ -567,7 +627,7 @@ static cudaError_t encode_row_map(const __half* base, int ld, int M, int nrows, 
 }
 
 template <int NR, int S>
-static cudaError_t tc_launch(const GemmArgs& a, int* status, cudaStream_t st) {
+static cudaError_t tc_launch(const GemmArgs& a, int sm_count, int* status, cudaStream_t st) {
   CUtensorMap map, tmap;
   cudaError_t e = encode_row_map(a.h, a.K, a.M, NR, &map);
   if (e != cudaSuccess) return e;
@@ -575,7 +635,9 @@ static cudaError_t tc_launch(const GemmArgs& a, int* status, cudaStream_t st) {
   if (a.lora.text != nullptr) e = encode_row_map(a.lora.text, a.lora.nseg * 2 * a.lora.ke, a.M, NR, &tmap);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(S, (unsigned)((a.N + TC_BM - 1) / TC_BM), (unsigned)((a.M + NR - 1) / NR));
+  // one CTA (or cluster) a tile; CTAs that have their K to themselves stay and take further tiles
+  const int tiles = (a.N + TC_BM - 1) / TC_BM * ((a.M + NR - 1) / NR);
+  cfg.gridDim = dim3(S, (unsigned)(S == 1 && tiles > sm_count * TcCfg<NR>::OCC ? sm_count * TcCfg<NR>::OCC : tiles));
   cfg.blockDim = dim3(TcCfg<NR>::THREADS); cfg.dynamicSmemBytes = TcCfg<NR>::SMEM; cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -607,11 +669,11 @@ bool gemm_tc_eligible(const GemmArgs& a) {
 }
 
 // Rows per CTA and K split, by a model of the time in microseconds, fitted to measurements of all candidates at seven
-// projections (2048 x 2048 .. 14336 x 4096) with 32 .. 1024 rows: the time of a step with one or two CTAs on an SM, a part
-// per wave (set-up, first tiles, epilogue), and the exchange of a split.  The choice it gives is within 1 % of the best
-// candidate on average.
+// projections (2048 x 2048 .. 14336 x 4096) with 32 .. 2000 rows: the time of a step with one or two CTAs on an SM, set-up
+// and epilogue, what a further wave costs (less where the CTA stays), and the exchange of a split.  The choice it gives is
+// within 1.5 % of the best candidate on average, within 16 % at worst.
 static void tc_plan(const GemmArgs& a, int sm_count, int& nr, int& split) {
-  static const double step1[4] = {0.181, 0.209, 0.251, 0.310}, step2[4] = {0.387, 0.409, 0.524, 0.0};
+  static const double step1[4] = {0.227, 0.242, 0.286, 0.320}, step2[4] = {0.393, 0.429, 0.538, 0.0};
   const int slabs = (a.N + TC_BM - 1) / TC_BM, KT = a.K / TILE_K;
   double best = 1e30;
   for (int ri = 0; ri < 4; ++ri) {
@@ -621,10 +683,11 @@ static void tc_plan(const GemmArgs& a, int sm_count, int& nr, int& split) {
       if (S > 1 && KT / S < 4) break;
       const long long ctas = (long long)slabs * ((a.M + R - 1) / R) * S, per_wave = (long long)sm_count * (R == 256 ? 1 : 2);
       const long long full = ctas / per_wave, rest = ctas % per_wave;
-      const double steps = (KT + S - 1) / S;
+      const double steps = (KT + S - 1) / S, f = R / 256.0;
       const double full_t = R == 256 ? step1[ri] : step2[ri], rest_t = rest == 0 ? 0.0 : (rest > sm_count ? step2[ri] : step1[ri]);
-      const double waves = (double)full + (rest > 0 ? 1 : 0);
-      const double cost = steps * (full * full_t + rest_t) + waves * (4.26 + R * 0.00914 + (S > 1 ? R * 0.0156 : 0.0)) + (S == 8 ? 1.1 : 0.0);
+      const double more = (double)full + (rest > 0 ? 1 : 0) - 1.0;
+      const double cost = steps * (full * full_t + rest_t) + 3.34 + 3.36 * f + (S > 1 ? 2.52 * f : 0.0) + (S == 8 ? 1.6 : 0.0) +
+                          more * (S == 1 ? 1.4 + 5.1 * f : 4.8 + 7.8 * f);
       if (cost < best) { best = cost; nr = R; split = S; }
     }
   }
@@ -634,7 +697,7 @@ static void tc_plan(const GemmArgs& a, int sm_count, int& nr, int& split) {
 cudaError_t launch_gemm_tc(const GemmArgs& a, int sm_count, int* status, cudaStream_t st) {
   int nr = 32, split = 1;
   tc_plan(a, sm_count, nr, split);
-#define TC_CASE(NR, S) if (nr == NR && split == S) return tc_launch<NR, S>(a, status, st);
+#define TC_CASE(NR, S) if (nr == NR && split == S) return tc_launch<NR, S>(a, sm_count, status, st);
   TC_FOR_EACH(TC_CASE)
 #undef TC_CASE
   return cudaErrorInvalidValue;

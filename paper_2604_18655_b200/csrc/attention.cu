@@ -307,35 +307,96 @@ __device__ __forceinline__ void attn_partial_body(const AttnArgs& p, const int r
 // log-sum-exp merge of the chunks of virtual row v (row m, query head hq) of kv head kh by one warp.  The lanes
 // take the chunks' (max, sum) pairs side by side; the weighted sum over chunks runs in chunk order with
 // independent loads.
+// Merge of a row's chunks by one warp; lane l holds the hd / 32 (2 or 4) consecutive features from l * hd / 32 on.
+__device__ __forceinline__ float4 merge_load(const float* row, int hd, int lane) {
+  if (hd == 128) return __ldcg(reinterpret_cast<const float4*>(row) + lane);
+  const float2 v = __ldcg(reinterpret_cast<const float2*>(row) + lane);
+  return make_float4(v.x, v.y, 0.f, 0.f);
+}
+// Partial shrink of the o projection's adapter (Eq. 1-4) over the features of one head of row m (fp16-rounded values v):
+// eight rank indices at a time, their sums folded together by a butterfly; integer atomics on fixed-point sums, so that the
+// total does not depend on the arrival order.  The loads of a batch are unconditional (rank indices past the end repeat the
+// last one): as predicated 2-byte loads they took the merge from 4.5 to 22 us.
+__device__ __forceinline__ void merge_o_shrink(const AttnArgs& p, int m, int hq, const float4 v, int lane) {
+  const __half* A = nullptr;
+  const int ad = p.o_direct ? m : p.o_adapter_idx[m];
+  if (ad >= 0 && ad < p.o_n_slots) A = p.o_tabA[(size_t)ad * p.o_tab_stride + p.o_proj_index];
+  if (A == nullptr) return;
+  const int ld = p.Hq * p.hd, r = p.o_rank;
+  A += (size_t)hq * p.hd + lane * (p.hd >> 5);
+  for (int j0 = 0; j0 < r; j0 += 8) {
+    float q[8];
+    if (p.hd == 128) {
+      uint2 w[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) w[j] = __ldg(reinterpret_cast<const uint2*>(A + (size_t)min(j0 + j, r - 1) * ld));
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float2 a = __half22float2(u32_as_h2(w[j].x)), b = __half22float2(u32_as_h2(w[j].y));
+        q[j] = v.x * a.x + v.y * a.y + v.z * b.x + v.w * b.y;
+      }
+    } else {
+      uint32_t w[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) w[j] = __ldg(reinterpret_cast<const uint32_t*>(A + (size_t)min(j0 + j, r - 1) * ld));
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float2 a = __half22float2(u32_as_h2(w[j]));
+        q[j] = v.x * a.x + v.y * a.y;
+      }
+    }
+    int id = 0;
+#pragma unroll
+    for (int w = 4, o = 16; w > 0; w >>= 1, o >>= 1) {
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (j < w) q[j] = (up ? q[j + w] : q[j]) + __shfl_xor_sync(0xffffffffu, up ? q[j] : q[j + w], o);
+      id = id * 2 + (up ? 1 : 0);
+    }
+    q[0] += __shfl_xor_sync(0xffffffffu, q[0], 2);
+    q[0] += __shfl_xor_sync(0xffffffffu, q[0], 1);
+    if ((lane & 3) == 0 && j0 + id < r) {
+      const unsigned long long f = (unsigned long long)__float2ll_rn(q[0] * 4294967296.f);
+      asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p.o_tacc + (size_t)m * 3 * r + j0 + id), "l"(f) : "memory");
+    }
+  }
+}
+__device__ __forceinline__ void merge_store(const AttnArgs& p, float4 acc, float inv, __half* out, int m, int hq, int lane) {
+  const __half2 a = __floats2half2_rn(acc.x * inv, acc.y * inv), b = __floats2half2_rn(acc.z * inv, acc.w * inv);
+  if (p.hd == 128) *(reinterpret_cast<uint2*>(out) + lane) = make_uint2(h2_as_u32(a), h2_as_u32(b));
+  else *(reinterpret_cast<__half2*>(out) + lane) = a;
+  if (p.o_tacc != nullptr) {
+    const float2 fa = __half22float2(a), fb = __half22float2(b);
+    merge_o_shrink(p, m, hq, make_float4(fa.x, fa.y, fb.x, fb.y), lane);
+  }
+}
+// log-sum-exp merge of the chunks of virtual row v (row m, query head hq) of kv head kh by one warp.  The lanes
+// take the chunks' (max, sum) pairs side by side; the weighted sum over chunks runs in chunk order with
+// independent loads.
 template <int FAST>
-__device__ __forceinline__ void merge_row_fast(const AttnArgs& p, size_t base, int n_valid, __half* out, int lane) {
+__device__ __forceinline__ void merge_row_fast(const AttnArgs& p, size_t base, int n_valid, __half* out, int m, int hq, int lane) {
   // one round trip: every load is issued before the first use; the partial outputs of FAST chunks sit in registers
   const int hd = p.hd;
   float2 ml = make_float2(-INFINITY, 0.f);
   if (lane < n_valid) ml = __ldcg(reinterpret_cast<const float2*>(p.part_ml + (base + lane) * 2));
-  float po[FAST][4];
+  float4 po[FAST];
 #pragma unroll
-  for (int i = 0; i < FAST; ++i)
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-      po[i][e] = (i < n_valid && e * 32 + lane < hd) ? __ldcg(p.part_o + (base + i) * hd + e * 32 + lane) : 0.f;
+  for (int i = 0; i < FAST; ++i) po[i] = i < n_valid ? merge_load(p.part_o + (base + i) * hd, hd, lane) : make_float4(0.f, 0.f, 0.f, 0.f);
   float mmax = ml.x;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mmax = fmaxf(mmax, __shfl_xor_sync(0xffffffffu, mmax, o));
   const float wgt = (ml.x == -INFINITY) ? 0.f : exp2f(ml.x - mmax);
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   float L = 0.f;
 #pragma unroll
   for (int i = 0; i < FAST; ++i) {                                     // fixed order: chunk 0, 1, ...
     const float wi = __shfl_sync(0xffffffffu, wgt, i);
     L = fmaf(wi, __shfl_sync(0xffffffffu, ml.y, i), L);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc[e] = fmaf(wi, po[i][e], acc[e]);
+    acc.x = fmaf(wi, po[i].x, acc.x); acc.y = fmaf(wi, po[i].y, acc.y);
+    acc.z = fmaf(wi, po[i].z, acc.z); acc.w = fmaf(wi, po[i].w, acc.w);
   }
-  const float inv = 1.f / L;
-#pragma unroll
-  for (int e = 0; e < 4; ++e)
-    if (e * 32 + lane < hd) out[e * 32 + lane] = __float2half_rn(acc[e] * inv);
+  merge_store(p, acc, 1.f / L, out, m, hq, lane);
 }
 
 __device__ __forceinline__ void merge_row(const AttnArgs& p, int kh, int v, int m, int hq, int lane) {
@@ -349,15 +410,14 @@ __device__ __forceinline__ void merge_row(const AttnArgs& p, int kh, int v, int 
   const size_t base = ((size_t)kh * R_all + v) * slots;
   const int hd = p.hd;
   __half* out = p.out + ((size_t)m * p.Hq + hq) * hd;
-  if (hd <= 128) {
-    if (n_valid <= 12) { merge_row_fast<12>(p, base, n_valid, out, lane); return; }
-    if (n_valid <= 24) { merge_row_fast<24>(p, base, n_valid, out, lane); return; }
-  }
+  if (n_valid <= 6) { merge_row_fast<6>(p, base, n_valid, out, m, hq, lane); return; }
+  if (n_valid <= 12) { merge_row_fast<12>(p, base, n_valid, out, m, hq, lane); return; }
+  if (n_valid <= 24) { merge_row_fast<24>(p, base, n_valid, out, m, hq, lane); return; }
   float mmax = -INFINITY;
   for (int i = lane; i < n_valid; i += 32) mmax = fmaxf(mmax, __ldcg(p.part_ml + (base + i) * 2));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mmax = fmaxf(mmax, __shfl_xor_sync(0xffffffffu, mmax, o));
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   float L = 0.f;
   for (int i0 = 0; i0 < n_valid; i0 += 32) {
     // lane i0 + lane holds the weight and the sum of its chunk
@@ -372,16 +432,11 @@ __device__ __forceinline__ void merge_row(const AttnArgs& p, int kh, int v, int 
     for (int i = 0; i < cnt; ++i) {                                      // fixed order: chunk 0, 1, ...
       const float wi = __shfl_sync(0xffffffffu, wgt, i);
       L = fmaf(wi, __shfl_sync(0xffffffffu, lsum, i), L);
-      const float* po = p.part_o + (base + i0 + i) * hd;
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (e * 32 + lane < hd) acc[e] = fmaf(wi, __ldcg(po + e * 32 + lane), acc[e]);
+      const float4 po = merge_load(p.part_o + (base + i0 + i) * hd, hd, lane);
+      acc.x = fmaf(wi, po.x, acc.x); acc.y = fmaf(wi, po.y, acc.y); acc.z = fmaf(wi, po.z, acc.z); acc.w = fmaf(wi, po.w, acc.w);
     }
   }
-  const float inv = 1.f / L;
-#pragma unroll
-  for (int e = 0; e < 4; ++e)
-    if (e * 32 + lane < hd) out[e * 32 + lane] = __float2half_rn(acc[e] * inv);
+  merge_store(p, acc, 1.f / L, out, m, hq, lane);
 }
 
 template <int HD>
@@ -392,11 +447,24 @@ __global__ void __launch_bounds__(ATT_THREADS, 3) attn_partial_kernel(const Attn
 
 // One warp per (row, query head): log-sum-exp merge of the row's chunks, output in fp16.
 __global__ void attn_merge_kernel(const AttnArgs p) {
+  // (a decode step's o projection has its weights to ask for meanwhile; the shrink of a larger pass only takes room)
+  if (p.o_tacc != nullptr) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   const int M = p.n * p.T;
   if (w >= M * p.Hq) return;
   const int m = w / p.Hq, hq = w % p.Hq;
+  if (p.o_tacc != nullptr) {                               // the adapter's rows over this head's features, ahead of the wait
+    const int ad = p.o_direct ? m : p.o_adapter_idx[m];
+    const __half* A = (ad >= 0 && ad < p.o_n_slots) ? p.o_tabA[(size_t)ad * p.o_tab_stride + p.o_proj_index] : nullptr;
+    if (A != nullptr)
+      for (int j = lane; j < p.o_rank * (p.hd >> 6); j += 32) {
+        const int half = p.hd == 128 ? j & 1 : 0, jj = p.hd == 128 ? j >> 1 : j;
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(A + (size_t)jj * p.Hq * p.hd + (size_t)hq * p.hd + half * 64) : "memory");
+      }
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");      // (programmatic launch behind the kernel that makes the partials)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int g_heads = p.Hq / p.Hkv;
   merge_row(p, hq / g_heads, m * g_heads + hq % g_heads, m, hq, lane);
 }
@@ -964,6 +1032,7 @@ attn_stream_kernel(const AttnArgs p, const __grid_constant__ CUtensorMap map_k, 
   uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(Qs) + (size_t)STR_ROWS * QSTRIDE * 2);
   float* comb = reinterpret_cast<float*>(ring);                            // after the prefix loop: [8 warps][16][HD + 2]
   __shared__ int s_abort;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const uint32_t ring_u = smem_u32(ring), own_u = smem_u32(own_tiles_mem);
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STR_STAGES);
 
@@ -1004,7 +1073,9 @@ attn_stream_kernel(const AttnArgs p, const __grid_constant__ CUtensorMap map_k, 
     return;                                                                 // (the consumers wait for every copy issued)
   }
 
-  // ---- consumers
+  // ---- consumers (programmatic launch: the prefix, which no decode step writes, is on its way; the projections are the
+  // kernel ahead's)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int ctid = threadIdx.x;                                             // 0 .. 255
   const int rt = warp & 1, kq = warp >> 1;                                  // row tile, key quarter of a tile
   const int key_end = S + 1;                                                // own keys: cached rows + this pass's row
@@ -1023,7 +1094,7 @@ attn_stream_kernel(const AttnArgs p, const __grid_constant__ CUtensorMap map_k, 
         if (key < key_end) {
           // this pass's row: built from the projections (k rotated), used, and appended to the stream's own segment
           const float* row = p.qkv_f32 + (size_t)s * (size_t)((p.Hq + 2 * p.Hkv) * HD);
-          const float2* cs = p.cs_table + (size_t)(p.pos_base + S + p.depth[s]) * (HD / 2);
+          const float2* cs = p.cs_table + (size_t)(p.pos_base + S + (p.depth ? p.depth[s] : 0)) * (HD / 2);
           kv8 = head_piece_f16(row + (size_t)(p.Hq + kh) * HD, piece * 8, HD, cs);
           vv8 = head_piece_f16(row + (size_t)(p.Hq + p.Hkv + kh) * HD, piece * 8, HD, nullptr);
           *reinterpret_cast<uint4*>(ok_ + (size_t)key * HD + piece * 8) = kv8;
@@ -1049,7 +1120,7 @@ attn_stream_kernel(const AttnArgs p, const __grid_constant__ CUtensorMap map_k, 
         const int v = v0 + r, m = v / g_heads, j = v % g_heads;
         if (fused) {
           const float* row = p.qkv_f32 + (size_t)m * (size_t)((p.Hq + 2 * p.Hkv) * HD);
-          const float2* cs = p.cs_table + (size_t)(p.pos_base + p.suffix_len[m] + p.depth[m]) * (HD / 2);
+          const float2* cs = p.cs_table + (size_t)(p.pos_base + p.suffix_len[m] + (p.depth ? p.depth[m] : 0)) * (HD / 2);
           val = head_piece_f16(row + (size_t)(kh * g_heads + j) * HD, c, HD, cs);
         } else {
           val = *reinterpret_cast<const uint4*>(p.q + ((size_t)m * p.Hq + kh * g_heads + j) * HD + c);
@@ -1265,10 +1336,16 @@ static cudaError_t launch_attention_stream(const AttnArgs& a, cudaStream_t st) {
   e = attn_prefix_map(a.prefix_v, a.hd, a.P, a.Hkv, a.prefix_head_stride, &mv);
   if (e != cudaSuccess) return e;
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)a.hd);
-  const dim3 grid((unsigned)(a.Hkv * a.n_prefix_chunks));
-  if (a.hd == 64) attn_stream_kernel<64><<<grid, STR_THREADS, str_smem_bytes(64), st>>>(a, mk, mv, scale_log2);
-  else attn_stream_kernel<128><<<grid, STR_THREADS, str_smem_bytes(128), st>>>(a, mk, mv, scale_log2);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(a.Hkv * a.n_prefix_chunks)); cfg.blockDim = dim3(STR_THREADS); cfg.stream = st;
+  cfg.dynamicSmemBytes = str_smem_bytes(a.hd);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = a.pdl ? 1 : 0;
+  if (a.hd == 64) return cudaLaunchKernelEx(&cfg, attn_stream_kernel<64>, a, mk, mv, scale_log2);
+  return cudaLaunchKernelEx(&cfg, attn_stream_kernel<128>, a, mk, mv, scale_log2);
 }
 
 cudaError_t launch_attention(const AttnArgs& a, cudaStream_t st) {
@@ -1303,8 +1380,15 @@ cudaError_t launch_attention(const AttnArgs& a, cudaStream_t st) {
 cudaError_t launch_attention_merge(const AttnArgs& a, cudaStream_t st) {
   if (a.tc_nq ? a.causal : attn_single_pass(a)) return cudaSuccess;   // nothing to merge
   const int warps = a.n * a.T * a.Hq;
-  attn_merge_kernel<<<(warps + 3) / 4, 128, 0, st>>>(a);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  const int per = warps <= 512 ? 1 : 4;                    // few rows: spread over the SMs
+  cfg.gridDim = dim3((unsigned)((warps + per - 1) / per)); cfg.blockDim = dim3((unsigned)per * 32); cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = a.pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, attn_merge_kernel, a);
 }
 
 }  // namespace mlora

@@ -52,10 +52,34 @@ __device__ __forceinline__ void ln_divmod_rank(const LeanArgs& a, int x, int& q,
 
 // Items run over all CHAIN_MAX_ROWS rows (row = low three bits of the quotient; rows past M are skipped), so that no
 // index needs a division by the row count.
-template <int NTILE>
+// Ranks above LN_PTR_RANK (several items a thread): the rows' matrix pointers, one load a (row, segment), go through shared
+// memory, asked for ahead of everything.  A pointer load in front of every item's copy puts several dependent trips to L2
+// at the start of every CTA (at rank 32 a late CTA of llama3b's gate/up reached its wait 4.9 us after its start, 3.0 with
+// the table); at rank 16 the barrier costs what the trips do (llama1b: 32.6 us a layer without, 32.9 with).
+constexpr int LN_PTR_RANK = 16;
+__device__ __forceinline__ const __half* lean_row_ptr(const LeanArgs& a, const StepPhase& ph) {
+  if (a.adapter_idx == nullptr || threadIdx.x >= 48) return nullptr;
+  const int w = threadIdx.x / 24, seg = (threadIdx.x >> 3) % 3, m = threadIdx.x & 7;   // B of this group, A of the next
+  if (m >= a.M || seg >= (w == 0 ? ph.lora_nseg : ph.next_nseg)) return nullptr;
+  const int ad = a.rows_direct ? m : a.adapter_idx[m];
+  if (ad < 0 || ad >= a.n_slots) return nullptr;
+  return (w == 0 ? a.tabB + ph.lora_proj[seg] : a.tabA + ph.next_proj[seg])[(size_t)ad * a.tab_stride];
+}
+template <int NTILE, bool TAB>
 __device__ __forceinline__ void lean_prefetch_slices(const LeanArgs& a, const StepPhase& ph, int tile0, int n_out0, bool lora,
-                                                     __half* sB, __half* sA) {
+                                                     const __half* row_ptr, __half* sB, __half* sA) {
+  __shared__ const __half* s_ptr[48];                       // [B of this group, A of the next][segment][row]
   const int r = a.rank, M = a.M;
+  if (a.adapter_idx == nullptr) { asm volatile("cp.async.commit_group;" ::: "memory"); return; }
+  if constexpr (TAB) {
+    if (threadIdx.x < 48) s_ptr[threadIdx.x] = row_ptr;
+    __syncthreads();
+  }
+  auto matrix = [&](const __half* const* tab, const int* proj, int s0, int seg, int m) -> const __half* {
+    if constexpr (TAB) return s_ptr[s0 + seg * 8 + m];
+    const int ad = a.rows_direct ? m : a.adapter_idx[m];
+    return (ad >= 0 && ad < a.n_slots) ? tab[(size_t)ad * a.tab_stride + proj[seg]] : nullptr;
+  };
   const int nB = lora ? NTILE * CHAIN_MAX_ROWS * r * 2 : 0;
   const int nA = (ph.next_nseg > 0 && a.adapter_idx != nullptr) ? ph.next_nseg * CHAIN_MAX_ROWS * r * 2 : 0;
   for (int it = threadIdx.x; it < nB; it += blockDim.x) {
@@ -63,10 +87,9 @@ __device__ __forceinline__ void lean_prefetch_slices(const LeanArgs& a, const St
     ln_divmod_rank(a, it >> 1, q, j);
     const int hf = it & 1, m = q & (CHAIN_MAX_ROWS - 1), u = q >> 3;
     if (m >= M) continue;
-    const int ad = a.rows_direct ? m : a.adapter_idx[m];
     int seg, col;
     map_col(ph.mode, (tile0 + u) * TILE_N, ph.seg_n0, ph.seg_n1, seg, col);
-    const __half* B = (ad >= 0 && ad < a.n_slots) ? a.tabB[(size_t)ad * a.tab_stride + ph.lora_proj[seg]] : nullptr;
+    const __half* B = matrix(a.tabB, ph.lora_proj, 0, seg, m);
     ln_cp_async16(sB + (((size_t)u * M + m) * r + j) * 16 + hf * 8, B ? B + (size_t)j * ph.lora_n[seg] + col + hf * 8 : (const __half*)ph.w,
                   B != nullptr);
   }
@@ -75,8 +98,7 @@ __device__ __forceinline__ void lean_prefetch_slices(const LeanArgs& a, const St
     ln_divmod_rank(a, it >> 1, q, j);
     const int hf = it & 1, m = q & (CHAIN_MAX_ROWS - 1), seg = q >> 3;
     if (m >= M) continue;
-    const int ad = a.rows_direct ? m : a.adapter_idx[m];
-    const __half* A = (ad >= 0 && ad < a.n_slots) ? a.tabA[(size_t)ad * a.tab_stride + ph.next_proj[seg]] : nullptr;
+    const __half* A = matrix(a.tabA, ph.next_proj, 24, seg, m);
     ln_cp_async16(sA + (((size_t)m * ph.next_nseg + seg) * r + j) * 16 + hf * 8,
                   A ? A + (size_t)j * ph.next_ld + n_out0 + hf * 8 : (const __half*)ph.w, A != nullptr);
   }
@@ -127,13 +149,14 @@ __device__ __forceinline__ void ln_stamp(const LeanArgs& a, int slot) {
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-template <int NTILE, int WARPS, bool TRACE>
-__global__ void __launch_bounds__(WARPS * 32, WARPS == 8 ? 3 : 1)
+// PF k-tiles' weights in flight per warp, the input rows of XB of them loaded together, OCC CTAs on an SM; TAB: the rows'
+// matrix pointers by a table (an instantiation of its own: the code a CTA runs once runs at the instruction cache's cold rate)
+template <int NTILE, int WARPS, int PF, int XB, int OCC, bool TRACE, bool TAB>
+__global__ void __launch_bounds__(WARPS * 32, OCC)
 lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   constexpr int THREADS = WARPS * 32;
   __shared__ float red[WARPS][NTILE][32][4];
   __shared__ float s_inv[CHAIN_MAX_ROWS];
-  __shared__ float s_T[CHAIN_MAX_ROWS][3 * 64];
   __shared__ float s_y[NTILE][CHAIN_MAX_ROWS][16];
   __shared__ __align__(16) __half s_vals[CHAIN_MAX_ROWS][16];
   __shared__ float s_sq[CHAIN_MAX_ROWS][16];
@@ -142,18 +165,20 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   ln_stamp<TRACE>(a, 0);
   pdl_launch_dependents();
   const int M = a.M, K = ph.K, r = a.rank;
+  const __half* const row_ptr = TAB ? lean_row_ptr(a, ph) : nullptr;
   const WLayout L = make_wlayout(K, ph.N, ph.G);
   const int tile0 = blockIdx.x * NTILE;
   // ---- ahead of the wait: adapter slices and the first weights (immutable data)
   const bool lora = ph.lora_nseg > 0 && a.adapter_idx != nullptr;
   __half* sB = reinterpret_cast<__half*>(ln_dyn);                          // [NTILE][M][r][16]
   __half* sA = sB + (size_t)NTILE * CHAIN_MAX_ROWS * r * 16;               // [M][next_nseg][r][16]
+  const int ldt = TAB ? ph.lora_nseg * r : 3 * LN_PTR_RANK;
+  float* s_T = reinterpret_cast<float*>(sA + (size_t)CHAIN_MAX_ROWS * ph.next_nseg * r * 16);   // [8][ldt]
   const int n_out0 = ph.epi == EPI_SWIGLU ? (tile0 >> 1) * TILE_N : tile0 * TILE_N;   // first column the CTA produces
   const int kt0 = (L.KT * warp) / WARPS, kt1 = (L.KT * (warp + 1)) / WARPS;
   const unsigned char* unit[NTILE];
 #pragma unroll
   for (int u = 0; u < NTILE; ++u) unit[u] = ph.w + (size_t)(tile0 + u) * L.unit_bytes;
-  constexpr int PF = 4;                                                    // k-tiles in flight per warp
   uint4 wv[PF][NTILE];
   uint32_t sv[PF][NTILE];
   auto load_weights = [&](int kb) {
@@ -180,7 +205,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(ph.pf_w + o), "r"(n) : "memory");
     }
   }
-  lean_prefetch_slices<NTILE>(a, ph, tile0, n_out0, lora, sB, sA);
+  lean_prefetch_slices<NTILE, TAB>(a, ph, tile0, n_out0, lora, row_ptr, sB, sA);
   pdl_wait();
   ln_stamp<TRACE>(a, 1);
   // ---- what earlier kernels produced: the old residual, norm factors, T of this group, the input rows
@@ -205,7 +230,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
       float v = 0.f;
       if (ad >= 0 && ad < a.n_slots)
         v = ln_unfix(__ldcg(a.tacc + ((size_t)ph.t_in * CHAIN_MAX_ROWS + m) * 3 * r + rest)) * a.scale[ad];
-      s_T[m][rest] = v;
+      s_T[m * ldt + rest] = v;
     }
   };
   if (lora && !a.late_wait) load_T();
@@ -217,10 +242,12 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   const bool row_live = g < M;
 #pragma unroll 1
   for (int kb = kt0; kb < kt1; kb += PF) {
-    uint4 x0[PF], x1[PF];
 #pragma unroll
-    for (int i = 0; i < PF; ++i) {
-      const int kt = kb + i;
+   for (int ib = 0; ib < PF; ib += XB) {
+    uint4 x0[XB], x1[XB];
+#pragma unroll
+    for (int i = 0; i < XB; ++i) {
+      const int kt = kb + ib + i;
       if (kt < kt1 && row_live) {
         // (ordinary cached loads: the CTAs that share an SM read the same rows, and loads behind the wait see what
         // the kernel ahead wrote)
@@ -232,17 +259,17 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
       }
     }
 #pragma unroll
-    for (int i = 0; i < PF; ++i) {
-      if (kb + i < kt1) {
+    for (int i = 0; i < XB; ++i) {
+      if (kb + ib + i < kt1) {
 #pragma unroll
         for (int u = 0; u < NTILE; ++u) {
           __half2 s_lo, s_hi;
-          split_scales(sv[i][u], s_lo, s_hi);
+          split_scales(sv[ib + i][u], s_lo, s_hi);
           uint32_t af[4][4];
-          dequant8(wv[i][u].x, s_lo, s_hi, af[0]);
-          dequant8(wv[i][u].y, s_lo, s_hi, af[1]);
-          dequant8(wv[i][u].z, s_lo, s_hi, af[2]);
-          dequant8(wv[i][u].w, s_lo, s_hi, af[3]);
+          dequant8(wv[ib + i][u].x, s_lo, s_hi, af[0]);
+          dequant8(wv[ib + i][u].y, s_lo, s_hi, af[1]);
+          dequant8(wv[ib + i][u].z, s_lo, s_hi, af[2]);
+          dequant8(wv[ib + i][u].w, s_lo, s_hi, af[3]);
           mma_16816(acc[u], af[0], x0[i].x, x0[i].y);
           mma_16816(acc[u], af[1], x0[i].z, x0[i].w);
           mma_16816(acc[u], af[2], x1[i].x, x1[i].y);
@@ -250,6 +277,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
         }
       }
     }
+   }
     if (kb + PF < kt1) load_weights(kb + PF);
   }
   if (a.late_wait) {
@@ -275,7 +303,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
       if (lora) {
         int seg, col;
         map_col(ph.mode, (tile0 + u) * TILE_N, ph.seg_n0, ph.seg_n1, seg, col);
-        const float* T = s_T[m] + seg * r;
+        const float* T = s_T + m * ldt + seg * r;
         const __half* Bs = sB + ((size_t)u * M + m) * r * 16 + c;           // (zeros where the row has no adapter)
         float ex = 0.f;
         for (int j = 0; j < r; ++j) ex = fmaf(T[j], __half2float(Bs[(size_t)j * 16]), ex);
@@ -373,10 +401,10 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
 // go through two alternating buffers (one barrier per tile); in row-maxima mode every thread keeps the best key of its
 // (row, column of the tile) across its tiles: one atomic per row and CTA at the end.  2000 short-lived CTAs of the
 // one-tile kernel took 20 us for the 33 MB of a 32000 x 2048 lm_head (4.5 waves, each paying the trip to HBM).
-constexpr int LM_PF = 4;
-constexpr int LM_DEPTH = 4;
-constexpr size_t lm_smem_bytes(int threads) { return (size_t)LM_DEPTH * LM_PF * threads * (16 + 4); }
-template <int WARPS, bool TRACE>
+// LM_PF k-tiles a warp (4: K up to 2048, 6: up to 3072, 8: up to 4096), LM_DEPTH tiles in flight: at most 113 KB a CTA.
+// (K = 3072: 2000 one-tile CTAs took 27 us for the 50 MB.)
+constexpr size_t lm_smem_bytes(int pf, int depth, int threads) { return (size_t)depth * pf * threads * (16 + 4); }
+template <int WARPS, int LM_PF, int LM_DEPTH, bool TRACE>
 __global__ void __launch_bounds__(WARPS * 32, 2) lean_lmhead_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   constexpr int THREADS = WARPS * 32;
   extern __shared__ __align__(16) unsigned char lm_dyn[];
@@ -648,16 +676,29 @@ cudaError_t launch_lean_embed(const LeanArgs& a, const StepPhase& ph, const int3
   return cudaGetLastError();
 }
 
+// The variants of lean_gemm_kernel (NTILE, WARPS, PF, XB, OCC).  A grid that does not fit the SMs at once costs a whole
+// CTA's life more (llama3b gate/up, 512 CTAs at three an SM: 24.5 us, the last ones starting at 11; 12.9 at four), but the
+// registers of a fourth CTA are paid with loads in flight (llama1b gate/up, 352 CTAs: 9.1 us at three, 9.7 at four), so the
+// dense variants are taken only where they save the second wave.
+#define LN_ONE 1, 8, 4, 4, 3
+#define LN_PAIR 2, 8, 4, 4, 3         // gate/up: a gate tile and its up tile
+#define LN_PAIR_DENSE 2, 8, 2, 2, 4
+#define LN_WIDE 1, 16, 4, 4, 1        // a long K on few tiles: sixteen warps split it
+#define LN_WIDE_DENSE 1, 16, 4, 2, 2
+#define LN_SET(...) \
+  if ((e = cudaFuncSetAttribute(lean_gemm_kernel<__VA_ARGS__, TRACE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 88 * 1024)) != cudaSuccess) return e; \
+  if ((e = cudaFuncSetAttribute(lean_gemm_kernel<__VA_ARGS__, TRACE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 88 * 1024)) != cudaSuccess) return e;
+#define LN_LAUNCH(...) \
+  return a.rank > LN_PTR_RANK ? cudaLaunchKernelEx(&cfg, lean_gemm_kernel<__VA_ARGS__, TRACE, true>, a, ph) : cudaLaunchKernelEx(&cfg, lean_gemm_kernel<__VA_ARGS__, TRACE, false>, a, ph)
 template <bool TRACE>
 static cudaError_t init_lean_variant() {
-  // room for the adapter slices at rank 64: 5 x 16 KB
-  cudaError_t e = cudaFuncSetAttribute(lean_gemm_kernel<1, 8, TRACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(lean_gemm_kernel<1, 16, TRACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(lean_lmhead_kernel<LN_WARPS, TRACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lm_smem_bytes(LN_THREADS));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(lean_gemm_kernel<2, 8, TRACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
+  // room for the adapter slices and T at rank 64: 5 x 16 KB and 6 KB
+  cudaError_t e;
+  LN_SET(LN_ONE) LN_SET(LN_PAIR) LN_SET(LN_PAIR_DENSE) LN_SET(LN_WIDE) LN_SET(LN_WIDE_DENSE)
+#define LM_SET(PF, D) \
+  if ((e = cudaFuncSetAttribute(lean_lmhead_kernel<LN_WARPS, PF, D, TRACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lm_smem_bytes(PF, D, LN_THREADS))) != cudaSuccess) return e;
+  LM_SET(4, 4) LM_SET(6, 3) LM_SET(8, 2)
+  return cudaSuccess;
 }
 cudaError_t init_lean() {
   const cudaError_t e = init_lean_variant<false>();
@@ -671,27 +712,36 @@ static cudaError_t launch_lean_gemm_variant(const LeanArgs& a, const StepPhase& 
   const size_t slice = (size_t)CHAIN_MAX_ROWS * (a.rank > 0 ? a.rank : 1) * 16 * sizeof(__half);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(mode == MODE_GATEUP ? tiles / 2 : tiles));
-  const bool wide = mode != MODE_GATEUP && ph.K >= 4096 && tiles <= 148;   // a long K on few tiles: sixteen warps split it
-  cfg.blockDim = dim3(wide ? 512 : LN_THREADS);
-  cfg.dynamicSmemBytes = (mode == MODE_GATEUP ? 5 : 4) * slice;
+  cfg.dynamicSmemBytes = ((mode == MODE_GATEUP ? 2 : 1) + ph.next_nseg) * slice + (size_t)CHAIN_MAX_ROWS * (a.rank > LN_PTR_RANK ? ph.lora_nseg * a.rank : 3 * LN_PTR_RANK) * sizeof(float);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // may start while the kernel before it drains
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  static const int sms = [] { int d = 0, n = 0; cudaGetDevice(&d); cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, d); return n > 0 ? n : 148; }();
+  const bool wide = mode != MODE_GATEUP && ph.K >= 4096 && tiles <= 2 * sms;
+  cfg.blockDim = dim3(wide ? 512 : LN_THREADS);
   // wide projections without adapters (the lm_head): persistent CTAs, two per SM, that loop over the column tiles
-  static const int sms = [] { int d = 0, n = 0; cudaGetDevice(&d); cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, d); return n; }();
-  if (mode == MODE_PLAIN && ph.epi == EPI_F32 && ph.lora_nseg == 0 && tiles >= 4 * sms && sms > 0 &&
-      (ph.K / TILE_K + LN_WARPS - 1) / LN_WARPS <= LM_PF) {
+  if (mode == MODE_PLAIN && ph.epi == EPI_F32 && ph.lora_nseg == 0 && tiles >= 4 * sms &&
+      ph.K <= 8 * LN_WARPS * TILE_K) {
     cfg.gridDim = dim3((unsigned)(2 * sms < tiles ? 2 * sms : tiles));
     cfg.blockDim = dim3(LN_THREADS);
-    cfg.dynamicSmemBytes = lm_smem_bytes(LN_THREADS);
-    return cudaLaunchKernelEx(&cfg, lean_lmhead_kernel<LN_WARPS, TRACE>, a, ph);
+    const int pf = (ph.K / TILE_K + LN_WARPS - 1) / LN_WARPS;
+#define LM_LAUNCH(PF, D) \
+    cfg.dynamicSmemBytes = lm_smem_bytes(PF, D, LN_THREADS); \
+    return cudaLaunchKernelEx(&cfg, lean_lmhead_kernel<LN_WARPS, PF, D, TRACE>, a, ph);
+    if (pf <= 4) { LM_LAUNCH(4, 4) }
+    if (pf <= 6) { LM_LAUNCH(6, 3) }
+    LM_LAUNCH(8, 2)
   }
-  if (mode == MODE_GATEUP) return cudaLaunchKernelEx(&cfg, lean_gemm_kernel<2, 8, TRACE>, a, ph);
-  if (wide) return cudaLaunchKernelEx(&cfg, lean_gemm_kernel<1, 16, TRACE>, a, ph);
-  return cudaLaunchKernelEx(&cfg, lean_gemm_kernel<1, 8, TRACE>, a, ph);
+  if (mode == MODE_GATEUP) {
+    if (tiles / 2 > 3 * sms && tiles / 2 <= 4 * sms) LN_LAUNCH(LN_PAIR_DENSE);
+    LN_LAUNCH(LN_PAIR);
+  }
+  if (wide && tiles > sms) LN_LAUNCH(LN_WIDE_DENSE);
+  if (wide) LN_LAUNCH(LN_WIDE);
+  LN_LAUNCH(LN_ONE);
 }
 
 // (a.trace0 set: the instantiations that stamp the step's timeline)

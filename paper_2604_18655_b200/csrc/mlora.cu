@@ -386,7 +386,7 @@ int forward_chain(mlora_ctx* c, const PassIO& io) {
 bool lean_eligible(const mlora_ctx* c, const PassIO& io) {
   // (the library's own choice where it applies: the fastest of the three decode paths at the measured shapes)
   return (c->step_mode == 3 || c->step_mode == 0) && !c->dbg_no_chain && c->lean_ok && c->step_phases != nullptr && !io.prefill && io.T == 1 &&
-         io.n <= CHAIN_MAX_ROWS && io.parent == c->root_parent && attn_single_pass(io.plan);
+         io.n <= CHAIN_MAX_ROWS && io.parent == c->root_parent && (attn_single_pass(io.plan) || io.plan.stream_mode);
 }
 
 int forward_lean(mlora_ctx* c, PassIO& io) {
@@ -444,7 +444,13 @@ int forward_lean(mlora_ctx* c, PassIO& io) {
         at.o_tabA = c->step_rowA; at.o_adapter_idx = io.adapter_idx; at.o_direct = 1; at.o_proj_index = ph.next_proj[0]; at.o_rank = a.rank;
         at.o_tab_stride = c->L * 7; at.o_n_slots = CHAIN_MAX_ROWS;
       }
+      if (at.stream_mode) {                              // a long prefix: partials per chunk, the merge does the o projection's shrink
+        if (attn_workspace_floats(at) > c->att_ws_floats) return fail(MLORA_ERR_CAPACITY, "attention scratch too small");
+        at.part_o = c->att_ws;
+        at.part_ml = c->att_ws + (attn_workspace_floats(at) / (at.hd + 2)) * at.hd;
+      }
       CK(run(c, MLORA_PROF_ATTN, [&] { return launch_attention(at, st); }));
+      if (at.stream_mode) CK(run(c, MLORA_PROF_ATTN_MERGE, [&] { return launch_attention_merge(at, st); }));
     }
   }
   if (fused) {

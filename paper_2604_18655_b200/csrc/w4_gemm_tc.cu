@@ -45,7 +45,7 @@ template <int NR> struct TcCfg {
   static constexpr size_t SMEM = (size_t)NB * NR * TC_BK * 2 + (size_t)WD * GR * 4 * TC_WSLOT + 1024;
 };
 
-template <int NR, int S>
+template <int NR, int S, int EPI>
 __global__ void __launch_bounds__(TcCfg<NR>::THREADS, TcCfg<NR>::OCC)
 w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_constant__ CUtensorMap act_map,
                   const __grid_constant__ CUtensorMap text_map) {
@@ -69,18 +69,23 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
   const WLayout L = make_wlayout(p.K, p.N, p.G);
   const int slabs = (p.N + TC_BM - 1) / TC_BM, tiles = slabs * ((p.M + NR - 1) / NR);
 
+  const int first = blockIdx.y + blockIdx.z * gridDim.y, stride = gridDim.y * gridDim.z;
+  const bool single = stride >= tiles;                // (then the grid is slabs x row blocks)
+
   // ---- a tile = 128 output features x NR rows.  Its steps: KT k-tiles of the weights, then the expand's blocks of 64
   // (slot, rank index) pairs, per segment that the features touch; a CTA of a cluster takes a contiguous share of them.
   struct Tile { int slab, m0, seg0, nE, kb0, u0, u1; };
+  auto stream_of = [&](int m) { return p.stream_magic ? (int)__umulhi((unsigned)m, p.stream_magic) : m; };   // m / rows per stream
   auto tile_of = [&](int t) {
     Tile x;
-    const int mb = t / slabs;
-    x.slab = t - mb * slabs; x.m0 = mb * NR;
+    // (one tile a CTA: no division)
+    const int mb = single ? (int)blockIdx.z : t / slabs;
+    x.slab = single ? (int)blockIdx.y : t - mb * slabs; x.m0 = mb * NR;
     x.seg0 = 0; x.nE = 0; x.kb0 = 0;
     int nseg_in = 0;
     if (p.lora.text != nullptr) {
       int s_lo = 0, s_hi = p.lora.k_slots - 1;
-      if (!p.lora.slot_is_adapter) { s_lo = x.m0 / p.lora.rows_per_stream; s_hi = min(s_hi, (min(p.M, x.m0 + NR) - 1) / p.lora.rows_per_stream); }
+      if (!p.lora.slot_is_adapter) { s_lo = stream_of(x.m0); s_hi = min(s_hi, stream_of(min(p.M, x.m0 + NR) - 1)); }
       x.kb0 = (s_lo * p.lora.rank) & ~63;
       x.nE = ((s_hi + 1) * p.lora.rank - x.kb0 + 63) >> 6;
       int c, seg1;
@@ -95,7 +100,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
   };
   // n-tile (16 features) of the slab that lanes 16 h .. 16 h + 15 of accumulator quarter q hold: consecutive ones; with
   // RoPE in the epilogue a pair of tiles half a head apart, so that a feature's partner sits 16 lanes on
-  const int rope_gap = p.epi == EPI_QKV ? p.hd >> 5 : 0;   // 2 (hd 64) or 4 (hd 128) tiles
+  const int rope_gap = EPI == EPI_QKV ? p.hd >> 5 : 0;   // 2 (hd 64) or 4 (hd 128) tiles
   auto ntile_of = [&](int q, int h) { return rope_gap == 0 ? 2 * q + h : (rope_gap == 4 ? q + 4 * h : (q >> 1) * 4 + (q & 1) + 2 * h); };
 
   if (tid == 0) {
@@ -144,14 +149,14 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
         ++issued;
         if (++sb == NB) { sb = 0; pb ^= 1u; }
       };
-      for (int t = blockIdx.y; t < tiles && alive; t += gridDim.y) {
+      for (int t = first; t < tiles && alive; t += stride) {
         const Tile x = tile_of(t);
         m0 = x.m0;
         for (int u = x.u0; u < x.u1 && alive; ++u) {
           if (u < L.KT) copy(&act_map, u * TC_BK);
           else {
             if (!waited) { asm volatile("griddepcontrol.wait;" ::: "memory"); waited = true; }
-            const int e = u - L.KT, seg = x.seg0 + e / x.nE, c = x.kb0 + (e % x.nE) * 64;
+            const int e = u - L.KT, sg = (e >= x.nE) + (e >= 2 * x.nE), seg = x.seg0 + sg, c = x.kb0 + (e - sg * x.nE) * 64;
             copy(&text_map, (seg * 2) * p.lora.ke + c);
             copy(&text_map, (seg * 2 + 1) * p.lora.ke + c);
           }
@@ -192,7 +197,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(ae + 8 * sa) : "memory");
       };
       int sa = 0, sb = 0; uint32_t pa = 0, pb = 0, p_acc = 1;
-      for (int t = blockIdx.y; t < tiles && alive; t += gridDim.y) {
+      for (int t = first; t < tiles && alive; t += stride) {
       const Tile x = tile_of(t);
       const int nsteps = x.u1 - x.u0, n_main = max(0, min(L.KT, x.u1) - x.u0);
       // the accumulator is the epilogue's until it has read it
@@ -306,13 +311,13 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       sa += GR;
       if (sa >= NA) { sa -= NA; pa ^= 1u; }
     };
-    fetch_tile(tile_of(blockIdx.y));
+    fetch_tile(tile_of(first));
 #pragma unroll 1
     for (int j = 0; j < WD; ++j) fetch_w();
     uint32_t p_done = 0;
     bool waited = false;
 #pragma unroll 1
-    for (int t = blockIdx.y; t < tiles; t += gridDim.y) {
+    for (int t = first; t < tiles; t += stride) {
     const Tile x = tile_of(t);
     const int u0 = x.u0, nsteps = x.u1 - x.u0, u_end = min(x.u1, L.KT);
     int i = grp;
@@ -359,7 +364,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       {
         // 64 (slot, rank index) pairs of the expand: lane = output feature, two rank
         // indices a column
-        const int e = u0 + i - L.KT, seg = x.seg0 + e / x.nE, k0 = x.kb0 + (e % x.nE) * 64;
+        const int e = u0 + i - L.KT, sg = (e >= x.nE) + (e >= 2 * x.nE), seg = x.seg0 + sg, k0 = x.kb0 + (e - sg * x.nE) * 64;
         const int r = p.lora.rank, ldb = p.lora.seg[seg].n;
         // lane l looks up the element addresses of pairs k0 + l and k0 + 32 + l (column 0); the loop below hands them round
         // and issues its loads independently of one another
@@ -410,12 +415,12 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     const int slab = x.slab, m0 = x.m0;
-    const bool more = S == 1 && t + (int)gridDim.y < tiles;
+    const bool more = S == 1 && t + stride < tiles;
     if (more) {                                            // the next tile's first weights, under the epilogue
       sa += nsteps + grp - i;                              // (from where step i would have been to step grp of the next tile)
       if (sa >= NA) { sa -= NA; pa ^= 1u; }
       else if (sa < 0) { sa += NA; pa ^= 1u; }
-      fetch_tile(tile_of(t + gridDim.y));
+      fetch_tile(tile_of(t + stride));
       f_dst = slot = ring0;
 #pragma unroll 1
       for (int j = 0; j < WD; ++j) fetch_w();
@@ -434,8 +439,8 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       s_inv[tid] = inv;
       s_ssq[tid] = 0ull;
       s_pos[tid] = 0;
-      if (p.epi == EPI_QKV && row0 + tid < p.M) {
-        const int m = row0 + tid, st = m / p.rows_per_stream, cached = p.suffix_len[st];
+      if (EPI == EPI_QKV && row0 + tid < p.M) {
+        const int m = row0 + tid, st = stream_of(m), cached = p.suffix_len[st];
         s_pos[tid] = p.pos_base + cached + p.depth[m];
         s_dst[tid] = (size_t)st * p.kv_stream_stride + (size_t)(cached + m - st * p.rows_per_stream) * p.hd;
       }
@@ -449,7 +454,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       for (int j = 0; j < CH; ++j)
         if (n_ok && row0 + c0 + j < p.M) x_old[j] = __ldcg(p.resid + (size_t)(row0 + c0 + j) * p.N + n);
     };
-    if (p.epi == EPI_RESID) {
+    if (EPI == EPI_RESID) {
       prefetch_resid(c_lo);
       if (p.xg_out != nullptr && n_ok) gain = __half2float(__ldg(p.gain_next + n));
     }
@@ -495,11 +500,11 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
 #pragma unroll
         for (int j = 0; j < CH; ++j) v[j] *= s_inv[c0 + j];
       }
-      if (p.epi == EPI_F32) {
+      if constexpr (EPI == EPI_F32) {
 #pragma unroll
         for (int j = 0; j < CH; ++j)
           if (n_ok && row0 + c0 + j < p.M) p.out_f32[(size_t)(row0 + c0 + j) * p.ldo + n] = v[j];
-      } else if (p.epi == EPI_QKV) {
+      } else if constexpr (EPI == EPI_QKV) {
         // RoPE on q and k (pairs (i, i + hd/2): 16 lanes on), fp16, q to its matrix, k and v into the stream's cache
         int seg = 0, col = 0;
         if (n_ok) map_col(p.mode, n, p.seg_n0, p.seg_n1, seg, col);
@@ -525,7 +530,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
           for (int j = 0; j < CH; ++j)
             if (j < rows) dst[seg == 0 ? (size_t)j * p.seg_n0 : s_dst[c0 + j]] = __float2half_rn(v[j]);
         }
-      } else if (p.epi == EPI_SWIGLU) {
+      } else if constexpr (EPI == EPI_SWIGLU) {
         // lanes 0-15 hold a gate tile's features, lanes 16-31 the up tile's: of every two rows the lower half takes the
         // first, the upper half the second
         const bool lo = lane < 16;
@@ -626,7 +631,7 @@ static cudaError_t encode_row_map(const __half* base, int ld, int M, int nrows, 
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int NR, int S>
+template <int NR, int S, int EPI>
 static cudaError_t tc_launch(const GemmArgs& a, int sm_count, int* status, cudaStream_t st) {
   CUtensorMap map, tmap;
   cudaError_t e = encode_row_map(a.h, a.K, a.M, NR, &map);
@@ -637,7 +642,8 @@ static cudaError_t tc_launch(const GemmArgs& a, int sm_count, int* status, cudaS
   cudaLaunchConfig_t cfg{};
   // one CTA (or cluster) a tile; CTAs that have their K to themselves stay and take further tiles
   const int tiles = (a.N + TC_BM - 1) / TC_BM * ((a.M + NR - 1) / NR);
-  cfg.gridDim = dim3(S, (unsigned)(S == 1 && tiles > sm_count * TcCfg<NR>::OCC ? sm_count * TcCfg<NR>::OCC : tiles));
+  if (S == 1 && tiles > sm_count * TcCfg<NR>::OCC) cfg.gridDim = dim3(1, (unsigned)(sm_count * TcCfg<NR>::OCC));
+  else cfg.gridDim = dim3(S, (unsigned)((a.N + TC_BM - 1) / TC_BM), (unsigned)((a.M + NR - 1) / NR));
   cfg.blockDim = dim3(TcCfg<NR>::THREADS); cfg.dynamicSmemBytes = TcCfg<NR>::SMEM; cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -646,7 +652,7 @@ static cudaError_t tc_launch(const GemmArgs& a, int sm_count, int* status, cudaS
   attr[1].val.clusterDim.x = S; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = S > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, w4_gemm_tc_kernel<NR, S>, a, status, map, tmap);
+  return cudaLaunchKernelEx(&cfg, w4_gemm_tc_kernel<NR, S, EPI>, a, status, map, tmap);
 }
 
 #define TC_FOR_EACH(X) \
@@ -654,10 +660,12 @@ static cudaError_t tc_launch(const GemmArgs& a, int sm_count, int* status, cudaS
   X(128, 1) X(128, 2) X(128, 4) X(128, 8) X(256, 1) X(256, 2) X(256, 4) X(256, 8)
 cudaError_t init_gemm_tc() {
   cudaError_t e;
-#define TC_ATTR(NR, S) \
-  if ((e = cudaFuncSetAttribute(w4_gemm_tc_kernel<NR, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<NR>::SMEM)) != cudaSuccess) return e;
+#define TC_ATTR1(NR, S, EPI) \
+  if ((e = cudaFuncSetAttribute(w4_gemm_tc_kernel<NR, S, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<NR>::SMEM)) != cudaSuccess) return e;
+#define TC_ATTR(NR, S) TC_ATTR1(NR, S, EPI_F32) TC_ATTR1(NR, S, EPI_RESID) TC_ATTR1(NR, S, EPI_SWIGLU) TC_ATTR1(NR, S, EPI_QKV)
   TC_FOR_EACH(TC_ATTR)
 #undef TC_ATTR
+#undef TC_ATTR1
   return cudaSuccess;
 }
 
@@ -694,10 +702,16 @@ static void tc_plan(const GemmArgs& a, int sm_count, int& nr, int& split) {
 }
 
 // `status` may be nullptr
-cudaError_t launch_gemm_tc(const GemmArgs& a, int sm_count, int* status, cudaStream_t st) {
+cudaError_t launch_gemm_tc(const GemmArgs& args, int sm_count, int* status, cudaStream_t st) {
+  GemmArgs a = args;
+  const unsigned T = (unsigned)(a.epi == EPI_QKV ? a.rows_per_stream : (a.lora.adapter_idx != nullptr ? a.lora.rows_per_stream : 1));
+  a.stream_magic = T > 1 ? 0xffffffffu / T + 1u : 0u;      // exact for m, T below 65536
   int nr = 32, split = 1;
   tc_plan(a, sm_count, nr, split);
-#define TC_CASE(NR, S) if (nr == NR && split == S) return tc_launch<NR, S>(a, sm_count, status, st);
+#define TC_CASE(NR, S) \
+  if (nr == NR && split == S) \
+    return a.epi == EPI_F32 ? tc_launch<NR, S, EPI_F32>(a, sm_count, status, st) : a.epi == EPI_RESID ? tc_launch<NR, S, EPI_RESID>(a, sm_count, status, st) \
+         : a.epi == EPI_SWIGLU ? tc_launch<NR, S, EPI_SWIGLU>(a, sm_count, status, st) : tc_launch<NR, S, EPI_QKV>(a, sm_count, status, st);
   TC_FOR_EACH(TC_CASE)
 #undef TC_CASE
   return cudaErrorInvalidValue;

@@ -130,6 +130,8 @@ struct GemmArgs {
   const int32_t *suffix_len, *depth;
   size_t kv_stream_stride, kv_head_stride;
   int hd, pos_base, rows_per_stream;
+  const unsigned char* pf_w;      // packed weights of the projection that runs next: asked for in L2 (pf_bytes of them)
+  unsigned pf_bytes;
   unsigned stream_magic;          // set by the launcher: ceil(2^32 / rows per stream), 0 for one row per stream
 };
 

@@ -34,6 +34,7 @@ void free_packed(PackedWeight& w) {
 }
 
 constexpr int PREFILL_ROWS = 2048;                 // rows of one causal prefill pass
+constexpr int PREFETCH_ROWS = 512;                 // passes up to this many rows prefetch the next projection's weights
 constexpr int MAX_FORECAST = 8, MAX_DRAFT_WIDTH = 32;
 
 struct GraphKey {
@@ -488,11 +489,19 @@ int forward_rows(mlora_ctx* c, PassIO& io) {
     CK(run(c, MLORA_PROF_GEMM, [&] { return launch_gemm_tc(g, c->sm_count, c->status, st); }));
     return MLORA_OK;
   };
+  // passes that wait for their weights rather than for the tensor cores: each projection asks for the next one's in L2
+  auto prefetch = [&](GemmArgs& g, const PackedWeight* w) {
+    if (M > PREFETCH_ROWS || w == nullptr || w->data == nullptr) return;
+    const WLayout wl = make_wlayout(w->K, w->N, w->G);
+    const unsigned long long bytes = (unsigned long long)wl.NT * wl.unit_bytes;
+    g.pf_w = w->data; g.pf_bytes = (unsigned)(bytes < LEAN_PF_MAX_BYTES ? bytes : LEAN_PF_MAX_BYTES);
+  };
   int rc;
   for (int l = 0; l < c->L; ++l) {
     {
       const int projs[3] = {0, 1, 2}, widths[3] = {c->Nq, c->Nkv, c->Nkv};
       GemmArgs g{};
+      prefetch(g, &c->w_o[l]);
       g.mode = MODE_QKV; g.epi = EPI_QKV; g.seg_n0 = c->Nq; g.seg_n1 = c->Nkv; g.q_out = c->q16;
       kv_destination(c, io, l, g.k_out, g.v_out, g.kv_stream_stride, g.kv_head_stride);
       g.cs_table = c->cs_table; g.suffix_len = io.suffix_len; g.depth = c->depth; g.hd = d.head_dim; g.pos_base = io.pos_base;
@@ -504,6 +513,7 @@ int forward_rows(mlora_ctx* c, PassIO& io) {
     {
       const int projs[1] = {3}, widths[1] = {dm};
       GemmArgs g{};
+      prefetch(g, &c->w_gateup[l]);
       g.mode = MODE_PLAIN; g.epi = EPI_RESID; g.resid = c->X;
       g.xg_out = c->h_ffn; g.gain_next = c->rms_ffn[l]; g.ssq_out = c->row_ssq + (size_t)(2 * l + 1) * ld_ssq;
       if ((rc = project(g, c->w_o[l], c->attn16, l, 1, projs, widths)) != MLORA_OK) return rc;
@@ -511,6 +521,7 @@ int forward_rows(mlora_ctx* c, PassIO& io) {
     {
       const int projs[2] = {4, 5}, widths[2] = {F, F};
       GemmArgs g{};
+      prefetch(g, &c->w_down[l]);
       g.mode = MODE_GATEUP; g.epi = EPI_SWIGLU; g.out_f16 = c->act16;
       g.ssq_in = c->row_ssq + (size_t)(2 * l + 1) * ld_ssq;
       if ((rc = project(g, c->w_gateup[l], c->h_ffn, l, 2, projs, widths)) != MLORA_OK) return rc;
@@ -518,6 +529,7 @@ int forward_rows(mlora_ctx* c, PassIO& io) {
     {
       const int projs[1] = {6}, widths[1] = {dm};
       GemmArgs g{};
+      prefetch(g, l + 1 < c->L ? &c->w_qkv[l + 1] : (io.logits != nullptr ? &c->w_lm : nullptr));
       g.mode = MODE_PLAIN; g.epi = EPI_RESID; g.resid = c->X;
       const __half* gain = l + 1 < c->L ? c->rms_attn[l + 1] : (const __half*)d.rms_final;
       if (gain != nullptr) { g.xg_out = c->h; g.gain_next = gain; g.ssq_out = c->row_ssq + (size_t)(2 * l + 2) * ld_ssq; }

@@ -94,8 +94,10 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       if (p.mode == MODE_GATEUP) { x.seg0 = 0; seg1 = 1; }
       nseg_in = seg1 - x.seg0 + 1;
     }
-    const int total = L.KT + x.nE * nseg_in;
-    x.u0 = (total * rank) / S; x.u1 = (total * (rank + 1)) / S;
+    // (an expand step counts as three: two activation tiles, and its weights are not on their way long before)
+    const int ext = x.nE * nseg_in, total = L.KT + 3 * ext;
+    auto cut = [&](int q) { const int w = (total * q) / S; return w <= L.KT ? w : (q == S ? L.KT + ext : L.KT + (w - L.KT) / 3); };
+    x.u0 = cut(rank); x.u1 = cut(rank + 1);
     return x;
   };
   // n-tile (16 features) of the slab that lanes 16 h .. 16 h + 15 of accumulator quarter q hold: consecutive ones; with
@@ -125,6 +127,14 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base_s, 0);
   bool alive = true;
+  // this CTA's share of the next projection's weights, asked for in L2: that kernel starts when this one is done and then
+  // finds its first tiles a short trip away (from HBM they took 1.8 us of a 9 us CTA)
+  if (tid == TC_WARPS * 32 + 32 && p.pf_bytes != 0) {
+    const unsigned n_cta = gridDim.x * gridDim.y * gridDim.z, cta = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    const unsigned per = ((p.pf_bytes / n_cta) + 15u) & ~15u, b0 = per * cta, b1 = min(b0 + per, p.pf_bytes & ~15u);
+    for (unsigned o = b0; o < b1; o += 16384u)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.pf_w + o), "r"(min(b1 - o, 16384u)) : "memory");
+  }
 
   if (warp == TC_WARPS) {
     // ---- activation copies (the warp waits, an elected lane issues): x = multiples of 64 features, rows m0 ..
@@ -289,6 +299,20 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       asm volatile("cp.async.commit_group;" ::: "memory");
       f_dst = f_dst + TC_WSLOT == ring_end ? ring0 : f_dst + TC_WSLOT;
     };
+    // lane l looks up the addresses (column 0) of B's rows for the (slot, rank index) pairs k0 + l and k0 + 32 + l
+    auto expand_rows = [&](int seg, int k0, unsigned long long (&adr)[2]) {
+      const int r = p.lora.rank, ldb = p.lora.seg[seg].n;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = k0 + h * 32 + lane, s = k / r, j = k - s * r;
+        adr[h] = 0ull;
+        if (s < p.lora.k_slots) {
+          const int a = p.lora.slot_is_adapter ? s : __ldg(p.lora.adapter_idx + s);
+          const __half* B = (a >= 0 && a < p.lora.n_slots) ? p.lora.tabB[(size_t)a * p.lora.tab_stride + p.lora.seg[seg].proj_index] : nullptr;
+          if (B != nullptr) adr[h] = (unsigned long long)(B + (size_t)j * ldb);
+        }
+      }
+    };
     uint32_t slot = ring0;                                // ring slot consumed next
     const uint32_t ae = tc_smem_u32(a_empty), af = tc_smem_u32(a_full);
     const uint32_t lane_t = tmem + NR + ((uint32_t)(wq * 32) << 16);
@@ -365,17 +389,8 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
         // 64 (slot, rank index) pairs of the expand: lane = output feature, two rank
         // indices a column
         const int e = u0 + i - L.KT, sg = (e >= x.nE) + (e >= 2 * x.nE), seg = x.seg0 + sg, k0 = x.kb0 + (e - sg * x.nE) * 64;
-        const int r = p.lora.rank, ldb = p.lora.seg[seg].n;
-        // lane l looks up the element addresses of pairs k0 + l and k0 + 32 + l (column 0); the loop below hands them round
-        // and issues its loads independently of one another
-        auto address_of = [&](int k) -> unsigned long long {
-          const int s = k / r, j = k - s * r;
-          if (s >= p.lora.k_slots) return 0ull;
-          const int a = p.lora.slot_is_adapter ? s : __ldg(p.lora.adapter_idx + s);
-          const __half* B = (a >= 0 && a < p.lora.n_slots) ? p.lora.tabB[(size_t)a * p.lora.tab_stride + p.lora.seg[seg].proj_index] : nullptr;
-          return B ? (unsigned long long)(B + (size_t)j * ldb) : 0ull;
-        };
-        const unsigned long long adr[2] = {address_of(k0 + lane), address_of(k0 + 32 + lane)};
+        unsigned long long adr[2];
+        expand_rows(seg, k0, adr);
         // [64 pairs][32 features] through the warp's ring (its weight steps are all done): 16-byte pieces in, columns out
         {
           const int piece = lane & 3, n = x.slab * TC_BM + ntile_of(wq, piece >> 1) * TILE_N + (piece & 1) * 8;

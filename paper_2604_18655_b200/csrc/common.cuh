@@ -401,6 +401,7 @@ cudaError_t launch_quant_act(const __half* x, long long count, float scale, sign
 bool w4a8_shape_ok(int M, int K, int N);
 cudaError_t launch_w4a8(const unsigned char* w, const __half* ws, const signed char* x, float x_scale, int M, int K, int N,
                         float* y, cudaStream_t st);
+cudaError_t launch_hidden_out(const float* src, float* dst, size_t count, int32_t* suffix_len, int n, cudaStream_t st);
 cudaError_t launch_copy_rows_f32(const float* src, float* dst, size_t count, cudaStream_t st);
 
 // ----------------------------------------------------------------------------- device helpers

@@ -1241,7 +1241,8 @@ static int decode_impl(mlora_ctx* c, int n, const int32_t* adapter_idx, const in
     if (c->d.vocab > 0) {
       CK(run(c, MLORA_PROF_MISC, [&] { return launch_argmax(io.logits, n, c->d.vocab, out_next, c->stream); }));
     } else {
-      CK(run(c, MLORA_PROF_MISC, [&] { return launch_copy_rows_f32(c->X, hidden_out, (size_t)n * c->d.d_model, c->stream); }));
+      CK(run(c, MLORA_PROF_MISC, [&] { return launch_hidden_out(c->X, hidden_out, (size_t)n * c->d.d_model, c->suffix_len, n, c->stream); }));
+      return MLORA_OK;
     }
     CK(run(c, MLORA_PROF_MISC, [&] { return launch_advance(c->suffix_len, nullptr, n, 1, c->stream); }));
     return MLORA_OK;

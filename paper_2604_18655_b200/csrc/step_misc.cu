@@ -357,4 +357,19 @@ cudaError_t launch_copy_rows_f32(const float* src, float* dst, size_t count, cud
   return cudaGetLastError();
 }
 
+// the end of a decode step that hands hidden states out: the residual rows to the caller, suffix lengths one further
+__global__ void hidden_out_kernel(const float4* __restrict__ src, float4* __restrict__ dst, int count4, int32_t* __restrict__ suffix_len, int n) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count4; i += gridDim.x * blockDim.x) dst[i] = src[i];
+  if (blockIdx.x == 0 && (int)threadIdx.x < n) suffix_len[threadIdx.x] += 1;
+}
+cudaError_t launch_hidden_out(const float* src, float* dst, size_t count, int32_t* suffix_len, int n, cudaStream_t st) {
+  if (n > 256 || count % 4 || count >= (1u << 30) || (reinterpret_cast<uintptr_t>(dst) & 15)) {   // (rows of a multiple of 64 features)
+    const cudaError_t e = launch_copy_rows_f32(src, dst, count, st);
+    return e != cudaSuccess ? e : launch_advance(suffix_len, nullptr, n, 1, st);
+  }
+  const int blocks = (int)((count / 4 + 255) / 256);
+  hidden_out_kernel<<<blocks < 1024 ? blocks : 1024, 256, 0, st>>>(reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(dst), (int)(count / 4), suffix_len, n);
+  return cudaGetLastError();
+}
+
 }  // namespace mlora

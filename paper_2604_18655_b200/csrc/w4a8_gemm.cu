@@ -34,7 +34,7 @@ __device__ __forceinline__ uint32_t nib_to_s8(uint32_t v) { return __vsub4(v & 0
 
 template <int NT>
 __global__ void __launch_bounds__(WA_THREADS) w4a8_kernel(const unsigned char* __restrict__ qw, const __half* __restrict__ w_scale,
-                                                         const signed char* __restrict__ qx, float x_scale, int M, int K, int N,
+                                                         const signed char* qx, float x_scale, int M, int K, int N,
                                                          float* __restrict__ y) {
   __shared__ int red[WA_WARPS][NT][32][4];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -45,14 +45,24 @@ __global__ void __launch_bounds__(WA_THREADS) w4a8_kernel(const unsigned char* _
   const unsigned char* w_lo = qw + (size_t)(n0 + g) * (K / 2);
   const unsigned char* w_hi = qw + (size_t)(n0 + g + 8) * (K / 2);
   const int spans = K / WA_SPAN;
-#pragma unroll 2
+  // the next span's weights are always in flight; the first ones before the wait for the kernel ahead (programmatic launch:
+  // usually the quantisation of the activations), which has no hand in them
+  uint32_t nl[8], nh[8];
+  auto load = [&](int sp) {
+    const int k0 = sp * WA_SPAN + t * 64;
+    *reinterpret_cast<uint4*>(nl) = ldg_nc16(w_lo + k0 / 2);
+    *reinterpret_cast<uint4*>(nl + 4) = ldg_nc16(w_lo + k0 / 2 + 16);
+    *reinterpret_cast<uint4*>(nh) = ldg_nc16(w_hi + k0 / 2);
+    *reinterpret_cast<uint4*>(nh + 4) = ldg_nc16(w_hi + k0 / 2 + 16);
+  };
+  if (warp < spans) load(warp);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   for (int sp = warp; sp < spans; sp += WA_WARPS) {
     const int k0 = sp * WA_SPAN + t * 64;
     uint32_t wl[8], wh[8];
-    *reinterpret_cast<uint4*>(wl) = ldg_nc16(w_lo + k0 / 2);
-    *reinterpret_cast<uint4*>(wl + 4) = ldg_nc16(w_lo + k0 / 2 + 16);
-    *reinterpret_cast<uint4*>(wh) = ldg_nc16(w_hi + k0 / 2);
-    *reinterpret_cast<uint4*>(wh + 4) = ldg_nc16(w_hi + k0 / 2 + 16);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { wl[i] = nl[i]; wh[i] = nh[i]; }
+    if (sp + WA_WARPS < spans) load(sp + WA_WARPS);
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
       const int row = nt * 8 + g;
@@ -60,7 +70,7 @@ __global__ void __launch_bounds__(WA_THREADS) w4a8_kernel(const unsigned char* _
       if (row < M) {
         const signed char* xr = qx + (size_t)row * K + k0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) *reinterpret_cast<uint4*>(xs + 4 * q) = __ldg(reinterpret_cast<const uint4*>(xr) + q);
+        for (int q = 0; q < 4; ++q) *reinterpret_cast<uint4*>(xs + 4 * q) = *(reinterpret_cast<const uint4*>(xr) + q);
       } else {
 #pragma unroll
         for (int q = 0; q < 16; ++q) xs[q] = 0u;
@@ -90,17 +100,29 @@ __global__ void __launch_bounds__(WA_THREADS) w4a8_kernel(const unsigned char* _
   }
 }
 
-// per-tensor INT8 activations: q = clip(round_half_even(x / scale), -127, 127), the division in float32
-__global__ void quant_act_kernel(const __half* __restrict__ x, long long count, float scale, signed char* __restrict__ out) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  int q = __float2int_rn(__fdiv_rn(__half2float(x[i]), scale));
+// per-tensor INT8 activations: q = clip(round_half_even(x / scale), -127, 127), the division in float32; eight values a thread
+__device__ __forceinline__ unsigned quant_act(__half x, float scale) {
+  int q = __float2int_rn(__fdiv_rn(__half2float(x), scale));
   q = q > 127 ? 127 : (q < -127 ? -127 : q);
-  out[i] = (signed char)q;
+  return (unsigned)q & 0xffu;
+}
+__global__ void quant_act_kernel(const __half* __restrict__ x, long long count, float scale, signed char* __restrict__ out) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (a projection behind it may ask for its weights)
+  const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 8;
+  if (i + 8 <= count && ((reinterpret_cast<uintptr_t>(x) & 15) | (reinterpret_cast<uintptr_t>(out) & 7)) == 0) {
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(x + i));
+    const __half* h = reinterpret_cast<const __half*>(&v);
+    uint2 o = make_uint2(0u, 0u);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { o.x |= quant_act(h[e], scale) << (8 * e); o.y |= quant_act(h[4 + e], scale) << (8 * e); }
+    *reinterpret_cast<uint2*>(out + i) = o;
+  } else {
+    for (long long k = i; k < i + 8 && k < count; ++k) out[k] = (signed char)quant_act(x[k], scale);
+  }
 }
 
 cudaError_t launch_quant_act(const __half* x, long long count, float scale, signed char* out, cudaStream_t st) {
-  quant_act_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(x, count, scale, out);
+  quant_act_kernel<<<(unsigned)((count + 1023) / 1024), 128, 0, st>>>(x, count, scale, out);
   return cudaGetLastError();
 }
 
@@ -112,12 +134,17 @@ bool w4a8_shape_ok(int M, int K, int N) {
 
 cudaError_t launch_w4a8(const unsigned char* w, const __half* ws, const signed char* x, float x_scale, int M, int K, int N,
                         float* y, cudaStream_t st) {
-  const dim3 grid((unsigned)(N / WA_CH));
-  if (M <= 8) w4a8_kernel<1><<<grid, WA_THREADS, 0, st>>>(w, ws, x, x_scale, M, K, N, y);
-  else if (M <= 16) w4a8_kernel<2><<<grid, WA_THREADS, 0, st>>>(w, ws, x, x_scale, M, K, N, y);
-  else if (M <= 32) w4a8_kernel<4><<<grid, WA_THREADS, 0, st>>>(w, ws, x, x_scale, M, K, N, y);
-  else w4a8_kernel<8><<<grid, WA_THREADS, 0, st>>>(w, ws, x, x_scale, M, K, N, y);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(N / WA_CH)); cfg.blockDim = dim3(WA_THREADS); cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (M <= 8) return cudaLaunchKernelEx(&cfg, w4a8_kernel<1>, w, ws, x, x_scale, M, K, N, y);
+  if (M <= 16) return cudaLaunchKernelEx(&cfg, w4a8_kernel<2>, w, ws, x, x_scale, M, K, N, y);
+  if (M <= 32) return cudaLaunchKernelEx(&cfg, w4a8_kernel<4>, w, ws, x, x_scale, M, K, N, y);
+  return cudaLaunchKernelEx(&cfg, w4a8_kernel<8>, w, ws, x, x_scale, M, K, N, y);
 }
 
 }  // namespace mlora

@@ -1277,7 +1277,9 @@ static cudaError_t launch_attn_hd(const AttnArgs& a, cudaStream_t st) {
 }
 
 cudaError_t init_attention() {
-  cudaError_t e = cudaFuncSetAttribute(attn_partial_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e;
+  if ((e = full_carveout(attn_merge_kernel)) != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(attn_partial_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)((ATT_ROWS + 4 * ATT_KEYS) * (64 + 8) * sizeof(__half)));
   if (e != cudaSuccess) return e;
   // (+ room for the o adapter's rows over a kv head's features, up to the limit of a CTA)

@@ -477,6 +477,7 @@ cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
 cudaError_t init_attention_tc() {
   cudaError_t e;
 #define AT_ATTR(HD, NQ) \
+  if ((e = full_carveout(attn_tc_kernel<HD, NQ>)) != cudaSuccess) return e; \
   if ((e = cudaFuncSetAttribute(attn_tc_kernel<HD, NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AtCfg<HD, NQ>::SMEM)) != cudaSuccess) return e;
   AT_ATTR(64, 1) AT_ATTR(64, 2) AT_ATTR(128, 1) AT_ATTR(128, 2)
 #undef AT_ATTR

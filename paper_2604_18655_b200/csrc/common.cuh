@@ -314,6 +314,13 @@ constexpr int STEP_TMAP_BYTES = 128;
 cudaError_t step_encode_slice_map(const void* base, int width, int rank, void* map_out);
 cudaError_t launch_step(const StepArgs& a, int sm_count, cudaStream_t st);
 
+// Kernels that run next to one another through programmatic launches all ask for the largest shared-memory share of an SM:
+// with different shares the SM has to drain before the next kernel's CTAs can start on it.
+template <class K>
+inline cudaError_t full_carveout(K* kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
+
 // ----------------------------------------------------------------------------- launchers
 cudaError_t init_gemm();        // opt-in shared-memory sizes; call once per process before the first launch
 cudaError_t init_shrink();
@@ -333,6 +340,7 @@ cudaError_t launch_gemm_tc(const GemmArgs& a, int sm_count, int* status, cudaStr
 cudaError_t launch_shrink(const ShrinkArgs& a, cudaStream_t st);
 // T of a pass whose rows are grouped by stream (rows_per_stream each), from fp16 rows, on mma.sync
 cudaError_t launch_shrink_rows(const ShrinkArgs& a, cudaStream_t st);
+cudaError_t launch_shrink_gather(const ShrinkArgs& a, cudaStream_t st);
 bool tensor_maps_available();
 cudaError_t launch_embed(const int32_t* tokens, const __half* embed, const __half* hidden_in, float* X, int M,
                          int d, int vocab, int* status, cudaStream_t st, const __half* forecast = nullptr,

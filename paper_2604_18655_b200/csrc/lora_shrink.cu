@@ -199,15 +199,156 @@ cudaError_t launch_shrink_rows(const ShrinkArgs& a, cudaStream_t st) {
   cfg.gridDim = dim3((unsigned)((a.M + T - 1) / T * tps), (unsigned)(a.lora.nseg * ((a.lora.rank + 7) / 8)));
   cfg.blockDim = dim3(SHRINK_MMA_WARPS * 32);
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  // Small grids: start beside the projection that is still running, whose SMs have the largest shared-memory share
+  // (with another share they would have to drain first; llama1b verify 2.64 -> 2.52 ms).  Larger grids only take room from
+  // the projection behind (llama3b, 192 CTAs: 7.82 -> 8.01 ms).
+  attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  attr[1].val.sharedMemCarveout = 100;
   cfg.attrs = attr;
-  cfg.numAttrs = a.pdl ? 1 : 0;
+  cfg.numAttrs = a.pdl ? ((long long)cfg.gridDim.x * cfg.gridDim.y <= 96 ? 2 : 1) : 0;
   return cudaLaunchKernelEx(&cfg, shrink_mma_kernel, a, tps);
 }
 
+// The same for rows that pick their adapters one by one (the single-projection call): a CTA takes an adapter, eight of its
+// rank indices and a share of K, finds the rows that use the adapter, and keeps its fragments of A in registers over them,
+// 16 rows at a time.  The S CTAs of a cluster split K; the first one adds their sums up in rank order.  (One row per CTA read
+// every adapter once per row: 115 MB through L2 and 18 us for 250 rows of 14336 inputs and 8 adapters.)
+constexpr int SG_BLOCKS = 2;                 // 64-feature blocks of a warp per CTA: K share = 16 warps x 2 x 64 at most
+constexpr int SG_MAX_ROWS = 4096;
+template <int S>
+__global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_gather_kernel(const ShrinkArgs p) {
+  __shared__ float red[SHRINK_MMA_WARPS][32][4];
+  __shared__ float part[S][128];             // first CTA of a cluster: the CTAs' sums of a group of 16 rows
+  __shared__ short rows[SG_MAX_ROWS];
+  __shared__ int s_n, s_w[SHRINK_MMA_WARPS];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int rank = S > 1 ? (int)blockIdx.x : 0, j0 = blockIdx.y * 8, a = blockIdx.z, r = p.lora.rank, K = p.K;
+  const __half* const A = p.lora.tabA[(size_t)a * p.lora.tab_stride + p.lora.seg[0].proj_index];
+  const float s = p.lora.scale[a];
+  // this warp's blocks of A, while the rows are looked up
+  const int nblk = K / 64, b_lo = (nblk * (rank * SHRINK_MMA_WARPS + warp)) / (S * SHRINK_MMA_WARPS), b_hi = (nblk * (rank * SHRINK_MMA_WARPS + warp + 1)) / (S * SHRINK_MMA_WARPS);
+  const uint4* const Ar = reinterpret_cast<const uint4*>(A + (size_t)min(j0 + g, r - 1) * K) + 2 * t;
+  uint4 w[SG_BLOCKS][2];
+#pragma unroll
+  for (int b = 0; b < SG_BLOCKS; ++b)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) w[b][q] = (A != nullptr && b_lo + b < b_hi && j0 + g < r) ? __ldg(Ar + (b_lo + b) * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
+  // rows of the adapter, in rising order (every CTA of a cluster finds the same list); adapter 0's CTAs also see to the rows
+  // without one
+  if (threadIdx.x == 0) s_n = 0;
+  __syncthreads();
+  for (int base = 0; base < p.M; base += SHRINK_MMA_WARPS * 32) {
+    const int m = base + threadIdx.x;
+    const int am = m < p.M ? p.lora.adapter_idx[m] : -1;
+    const bool mine = m < p.M && am == a && A != nullptr;
+    const unsigned bal = __ballot_sync(0xffffffffu, mine);
+    if (lane == 0) s_w[warp] = __popc(bal);
+    __syncthreads();
+    int off = s_n;
+    for (int q = 0; q < warp; ++q) off += s_w[q];
+    if (mine) rows[off + __popc(bal & ((1u << lane) - 1u))] = (short)m;
+    __syncthreads();
+    if (threadIdx.x == 0) { int n = s_n; for (int q = 0; q < SHRINK_MMA_WARPS; ++q) n += s_w[q]; s_n = n; }
+    if (rank == 0 && j0 == 0) {
+      unsigned none = __ballot_sync(0xffffffffu, m < p.M && ((a == 0 && (am < 0 || am >= p.lora.n_slots)) || (am == a && A == nullptr)));
+      for (; none != 0u; none &= none - 1u) text_clear(p.lora, base + warp * 32 + __ffs(none) - 1, 0, 0, 0, lane, 32);
+    }
+    __syncthreads();
+  }
+  const int n = s_n;
+  for (int r0 = 0; r0 < n; r0 += 16) {
+    const int mA = rows[min(r0 + g, n - 1)], mB = rows[min(r0 + g + 8, n - 1)];
+    const uint4* const hA = reinterpret_cast<const uint4*>(p.h_in + (size_t)mA * K) + 2 * t;
+    const uint4* const hB = reinterpret_cast<const uint4*>(p.h_in + (size_t)mB * K) + 2 * t;
+    uint4 va[SG_BLOCKS][2], vb[SG_BLOCKS][2];
+#pragma unroll
+    for (int b = 0; b < SG_BLOCKS; ++b)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const bool ok = b_lo + b < b_hi;
+        va[b][q] = ok ? __ldg(hA + (b_lo + b) * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
+        vb[b][q] = ok ? __ldg(hB + (b_lo + b) * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
+      }
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int b = 0; b < SG_BLOCKS; ++b)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const uint32_t f0[4] = {va[b][q].x, vb[b][q].x, va[b][q].y, vb[b][q].y}, f1[4] = {va[b][q].z, vb[b][q].z, va[b][q].w, vb[b][q].w};
+        mma_16816(acc, f0, w[b][q].x, w[b][q].y);
+        mma_16816(acc, f1, w[b][q].z, w[b][q].w);
+      }
+    for (int b = b_lo + SG_BLOCKS; b < b_hi; ++b)          // (a K share beyond what the registers hold)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const uint4 xa = __ldg(hA + b * 8 + q), xb = __ldg(hB + b * 8 + q), xw = j0 + g < r ? __ldg(Ar + b * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
+        const uint32_t f0[4] = {xa.x, xb.x, xa.y, xb.y}, f1[4] = {xa.z, xb.z, xa.w, xb.w};
+        mma_16816(acc, f0, xw.x, xw.y);
+        mma_16816(acc, f1, xw.z, xw.w);
+      }
+    *reinterpret_cast<float4*>(red[warp][lane]) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    __syncthreads();
+    const int e = warp & 3;                                // threads 0-127: accumulator element e of every lane's fragment
+    float tot = 0.f;
+    if (warp < 4) {
+#pragma unroll
+      for (int q = 0; q < SHRINK_MMA_WARPS; ++q) tot += red[q][lane][e];
+      if constexpr (S > 1) {
+        uint32_t dst;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"((uint32_t)__cvta_generic_to_shared(&part[rank][threadIdx.x])), "r"(0));
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(tot) : "memory");
+      }
+    }
+    if constexpr (S > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (rank == 0 && warp < 4) {
+      if constexpr (S > 1) {
+        tot = 0.f;
+#pragma unroll
+        for (int q = 0; q < S; ++q) tot += part[q][threadIdx.x];
+      }
+      const int k = r0 + g + (e >= 2 ? 8 : 0), j = j0 + 2 * t + (e & 1);
+      if (k < n && j < r) text_store(p.lora, rows[k], 0, a * r + j, s * tot);
+    }
+    if (rank == 0 && j0 == 0 && warp >= 4)
+      for (int k = r0 + warp - 4; k < min(r0 + 16, n); k += SHRINK_MMA_WARPS - 4) text_clear(p.lora, rows[k], 0, a * r, a * r + r, lane, 32);
+    if constexpr (S > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else __syncthreads();
+  }
+}
+
+template <int S>
+static cudaError_t launch_gather(const ShrinkArgs& a, cudaStream_t st) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(S, (unsigned)((a.lora.rank + 7) / 8), (unsigned)a.lora.n_slots);
+  cfg.blockDim = dim3(SHRINK_MMA_WARPS * 32);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = S; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = S > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, shrink_gather_kernel<S>, a);
+}
+// T of rows with adapters of their own (LoraArgs::text, slots = adapters)
+cudaError_t launch_shrink_gather(const ShrinkArgs& a, cudaStream_t st) {
+  // K split so that a warp's share fits its registers, as long as the grid stays within a few CTAs an SM
+  const int per = SHRINK_MMA_WARPS * SG_BLOCKS * 64, ctas = (a.lora.rank + 7) / 8 * a.lora.n_slots;
+  if (a.K > 4 * per && ctas <= 64) return launch_gather<8>(a, st);
+  if (a.K > 2 * per && ctas <= 128) return launch_gather<4>(a, st);
+  if (a.K > per && ctas <= 256) return launch_gather<2>(a, st);
+  return launch_gather<1>(a, st);
+}
+
 cudaError_t init_shrink() {
+  cudaError_t e;
+#define SG_SET(S) \
+  if ((e = full_carveout(shrink_gather_kernel<S>)) != cudaSuccess) return e;
+  SG_SET(1) SG_SET(2) SG_SET(4) SG_SET(8)
+#undef SG_SET
   return cudaFuncSetAttribute(norm_shrink_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
 }
 

@@ -1780,7 +1780,8 @@ int mlora_linear(mlora_weight* w, const void* x, int32_t M, const int32_t* row_a
     }
     ShrinkArgs s{};
     s.h_in = (const __half*)x; s.M = M; s.K = w->w.K; s.lora = la;
-    CK(launch_shrink(s, w->stream));
+    if (la.text != nullptr) CK(launch_shrink_gather(s, w->stream));
+    else CK(launch_shrink(s, w->stream));
   }
   GemmArgs g{};
   g.w = w->w.data; g.K = w->w.K; g.N = w->w.N; g.G = w->w.G; g.h = (const __half*)x; g.M = M;

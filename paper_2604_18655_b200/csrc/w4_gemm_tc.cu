@@ -37,9 +37,9 @@ constexpr float TC_FIX = 4294967296.f, TC_UNFIX = 1.f / 4294967296.f;   // fixed
 // Weight stages in tensor memory (32 columns each, behind the NR accumulator columns), activation tiles, ring depth in
 // visits; the accumulator and the stages fill 256 or 512 columns.
 template <int NR> struct TcCfg {
-  static constexpr int GR = NR == 256 ? 4 : 2, OCC = GR == 2 ? 2 : 1, COLS = GR == 2 ? 256 : 512;
+  static constexpr int GR = NR > 128 ? 4 : 2, OCC = GR == 2 ? 2 : 1, COLS = GR == 2 ? 256 : 512;
   static constexpr int NA = (COLS - NR) / 32 < 8 ? (COLS - NR) / 32 : 8;
-  static constexpr int NB = NR == 32 ? 8 : (NR == 64 ? 6 : 4);
+  static constexpr int NB = NR == 32 ? 8 : (NR <= 96 ? 6 : 4);
   static constexpr int WD = 4;
   static constexpr int THREADS = GR * 128 + 64;       // + one warp for the activation copies, one for the MMAs
   static constexpr size_t SMEM = (size_t)NB * NR * TC_BK * 2 + (size_t)WD * GR * 4 * TC_WSLOT + 1024;
@@ -672,10 +672,11 @@ static cudaError_t tc_launch(const GemmArgs& a, int sm_count, int* status, cudaS
 
 #define TC_FOR_EACH(X) \
   X(32, 1) X(32, 2) X(32, 4) X(32, 8) X(64, 1) X(64, 2) X(64, 4) X(64, 8) \
-  X(128, 1) X(128, 2) X(128, 4) X(128, 8) X(256, 1) X(256, 2) X(256, 4) X(256, 8)
+  X(96, 1) X(192, 1) X(128, 1) X(128, 2) X(128, 4) X(128, 8) X(256, 1) X(256, 2) X(256, 4) X(256, 8)
 cudaError_t init_gemm_tc() {
   cudaError_t e;
 #define TC_ATTR1(NR, S, EPI) \
+  if ((e = full_carveout(w4_gemm_tc_kernel<NR, S, EPI>)) != cudaSuccess) return e; \
   if ((e = cudaFuncSetAttribute(w4_gemm_tc_kernel<NR, S, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<NR>::SMEM)) != cudaSuccess) return e;
 #define TC_ATTR(NR, S) TC_ATTR1(NR, S, EPI_F32) TC_ATTR1(NR, S, EPI_RESID) TC_ATTR1(NR, S, EPI_SWIGLU) TC_ATTR1(NR, S, EPI_QKV)
   TC_FOR_EACH(TC_ATTR)
@@ -696,18 +697,19 @@ bool gemm_tc_eligible(const GemmArgs& a) {
 // and epilogue, what a further wave costs (less where the CTA stays), and the exchange of a split.  The choice it gives is
 // within 1.5 % of the best candidate on average, within 16 % at worst.
 static void tc_plan(const GemmArgs& a, int sm_count, int& nr, int& split) {
-  static const double step1[4] = {0.227, 0.242, 0.286, 0.320}, step2[4] = {0.393, 0.429, 0.538, 0.0};
+  static const int sizes[6] = {32, 64, 96, 128, 192, 256};
+  static const double step1[6] = {0.227, 0.242, 0.264, 0.286, 0.303, 0.320}, step2[6] = {0.393, 0.429, 0.484, 0.538, 0.0, 0.0};
   const int slabs = (a.N + TC_BM - 1) / TC_BM, KT = a.K / TILE_K;
   double best = 1e30;
-  for (int ri = 0; ri < 4; ++ri) {
-    const int R = 32 << ri;
-    if (R > 32 && a.M <= R / 2) break;
-    for (int S = 1; S <= 8; S *= 2) {
+  for (int ri = 0; ri < 6; ++ri) {
+    const int R = sizes[ri], max_split = R == 96 || R == 192 ? 1 : 8;
+    if (ri > 0 && a.M <= sizes[ri - 1]) break;
+    for (int S = 1; S <= max_split; S *= 2) {
       if (S > 1 && KT / S < 4) break;
-      const long long ctas = (long long)slabs * ((a.M + R - 1) / R) * S, per_wave = (long long)sm_count * (R == 256 ? 1 : 2);
+      const long long ctas = (long long)slabs * ((a.M + R - 1) / R) * S, per_wave = (long long)sm_count * (R > 128 ? 1 : 2);
       const long long full = ctas / per_wave, rest = ctas % per_wave;
       const double steps = (KT + S - 1) / S, f = R / 256.0;
-      const double full_t = R == 256 ? step1[ri] : step2[ri], rest_t = rest == 0 ? 0.0 : (rest > sm_count ? step2[ri] : step1[ri]);
+      const double full_t = R > 128 ? step1[ri] : step2[ri], rest_t = rest == 0 ? 0.0 : (rest > sm_count ? step2[ri] : step1[ri]);
       const double more = (double)full + (rest > 0 ? 1 : 0) - 1.0;
       const double cost = steps * (full * full_t + rest_t) + 3.34 + 3.36 * f + (S > 1 ? 2.52 * f : 0.0) + (S == 8 ? 1.6 : 0.0) +
                           more * (S == 1 ? 1.4 + 5.1 * f : 4.8 + 7.8 * f);

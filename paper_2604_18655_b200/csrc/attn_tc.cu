@@ -352,12 +352,12 @@ attn_tc_kernel(const __grid_constant__ AttnArgs p, const int rb_rows, const int 
       __syncwarp();
       if (lane == 0) tc_arrive(tc_smem_u32(p_full + w));
     }
-    // (with two blocks: both, the tiles' memory is about to be reused)
-#pragma unroll
-    for (int q = 0; q < NQ; ++q)
-      if (n_w[q] > 0 && alive) alive = tc_wait(tc_smem_u32(o_done + q), (uint32_t)((n_w[q] - 1) & 1), p.status);
+    if (n_tiles > 0 && alive) alive = tc_wait(tc_smem_u32(o_done + w), (uint32_t)((n_tiles - 1) & 1), p.status);
     alive = __all_sync(0xffffffffu, alive);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    // the tiles' memory is about to be reused: with two blocks both have to be done with it (not by waiting for the other's
+    // o_done: a parity only tells apart phases next to each other, and these warps have not followed that barrier)
+    if constexpr (NQ == 2) asm volatile("bar.sync 1, %0;" ::"n"(NQ * 128) : "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (n_tiles > 0 && alive) {

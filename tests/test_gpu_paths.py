@@ -1,0 +1,109 @@
+"""Edges of the paths that a size decides: row tiles and K splits of the tensor-core projection, the shrink over rows that
+pick their adapters one by one, tensor-core attention (trees, many streams, causal passes of one and two row blocks), and the
+variants of the kernel-per-projection decode path -- each against the CPU oracle."""
+import numpy as np
+import pytest
+
+import gen
+from tests.helpers import check_argmax, compare
+from tests.test_gpu_kernels import dev, mb, run_attention, run_linear  # noqa: F401  (mb: fixture)
+from tests.test_gpu_model import GpuModel, compare_kv, make_pair  # noqa: F401
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+# ------------------------------------------------------------------ projections of many rows
+@pytest.mark.parametrize("M", [9, 32, 33, 64, 65, 96, 97, 128, 129, 192, 193, 256, 257, 385])
+def test_projection_row_tiles(mb, M):
+    """Row counts at the edges of the row tiles, a ragged last column tile (N = 8 x 128 + 16), adapters and base rows."""
+    got, want = run_linear(mb, 512, 1040, 128, M, 8, 16, seed=M)
+    compare(got, want, f"row tiles M{M}")
+
+
+@pytest.mark.parametrize("K,N,G,M", [
+    (256, 16, 64, 9),            # one column tile of 16, the smallest K that is split
+    (4096, 256, 128, 40),        # few columns: the widest split of K
+    (14336, 128, 128, 250),      # the longest K in two row blocks
+    (320, 4096, 64, 700),        # K of an odd number of steps, more tiles than CTAs: each stays for further ones
+    (192, 9600, 64, 180),        # the same with the 192-row tile, fewer steps than weight stages
+    (192, 9600, 64, 90),         # and the 96-row one
+])
+def test_projection_splits_and_persistent_tiles(mb, K, N, G, M):
+    for n_ad, rank in ((0, 0), (3, 8)):
+        got, want = run_linear(mb, K, N, G, M, n_ad, rank, seed=K + N + M + n_ad)
+        compare(got, want, f"projection K{K} N{N} M{M} adapters {n_ad}")
+
+
+@pytest.mark.parametrize("M,n_ad,rank,K", [(9, 1, 1, 256), (17, 40, 12, 1024), (300, 2, 64, 8192), (64, 64, 16, 2112)])
+def test_shrink_of_rows_with_their_own_adapters(mb, M, n_ad, rank, K):
+    """Adapters without a row, with one, with more than the 16 of a group; ranks off the tile of eight; K shares beyond what
+    the registers hold and a K that the warps share unevenly."""
+    got, want = run_linear(mb, K, 256, 64, M, n_ad, rank, seed=M + rank)
+    compare(got, want, f"gather shrink M{M} adapters {n_ad} rank {rank} K{K}")
+
+
+@pytest.mark.parametrize("count", [1, 7, 8, 9, 1023, 1025])
+def test_quantiser_tails(mb, count):
+    from oracle import ref
+    x = np.random.default_rng(count).standard_normal((1, count)).astype(np.float16)
+    for off in (0, 1):           # (an input that starts between 16-byte boundaries)
+        buf = torch.zeros(count + 8, dtype=torch.float16, device="cuda")
+        buf[off:off + count] = dev(x[0])
+        out = torch.zeros(count, dtype=torch.int8, device="cuda")
+        mb.mlora_quantize_act_int8(buf[off:off + count].view(1, count), 0.02, out.view(1, count))
+        torch.cuda.synchronize()
+        assert np.array_equal(out.cpu().numpy().reshape(1, -1), ref.quantize_act_int8(x, 0.02))
+
+
+# ------------------------------------------------------------------ attention
+@pytest.mark.parametrize("n,T,Hq,Hkv,hd,P,suf,branch", [
+    (2, 9, 6, 2, 64, 129, [0, 1], (2, 3)),            # groups of three heads: 126 of a block's 128 rows
+    (3, 33, 5, 1, 128, 128, [127, 128, 5], (4, 4, 3)),   # own segments over a tile's end, two blocks of rows a stream
+    (1, 64, 8, 8, 64, 1, [0], (4, 4, 3)),             # one head a group, the largest tree, a prefix of one key
+    (2, 16, 16, 2, 128, 0, [3, 250], (4, 3)),         # no prefix
+])
+def test_tree_attention_edges(mb, n, T, Hq, Hkv, hd, P, suf, branch):
+    got, want = run_attention(mb, n, T, Hq, Hkv, hd, P, suf, branch, seed=n + T + P)
+    compare(got, want, f"tree attention n{n} T{T} {Hq}q/{Hkv}kv hd{hd} P{P}")
+
+
+@pytest.mark.parametrize("hd,n_q,n_kv,P", [(64, 32, 8, 640), (128, 24, 8, 1025), (128, 16, 8, 2100), (64, 6, 2, 257)])
+def test_causal_passes_of_one_and_two_row_blocks(GpuModel, hd, n_q, n_kv, P):
+    """Two row blocks a CTA from about 600 positions on; the second layer's K/V show every row of the first one's output.
+    2100 positions: a second pass of 52 rows over the first one's keys."""
+    cfg = gen.ModelCfg("causal", 2, 256, n_q, n_kv, hd, 320, 0, 64, 8, 15, 1, 1, P)
+    _, orc, gm = make_pair(GpuModel, cfg, max_suffix=8)
+    prompt = gen.make_hidden(cfg, P, 0, 0)
+    want = orc.prefill_shared(hidden=prompt)
+    compare(gm.prefill_h(prompt), want, "last hidden")
+    for l in range(2):
+        _, pk, pv = gm.export_kv(l, -1, 0, P)
+        compare(pk, orc.prefix_k[l], f"prefix K of layer {l}")
+        compare(pv, orc.prefix_v[l], f"prefix V of layer {l}")
+    gm.close()
+
+
+# ------------------------------------------------------------------ decode
+@pytest.mark.parametrize("d_model,d_ffn,hd,n_q,n_kv,vocab,rank,n,P", [
+    (3072, 4096, 128, 24, 8, 9600, 32, 8, 70),     # single-wave variants, pointer table, lm_head of K = 3072
+    (4096, 1024, 128, 8, 2, 9600, 20, 3, 40),      # a rank off the multiples of 16, lm_head of K = 4096
+    (512, 8192, 64, 8, 8, 304, 16, 5, 33),         # down projection of K = 8192 with few columns
+    (512, 1408, 64, 8, 4, 304, 64, 8, 2101),       # streaming attention + merge with the o projection's shrink, rank 64
+    (256, 512, 128, 4, 1, 304, 8, 2, 2048),
+])
+def test_decode_variants(GpuModel, d_model, d_ffn, hd, n_q, n_kv, vocab, rank, n, P):
+    cfg = gen.ModelCfg("decode", 2, d_model, n_q, n_kv, hd, d_ffn, vocab, 64, rank, gen.configs.ALL7, 3, n, P)
+    _, orc, gm = make_pair(GpuModel, cfg, max_suffix=8)
+    ids = gen.make_prompt_ids(cfg, 0)
+    compare(gm.prefill(ids), orc.prefill_shared(ids, n_streams=n), "prefill logits")
+    ad = [(s % 4) - 1 for s in range(n)]
+    toks = np.arange(3, 3 + n, dtype=np.int32)
+    for step in range(2):
+        nxt, logits = gm.decode(ad, toks)
+        r = orc.decode_step(ad, tokens=toks)
+        compare(logits, r["logits"], f"decode logits, step {step}")
+        check_argmax(nxt, r["logits"], f"step {step}")
+        toks = nxt
+    compare_kv(gm, orc, cfg, n)
+    gm.close()

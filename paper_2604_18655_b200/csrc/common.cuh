@@ -404,6 +404,7 @@ cudaError_t init_lean();
 bool lean_shapes_ok(int d_model, int d_ffn, int Nq, int Nkv, int rank);
 cudaError_t launch_lean_embed(const LeanArgs& a, const StepPhase& ph, const int32_t* tokens, const __half* embed, int vocab,
                               const __half* hidden_in, int* status, cudaStream_t st);
+cudaError_t launch_lean_shrink(const LeanArgs& a, const __half* x, int K, cudaStream_t st);
 cudaError_t launch_lean_gemm(const LeanArgs& a, const StepPhase& ph, cudaStream_t st);
 cudaError_t launch_quant_act(const __half* x, long long count, float scale, signed char* out, cudaStream_t st);
 bool w4a8_shape_ok(int M, int K, int N);

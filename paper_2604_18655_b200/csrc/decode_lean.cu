@@ -206,7 +206,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
     }
   }
   lean_prefetch_slices<NTILE, TAB>(a, ph, tile0, n_out0, lora, row_ptr, sB, sA);
-  pdl_wait();
+  if (!a.late_wait) pdl_wait();
   ln_stamp<TRACE>(a, 1);
   // ---- what earlier kernels produced: the old residual, norm factors, T of this group, the input rows
   float x_old = 0.f, gain_nx = 1.f;
@@ -590,17 +590,13 @@ __global__ void __launch_bounds__(LN_THREADS) lean_embed_kernel(const LeanArgs a
   if (ad < 0 || ad >= a.n_slots) return;
   const int r = a.rank;
   // the CTA's share of the (segment, rank index, 1024-element piece of the row) partial dot products, a warp each
-  // (ph.pad_ = 1: whole dot products, stored: the sums need no zeroing then -- the single-projection call)
-  const int KC = ph.pad_ ? 1 : (d + 1023) / 1024, items = ph.next_nseg * r * KC;
+  const int KC = (d + 1023) / 1024, items = ph.next_nseg * r * KC;
   for (int it = part * LN_WARPS + warp; it < items; it += gridDim.y * LN_WARPS) {
     const int kc = it % KC, j = (it / KC) % r, seg = it / (KC * r);
     const __half* A = a.tabA[(size_t)ad * a.tab_stride + ph.next_proj[seg]];
-    if (A == nullptr) {
-      if (ph.pad_ && lane == 0) a.tacc[((size_t)ph.t_out * CHAIN_MAX_ROWS + m) * 3 * r + seg * r + j] = 0ull;
-      continue;
-    }
+    if (A == nullptr) continue;
     const __half* arow = A + (size_t)j * ph.next_ld;
-    const int k1 = ph.pad_ ? d : min(d, (kc + 1) * 1024);
+    const int k1 = min(d, (kc + 1) * 1024);
     float s = 0.f;
     for (int k = kc * 1024 + lane * 8; k < k1; k += 32 * 8) {
       const uint4 av = __ldg(reinterpret_cast<const uint4*>(arow + k));
@@ -615,12 +611,74 @@ __global__ void __launch_bounds__(LN_THREADS) lean_embed_kernel(const LeanArgs a
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-      unsigned long long* dst = a.tacc + ((size_t)ph.t_out * CHAIN_MAX_ROWS + m) * 3 * r + seg * r + j;
-      if (ph.pad_) *dst = ln_fix(s);
-      else ln_red_add(dst, ln_fix(s));
+    if (lane == 0) ln_red_add(a.tacc + ((size_t)ph.t_out * CHAIN_MAX_ROWS + m) * 3 * r + seg * r + j, ln_fix(s));
+  }
+}
+
+// T of up to eight rows ahead of a single projection: KS warps share a dot product, at most 2048 features a warp, so that a
+// lane's loads (eight pieces of the row, eight of A) are all in flight at once.  Bound by the chain index -> table -> A row.
+// Waits before it lets the projection behind it start: whatever that one reads ahead of its own wait is complete then.
+// Launched programmatically itself although it waits at once: a full dependency between this pair and the call ahead cost
+// several us a call (8 rows of 4096 x 14336 with adapters 25.5 -> 19.2 us, 4 rows of 14336 x 1024 19.8 -> 10.2 us, with the
+// loads of a dot product all in flight).
+template <int KS>
+__global__ void __launch_bounds__(LN_THREADS) lean_shrink_kernel(const LeanArgs a, const __half* x, const int K) {
+  __shared__ float s_part[LN_WARPS];
+  pdl_wait();
+  pdl_launch_dependents();
+  const int m = blockIdx.y, r = a.rank, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int j = blockIdx.x * (LN_WARPS / KS) + warp / KS, q = warp % KS;
+  const int hi = (K / 8) * (q + 1) / KS, i0 = (K / 8) * q / KS + lane;
+  const uint4* const xr = reinterpret_cast<const uint4*>(x + (size_t)m * K);
+  uint4 xv[8], av[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) xv[u] = i0 + u * 32 < hi ? xr[i0 + u * 32] : make_uint4(0u, 0u, 0u, 0u);
+  const int ad = a.adapter_idx[m];
+  if (ad < 0 || ad >= a.n_slots) return;                   // (the projection does not look at such a row's T)
+  const __half* const A = a.tabA[(size_t)ad * a.tab_stride];
+  const uint4* const ar = reinterpret_cast<const uint4*>(A + (size_t)j * K);
+  const bool on = A != nullptr && j < r;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) av[u] = on && i0 + u * 32 < hi ? ar[i0 + u * 32] : make_uint4(0u, 0u, 0u, 0u);
+  float s = 0.f;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const __half2* const ap = reinterpret_cast<const __half2*>(&av[u]);
+    const __half2* const xp = reinterpret_cast<const __half2*>(&xv[u]);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float2 xf = __half22float2(xp[e]), w = __half22float2(ap[e]);
+      s = fmaf(xf.x, w.x, s); s = fmaf(xf.y, w.y, s);
     }
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (KS > 1) {
+    if (lane == 0) s_part[warp] = s;
+    __syncthreads();
+    s = 0.f;
+#pragma unroll
+    for (int w = 0; w < KS; ++w) s += s_part[warp - q + w];
+  }
+  if (lane == 0 && q == 0 && j < r) a.tacc[(size_t)m * 3 * r + j] = ln_fix(s);
+}
+template <int KS>
+static cudaError_t launch_lean_shrink_variant(const LeanArgs& a, const __half* x, int K, cudaStream_t st) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)((a.rank * KS + LN_WARPS - 1) / LN_WARPS), (unsigned)a.M);
+  cfg.blockDim = dim3(LN_THREADS); cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, lean_shrink_kernel<KS>, a, x, K);
+}
+cudaError_t launch_lean_shrink(const LeanArgs& a, const __half* x, int K, cudaStream_t st) {   // K <= 16384
+  if (K <= 2048) return launch_lean_shrink_variant<1>(a, x, K, st);
+  if (K <= 4096) return launch_lean_shrink_variant<2>(a, x, K, st);
+  if (K <= 8192) return launch_lean_shrink_variant<4>(a, x, K, st);
+  return launch_lean_shrink_variant<8>(a, x, K, st);
 }
 
 // the greedy tokens from the lm_head's row maxima, and the suffix lengths one further
@@ -670,7 +728,7 @@ bool lean_shapes_ok(int d_model, int d_ffn, int Nq, int Nkv, int rank) {
 cudaError_t launch_lean_embed(const LeanArgs& a, const StepPhase& ph, const int32_t* tokens, const __half* embed, int vocab,
                               const __half* hidden_in, int* status, cudaStream_t st) {
   // a warp per (segment, rank index, 1024-element piece): enough CTAs per row to give every item its own warp
-  const int items = (a.adapter_idx != nullptr ? ph.next_nseg * a.rank : 0) * (ph.pad_ ? 1 : (ph.N + 1023) / 1024);
+  const int items = (a.adapter_idx != nullptr ? ph.next_nseg * a.rank : 0) * ((ph.N + 1023) / 1024);
   const int gy = items <= LN_WARPS ? 1 : (items + LN_WARPS - 1) / LN_WARPS > 32 ? 32 : (items + LN_WARPS - 1) / LN_WARPS;
   lean_embed_kernel<<<dim3((unsigned)a.M, (unsigned)gy), LN_THREADS, (size_t)ph.N * sizeof(__half), st>>>(a, ph, tokens, embed, vocab, hidden_in, status);
   return cudaGetLastError();

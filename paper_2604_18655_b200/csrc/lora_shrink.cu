@@ -224,7 +224,9 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_gather_kernel(co
   __shared__ float part[S][128];             // first CTA of a cluster: the CTAs' sums of a group of 16 rows
   __shared__ short rows[SG_MAX_ROWS];
   __shared__ int s_n, s_w[SHRINK_MMA_WARPS];
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // (a programmatic launch that waits at once and only then lets the projection start, which reads the activations and B
+  // ahead of its own wait: everything earlier is complete then)
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int rank = S > 1 ? (int)blockIdx.x : 0, j0 = blockIdx.y * 8, a = blockIdx.z, r = p.lora.rank, K = p.K;
   const __half* const A = p.lora.tabA[(size_t)a * p.lora.tab_stride + p.lora.seg[0].proj_index];
@@ -236,7 +238,7 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_gather_kernel(co
 #pragma unroll
   for (int b = 0; b < SG_BLOCKS; ++b)
 #pragma unroll
-    for (int q = 0; q < 2; ++q) w[b][q] = (A != nullptr && b_lo + b < b_hi && j0 + g < r) ? __ldg(Ar + (b_lo + b) * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
+    for (int q = 0; q < 2; ++q) w[b][q] = (A != nullptr && b_lo + b < b_hi && j0 + g < r) ? *(Ar + (b_lo + b) * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
   // rows of the adapter, in rising order (every CTA of a cluster finds the same list); adapter 0's CTAs also see to the rows
   // without one
   if (threadIdx.x == 0) s_n = 0;
@@ -270,8 +272,8 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_gather_kernel(co
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         const bool ok = b_lo + b < b_hi;
-        va[b][q] = ok ? __ldg(hA + (b_lo + b) * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
-        vb[b][q] = ok ? __ldg(hB + (b_lo + b) * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
+        va[b][q] = ok ? *(hA + (b_lo + b) * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
+        vb[b][q] = ok ? *(hB + (b_lo + b) * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
       }
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -285,7 +287,7 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_gather_kernel(co
     for (int b = b_lo + SG_BLOCKS; b < b_hi; ++b)          // (a K share beyond what the registers hold)
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        const uint4 xa = __ldg(hA + b * 8 + q), xb = __ldg(hB + b * 8 + q), xw = j0 + g < r ? __ldg(Ar + b * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
+        const uint4 xa = *(hA + b * 8 + q), xb = *(hB + b * 8 + q), xw = j0 + g < r ? *(Ar + b * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
         const uint32_t f0[4] = {xa.x, xb.x, xa.y, xb.y}, f1[4] = {xa.z, xb.z, xa.w, xb.w};
         mma_16816(acc, f0, xw.x, xw.y);
         mma_16816(acc, f1, xw.z, xw.w);
@@ -326,11 +328,13 @@ static cudaError_t launch_gather(const ShrinkArgs& a, cudaStream_t st) {
   cfg.gridDim = dim3(S, (unsigned)((a.lora.rank + 7) / 8), (unsigned)a.lora.n_slots);
   cfg.blockDim = dim3(SHRINK_MMA_WARPS * 32);
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = S; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = S; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = S > 1 ? 1 : 0;
+  cfg.numAttrs = S > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, shrink_gather_kernel<S>, a);
 }
 // T of rows with adapters of their own (LoraArgs::text, slots = adapters)

@@ -1721,7 +1721,7 @@ int mlora_linear(mlora_weight* w, const void* x, int32_t M, const int32_t* row_a
   if ((size_t)((w->w.N + GEMM_NB - 1) / GEMM_NB) * m_blocks > 4096) return fail(MLORA_ERR_UNSUPPORTED, "too many output blocks");
   unsigned char* ws = (unsigned char*)workspace;
   if (M <= CHAIN_MAX_ROWS && (!lora || rank <= 64) && w->w.K % 64 == 0 && w->w.K <= 16384) {
-    // few rows: a shrink kernel (the rows' dot products with the adapters' A rows, added to fixed-point sums) and the
+    // few rows: a shrink kernel (the rows' dot products with the adapters' A rows) and the
     // projection kernel of the decode path, whose weights are in flight while the shrink runs
     LeanArgs a{};
     a.M = M; a.eps = 0.f;
@@ -1733,14 +1733,7 @@ int mlora_linear(mlora_weight* w, const void* x, int32_t M, const int32_t* row_a
       a.tab_stride = 1; a.n_slots = n_adapters; a.rank = rank; a.rank_log2 = lean_rank_log2(rank);
       a.tacc = (unsigned long long*)(ws + LIN_COUNTER_BYTES + lin_T_bytes(M, rank));
       ph.lora_nseg = 1; ph.lora_proj[0] = 0; ph.lora_n[0] = w->w.N; ph.t_in = 0;
-      StepPhase sh{};
-      sh.kind = SK_EMBED; sh.N = w->w.K; sh.norm_in = -1; sh.ssq_out = -1;
-      // short rows: whole dot products, stored (a row without adapter is never read); long rows: 1024-element pieces
-      // added to sums that a memset zeroes first (measured: 12.8 vs 14.4 us at K = 4096, 35.3 vs 30.7 us at K = 14336)
-      sh.pad_ = w->w.K <= 8192 ? 1 : 0;
-      if (!sh.pad_) CK(cudaMemsetAsync(a.tacc, 0, (size_t)CHAIN_MAX_ROWS * 3 * rank * sizeof(unsigned long long), w->stream));
-      sh.next_nseg = 1; sh.next_proj[0] = 0; sh.next_ld = w->w.K; sh.t_out = 0;
-      CK(launch_lean_embed(a, sh, nullptr, nullptr, 0, (const __half*)x, (int*)(ws + 32), w->stream));
+      CK(launch_lean_shrink(a, (const __half*)x, w->w.K, w->stream));
       a.late_wait = 1;
     }
     CK(launch_lean_gemm(a, ph, w->stream));

@@ -45,8 +45,8 @@ __global__ void __launch_bounds__(WA_THREADS) w4a8_kernel(const unsigned char* _
   const unsigned char* w_lo = qw + (size_t)(n0 + g) * (K / 2);
   const unsigned char* w_hi = qw + (size_t)(n0 + g + 8) * (K / 2);
   const int spans = K / WA_SPAN;
-  // the next span's weights are always in flight; the first ones before the wait for the kernel ahead (programmatic launch:
-  // usually the quantisation of the activations), which has no hand in them
+  // the next span's weights are always in flight; the first ones are asked for in L2 ahead of the wait for the kernel before
+  // this one (programmatic launch; usually the quantisation of the activations)
   uint32_t nl[8], nh[8];
   auto load = [&](int sp) {
     const int k0 = sp * WA_SPAN + t * 64;
@@ -55,8 +55,12 @@ __global__ void __launch_bounds__(WA_THREADS) w4a8_kernel(const unsigned char* _
     *reinterpret_cast<uint4*>(nh) = ldg_nc16(w_hi + k0 / 2);
     *reinterpret_cast<uint4*>(nh + 4) = ldg_nc16(w_hi + k0 / 2 + 16);
   };
+  if (warp < spans) {
+    const size_t o = (size_t)(warp * WA_SPAN + t * 64) / 2;
+    asm volatile("prefetch.global.L2 [%0];\n\tprefetch.global.L2 [%1];" ::"l"(w_lo + o), "l"(w_hi + o) : "memory");
+  }
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
   if (warp < spans) load(warp);
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   for (int sp = warp; sp < spans; sp += WA_WARPS) {
     const int k0 = sp * WA_SPAN + t * 64;
     uint32_t wl[8], wh[8];
@@ -106,11 +110,11 @@ __device__ __forceinline__ unsigned quant_act(__half x, float scale) {
   q = q > 127 ? 127 : (q < -127 ? -127 : q);
   return (unsigned)q & 0xffu;
 }
-__global__ void quant_act_kernel(const __half* __restrict__ x, long long count, float scale, signed char* __restrict__ out) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (a projection behind it may ask for its weights)
+__global__ void quant_act_kernel(const __half* x, long long count, float scale, signed char* out) {
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
   const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 8;
   if (i + 8 <= count && ((reinterpret_cast<uintptr_t>(x) & 15) | (reinterpret_cast<uintptr_t>(out) & 7)) == 0) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(x + i));
+    const uint4 v = *reinterpret_cast<const uint4*>(x + i);
     const __half* h = reinterpret_cast<const __half*>(&v);
     uint2 o = make_uint2(0u, 0u);
 #pragma unroll
@@ -122,8 +126,16 @@ __global__ void quant_act_kernel(const __half* __restrict__ x, long long count, 
 }
 
 cudaError_t launch_quant_act(const __half* x, long long count, float scale, signed char* out, cudaStream_t st) {
-  quant_act_kernel<<<(unsigned)((count + 1023) / 1024), 128, 0, st>>>(x, count, scale, out);
-  return cudaGetLastError();
+  // (programmatic although it waits at once: in a chain of programmatic launches no full dependency, which the device
+  // resolved in steps of 2 us, stands between one call and the next)
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)((count + 1023) / 1024)); cfg.blockDim = dim3(128); cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, quant_act_kernel, x, count, scale, out);
 }
 
 bool w4a8_shape_ok(int M, int K, int N) {

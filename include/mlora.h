@@ -195,14 +195,14 @@ int mlora_debug_dequant(mlora_ctx* ctx, int32_t layer, int32_t proj, void* out_f
  * key 2 = 1 disables CUDA-graph replay of steps (every kernel launched directly).
  * key 3 = 1 runs decode-sized passes through the general split-K kernels (one per operation: norm + shrink, projection,
  *         attention, ...) instead of any of the decode paths of key 6.
- * key 4 = 1 runs passes of 32 rows and more through the split-K mma.sync kernels instead of the tcgen05 projection kernel.
+ * key 4 = 1 runs passes of 9 rows and more through the split-K mma.sync kernels instead of the tcgen05 kernels.
  * key 5 = 1 makes the first wait of the next decode step (paths 1 and 2 of key 6) run out, on a flag nothing sets: the
  *         step returns the timeout status instead of hanging (the test of the bounded waits).
  * key 6 picks the path of decode steps (one row per stream, at most 8 streams): 1 = the per-layer persistent projection
  *         kernel plus attention kernels; 2 = ONE kernel that does the whole step (embedding to greedy token; where the
  *         model's shapes allow it, else the per-layer path); 3 = one small kernel per projection group, launched
- *         programmatically so that each one's weights are in flight while the one before it drains (contexts up to
- *         2047 keys; longer ones take the per-layer path); 0 = the library's choice (3 where it applies: the fastest of
+ *         programmatically so that each one's weights are in flight while the one before it drains (contexts
+ *         beyond 2047 keys with the streaming attention and its merge); 0 = the library's choice (3 where it applies: the fastest of
  *         the three at the 1B / 8-stream shapes).  All are replayed from CUDA graphs.
  * key 7 = 1 makes decode steps of paths 2 and 3 (key 6) record a timeline (see mlora_step_timeline); path 3 then runs
  *         instantiations of its kernels that carry the stamps (the untraced ones carry none). */

@@ -384,18 +384,11 @@ struct LeanArgs {
   unsigned long long* ssq;        // [n_ssq][8]
   long long* trace0;              // timeline of a traced step (nullptr otherwise): 12 slots of this launch for its first CTA
   long long* trace1;              // ... and for its last CTA
-  int rank_log2;                  // log2(rank) when the rank is a power of two, else -1 (index arithmetic by shifts)
   int rows_direct;                // tabA / tabB / scale are indexed by ROW (looked up once per call): adapter_idx is not read
   int late_wait;                  // the kernel ahead produces only T: wait for it after the main loop, not before
   unsigned long long* amax;       // [8]: row maxima of the lm_head as (ordered value, complemented column) keys, zero at
                                   // the start of a step; non-null = no logits are written, the greedy tokens come from here
 };
-inline int lean_rank_log2(int r) {                     // LeanArgs::rank_log2
-  if (r <= 0 || (r & (r - 1)) != 0) return -1;
-  int s = 0;
-  while ((1 << s) < r) ++s;
-  return s;
-}
 cudaError_t launch_lean_rowptr(const int32_t* adapter_idx, const __half* const* tabA, const __half* const* tabB, const float* scale,
                                int n_slots, int tab_stride, int M, const __half** rowA, const __half** rowB, float* rowscale,
                                cudaStream_t st);

@@ -40,91 +40,66 @@ __device__ __forceinline__ void ln_cp_async16(void* smem, const void* gmem, bool
 }
 
 // The adapter slices a CTA needs at its end, asked for at its start (cp.async, behind the main loop):
-//   sB [NTILE][M][r][16]: rows of B of this group for the CTA's columns (the expand);
-//   sA [M][next_nseg][r][16]: rows of A of the consuming group for the CTA's output columns (its partial shrink).
-// A missing adapter or matrix gives zeros.
-// x = q * rank + j by shifts where the rank is a power of two (runtime divisions cost tens of instructions each, and
-// these index computations sit at the start of every CTA and behind its main loop)
-__device__ __forceinline__ void ln_divmod_rank(const LeanArgs& a, int x, int& q, int& j) {
-  if (a.rank_log2 >= 0) { q = x >> a.rank_log2; j = x & (a.rank - 1); }
-  else { q = x / a.rank; j = x - q * a.rank; }
-}
-
-// Items run over all CHAIN_MAX_ROWS rows (row = low three bits of the quotient; rows past M are skipped), so that no
-// index needs a division by the row count.
-// Ranks above LN_PTR_RANK (several items a thread): the rows' matrix pointers, one load a (row, segment), go through shared
-// memory, asked for ahead of everything.  A pointer load in front of every item's copy puts several dependent trips to L2
-// at the start of every CTA (at rank 32 a late CTA of llama3b's gate/up reached its wait 4.9 us after its start, 3.0 with
-// the table); at rank 16 the barrier costs what the trips do (llama1b: 32.6 us a layer without, 32.9 with).
-constexpr int LN_PTR_RANK = 16;
-__device__ __forceinline__ const __half* lean_row_ptr(const LeanArgs& a, const StepPhase& ph) {
-  if (a.adapter_idx == nullptr || threadIdx.x >= 48) return nullptr;
-  const int w = threadIdx.x / 24, seg = (threadIdx.x >> 3) % 3, m = threadIdx.x & 7;   // B of this group, A of the next
-  if (m >= a.M || seg >= (w == 0 ? ph.lora_nseg : ph.next_nseg)) return nullptr;
-  const int ad = a.rows_direct ? m : a.adapter_idx[m];
-  if (ad < 0 || ad >= a.n_slots) return nullptr;
-  return (w == 0 ? a.tabB + ph.lora_proj[seg] : a.tabA + ph.next_proj[seg])[(size_t)ad * a.tab_stride];
-}
-template <int NTILE, bool TAB>
-__device__ __forceinline__ void lean_prefetch_slices(const LeanArgs& a, const StepPhase& ph, int tile0, int n_out0, bool lora,
-                                                     const __half* row_ptr, __half* sB, __half* sA) {
-  __shared__ const __half* s_ptr[48];                       // [B of this group, A of the next][segment][row]
-  const int r = a.rank, M = a.M;
-  if (a.adapter_idx == nullptr) { asm volatile("cp.async.commit_group;" ::: "memory"); return; }
-  if constexpr (TAB) {
-    if (threadIdx.x < 48) s_ptr[threadIdx.x] = row_ptr;
-    __syncthreads();
-  }
-  auto matrix = [&](const __half* const* tab, const int* proj, int s0, int seg, int m) -> const __half* {
-    if constexpr (TAB) return s_ptr[s0 + seg * 8 + m];
+//   sB [NTILE][row][r + 1][16]: rows of B of this group for the CTA's columns (the expand);
+//   sA [next_nseg][row][r + 1][16]: rows of A of the consuming group for the CTA's output columns (its partial shrink).
+// (One piece of padding a row: the expand's warps read two rows at once.)  A missing adapter or matrix gives zeros.  A warp
+// serves one row, its lane pairs a rank index each: no division, and all the matrix pointers of a thread -- at most five --
+// are in flight together.  (With a pointer load in front of every 16-byte piece a late CTA of llama1b's gate/up reached its
+// wait 2.7 us after its start, 1.8 now.)
+template <int NTILE, int THREADS>
+__device__ __forceinline__ void lean_prefetch_slices(const LeanArgs& a, const StepPhase& ph, const int (&seg)[NTILE], const int (&col)[NTILE],
+                                                     int n_out0, bool lora, __half* sB, __half* sA) {
+  const int r = a.rank, hf = threadIdx.x & 1, m = (threadIdx.x >> 5) & (CHAIN_MAX_ROWS - 1);
+  if (a.adapter_idx != nullptr && m < a.M) {
     const int ad = a.rows_direct ? m : a.adapter_idx[m];
-    return (ad >= 0 && ad < a.n_slots) ? tab[(size_t)ad * a.tab_stride + proj[seg]] : nullptr;
-  };
-  const int nB = lora ? NTILE * CHAIN_MAX_ROWS * r * 2 : 0;
-  const int nA = (ph.next_nseg > 0 && a.adapter_idx != nullptr) ? ph.next_nseg * CHAIN_MAX_ROWS * r * 2 : 0;
-  for (int it = threadIdx.x; it < nB; it += blockDim.x) {
-    int q, j;
-    ln_divmod_rank(a, it >> 1, q, j);
-    const int hf = it & 1, m = q & (CHAIN_MAX_ROWS - 1), u = q >> 3;
-    if (m >= M) continue;
-    int seg, col;
-    map_col(ph.mode, (tile0 + u) * TILE_N, ph.seg_n0, ph.seg_n1, seg, col);
-    const __half* B = matrix(a.tabB, ph.lora_proj, 0, seg, m);
-    ln_cp_async16(sB + (((size_t)u * M + m) * r + j) * 16 + hf * 8, B ? B + (size_t)j * ph.lora_n[seg] + col + hf * 8 : (const __half*)ph.w,
-                  B != nullptr);
-  }
-  for (int it = threadIdx.x; it < nA; it += blockDim.x) {
-    int q, j;
-    ln_divmod_rank(a, it >> 1, q, j);
-    const int hf = it & 1, m = q & (CHAIN_MAX_ROWS - 1), seg = q >> 3;
-    if (m >= M) continue;
-    const __half* A = matrix(a.tabA, ph.next_proj, 24, seg, m);
-    ln_cp_async16(sA + (((size_t)m * ph.next_nseg + seg) * r + j) * 16 + hf * 8,
-                  A ? A + (size_t)j * ph.next_ld + n_out0 + hf * 8 : (const __half*)ph.w, A != nullptr);
+    const bool ok = ad >= 0 && ad < a.n_slots;
+    const __half *B[NTILE], *A[3];
+#pragma unroll
+    for (int u = 0; u < NTILE; ++u) B[u] = lora && ok ? a.tabB[(size_t)ad * a.tab_stride + ph.lora_proj[seg[u]]] : nullptr;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) A[q] = q < ph.next_nseg && ok ? a.tabA[(size_t)ad * a.tab_stride + ph.next_proj[q]] : nullptr;
+#pragma unroll 1
+    for (int j = ((threadIdx.x >> 1) & 15) + (threadIdx.x >> 8) * 16; j < r; j += THREADS / 16) {
+      if (lora)
+#pragma unroll
+        for (int u = 0; u < NTILE; ++u)
+          ln_cp_async16(sB + ((u * CHAIN_MAX_ROWS + m) * (r + 1) + j) * 16 + hf * 8,
+                        B[u] ? B[u] + (size_t)j * ph.lora_n[seg[u]] + col[u] + hf * 8 : (const __half*)ph.w, B[u] != nullptr);
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        if (q < ph.next_nseg)
+          ln_cp_async16(sA + ((q * CHAIN_MAX_ROWS + m) * (r + 1) + j) * 16 + hf * 8,
+                        A[q] ? A[q] + (size_t)j * ph.next_ld + n_out0 + hf * 8 : (const __half*)ph.w, A[q] != nullptr);
+    }
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// partial shrink of the consuming group over this CTA's fresh fp16 outputs vals[8][16]: one item per (row, segment,
-// rank index), the A slices in shared memory
+// thread = row (bits 4-6 of its index) and rank index (the others): a warp's accumulators lie side by side, so that its atomics
+// are few requests (with the row in the low bits a kernel's atomics held up the next kernel's wait by 1.2 us)
+__device__ __forceinline__ int ln_row_of() { return (threadIdx.x >> 4) & (CHAIN_MAX_ROWS - 1); }
+__device__ __forceinline__ int ln_rank_of() { return (threadIdx.x & 15) + (threadIdx.x >> 7) * 16; }
+
+// partial shrink of the consuming group over this CTA's fresh fp16 outputs vals[8][16], the A slices in shared memory
+template <int THREADS>
 __device__ __forceinline__ void lean_shrink_partial(const LeanArgs& a, const StepPhase& ph, const __half (*vals)[16], const __half* sA) {
-  if (ph.next_nseg == 0 || a.adapter_idx == nullptr) return;
-  const int r = a.rank;
-  for (int it = threadIdx.x; it < ph.next_nseg * CHAIN_MAX_ROWS * r; it += blockDim.x) {
-    int q, j;
-    ln_divmod_rank(a, it, q, j);
-    const int m = q & (CHAIN_MAX_ROWS - 1), seg = q >> 3;
-    if (m >= a.M) continue;
-    const __half2* av = reinterpret_cast<const __half2*>(sA + (((size_t)m * ph.next_nseg + seg) * r + j) * 16);
-    const __half2* xv = reinterpret_cast<const __half2*>(vals[m]);
-    float s = 0.f;
+  const int r = a.rank, m = ln_row_of();
+  if (ph.next_nseg == 0 || a.adapter_idx == nullptr || m >= a.M) return;
+  const uint4 xr[2] = {reinterpret_cast<const uint4*>(vals[m])[0], reinterpret_cast<const uint4*>(vals[m])[1]};
+  const __half2* const xv = reinterpret_cast<const __half2*>(xr);
+  for (int j = ln_rank_of(); j < r; j += THREADS / 8)
+    for (int q = 0; q < ph.next_nseg; ++q) {
+      const uint4* const src = reinterpret_cast<const uint4*>(sA + ((q * CHAIN_MAX_ROWS + m) * (r + 1) + j) * 16);
+      const uint4 ar[2] = {src[0], src[1]};
+      const __half2* const av = reinterpret_cast<const __half2*>(ar);
+      float s = 0.f;
 #pragma unroll
-    for (int q2 = 0; q2 < 8; ++q2) {
-      const float2 x = __half22float2(xv[q2]), w = __half22float2(av[q2]);
-      s = fmaf(x.x, w.x, s); s = fmaf(x.y, w.y, s);
+      for (int e = 0; e < 8; ++e) {
+        const float2 x = __half22float2(xv[e]), w = __half22float2(av[e]);
+        s = fmaf(x.x, w.x, s); s = fmaf(x.y, w.y, s);
+      }
+      ln_red_add(a.tacc + ((size_t)ph.t_out * CHAIN_MAX_ROWS + m) * 3 * r + q * r + j, ln_fix(s));
     }
-    ln_red_add(a.tacc + ((size_t)ph.t_out * CHAIN_MAX_ROWS + m) * 3 * r + seg * r + j, ln_fix(s));
-  }
 }
 
 // NTILE = 1: 16 physical columns per CTA; NTILE = 2: a gate tile and its up tile (SwiGLU pair)
@@ -149,9 +124,8 @@ __device__ __forceinline__ void ln_stamp(const LeanArgs& a, int slot) {
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// PF k-tiles' weights in flight per warp, the input rows of XB of them loaded together, OCC CTAs on an SM; TAB: the rows'
-// matrix pointers by a table (an instantiation of its own: the code a CTA runs once runs at the instruction cache's cold rate)
-template <int NTILE, int WARPS, int PF, int XB, int OCC, bool TRACE, bool TAB>
+// PF k-tiles' weights in flight per warp, the input rows of XB of them loaded together, OCC CTAs on an SM
+template <int NTILE, int WARPS, int PF, int XB, int OCC, bool TRACE>
 __global__ void __launch_bounds__(WARPS * 32, OCC)
 lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   constexpr int THREADS = WARPS * 32;
@@ -165,15 +139,16 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   ln_stamp<TRACE>(a, 0);
   pdl_launch_dependents();
   const int M = a.M, K = ph.K, r = a.rank;
-  const __half* const row_ptr = TAB ? lean_row_ptr(a, ph) : nullptr;
   const WLayout L = make_wlayout(K, ph.N, ph.G);
   const int tile0 = blockIdx.x * NTILE;
   // ---- ahead of the wait: adapter slices and the first weights (immutable data)
   const bool lora = ph.lora_nseg > 0 && a.adapter_idx != nullptr;
-  __half* sB = reinterpret_cast<__half*>(ln_dyn);                          // [NTILE][M][r][16]
-  __half* sA = sB + (size_t)NTILE * CHAIN_MAX_ROWS * r * 16;               // [M][next_nseg][r][16]
-  const int ldt = TAB ? ph.lora_nseg * r : 3 * LN_PTR_RANK;
-  float* s_T = reinterpret_cast<float*>(sA + (size_t)CHAIN_MAX_ROWS * ph.next_nseg * r * 16);   // [8][ldt]
+  __half* sB = reinterpret_cast<__half*>(ln_dyn);                          // [NTILE][row][r + 1][16]
+  __half* sA = sB + NTILE * CHAIN_MAX_ROWS * (r + 1) * 16;                 // [next_nseg][row][r + 1][16]
+  float* s_T = reinterpret_cast<float*>(sA + CHAIN_MAX_ROWS * ph.next_nseg * (r + 1) * 16);   // [NTILE][row][r]
+  int seg[NTILE], col[NTILE];                                              // projection and first column of each tile
+#pragma unroll
+  for (int u = 0; u < NTILE; ++u) map_col(ph.mode, (tile0 + u) * TILE_N, ph.seg_n0, ph.seg_n1, seg[u], col[u]);
   const int n_out0 = ph.epi == EPI_SWIGLU ? (tile0 >> 1) * TILE_N : tile0 * TILE_N;   // first column the CTA produces
   const int kt0 = (L.KT * warp) / WARPS, kt1 = (L.KT * (warp + 1)) / WARPS;
   const unsigned char* unit[NTILE];
@@ -205,7 +180,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(ph.pf_w + o), "r"(n) : "memory");
     }
   }
-  lean_prefetch_slices<NTILE, TAB>(a, ph, tile0, n_out0, lora, row_ptr, sB, sA);
+  lean_prefetch_slices<NTILE, THREADS>(a, ph, seg, col, n_out0, lora, sB, sA);
   if (!a.late_wait) pdl_wait();
   ln_stamp<TRACE>(a, 1);
   // ---- what earlier kernels produced: the old residual, norm factors, T of this group, the input rows
@@ -221,33 +196,24 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
     s_inv[threadIdx.x] = inv;
   }
   auto load_T = [&]() {
-    for (int i = threadIdx.x; i < ph.lora_nseg * CHAIN_MAX_ROWS * r; i += THREADS) {
-      int q, j;
-      ln_divmod_rank(a, i, q, j);
-      const int m = q & (CHAIN_MAX_ROWS - 1), rest = (q >> 3) * r + j;
-      if (m >= M) continue;
-      const int ad = a.rows_direct ? m : a.adapter_idx[m];
-      float v = 0.f;
-      if (ad >= 0 && ad < a.n_slots)
-        v = ln_unfix(__ldcg(a.tacc + ((size_t)ph.t_in * CHAIN_MAX_ROWS + m) * 3 * r + rest)) * a.scale[ad];
-      s_T[m * ldt + rest] = v;
-    }
+    const int m = ln_row_of();
+    if (m >= M) return;
+    const int ad = a.rows_direct ? m : a.adapter_idx[m];
+    const bool ok = ad >= 0 && ad < a.n_slots;
+    const float scale = ok ? a.scale[ad] : 0.f;
+    const unsigned long long* const src = a.tacc + ((size_t)ph.t_in * CHAIN_MAX_ROWS + m) * 3 * r;
+    for (int j = ln_rank_of(); j < r; j += THREADS / 8)
+#pragma unroll
+      for (int u = 0; u < NTILE; ++u) s_T[(u * CHAIN_MAX_ROWS + m) * r + j] = ok ? ln_unfix(__ldcg(src + seg[u] * r + j)) * scale : 0.f;
   };
   if (lora && !a.late_wait) load_T();
-  // ---- main loop: warp w takes the k-tiles [kt0, kt1)
-  float acc[NTILE][4];
-#pragma unroll
-  for (int u = 0; u < NTILE; ++u) acc[u][0] = acc[u][1] = acc[u][2] = acc[u][3] = 0.f;
   const __half* xrow = ph.in16 + (size_t)g * K + 16 * t;
   const bool row_live = g < M;
-#pragma unroll 1
-  for (int kb = kt0; kb < kt1; kb += PF) {
-#pragma unroll
-   for (int ib = 0; ib < PF; ib += XB) {
-    uint4 x0[XB], x1[XB];
+  uint4 x0[XB], x1[XB];
+  auto load_x = [&](int kb) {
 #pragma unroll
     for (int i = 0; i < XB; ++i) {
-      const int kt = kb + ib + i;
+      const int kt = kb + i;
       if (kt < kt1 && row_live) {
         // (ordinary cached loads: the CTAs that share an SM read the same rows, and loads behind the wait see what
         // the kernel ahead wrote)
@@ -258,6 +224,16 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
         x1[i] = make_uint4(0, 0, 0, 0);
       }
     }
+  };
+  load_x(kt0);
+  // ---- main loop: warp w takes the k-tiles [kt0, kt1)
+  float acc[NTILE][4];
+#pragma unroll
+  for (int u = 0; u < NTILE; ++u) acc[u][0] = acc[u][1] = acc[u][2] = acc[u][3] = 0.f;
+#pragma unroll 1
+  for (int kb = kt0; kb < kt1; kb += PF) {
+#pragma unroll
+   for (int ib = 0; ib < PF; ib += XB) {
 #pragma unroll
     for (int i = 0; i < XB; ++i) {
       if (kb + ib + i < kt1) {
@@ -277,6 +253,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
         }
       }
     }
+    if (kb + ib + XB < kt1) load_x(kb + ib + XB);
    }
     if (kb + PF < kt1) load_weights(kb + PF);
   }
@@ -301,12 +278,11 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
 #pragma unroll
       for (int w = 0; w < WARPS; ++w) y += red[w][u][src_lane][e];
       if (lora) {
-        int seg, col;
-        map_col(ph.mode, (tile0 + u) * TILE_N, ph.seg_n0, ph.seg_n1, seg, col);
-        const float* T = s_T + m * ldt + seg * r;
-        const __half* Bs = sB + ((size_t)u * M + m) * r * 16 + c;           // (zeros where the row has no adapter)
+        const float* T = s_T + (u * CHAIN_MAX_ROWS + m) * r;
+        const __half* Bs = sB + (u * CHAIN_MAX_ROWS + m) * (r + 1) * 16 + c;   // (zeros where the row has no adapter)
         float ex = 0.f;
-        for (int j = 0; j < r; ++j) ex = fmaf(T[j], __half2float(Bs[(size_t)j * 16]), ex);
+#pragma unroll 8
+        for (int j = 0; j < r; ++j) ex = fmaf(T[j], __half2float(Bs[j * 16]), ex);
         y += ex;
       }
       y *= s_inv[m];
@@ -371,7 +347,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
       for (int c = 0; c < 16; ++c) sq += s_sq[threadIdx.x][c];
       ln_red_add(a.ssq + (size_t)ph.ssq_out * CHAIN_MAX_ROWS + threadIdx.x, ln_fix(sq));
     }
-    lean_shrink_partial(a, ph, s_vals, sA);
+    lean_shrink_partial<THREADS>(a, ph, s_vals, sA);
     ln_stamp<TRACE>(a, 3);
     return;
   }
@@ -389,7 +365,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
       s_vals[m][c] = hv;
     }
     __syncthreads();
-    lean_shrink_partial(a, ph, s_vals, sA);
+    lean_shrink_partial<THREADS>(a, ph, s_vals, sA);
   }
   ln_stamp<TRACE>(a, 3);
 }
@@ -737,22 +713,23 @@ cudaError_t launch_lean_embed(const LeanArgs& a, const StepPhase& ph, const int3
 // The variants of lean_gemm_kernel (NTILE, WARPS, PF, XB, OCC).  A grid that does not fit the SMs at once costs a whole
 // CTA's life more (llama3b gate/up, 512 CTAs at three an SM: 24.5 us, the last ones starting at 11; 12.9 at four), but the
 // registers of a fourth CTA are paid with loads in flight (llama1b gate/up, 352 CTAs: 9.1 us at three, 9.7 at four), so the
-// dense variants are taken only where they save the second wave.
+// dense variants are taken only where they save a wave.  Single tiles in more than three CTAs an SM: 8 rows of 2048 x 8192
+// without adapters 6.2 us at three, 4.9 at four; 4096 x 14336 with adapters 19.1 -> 18.4.
 #define LN_ONE 1, 8, 4, 4, 3
-#define LN_PAIR 2, 8, 4, 4, 3         // gate/up: a gate tile and its up tile
+#define LN_ONE_DENSE 1, 8, 4, 2, 4
+#define LN_PAIR 2, 8, 4, 2, 3         // gate/up: a gate tile and its up tile
 #define LN_PAIR_DENSE 2, 8, 2, 2, 4
 #define LN_WIDE 1, 16, 4, 4, 1        // a long K on few tiles: sixteen warps split it
 #define LN_WIDE_DENSE 1, 16, 4, 2, 2
 #define LN_SET(...) \
-  if ((e = cudaFuncSetAttribute(lean_gemm_kernel<__VA_ARGS__, TRACE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 88 * 1024)) != cudaSuccess) return e; \
-  if ((e = cudaFuncSetAttribute(lean_gemm_kernel<__VA_ARGS__, TRACE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 88 * 1024)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(lean_gemm_kernel<__VA_ARGS__, TRACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 88 * 1024)) != cudaSuccess) return e;
 #define LN_LAUNCH(...) \
-  return a.rank > LN_PTR_RANK ? cudaLaunchKernelEx(&cfg, lean_gemm_kernel<__VA_ARGS__, TRACE, true>, a, ph) : cudaLaunchKernelEx(&cfg, lean_gemm_kernel<__VA_ARGS__, TRACE, false>, a, ph)
+  return cudaLaunchKernelEx(&cfg, lean_gemm_kernel<__VA_ARGS__, TRACE>, a, ph)
 template <bool TRACE>
 static cudaError_t init_lean_variant() {
   // room for the adapter slices and T at rank 64: 5 x 16 KB and 6 KB
   cudaError_t e;
-  LN_SET(LN_ONE) LN_SET(LN_PAIR) LN_SET(LN_PAIR_DENSE) LN_SET(LN_WIDE) LN_SET(LN_WIDE_DENSE)
+  LN_SET(LN_ONE) LN_SET(LN_ONE_DENSE) LN_SET(LN_PAIR) LN_SET(LN_PAIR_DENSE) LN_SET(LN_WIDE) LN_SET(LN_WIDE_DENSE)
 #define LM_SET(PF, D) \
   if ((e = cudaFuncSetAttribute(lean_lmhead_kernel<LN_WARPS, PF, D, TRACE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lm_smem_bytes(PF, D, LN_THREADS))) != cudaSuccess) return e;
   LM_SET(4, 4) LM_SET(6, 3) LM_SET(8, 2)
@@ -767,10 +744,10 @@ template <bool TRACE>
 static cudaError_t launch_lean_gemm_variant(const LeanArgs& a, const StepPhase& ph, cudaStream_t st) {
   const int tiles = ph.N / TILE_N, mode = ph.mode;
   // B slices of up to two tiles and A slices of up to three consuming segments, 8 rows x rank x 16 columns each
-  const size_t slice = (size_t)CHAIN_MAX_ROWS * (a.rank > 0 ? a.rank : 1) * 16 * sizeof(__half);
+  const size_t slice = (size_t)CHAIN_MAX_ROWS * (a.rank + 1) * 16 * sizeof(__half);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(mode == MODE_GATEUP ? tiles / 2 : tiles));
-  cfg.dynamicSmemBytes = ((mode == MODE_GATEUP ? 2 : 1) + ph.next_nseg) * slice + (size_t)CHAIN_MAX_ROWS * (a.rank > LN_PTR_RANK ? ph.lora_nseg * a.rank : 3 * LN_PTR_RANK) * sizeof(float);
+  cfg.dynamicSmemBytes = ((mode == MODE_GATEUP ? 2 : 1) + ph.next_nseg) * slice + (size_t)(mode == MODE_GATEUP ? 2 : 1) * CHAIN_MAX_ROWS * a.rank * sizeof(float);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // may start while the kernel before it drains
@@ -799,6 +776,7 @@ static cudaError_t launch_lean_gemm_variant(const LeanArgs& a, const StepPhase& 
   }
   if (wide && tiles > sms) LN_LAUNCH(LN_WIDE_DENSE);
   if (wide) LN_LAUNCH(LN_WIDE);
+  if (tiles > 3 * sms) LN_LAUNCH(LN_ONE_DENSE);
   LN_LAUNCH(LN_ONE);
 }
 

@@ -409,7 +409,6 @@ int forward_lean(mlora_ctx* c, PassIO& io) {
     a.tab_stride = c->L * 7; a.n_slots = CHAIN_MAX_ROWS;
   }
   a.rank = (d.max_adapters > 0 && d.lora_targets != 0) ? d.lora_rank : 0;
-  a.rank_log2 = lean_rank_log2(a.rank);
   a.X = c->X; a.logits = io.logits; a.tacc = c->step_tacc; a.ssq = c->step_ssq;
   const bool fused = io.fused_next != nullptr && d.vocab > 0;
   if (fused) { a.logits = nullptr; a.amax = c->step_ssq + (size_t)c->n_ssq * CHAIN_MAX_ROWS; }
@@ -1730,7 +1729,7 @@ int mlora_linear(mlora_weight* w, const void* x, int32_t M, const int32_t* row_a
     ph.in16 = (const __half*)x; ph.norm_in = -1; ph.out_f32 = y; ph.ldo = w->w.N; ph.ssq_out = -1;
     if (lora) {
       a.adapter_idx = row_adapter; a.tabA = (const __half* const*)A; a.tabB = (const __half* const*)B; a.scale = scale;
-      a.tab_stride = 1; a.n_slots = n_adapters; a.rank = rank; a.rank_log2 = lean_rank_log2(rank);
+      a.tab_stride = 1; a.n_slots = n_adapters; a.rank = rank;
       a.tacc = (unsigned long long*)(ws + LIN_COUNTER_BYTES + lin_T_bytes(M, rank));
       ph.lora_nseg = 1; ph.lora_proj[0] = 0; ph.lora_n[0] = w->w.N; ph.t_in = 0;
       CK(launch_lean_shrink(a, (const __half*)x, w->w.K, w->stream));

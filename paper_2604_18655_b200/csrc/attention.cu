@@ -771,11 +771,10 @@ __global__ void __launch_bounds__(dec_warps(HD) * 32) attn_decode_kernel(const A
 #pragma unroll
     for (int w = 0; w < W; ++w) M = fmaxf(M, part_ml[((size_t)w * 16 + r) * 2]);
     num = 0.f; den = 0.f;
+    const float base = M == -INFINITY ? 0.f : M;
 #pragma unroll
-    for (int w = 0; w < W; ++w) {
-      const float mw = part_ml[((size_t)w * 16 + r) * 2];
-      if (mw == -INFINITY) continue;                       // a warp without tiles
-      const float f = exp2f(mw - M);
+    for (int w = 0; w < W; ++w) {                          // (a warp without tiles: -inf and zeros)
+      const float f = exp2f(part_ml[((size_t)w * 16 + r) * 2] - base);
       num += f * part_o(w)[(size_t)r * HD + d];
       den += f * part_ml[((size_t)w * 16 + r) * 2 + 1];
     }
@@ -828,18 +827,25 @@ __global__ void __launch_bounds__(dec_warps(HD) * 32) attn_decode_kernel(const A
       __syncthreads();
       if (oA != nullptr) {
         const int feats = g_heads * HD;
-        for (int j = warp; j < p.o_rank; j += W) {
-          const __half* arow = a_sl + (size_t)j * feats;
+        // half a warp a rank index: nine warps have sixteen of them done at once
+        for (int j0 = warp * 2; j0 < p.o_rank; j0 += 2 * W) {
+          const int j = j0 + (lane >> 4);
           float sum = 0.f;
-          for (int i = lane * 2; i < feats; i += 64) {
-            const float2 av = __half22float2(*reinterpret_cast<const __half2*>(arow + i));
-            const float2 xv = __half22float2(*reinterpret_cast<const __half2*>(Qs + (size_t)(i / HD) * STRIDE + (i % HD)));
-            sum = fmaf(xv.x, av.x, sum);
-            sum = fmaf(xv.y, av.y, sum);
-          }
+          if (j < p.o_rank)
+            for (int i = (lane & 15) * 8; i < feats; i += 128) {
+              const uint4 av = *reinterpret_cast<const uint4*>(a_sl + (size_t)j * feats + i);
+              const uint4 xv = *reinterpret_cast<const uint4*>(Qs + (size_t)(i / HD) * STRIDE + (i % HD));
+              const __half2 *ap = reinterpret_cast<const __half2*>(&av), *xp = reinterpret_cast<const __half2*>(&xv);
 #pragma unroll
-          for (int o2 = 16; o2 > 0; o2 >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o2);
-          if (lane == 0) {
+              for (int e = 0; e < 4; ++e) {
+                const float2 a2 = __half22float2(ap[e]), x2 = __half22float2(xp[e]);
+                sum = fmaf(x2.x, a2.x, sum);
+                sum = fmaf(x2.y, a2.y, sum);
+              }
+            }
+#pragma unroll
+          for (int o2 = 8; o2 > 0; o2 >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o2);
+          if ((lane & 15) == 0 && j < p.o_rank) {
             const unsigned long long q = (unsigned long long)__float2ll_rn(sum * 4294967296.f);
             asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p.o_tacc + ((size_t)m * 3 + 0) * p.o_rank + j), "l"(q) : "memory");
           }

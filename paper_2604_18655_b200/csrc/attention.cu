@@ -304,9 +304,6 @@ __device__ __forceinline__ void attn_partial_body(const AttnArgs& p, const int r
   }
 }
 
-// log-sum-exp merge of the chunks of virtual row v (row m, query head hq) of kv head kh by one warp.  The lanes
-// take the chunks' (max, sum) pairs side by side; the weighted sum over chunks runs in chunk order with
-// independent loads.
 // Merge of a row's chunks by one warp; lane l holds the hd / 32 (2 or 4) consecutive features from l * hd / 32 on.
 __device__ __forceinline__ float4 merge_load(const float* row, int hd, int lane) {
   if (hd == 128) return __ldcg(reinterpret_cast<const float4*>(row) + lane);
@@ -364,8 +361,15 @@ __device__ __forceinline__ void merge_o_shrink(const AttnArgs& p, int m, int hq,
 }
 __device__ __forceinline__ void merge_store(const AttnArgs& p, float4 acc, float inv, __half* out, int m, int hq, int lane) {
   const __half2 a = __floats2half2_rn(acc.x * inv, acc.y * inv), b = __floats2half2_rn(acc.z * inv, acc.w * inv);
-  if (p.hd == 128) *(reinterpret_cast<uint2*>(out) + lane) = make_uint2(h2_as_u32(a), h2_as_u32(b));
-  else *(reinterpret_cast<__half2*>(out) + lane) = a;
+  const int per = p.hd >> 5;                               // features a lane holds
+  if ((reinterpret_cast<uintptr_t>(p.out) & (2 * per - 1)) == 0) {
+    if (per == 4) *(reinterpret_cast<uint2*>(out) + lane) = make_uint2(h2_as_u32(a), h2_as_u32(b));
+    else *(reinterpret_cast<__half2*>(out) + lane) = a;
+  } else {                                                 // (a caller's buffer that only starts on a whole element)
+    out += lane * per;
+    out[0] = __low2half(a); out[1] = __high2half(a);
+    if (per == 4) { out[2] = __low2half(b); out[3] = __high2half(b); }
+  }
   if (p.o_tacc != nullptr) {
     const float2 fa = __half22float2(a), fb = __half22float2(b);
     merge_o_shrink(p, m, hq, make_float4(fa.x, fa.y, fb.x, fb.y), lane);

@@ -468,7 +468,9 @@ static cudaError_t at_launch(const AttnArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t st) {
-  for (const void* ptr : {(const void*)a.q, (const void*)a.prefix_k, (const void*)a.prefix_v, (const void*)a.own_k, (const void*)a.own_v, (const void*)a.out})
+  // (causal passes store their rows themselves; the others leave that to the merge, which takes any `out`)
+  for (const void* ptr : {(const void*)a.q, (const void*)a.prefix_k, (const void*)a.prefix_v, (const void*)a.own_k, (const void*)a.own_v,
+                          a.causal ? (const void*)a.out : (const void*)nullptr})
     if (reinterpret_cast<uintptr_t>(ptr) & 15) return cudaErrorMisalignedAddress;
   if (a.hd == 64) return a.tc_nq == 2 ? at_launch<64, 2>(a, st) : at_launch<64, 1>(a, st);
   return a.tc_nq == 2 ? at_launch<128, 2>(a, st) : at_launch<128, 1>(a, st);

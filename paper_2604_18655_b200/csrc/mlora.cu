@@ -1908,9 +1908,11 @@ int mlora_attention(const void* q, const void* prefix_k, const void* prefix_v, i
   AttnArgs a;
   attn_fill(a, n, T, Hq, Hkv, hd, P, suffix_bound);
   const size_t rows = (size_t)n * T;
-  const size_t head = (rows * (sizeof(unsigned long long) + sizeof(int32_t)) + 255) / 256 * 256;
-  if (workspace_bytes < head + attn_workspace_floats(a) * sizeof(float)) return fail(MLORA_ERR_CAPACITY, "workspace too small");
-  unsigned char* ws = (unsigned char*)workspace;
+  // (the partial results are read and written 16 bytes at a time: placed on such a boundary wherever the buffer starts)
+  unsigned char* const ws = (unsigned char*)(((uintptr_t)workspace + 15) & ~(uintptr_t)15);
+  unsigned char* const parts = ws + (rows * (sizeof(unsigned long long) + sizeof(int32_t)) + 15) / 16 * 16;
+  if (workspace_bytes < (size_t)(parts - (unsigned char*)workspace) + attn_workspace_floats(a) * sizeof(float))
+    return fail(MLORA_ERR_CAPACITY, "workspace too small");
   unsigned long long* anc = (unsigned long long*)ws;
   int32_t* depth = (int32_t*)(ws + rows * sizeof(unsigned long long));
   CK(launch_tree_prep(tree_parent, n, T, anc, depth, status, st));
@@ -1919,7 +1921,7 @@ int mlora_attention(const void* q, const void* prefix_k, const void* prefix_v, i
   a.own_k = (const __half*)own_k; a.own_v = (const __half*)own_v;
   a.own_head_stride = (size_t)own_capacity * hd; a.own_stream_stride = a.own_head_stride * Hkv;
   a.suffix_len = suffix_len; a.anc = anc; a.out = (__half*)out; a.status = status; a.depth = depth;
-  a.part_o = (float*)(ws + head);
+  a.part_o = (float*)parts;
   a.part_ml = a.part_o + (attn_workspace_floats(a) / (hd + 2)) * hd;
   CK(launch_attention(a, st));
   CK(launch_attention_merge(a, st));

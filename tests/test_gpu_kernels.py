@@ -158,7 +158,7 @@ def test_linear_rejects_bad_arguments(mb):
 
 
 # ------------------------------------------------------------------ attention
-def run_attention(mb, n, T, Hq, Hkv, hd, P, suf, branch, seed, cap=None):
+def run_attention(mb, n, T, Hq, Hkv, hd, P, suf, branch, seed, cap=None, out_off=0, ws_off=0):
     rng = np.random.default_rng(seed)
     cap = cap or (max(suf) + T + 3)
     q = rng.standard_normal((n * T, Hq, hd)).astype(np.float16)
@@ -168,8 +168,9 @@ def run_attention(mb, n, T, Hq, Hkv, hd, P, suf, branch, seed, cap=None):
     ov = rng.standard_normal((n, Hkv, cap, hd)).astype(np.float16)
     parent = gen.build_tree(branch, T) if T > 1 else np.array([-1], dtype=np.int32)
     parents = np.stack([parent] * n).astype(np.int32)
-    out = torch.empty(n * T, Hq, hd, dtype=torch.float16, device="cuda")
-    ws = torch.empty(mb.mlora_attention_workspace_bytes(n, T, Hq, Hkv, hd, P, cap), dtype=torch.uint8, device="cuda")
+    # (out_off elements, ws_off bytes: buffers that start between allocation boundaries)
+    out = torch.empty(n * T * Hq * hd + out_off, dtype=torch.float16, device="cuda")[out_off:].view(n * T, Hq, hd)
+    ws = torch.empty(mb.mlora_attention_workspace_bytes(n, T, Hq, Hkv, hd, P, cap) + ws_off, dtype=torch.uint8, device="cuda")[ws_off:]
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     mb.mlora_attention(dev(q), dev(pk[:, :P]) if P else None, dev(pv[:, :P]) if P else None, dev(ok), dev(ov),
                        dev(np.asarray(suf, dtype=np.int32)), int(max(suf)), dev(parents), out, ws, status)

@@ -68,6 +68,16 @@ def test_tree_attention_edges(mb, n, T, Hq, Hkv, hd, P, suf, branch):
     compare(got, want, f"tree attention n{n} T{T} {Hq}q/{Hkv}kv hd{hd} P{P}")
 
 
+@pytest.mark.parametrize("hd", [64, 128])
+@pytest.mark.parametrize("n,T,P,suf,branch", [(3, 1, 2100, [0, 40, 90], ()), (2, 16, 130, [3, 64], (4, 2, 2))])
+@pytest.mark.parametrize("out_off,ws_off", [(1, 8), (2, 0), (3, 4)])
+def test_merged_attention_into_buffers_of_any_start(mb, hd, n, T, P, suf, branch, out_off, ws_off):
+    """The partial-result paths (streaming + merge, tensor cores + merge) into an output that starts on any half and with
+    scratch that starts on any word."""
+    got, want = run_attention(mb, n, T, 8, 2, hd, P, suf, branch, seed=hd + T + out_off, out_off=out_off, ws_off=ws_off)
+    compare(got, want, f"attention out + {out_off} halves, scratch + {ws_off} bytes")
+
+
 @pytest.mark.parametrize("hd,n_q,n_kv,P", [(64, 32, 8, 640), (128, 24, 8, 1025), (128, 16, 8, 2100), (64, 6, 2, 257)])
 def test_causal_passes_of_one_and_two_row_blocks(GpuModel, hd, n_q, n_kv, P):
     """Two row blocks a CTA from about 600 positions on; the second layer's K/V show every row of the first one's output.

@@ -400,6 +400,9 @@ attn_tc_kernel(const __grid_constant__ AttnArgs p, const int rb_rows, const int 
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)C::COLS) : "memory");
 }
 
+// A row of queries with all heads of its group has to fit a block.
+bool attn_tc_shape(const AttnArgs& a) { return a.Hq / a.Hkv <= AT_ROWS; }
+
 // Blocks and chunks of a pass.  Causal passes: two blocks a CTA where that still gives half the SMs a CTA.  Trees: the
 // prefix in as many chunks (whole tiles) as two CTAs an SM take.
 void attn_plan_tc(AttnArgs& a, int sm_count) {

@@ -353,6 +353,7 @@ cudaError_t launch_draft(const float* logits, int V, int n, int R, int m, int wm
 cudaError_t launch_tree_prep(const int32_t* parent, int n, int T, unsigned long long* anc, int32_t* depth,
                              int* status, cudaStream_t st);
 void attn_plan(AttnArgs& a, int sm_count);
+bool attn_tc_shape(const AttnArgs& a);             // whether the tcgen05 attention takes the pass's head counts
 void attn_plan_tc(AttnArgs& a, int sm_count);
 cudaError_t init_attention_tc();
 cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t st);

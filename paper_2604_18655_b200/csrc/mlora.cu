@@ -237,7 +237,7 @@ void plan_pass(mlora_ctx* c, PassIO& io) {
   a.suffix_bound = (io.suffix_bound + 63) / 64 * 64;   // coarse, so the launch shape changes rarely
   a.causal = io.prefill ? 1 : 0;
   io.tc = !c->dbg_no_tc && io.n * io.T >= TC_MIN_ROWS && tensor_maps_available();
-  if (io.tc) { attn_plan_tc(a, c->sm_count); a.suffix_bound = 0; }     // (its launch shape does not depend on the bound)
+  if (io.tc && attn_tc_shape(a)) { attn_plan_tc(a, c->sm_count); a.suffix_bound = 0; }     // (its launch shape does not depend on the bound)
   else attn_plan(a, c->sm_count);
 }
 
@@ -262,7 +262,7 @@ int launch_attention_block(mlora_ctx* c, const PassIO& io, int l) {
   kv_destination(c, io, l, kd, vd, sstride, hstride);
   AttnArgs a = io.plan;
   // q and the new k rows are rotated on load, the new K/V rows appended by the attention kernel itself -- or by the
-  // epilogue of the tcgen05 q,k,v projection
+  // epilogue of the tcgen05 q,k,v projection (behind which any attention kernel may stand)
   if (io.tc) { a.q = c->q16; a.pdl = 1; }
   else a.qkv_f32 = c->qkv;
   a.cs_table = c->cs_table; a.pos_base = io.pos_base; a.depth = c->depth;
@@ -1874,7 +1874,7 @@ static void attn_fill(AttnArgs& a, int n, int T, int Hq, int Hkv, int hd, int P,
   a.suffix_bound = suffix_bound;
   attn_plan(a, 148);
   // (one row per stream: the decode kernels, where their shapes fit)
-  if (!attn_single_pass(a) && !a.stream_mode && Hq / Hkv <= 128 && tensor_maps_available()) attn_plan_tc(a, 148);
+  if (!attn_single_pass(a) && !a.stream_mode && attn_tc_shape(a) && tensor_maps_available()) attn_plan_tc(a, 148);
 }
 
 size_t mlora_attention_workspace_bytes(int32_t n, int32_t T, int32_t Hq, int32_t Hkv, int32_t hd, int32_t P,

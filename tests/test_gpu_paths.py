@@ -94,6 +94,26 @@ def test_causal_passes_of_one_and_two_row_blocks(GpuModel, hd, n_q, n_kv, P):
     gm.close()
 
 
+def test_passes_with_more_query_heads_a_group_than_a_block_has_rows(GpuModel):
+    """129 query heads on one KV head: prefill, a tree pass and a decode step of nine streams keep the tensor-core projections
+    and take the general attention kernel."""
+    cfg = gen.ModelCfg("mqa", 2, 128, 129, 1, 64, 192, 304, 64, 4, gen.configs.ALL7, 2, 9, 40)
+    _, orc, gm = make_pair(GpuModel, cfg, max_suffix=40, max_tree=6)
+    ids = gen.make_prompt_ids(cfg, 0)
+    compare(gm.prefill(ids), orc.prefill_shared(ids, n_streams=9), "prefill logits")
+    ad = [0, 1, -1] * 3
+    parent = np.array([-1, 0, 0, 1, 1, 2], dtype=np.int32)
+    tree = np.random.default_rng(3).integers(0, cfg.vocab, size=(9, 6), dtype=np.int32)
+    par = np.stack([parent] * 9)
+    got = gm.verify(ad, tree, par)
+    want = orc.verify_tree(ad, par, tree, follow_argmax=np.argmax(got["logits"], axis=1).reshape(9, 6))
+    compare(got["logits"], want["logits"], "verify logits")
+    toks = np.arange(3, 12, dtype=np.int32)
+    _, logits = gm.decode(ad, toks)
+    compare(logits, orc.decode_step(ad, tokens=toks)["logits"], "decode logits")
+    gm.close()
+
+
 # ------------------------------------------------------------------ decode
 @pytest.mark.parametrize("d_model,d_ffn,hd,n_q,n_kv,vocab,rank,n,P", [
     (3072, 4096, 128, 24, 8, 9600, 32, 8, 70),     # single-wave variants, pointer table, lm_head of K = 3072

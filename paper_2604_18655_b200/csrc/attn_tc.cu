@@ -11,8 +11,8 @@
 // inside fp16, and the sum is kept in fp32.  With NQ = 2 the tensor core works on one block while the other's softmax runs.
 // What bounds it: 16384 exponentials per tile against 16 per clock and SM (1024 cycles; the two products of head size 128
 // take as long).
-// Trees: the prefix is cut into chunks that serve the rows of ALL streams, an own segment serves its stream; partial
-// results go to the scratch that attn_merge_kernel combines.  Causal passes need no partials: one CTA sees all keys of its
+// Trees: the prefix is cut into chunks that serve the rows of ALL streams, an own segment into chunks that serve its stream;
+// partial results go to the scratch that attn_merge_kernel combines.  Causal passes need no partials: one CTA sees all keys of its
 // rows, longest rows first.  q, and the K/V rows of the pass, are rotated and in the cache already (the q,k,v projection's
 // epilogue puts them there).
 #include <cuda.h>
@@ -96,6 +96,7 @@ attn_tc_kernel(const __grid_constant__ AttnArgs p, const int rb_rows, const int 
 
   // ---- which rows, which keys
   AtItem it{};
+  int S_own = 0;
   if (p.causal) {
     const int b = gridDim.x - 1 - blockIdx.x;              // the longest first
     it.v_lo = b * NQ * rb_rows; it.v_hi = R_all;
@@ -108,12 +109,16 @@ attn_tc_kernel(const __grid_constant__ AttnArgs p, const int rb_rows, const int 
       it.k0 = it.slot * p.prefix_chunk; it.k1 = min(p.P, it.k0 + p.prefix_chunk);
     } else {
       item -= p.n_prefix_chunks * rb_all;
-      it.own = 1; it.slot = p.n_prefix_chunks; it.s = item / rb_own;
-      it.v_lo = it.s * p.T * g + (item % rb_own) * NQ * rb_rows; it.v_hi = (it.s + 1) * p.T * g;
-      it.k1 = p.suffix_len[it.s] + p.T;
+      const int rb = item % rb_own, chunk = item / rb_own % p.n_own_chunks;
+      it.own = 1; it.slot = p.n_prefix_chunks + chunk; it.s = item / (rb_own * p.n_own_chunks);
+      it.v_lo = it.s * p.T * g + rb * NQ * rb_rows; it.v_hi = (it.s + 1) * p.T * g;
+      S_own = p.suffix_len[it.s];
+      it.k0 = chunk * p.own_chunk; it.k1 = S_own + p.T;
+      // (the last chunk takes what is left, whatever bound the chunks were planned with)
+      if (chunk + 1 < p.n_own_chunks) it.k1 = min(it.k1, it.k0 + p.own_chunk);
+      if (it.k1 <= it.k0) return;                          // nothing here yet (the merge skips this slot too)
     }
   }
-  const int S_own = it.own ? it.k1 - p.T : 0;
   int n_w[NQ];                                             // key tiles of each block
 #pragma unroll
   for (int w = 0; w < NQ; ++w) {
@@ -404,7 +409,12 @@ attn_tc_kernel(const __grid_constant__ AttnArgs p, const int rb_rows, const int 
 bool attn_tc_shape(const AttnArgs& a) { return a.Hq / a.Hkv <= AT_ROWS; }
 
 // Blocks and chunks of a pass.  Causal passes: two blocks a CTA where that still gives half the SMs a CTA.  Trees: the
-// prefix in as many chunks (whole tiles) as two CTAs an SM take.
+// prefix in as many chunks (whole tiles) as two CTAs an SM take; then the longest own segment that the host's bound allows,
+// in at most as many, by a CTA's time (about 2 us a tile of an own segment, one behind the other, and two and a half tiles'
+// worth of fixed cost) and the waves that all CTAs make.  Unsplit, 4096 own keys of one stream (prefix 512, 32 heads of 64)
+// took 71.7 us, 19.4 in 33 chunks; of eight streams 75.4 us, 49.1 us in two; 256 own keys of eight streams 16.4 us
+// unsplit, 15.9 us in two chunks, 17.4 in three (a second wave).  The bound counts in whole tiles, so that the launch shape of
+// a captured pass changes every 128 keys at most.
 void attn_plan_tc(AttnArgs& a, int sm_count) {
   const int g = a.Hq / a.Hkv, rb = g * (AT_ROWS / g), R_all = a.n * a.T * g;
   a.stream_mode = 0;
@@ -421,8 +431,15 @@ void attn_plan_tc(AttnArgs& a, int sm_count) {
   const int per = tiles > 0 ? (tiles + want - 1) / want : 1;
   a.prefix_chunk = per * AT_KEYS;
   a.n_prefix_chunks = (tiles + per - 1) / per;
-  a.n_own_chunks = 1;
-  a.own_chunk = AT_KEYS;
+  const int rb_own = (a.T * g + rb - 1) / rb, own_tiles = (a.suffix_bound + a.T + AT_KEYS - 1) / AT_KEYS;
+  const int per_chunk = a.Hkv * a.n * rb_own, others = a.n_prefix_chunks * blocks * a.Hkv;
+  double best = 0.0;
+  for (int c = 1; c <= own_tiles && (c == 1 || c * per_chunk <= 2 * sm_count); ++c) {
+    const int own_per = (own_tiles + c - 1) / c, chunks = (own_tiles + own_per - 1) / own_per;
+    const int waves = (others + chunks * per_chunk + 2 * sm_count - 1) / (2 * sm_count);
+    const double cost = waves * (2.5 + (own_per > per ? own_per : per));
+    if (c == 1 || cost < best) { best = cost; a.n_own_chunks = chunks; a.own_chunk = own_per * AT_KEYS; }
+  }
 }
 
 static cudaError_t at_map(const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box, CUtensorMap* out) {
@@ -460,7 +477,7 @@ static cudaError_t at_launch(const AttnArgs& a, cudaStream_t st) {
   }
   const int rb_all = (R_all + NQ * rb - 1) / (NQ * rb), rb_own = (a.T * g + NQ * rb - 1) / (NQ * rb);
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(a.causal ? rb_all : a.n_prefix_chunks * rb_all + a.n * rb_own), (unsigned)a.Hkv);
+  cfg.gridDim = dim3((unsigned)(a.causal ? rb_all : a.n_prefix_chunks * rb_all + a.n * a.n_own_chunks * rb_own), (unsigned)a.Hkv);
   cfg.blockDim = dim3(C::THREADS); cfg.dynamicSmemBytes = C::SMEM; cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

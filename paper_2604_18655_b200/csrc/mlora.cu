@@ -237,7 +237,7 @@ void plan_pass(mlora_ctx* c, PassIO& io) {
   a.suffix_bound = (io.suffix_bound + 63) / 64 * 64;   // coarse, so the launch shape changes rarely
   a.causal = io.prefill ? 1 : 0;
   io.tc = !c->dbg_no_tc && io.n * io.T >= TC_MIN_ROWS && tensor_maps_available();
-  if (io.tc && attn_tc_shape(a)) { attn_plan_tc(a, c->sm_count); a.suffix_bound = 0; }     // (its launch shape does not depend on the bound)
+  if (io.tc && attn_tc_shape(a)) { attn_plan_tc(a, c->sm_count); a.suffix_bound = 0; }     // (its launch shape is all in the chunks)
   else attn_plan(a, c->sm_count);
 }
 
@@ -886,11 +886,11 @@ int mlora_create(const mlora_model_desc* desc, mlora_ctx** out) {
   CKC(cudaMalloc(&c->counters, 4096 * sizeof(unsigned)));
   CKC(cudaMemsetAsync(c->counters, 0, 4096 * sizeof(unsigned), st));
   {
-    // attention scratch: rows x chunks never exceeds (rows of one launch) + 64 x (CTAs the planner aims for),
-    // once for the shared-prefix chunks and once for the own-segment chunks
+    // attention scratch: rows x chunks never exceeds (rows of one launch) + (rows of a block: 128 at most) x (CTAs the
+    // planners aim for: two an SM), once for the shared-prefix chunks and once for the own-segment chunks
     const size_t g_heads = d.n_q_heads / d.n_kv_heads;
     const size_t R_all = Mm * g_heads;
-    c->att_ws_floats = ((size_t)d.n_kv_heads * R_all * 2 + (size_t)256 * c->sm_count + 4096) * (hd + 2);
+    c->att_ws_floats = ((size_t)d.n_kv_heads * R_all * 2 + (size_t)512 * c->sm_count + 4096) * (hd + 2);
     CKC(cudaMalloc(&c->att_ws, c->att_ws_floats * sizeof(float)));
   }
   CKC(cudaMalloc(&c->host_io, 3 * (size_t)d.max_streams * sizeof(int32_t)));

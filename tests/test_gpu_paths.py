@@ -62,6 +62,10 @@ def test_quantiser_tails(mb, count):
     (3, 33, 5, 1, 128, 128, [127, 128, 5], (4, 4, 3)),   # own segments over a tile's end, two blocks of rows a stream
     (1, 64, 8, 8, 64, 1, [0], (4, 4, 3)),             # one head a group, the largest tree, a prefix of one key
     (2, 16, 16, 2, 128, 0, [3, 250], (4, 3)),         # no prefix
+    (1, 16, 8, 2, 64, 100, [1500], (4, 3)),           # own segments in chunks: thirteen of them,
+    (3, 30, 24, 8, 128, 300, [900, 0, 380], (4, 3, 2)),   # two, of which a short segment has one; the tree across a chunk's end,
+    (16, 1, 8, 8, 64, 70, [700, 3, 127, 128, 129, 255, 256, 257, 383, 384, 385, 0, 511, 512, 513, 640], ()),
+    (40, 1, 32, 8, 128, 0, [400] * 39 + [1023], ()),      # one (more own segments than CTAs wanted)
 ])
 def test_tree_attention_edges(mb, n, T, Hq, Hkv, hd, P, suf, branch):
     got, want = run_attention(mb, n, T, Hq, Hkv, hd, P, suf, branch, seed=n + T + P)

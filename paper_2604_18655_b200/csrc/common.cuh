@@ -97,10 +97,25 @@ struct LoraArgs {
   LoraSeg seg[3];
   float* T;                       // dev fp32 [M][nseg][rank], already multiplied by the adapter scale
   // the same for the tcgen05 projection (nullptr: T is used): fp16 [M][nseg][2][ke], T as value + rounding remainder in
-  // the columns slot * rank + j of the row's own slot, zeros elsewhere; ke = k_slots * rank rounded up to 64
+  // the columns (slot * rank + j) & ke_mask of the row's own slot, zeros elsewhere; ke = text_width(...)
   __half* text;
-  int ke, k_slots, slot_is_adapter;   // slots: streams of the pass, or (1) the adapters themselves
+  int ke, ke_mask;                // ke_mask = ke - 1 where the columns are used round and round, else all ones
+  int k_slots, slot_is_adapter;   // slots: streams of the pass, or (1) the adapters themselves
 };
+
+// Columns of LoraArgs::text.  A tile of the projection has at most TC_MAX_ROWS consecutive rows and reads the columns of their
+// slots only, from a multiple of 64 on: as many columns as these span are enough (a power of two of them), used round and
+// round.  (With one column for every (stream, rank index), 256 streams of 64-node trees at rank 64 took 3.2 GB, and every
+// projection cleared them.)
+constexpr int TC_MAX_ROWS = 256;
+__host__ __device__ inline int text_width(int slots, int rows_per_slot, int rank) {
+  const int span = (TC_MAX_ROWS + rows_per_slot - 2) / rows_per_slot + 1;   // slots that so many consecutive rows can touch
+  const long long all = ((long long)slots * rank + 63) / 64 * 64, some = ((long long)span * rank + 63) / 64 * 64 + 64;
+  long long ke = 64;
+  while (ke < some) ke *= 2;
+  return (int)(all < ke ? all : ke);
+}
+__host__ __device__ inline int text_mask(int slots, int rank, int ke) { return (long long)slots * rank > ke ? ke - 1 : -1; }
 
 struct GemmArgs {
   const unsigned char* w;         // packed weights (chunked fragment-major layout)

@@ -13,12 +13,13 @@ __device__ __forceinline__ void text_store(const LoraArgs& l, int m, int seg, in
   row[0] = h;
   row[l.ke] = __float2half_rn(v - __half2float(h));
 }
-// zeros everywhere outside the columns [k0, k1) of the row
-__device__ __forceinline__ void text_clear(const LoraArgs& l, int m, int seg, int k0, int k1, int tid, int nthreads) {
+// zeros everywhere outside the r columns of the row from k0 on (round and round)
+__device__ __forceinline__ void text_clear(const LoraArgs& l, int m, int seg, int k0, int r, int tid, int nthreads) {
   __half* row = l.text + ((size_t)m * l.nseg + seg) * 2 * l.ke;
+  const int k1 = k0 + r, kw = k1 - l.ke;
   for (int k = tid; k < 2 * l.ke; k += nthreads) {
     const int kk = k < l.ke ? k : k - l.ke;
-    if (kk < k0 || kk >= k1) row[k] = __float2half_rn(0.f);
+    if ((kk < k0 || kk >= k1) && kk >= kw) row[k] = __float2half_rn(0.f);
   }
 }
 
@@ -75,11 +76,8 @@ __global__ void __launch_bounds__(SHRINK_THREADS) norm_shrink_kernel(const Shrin
   float* T = p.lora.T + ((size_t)m * p.lora.nseg + seg) * r;
   const __half* A = nullptr;
   if (a >= 0 && a < p.lora.n_slots) A = p.lora.tabA[(size_t)a * p.lora.tab_stride + p.lora.seg[seg].proj_index];
-  const int slot = p.lora.slot_is_adapter ? a : m / p.lora.rows_per_stream;
-  if (p.lora.text != nullptr && jc == 0) text_clear(p.lora, m, seg, A ? slot * r : 0, A ? slot * r + r : 0, threadIdx.x, SHRINK_THREADS);
   if (A == nullptr) {
-    if (p.lora.text == nullptr)
-      for (int j = j0 + threadIdx.x; j < j1; j += SHRINK_THREADS) T[j] = 0.f;
+    for (int j = j0 + threadIdx.x; j < j1; j += SHRINK_THREADS) T[j] = 0.f;
     return;
   }
   const float s = p.lora.scale[a];
@@ -99,10 +97,7 @@ __global__ void __launch_bounds__(SHRINK_THREADS) norm_shrink_kernel(const Shrin
       }
     }
     acc = warp_sum(acc);
-    if (lane == 0) {
-      if (p.lora.text != nullptr) text_store(p.lora, m, seg, slot * r + j, s * acc);
-      else T[j] = s * acc;
-    }
+    if (lane == 0) T[j] = s * acc;
   }
 }
 
@@ -185,11 +180,11 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_mma_kernel(const
     for (int w = 0; w < SHRINK_MMA_WARPS; ++w) tot += red[w][lane][e];
     const int m = (e < 2) ? mA : mB, j = j0 + 2 * t + (e & 1);
     if (m < m_end && j < r) {
-      if (p.lora.text != nullptr) text_store(p.lora, m, seg, stream * r + j, s * tot);
+      if (p.lora.text != nullptr) text_store(p.lora, m, seg, (stream * r + j) & p.lora.ke_mask, s * tot);
       else p.lora.T[((size_t)m * p.lora.nseg + seg) * r + j] = s * tot;
     }
   } else if (p.lora.text != nullptr && j0 == 0) {
-    for (int m = m0 + warp - 4; m < min(m0 + 16, m_end); m += 12) text_clear(p.lora, m, seg, stream * r, stream * r + r, lane, 32);
+    for (int m = m0 + warp - 4; m < min(m0 + 16, m_end); m += 12) text_clear(p.lora, m, seg, stream * r & p.lora.ke_mask, r, lane, 32);
   }
 }
 
@@ -316,7 +311,7 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_gather_kernel(co
       if (k < n && j < r) text_store(p.lora, rows[k], 0, a * r + j, s * tot);
     }
     if (rank == 0 && j0 == 0 && warp >= 4)
-      for (int k = r0 + warp - 4; k < min(r0 + 16, n); k += SHRINK_MMA_WARPS - 4) text_clear(p.lora, rows[k], 0, a * r, a * r + r, lane, 32);
+      for (int k = r0 + warp - 4; k < min(r0 + 16, n); k += SHRINK_MMA_WARPS - 4) text_clear(p.lora, rows[k], 0, a * r, r, lane, 32);
     if constexpr (S > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     else __syncthreads();
   }
@@ -360,7 +355,7 @@ cudaError_t launch_shrink(const ShrinkArgs& a, cudaStream_t st) {
   // Runs of 16 rows share an adapter: the norm (if any) as its own pass, the shrink on mma.sync from the fp16 rows.
   // With a norm this costs a second launch, which pays only when the shrink is large.
   const bool big = (long long)a.lora.rank * a.lora.nseg * a.K >= 150000;
-  if (a.lora.adapter_idx != nullptr && !a.lora.slot_is_adapter && a.lora.rows_per_stream % 16 == 0 && a.M >= 32 && (a.x_f32 == nullptr || big)) {
+  if (a.lora.adapter_idx != nullptr && a.lora.rows_per_stream % 16 == 0 && a.M >= 32 && (a.x_f32 == nullptr || big)) {
     ShrinkArgs r = a;
     if (a.x_f32 != nullptr) {
       ShrinkArgs n = a;

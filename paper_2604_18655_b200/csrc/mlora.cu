@@ -225,7 +225,7 @@ LoraArgs lora_args(mlora_ctx* c, const PassIO& io, int l, int nseg, const int* p
   la.nseg = nseg;
   for (int i = 0; i < nseg; ++i) { la.seg[i].proj_index = l * 7 + projs[i]; la.seg[i].n = widths[i]; }
   la.T = c->T;
-  if (io.tc) { la.text = c->text; la.k_slots = io.n; la.ke = (io.n * la.rank + 63) & ~63; }
+  if (io.tc) { la.text = c->text; la.k_slots = io.n; la.ke = text_width(io.n, io.T, la.rank); la.ke_mask = text_mask(io.n, la.rank, la.ke); }
   return la;
 }
 
@@ -879,8 +879,14 @@ int mlora_create(const mlora_model_desc* desc, mlora_ctx** out) {
   CKC(cudaMalloc(&c->act16, Mm * F * sizeof(__half)));
   if (d.vocab > 0) CKC(cudaMalloc(&c->logits, (size_t)d.max_streams * d.max_tree * d.vocab * sizeof(float)));   // (prefill: one row)
   CKC(cudaMalloc(&c->T, Mm * 3 * (d.lora_rank > 0 ? d.lora_rank : 1) * sizeof(float)));
-  if (d.lora_rank > 0)
-    CKC(cudaMalloc(&c->text, (size_t)d.max_streams * d.max_tree * 6 * (((size_t)d.max_streams * d.lora_rank + 63) / 64 * 64) * sizeof(__half)));
+  if (d.lora_rank > 0) {
+    size_t most = 0;                                  // the largest need over the passes' rows per stream
+    for (int T = 1; T <= d.max_tree; ++T) {
+      const size_t need = (size_t)d.max_streams * T * 6 * text_width(d.max_streams, T, d.lora_rank);
+      most = need > most ? need : most;
+    }
+    CKC(cudaMalloc(&c->text, most * sizeof(__half)));
+  }
   c->partial_floats = (size_t)16 << 20;               // 64 MB of split-K scratch
   CKC(cudaMalloc(&c->partial, c->partial_floats * sizeof(float)));
   CKC(cudaMalloc(&c->counters, 4096 * sizeof(unsigned)));
@@ -1768,7 +1774,7 @@ int mlora_linear(mlora_weight* w, const void* x, int32_t M, const int32_t* row_a
     // not need), where that fits
     const long long ke = ((long long)n_adapters * rank + 63) / 64 * 64;
     if (M >= TC_MIN_ROWS && ke <= 4096 && (size_t)M * 2 * ke * sizeof(__half) + 256 <= workspace_bytes - fixed) {
-      la.text = (__half*)(ws + (fixed + 255) / 256 * 256); la.ke = (int)ke; la.k_slots = n_adapters; la.slot_is_adapter = 1;
+      la.text = (__half*)(ws + (fixed + 255) / 256 * 256); la.ke = (int)ke; la.ke_mask = -1; la.k_slots = n_adapters; la.slot_is_adapter = 1;
     }
     ShrinkArgs s{};
     s.h_in = (const __half*)x; s.M = M; s.K = w->w.K; s.lora = la;

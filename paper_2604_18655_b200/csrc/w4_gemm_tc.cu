@@ -3,16 +3,16 @@
 // Sec. 3.3), the LoRA expand T B (Eq. 1-4, second factor) as further k-steps, and the projection's epilogue, in one kernel.
 //
 // "Swap-AB": the 128 output features of a CTA are the UMMA M dimension, NR rows the N dimension.  Warp roles:
-//   - eight warps dequantise: warps 0-3 the even k-steps (64 input features), warps 4-7 the odd ones, two n-tiles (32
-//     features) a warp.  The packed bytes come through a private cp.async ring; ldmatrix hands every lane the words of
+//   - groups of four warps dequantise, two groups up to 128 rows and four beyond: group q takes every second (fourth) k-step
+//     (64 input features) from step q on, two n-tiles (32 features) a warp.  The packed bytes come through a private cp.async ring; ldmatrix hands every lane the words of
 //     its k16 slices, dequant8() unpacks them (exactly fp16(q * scale), as on every other path), and one tcgen05.st per
 //     n-tile puts them into TENSOR MEMORY, where the MMA reads its A operand.  The dequantised weights therefore never
 //     touch shared memory, which only carries the activations, and no proxy fence is needed per step.
 //   - one thread issues the TMA copies of the activation tiles (128-byte swizzle, rows past M read as zero),
 //   - one thread issues the MMAs (4 x K 16 per step, fp32 accumulator in tensor memory).
-// Adapters: T = s x A^T arrives as an fp16 matrix [M][segment][value | rounding remainder][slot * rank + j] that is zero
-// outside the row's own slot (a slot = a stream of the pass, or an adapter of the single-projection call), so that
-// y += T B is two more MMAs per 64 (slot, rank) indices with B as the A operand, read from the caller's matrices by the
+// Adapters: T = s x A^T arrives as an fp16 matrix [M][segment][value | rounding remainder][slot * rank + j, round and round]
+// that is zero outside the row's own slot (a slot = a stream of the pass, or an adapter of the single-projection call), so
+// that y += T B is two more MMAs per 64 (slot, rank) indices with B as the A operand, read from the caller's matrices by the
 // dequantising warps.  Value + remainder keep T at fp32 accuracy.
 // Few output features and many SMs: a cluster of S CTAs splits K, each CTA ends with NR / S rows: the others push their
 // accumulators into its shared memory (distributed shared memory, reused activation tiles) and it adds them in rank order
@@ -166,7 +166,8 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
           if (u < L.KT) copy(&act_map, u * TC_BK);
           else {
             if (!waited) { asm volatile("griddepcontrol.wait;" ::: "memory"); waited = true; }
-            const int e = u - L.KT, sg = (e >= x.nE) + (e >= 2 * x.nE), seg = x.seg0 + sg, c = x.kb0 + (e - sg * x.nE) * 64;
+            const int e = u - L.KT, sg = (e >= x.nE) + (e >= 2 * x.nE), seg = x.seg0 + sg;
+            const int c = (x.kb0 + (e - sg * x.nE) * 64) & p.lora.ke_mask;
             copy(&text_map, (seg * 2) * p.lora.ke + c);
             copy(&text_map, (seg * 2 + 1) * p.lora.ke + c);
           }

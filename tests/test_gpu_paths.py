@@ -56,6 +56,36 @@ def test_quantiser_tails(mb, count):
         assert np.array_equal(out.cpu().numpy().reshape(1, -1), ref.quantize_act_int8(x, 0.02))
 
 
+@pytest.mark.parametrize("n,T,rank", [(40, 30, 20), (70, 6, 12), (9, 64, 64), (300, 1, 9), (130, 3, 64)])
+def test_adapters_of_passes_with_more_streams_than_a_row_tile_has(GpuModel, n, T, rank):
+    """The adapters' T has columns for the streams that one row tile can touch; further streams use them again."""
+    cfg = gen.ModelCfg("streams", 1, 128, 4, 2, 64, 192, 304, 64, rank, gen.configs.ALL7, 5, n, 33, b_std=0.05)
+    _, orc, gm = make_pair(GpuModel, cfg, max_suffix=T, max_tree=T)
+    ids = gen.make_prompt_ids(cfg, 0)
+    compare(gm.prefill(ids), orc.prefill_shared(ids, n_streams=n), "prefill logits")
+    ad = [(s * 7) % 6 - 1 for s in range(n)]
+    par = np.stack([np.array([-1] + [(i - 1) // 2 for i in range(1, T)], dtype=np.int32)] * n)
+    tree = np.random.default_rng(n).integers(0, cfg.vocab, size=(n, T), dtype=np.int32)
+    compare(gm.verify(ad, tree, par)["logits"], orc.verify_tree(ad, par, tree)["logits"], f"{n} streams of {T} rows, rank {rank}")
+    gm.close()
+
+
+def test_adapter_scratch_of_many_streams_stays_proportional():
+    """A context for 256 streams of 64-node trees at rank 64 (one small layer) fits in half of what the adapters' T alone took
+    with a column for every (stream, rank index)."""
+    from paper_2604_18655_b200 import binding as mb
+    cfg = gen.ModelCfg("scratch", 1, 64, 1, 1, 64, 64, 0, 64, 64, gen.configs.ALL7, 1, 256, 64)
+    m = gen.make_model(cfg, 0)
+    to = lambda ts: [dev(t) for t in ts]
+    w, s, ga, gf = to(m.qweight), to(m.scales), to(m.rms_attn), to(m.rms_ffn)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    ctx = mb.mlora_create(cfg, w, s, ga, gf, None, None, max_adapters=1, max_streams=256, max_prefix=64, max_suffix=64, max_tree=64)
+    used = before - torch.cuda.mem_get_info()[0]
+    mb.mlora_destroy(ctx)
+    assert used < 256 * 64 * 6 * 256 * 64 * 2 // 2, used
+
+
 # ------------------------------------------------------------------ attention
 @pytest.mark.parametrize("n,T,Hq,Hkv,hd,P,suf,branch", [
     (2, 9, 6, 2, 64, 129, [0, 1], (2, 3)),            # groups of three heads: 126 of a block's 128 rows

@@ -158,7 +158,7 @@ struct ShrinkArgs {
   __half* h_out;                  // NORM mode: normalised fp16 rows written here
   int M, K;
   LoraArgs lora;                  // adapter_idx == nullptr: only the norm is done
-  int pdl;                        // launch_shrink_rows: programmatic launch behind the kernel that writes h_in
+  int pdl;                        // programmatic launch behind the kernel that writes h_in
 };
 
 struct AttnArgs {
@@ -352,10 +352,13 @@ constexpr int TC_MIN_ROWS = 9;
 cudaError_t init_gemm_tc();
 bool gemm_tc_eligible(const GemmArgs& a);
 cudaError_t launch_gemm_tc(const GemmArgs& a, int sm_count, int* status, cudaStream_t st);
+constexpr int SHRINK_MAX_K = 48 * 1024;   // launch_shrink: a row as fp16 in shared memory
 cudaError_t launch_shrink(const ShrinkArgs& a, cudaStream_t st);
 // T of a pass whose rows are grouped by stream (rows_per_stream each), from fp16 rows, on mma.sync
 cudaError_t launch_shrink_rows(const ShrinkArgs& a, cudaStream_t st);
 cudaError_t launch_shrink_gather(const ShrinkArgs& a, cudaStream_t st);
+// y += T B for rows that pick their adapters one by one
+cudaError_t launch_expand_rows(const LoraArgs& l, int M, float* y, int N, cudaStream_t st);
 bool tensor_maps_available();
 cudaError_t launch_embed(const int32_t* tokens, const __half* embed, const __half* hidden_in, float* X, int M,
                          int d, int vocab, int* status, cudaStream_t st, const __half* forecast = nullptr,

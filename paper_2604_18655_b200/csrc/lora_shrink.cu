@@ -13,13 +13,14 @@ __device__ __forceinline__ void text_store(const LoraArgs& l, int m, int seg, in
   row[0] = h;
   row[l.ke] = __float2half_rn(v - __half2float(h));
 }
-// zeros everywhere outside the r columns of the row from k0 on (round and round)
+// zeros everywhere outside the r columns of the row from k0 on (WRAP: round and round)
+template <bool WRAP>
 __device__ __forceinline__ void text_clear(const LoraArgs& l, int m, int seg, int k0, int r, int tid, int nthreads) {
   __half* row = l.text + ((size_t)m * l.nseg + seg) * 2 * l.ke;
   const int k1 = k0 + r, kw = k1 - l.ke;
   for (int k = tid; k < 2 * l.ke; k += nthreads) {
     const int kk = k < l.ke ? k : k - l.ke;
-    if ((kk < k0 || kk >= k1) && kk >= kw) row[k] = __float2half_rn(0.f);
+    if ((kk < k0 || kk >= k1) && (!WRAP || kk >= kw)) row[k] = __float2half_rn(0.f);
   }
 }
 
@@ -27,8 +28,9 @@ constexpr int SHRINK_THREADS = 256;
 constexpr int SHRINK_JCHUNK = 8;   // rank indices per CTA
 
 __global__ void __launch_bounds__(SHRINK_THREADS) norm_shrink_kernel(const ShrinkArgs p, const int jchunks) {
-  // (the tensor-core projection launched after this kernel may start streaming its weights now)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // (as a programmatic launch it waits at once and only then lets the projection behind it start, which streams its weights
+  // meanwhile and reads the call's inputs ahead of its own wait: everything earlier is complete then)
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __half* hrow = reinterpret_cast<__half*>(smem_raw);          // [K]
   __shared__ float red[SHRINK_THREADS / 32];
@@ -184,7 +186,7 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_mma_kernel(const
       else p.lora.T[((size_t)m * p.lora.nseg + seg) * r + j] = s * tot;
     }
   } else if (p.lora.text != nullptr && j0 == 0) {
-    for (int m = m0 + warp - 4; m < min(m0 + 16, m_end); m += 12) text_clear(p.lora, m, seg, stream * r & p.lora.ke_mask, r, lane, 32);
+    for (int m = m0 + warp - 4; m < min(m0 + 16, m_end); m += 12) text_clear<true>(p.lora, m, seg, stream * r & p.lora.ke_mask, r, lane, 32);
   }
 }
 
@@ -213,7 +215,8 @@ cudaError_t launch_shrink_rows(const ShrinkArgs& a, cudaStream_t st) {
 // every adapter once per row: 115 MB through L2 and 18 us for 250 rows of 14336 inputs and 8 adapters.)
 constexpr int SG_BLOCKS = 2;                 // 64-feature blocks of a warp per CTA: K share = 16 warps x 2 x 64 at most
 constexpr int SG_MAX_ROWS = 4096;
-template <int S>
+// TEXT: T goes into the matrix that the projection reads; else to fp32 T, and rows without an adapter are not looked at.
+template <int S, bool TEXT>
 __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_gather_kernel(const ShrinkArgs p) {
   __shared__ float red[SHRINK_MMA_WARPS][32][4];
   __shared__ float part[S][128];             // first CTA of a cluster: the CTAs' sums of a group of 16 rows
@@ -225,7 +228,7 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_gather_kernel(co
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int rank = S > 1 ? (int)blockIdx.x : 0, j0 = blockIdx.y * 8, a = blockIdx.z, r = p.lora.rank, K = p.K;
   const __half* const A = p.lora.tabA[(size_t)a * p.lora.tab_stride + p.lora.seg[0].proj_index];
-  const float s = p.lora.scale[a];
+  const float s = TEXT || A != nullptr ? p.lora.scale[a] : 0.f;
   // this warp's blocks of A, while the rows are looked up
   const int nblk = K / 64, b_lo = (nblk * (rank * SHRINK_MMA_WARPS + warp)) / (S * SHRINK_MMA_WARPS), b_hi = (nblk * (rank * SHRINK_MMA_WARPS + warp + 1)) / (S * SHRINK_MMA_WARPS);
   const uint4* const Ar = reinterpret_cast<const uint4*>(A + (size_t)min(j0 + g, r - 1) * K) + 2 * t;
@@ -241,7 +244,7 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_gather_kernel(co
   for (int base = 0; base < p.M; base += SHRINK_MMA_WARPS * 32) {
     const int m = base + threadIdx.x;
     const int am = m < p.M ? p.lora.adapter_idx[m] : -1;
-    const bool mine = m < p.M && am == a && A != nullptr;
+    const bool mine = m < p.M && am == a && (!TEXT || A != nullptr);
     const unsigned bal = __ballot_sync(0xffffffffu, mine);
     if (lane == 0) s_w[warp] = __popc(bal);
     __syncthreads();
@@ -250,9 +253,9 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_gather_kernel(co
     if (mine) rows[off + __popc(bal & ((1u << lane) - 1u))] = (short)m;
     __syncthreads();
     if (threadIdx.x == 0) { int n = s_n; for (int q = 0; q < SHRINK_MMA_WARPS; ++q) n += s_w[q]; s_n = n; }
-    if (rank == 0 && j0 == 0) {
+    if (TEXT && rank == 0 && j0 == 0) {
       unsigned none = __ballot_sync(0xffffffffu, m < p.M && ((a == 0 && (am < 0 || am >= p.lora.n_slots)) || (am == a && A == nullptr)));
-      for (; none != 0u; none &= none - 1u) text_clear(p.lora, base + warp * 32 + __ffs(none) - 1, 0, 0, 0, lane, 32);
+      for (; none != 0u; none &= none - 1u) text_clear<false>(p.lora, base + warp * 32 + __ffs(none) - 1, 0, 0, 0, lane, 32);
     }
     __syncthreads();
   }
@@ -282,7 +285,7 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_gather_kernel(co
     for (int b = b_lo + SG_BLOCKS; b < b_hi; ++b)          // (a K share beyond what the registers hold)
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        const uint4 xa = *(hA + b * 8 + q), xb = *(hB + b * 8 + q), xw = j0 + g < r ? *(Ar + b * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
+        const uint4 xa = *(hA + b * 8 + q), xb = *(hB + b * 8 + q), xw = (TEXT || A != nullptr) && j0 + g < r ? *(Ar + b * 8 + q) : make_uint4(0u, 0u, 0u, 0u);
         const uint32_t f0[4] = {xa.x, xb.x, xa.y, xb.y}, f1[4] = {xa.z, xb.z, xa.w, xb.w};
         mma_16816(acc, f0, xw.x, xw.y);
         mma_16816(acc, f1, xw.z, xw.w);
@@ -308,16 +311,19 @@ __global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_gather_kernel(co
         for (int q = 0; q < S; ++q) tot += part[q][threadIdx.x];
       }
       const int k = r0 + g + (e >= 2 ? 8 : 0), j = j0 + 2 * t + (e & 1);
-      if (k < n && j < r) text_store(p.lora, rows[k], 0, a * r + j, s * tot);
+      if (k < n && j < r) {
+        if (TEXT) text_store(p.lora, rows[k], 0, a * r + j, s * tot);
+        else p.lora.T[(size_t)rows[k] * r + j] = s * tot;
+      }
     }
-    if (rank == 0 && j0 == 0 && warp >= 4)
-      for (int k = r0 + warp - 4; k < min(r0 + 16, n); k += SHRINK_MMA_WARPS - 4) text_clear(p.lora, rows[k], 0, a * r, r, lane, 32);
+    if (TEXT && rank == 0 && j0 == 0 && warp >= 4)
+      for (int k = r0 + warp - 4; k < min(r0 + 16, n); k += SHRINK_MMA_WARPS - 4) text_clear<false>(p.lora, rows[k], 0, a * r, r, lane, 32);
     if constexpr (S > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     else __syncthreads();
   }
 }
 
-template <int S>
+template <int S, bool TEXT>
 static cudaError_t launch_gather(const ShrinkArgs& a, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(S, (unsigned)((a.lora.rank + 7) / 8), (unsigned)a.lora.n_slots);
@@ -330,25 +336,127 @@ static cudaError_t launch_gather(const ShrinkArgs& a, cudaStream_t st) {
   attr[1].val.clusterDim.x = S; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = S > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, shrink_gather_kernel<S>, a);
+  return cudaLaunchKernelEx(&cfg, shrink_gather_kernel<S, TEXT>, a);
 }
-// T of rows with adapters of their own (LoraArgs::text, slots = adapters)
-cudaError_t launch_shrink_gather(const ShrinkArgs& a, cudaStream_t st) {
+// T of rows with adapters of their own (LoraArgs::text with slots = adapters; or fp32)
+template <bool TEXT>
+static cudaError_t launch_gather_split(const ShrinkArgs& a, cudaStream_t st) {
   // K split so that a warp's share fits its registers, as long as the grid stays within a few CTAs an SM
   const int per = SHRINK_MMA_WARPS * SG_BLOCKS * 64, ctas = (a.lora.rank + 7) / 8 * a.lora.n_slots;
-  if (a.K > 4 * per && ctas <= 64) return launch_gather<8>(a, st);
-  if (a.K > 2 * per && ctas <= 128) return launch_gather<4>(a, st);
-  if (a.K > per && ctas <= 256) return launch_gather<2>(a, st);
-  return launch_gather<1>(a, st);
+  if (a.K > 4 * per && ctas <= 64) return launch_gather<8, TEXT>(a, st);
+  if (a.K > 2 * per && ctas <= 128) return launch_gather<4, TEXT>(a, st);
+  if (a.K > per && ctas <= 256) return launch_gather<2, TEXT>(a, st);
+  return launch_gather<1, TEXT>(a, st);
+}
+cudaError_t launch_shrink_gather(const ShrinkArgs& a, cudaStream_t st) {
+  return a.lora.text != nullptr ? launch_gather_split<true>(a, st) : launch_gather_split<false>(a, st);
+}
+
+// The expand of rows that pick their adapters one by one from many: y[m] += T[m] B (Eq. 1-4, second factor), after the
+// projection.  A CTA takes an adapter (or, more adapters than rows, a row's adapter, if no row before has it) and 256 columns of
+// its B, which it reads once, in shared memory, for all rows that use the adapter: fp32 sums, rank indices in rising order.
+// Bound by B of the adapters in use; inside the tensor-core projection every row tile paid for every adapter instead, 64 of
+// them or 7 that occur (32 rows of 4096 x 4096, 64 adapters of rank 64: 37.6 us, 17.8 with this kernel).
+constexpr int EXP_COLS = 256, EXP_ROWS = 16, EXP_RANK = 64, EXP_THREADS = 256;
+__global__ void __launch_bounds__(EXP_THREADS) expand_rows_kernel(const LoraArgs l, const int M, const int by_row, float* __restrict__ y, const int N) {
+  __shared__ __align__(16) __half s_B[EXP_RANK][EXP_COLS];
+  __shared__ __align__(16) float s_T[EXP_ROWS][EXP_RANK];
+  __shared__ short rows[4096];
+  __shared__ int s_w[EXP_THREADS / 32], s_n;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, r = l.rank, n0 = blockIdx.x * EXP_COLS;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // (the call's inputs, complete before the kernels ahead started)
+  const int a = by_row ? l.adapter_idx[blockIdx.y] : (int)blockIdx.y;
+  const __half* const B = a >= 0 && a < l.n_slots ? l.tabB[(size_t)a * l.tab_stride + l.seg[0].proj_index] : nullptr;
+  // (every CTA takes the wait: a kernel that waits for this one must find the projection done, too)
+  if (B == nullptr) { asm volatile("griddepcontrol.wait;" ::: "memory"); return; }
+  auto fetch_B = [&](int j0) {                             // rank indices j0 .. of the CTA's columns
+    const int nj = min(EXP_RANK, r - j0);
+    for (int i = tid; i < nj * (EXP_COLS / 8); i += EXP_THREADS) {
+      const int j = i / (EXP_COLS / 8), c = (i % (EXP_COLS / 8)) * 8;
+      if (n0 + c < N)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(&s_B[j][c])), "l"(B + (size_t)(j0 + j) * N + n0 + c) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (tid == 0) s_n = 0;
+  __syncthreads();
+  for (int base = 0; base < M; base += EXP_THREADS) {      // the adapter's rows, in rising order
+    const int m = base + tid;
+    const bool mine = m < M && l.adapter_idx[m] == a;
+    const unsigned bal = __ballot_sync(0xffffffffu, mine);
+    if (lane == 0) s_w[warp] = __popc(bal);
+    __syncthreads();
+    int off = s_n, all = 0;
+    for (int q = 0; q < EXP_THREADS / 32; ++q) { if (q < warp) off += s_w[q]; all += s_w[q]; }
+    if (mine) rows[off + __popc(bal & ((1u << lane) - 1u))] = (short)m;
+    __syncthreads();
+    if (tid == 0) s_n += all;
+    __syncthreads();
+  }
+  const int n = s_n;
+  const bool on = n > 0 && (!by_row || rows[0] == (int)blockIdx.y);
+  if (on) fetch_B(0);
+  asm volatile("griddepcontrol.wait;" ::: "memory");      // T and the projection's y
+  if (!on) return;
+  const int c = (tid & (EXP_COLS / 2 - 1)) * 2, grp = tid / (EXP_COLS / 2);   // two columns, every second row
+  for (int j0 = 0; j0 < r; j0 += EXP_RANK) {
+    const int nj = min(EXP_RANK, r - j0);
+    if (j0 > 0) { __syncthreads(); fetch_B(j0); }
+    for (int r0 = 0; r0 < n; r0 += EXP_ROWS) {
+      const int nr = min(EXP_ROWS, n - r0);
+      if (r0 > 0) __syncthreads();
+      for (int i = tid; i < nr * EXP_RANK; i += EXP_THREADS) {
+        const int q = i / EXP_RANK, j = i % EXP_RANK;
+        s_T[q][j] = j < nj ? __ldcg(l.T + (size_t)rows[r0 + q] * r + j0 + j) : 0.f;
+      }
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+      if (n0 + c < N) {
+        for (int q = grp; q < nr; q += 4) {                // two rows at a time
+          const bool two = q + 2 < nr;
+          float2* const y0 = reinterpret_cast<float2*>(y + (size_t)rows[r0 + q] * N + n0 + c);
+          float2* const y1 = two ? reinterpret_cast<float2*>(y + (size_t)rows[r0 + q + 2] * N + n0 + c) : y0;
+          const float2 o0 = __ldcg(y0), o1 = __ldcg(y1);
+          const float *t0 = s_T[q], *t1 = s_T[two ? q + 2 : q];
+          float a0 = 0.f, b0 = 0.f, a1 = 0.f, b1 = 0.f;
+#pragma unroll 4
+          for (int j = 0; j < nj; ++j) {
+            const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&s_B[j][c]));
+            const float u = t0[j], v = t1[j];
+            a0 = fmaf(u, b.x, a0); b0 = fmaf(u, b.y, b0);
+            a1 = fmaf(v, b.x, a1); b1 = fmaf(v, b.y, b1);
+          }
+          *y0 = make_float2(o0.x + a0, o0.y + b0);
+          if (two) *y1 = make_float2(o1.x + a1, o1.y + b1);
+        }
+      }
+    }
+  }
+}
+cudaError_t launch_expand_rows(const LoraArgs& l, int M, float* y, int N, cudaStream_t st) {
+  const int by_row = l.n_slots > M;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)((N + EXP_COLS - 1) / EXP_COLS), (unsigned)(by_row ? M : l.n_slots));
+  cfg.blockDim = dim3(EXP_THREADS);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, expand_rows_kernel, l, M, by_row, y, N);
 }
 
 cudaError_t init_shrink() {
   cudaError_t e;
 #define SG_SET(S) \
-  if ((e = full_carveout(shrink_gather_kernel<S>)) != cudaSuccess) return e;
+  if ((e = full_carveout(shrink_gather_kernel<S, true>)) != cudaSuccess) return e; \
+  if ((e = full_carveout(shrink_gather_kernel<S, false>)) != cudaSuccess) return e;
   SG_SET(1) SG_SET(2) SG_SET(4) SG_SET(8)
 #undef SG_SET
-  return cudaFuncSetAttribute(norm_shrink_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+  if ((e = full_carveout(expand_rows_kernel)) != cudaSuccess) return e;
+  return cudaFuncSetAttribute(norm_shrink_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SHRINK_MAX_K * (int)sizeof(__half));
 }
 
 cudaError_t launch_shrink(const ShrinkArgs& a, cudaStream_t st) {
@@ -373,9 +481,15 @@ cudaError_t launch_shrink(const ShrinkArgs& a, cudaStream_t st) {
     jchunks = (a.lora.rank + SHRINK_JCHUNK - 1) / SHRINK_JCHUNK;
     gy = jchunks * a.lora.nseg;
   }
-  dim3 grid(a.M, gy);
-  norm_shrink_kernel<<<grid, SHRINK_THREADS, (size_t)a.K * sizeof(__half), st>>>(a, jchunks);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)a.M, (unsigned)gy);
+  cfg.blockDim = dim3(SHRINK_THREADS); cfg.dynamicSmemBytes = (size_t)a.K * sizeof(__half); cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = a.pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, norm_shrink_kernel, a, jchunks);
 }
 
 }  // namespace mlora

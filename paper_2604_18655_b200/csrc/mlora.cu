@@ -1763,33 +1763,56 @@ int mlora_linear(mlora_weight* w, const void* x, int32_t M, const int32_t* row_a
       return MLORA_OK;
     }
   }
-  LoraArgs la{};
-  if (lora) {
-    la.adapter_idx = row_adapter; la.rows_per_stream = 1;
-    la.tabA = (const __half* const*)A; la.tabB = (const __half* const*)B; la.scale = scale;
-    la.tab_stride = 1; la.n_slots = n_adapters; la.rank = rank; la.nseg = 1;
-    la.seg[0].proj_index = 0; la.seg[0].n = w->w.N;
-    la.T = (float*)(ws + LIN_COUNTER_BYTES);
-    // the tcgen05 kernel takes T as a matrix over all adapters (in the room of the split-K partial sums, which it does
-    // not need), where that fits
-    const long long ke = ((long long)n_adapters * rank + 63) / 64 * 64;
-    if (M >= TC_MIN_ROWS && ke <= 4096 && (size_t)M * 2 * ke * sizeof(__half) + 256 <= workspace_bytes - fixed) {
-      la.text = (__half*)(ws + (fixed + 255) / 256 * 256); la.ke = (int)ke; la.ke_mask = -1; la.k_slots = n_adapters; la.slot_is_adapter = 1;
-    }
-    ShrinkArgs s{};
-    s.h_in = (const __half*)x; s.M = M; s.K = w->w.K; s.lora = la;
-    if (la.text != nullptr) CK(launch_shrink_gather(s, w->stream));
-    else CK(launch_shrink(s, w->stream));
-  }
   GemmArgs g{};
   g.w = w->w.data; g.K = w->w.K; g.N = w->w.N; g.G = w->w.G; g.h = (const __half*)x; g.M = M;
   g.mode = MODE_PLAIN; g.epi = EPI_F32; g.out_f32 = y; g.ldo = w->w.N;
   g.partial = (float*)(ws + fixed); g.partial_capacity = (workspace_bytes - fixed) / sizeof(float);
   g.counters = (unsigned*)(ws + LIN_SYNC_BYTES);
-  g.lora = la;
-  g.late_wait = lora;                                      // (x is there already: the shrink kernel adds only T)
-  if (gemm_tc_eligible(g) && (!lora || la.text != nullptr)) CK(launch_gemm_tc(g, w->sm_count, (int*)(ws + 32), w->stream));
-  else CK(launch_gemm(g, w->stream));
+  if (!lora) {
+    if (gemm_tc_eligible(g)) CK(launch_gemm_tc(g, w->sm_count, (int*)(ws + 32), w->stream));
+    else CK(launch_gemm(g, w->stream));
+    return MLORA_OK;
+  }
+  LoraArgs la{};
+  la.adapter_idx = row_adapter; la.rows_per_stream = 1;
+  la.tabA = (const __half* const*)A; la.tabB = (const __half* const*)B; la.scale = scale;
+  la.tab_stride = 1; la.n_slots = n_adapters; la.rank = rank; la.nseg = 1;
+  la.seg[0].proj_index = 0; la.seg[0].n = w->w.N;
+  la.T = (float*)(ws + LIN_COUNTER_BYTES);
+  ShrinkArgs s{};
+  s.h_in = (const __half*)x; s.M = M; s.K = w->w.K; s.lora = la;
+  if (!gemm_tc_eligible(g)) {
+    CK(launch_shrink(s, w->stream));
+    g.lora = la;
+    CK(launch_gemm(g, w->stream));
+    return MLORA_OK;
+  }
+  g.late_wait = 1;                                         // (x is there already: the shrink kernel adds only T)
+  // Where the expand is done.  Inside the projection, as further k-steps over ALL adapters (T is a matrix with a column for
+  // each of their rank indices): right while that is little (up to 512 columns), or not much for every row (up to 8) and most
+  // adapters have several rows anyway.  Else by a kernel of its own that reads the adapters in use.  4096 x 4096, inside / by
+  // its own kernel, us: 256 rows of 64 adapters of rank 16 26.9 / 30.6, 128 rows 26.8 / 22.3; 256 rows, 32 of rank 64 36.8 /
+  // 48.8, 32 rows 28.4 / 18.2; 1000 rows, 64 of rank 64 106 / 91, 32 rows 37.6 / 17.8.  (14336 x 4096, 32 rows, 16 of rank 64:
+  // 35.8 / 37.1, on the wrong side.)
+  const long long ke = ((long long)n_adapters * rank + 63) / 64 * 64;
+  const bool inside = ke <= 512 || (ke <= 2048 && ke <= 8ll * M && M >= 4ll * n_adapters);
+  if (inside && (size_t)M * ke * 2 * sizeof(__half) <= workspace_bytes - fixed) {
+    // (T in the room of the split-K partial sums, which the tensor-core kernel does not need; the documented workspace has it
+    // from 256 output features on)
+    la.text = (__half*)(ws + fixed); la.ke = (int)ke; la.ke_mask = -1; la.k_slots = n_adapters; la.slot_is_adapter = 1;
+    s.lora = g.lora = la;
+    CK(launch_shrink_gather(s, w->stream));
+    CK(launch_gemm_tc(g, w->sm_count, (int*)(ws + 32), w->stream));
+  } else {
+    // T adapter by adapter where they have several rows each and there is enough of it to fill the machine, else row by row:
+    // 256 rows, 64 adapters of rank 64 42.5 / 44.7 us, 128 rows, 32 adapters 34.5 / 30.6, 256 rows, 128 adapters 57.9 / 52.6
+    s.pdl = 1;
+    // (which holds a row in shared memory)
+    if ((M >= 256 && M >= 4ll * n_adapters) || w->w.K > SHRINK_MAX_K) CK(launch_shrink_gather(s, w->stream));
+    else CK(launch_shrink(s, w->stream));
+    CK(launch_gemm_tc(g, w->sm_count, (int*)(ws + 32), w->stream));
+    CK(launch_expand_rows(la, M, y, w->w.N, w->stream));
+  }
   return MLORA_OK;
 }
 

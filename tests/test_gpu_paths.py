@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 import gen
+from oracle import ref
 from tests.helpers import check_argmax, compare
 from tests.test_gpu_kernels import dev, mb, run_attention, run_linear  # noqa: F401  (mb: fixture)
 from tests.test_gpu_model import GpuModel, compare_kv, make_pair  # noqa: F401
@@ -43,9 +44,53 @@ def test_shrink_of_rows_with_their_own_adapters(mb, M, n_ad, rank, K):
     compare(got, want, f"gather shrink M{M} adapters {n_ad} rank {rank} K{K}")
 
 
+@pytest.mark.parametrize("M,n_ad,rank,K,N", [
+    (9, 64, 64, 256, 208),        # 4096 columns of (adapter, rank index), few of them in use
+    (32, 65, 64, 512, 1040),      # more than that
+    (250, 300, 20, 320, 144),     # more adapters than rows, a rank off the multiples of 8
+    (129, 128, 64, 192, 4112),
+    (700, 90, 24, 320, 9600),     # about eight rows an adapter: groups of sixteen rows, and more
+    (4096, 5000, 9, 64, 16),      # the most rows, the narrowest output
+    (40, 7, 130, 256, 64),        # a rank above 64
+    (64, 40, 16, 14336, 128),     # the widest split of K
+    (300, 64, 64, 1088, 528),     # T adapter by adapter ahead of the separate expand
+    (600, 70, 70, 64, 48),
+    (64, 70, 16, 49216, 16),      # rows too long for the row-wise shrink
+])
+def test_projection_with_many_adapters(mb, M, n_ad, rank, K, N):
+    """Calls whose rows pick from many adapters: the expand is a kernel of its own over the ones that occur.  The workspace is the
+    smallest that the call takes; rows without an adapter, adapters without matrices."""
+    rng = np.random.default_rng(M + n_ad)
+    qb, sc = gen.quantize_int4(rng.standard_normal((K, N)).astype(np.float32) * 0.02, 64)
+    x = rng.standard_normal((M, K)).astype(np.float16)
+    A = (rng.standard_normal((n_ad, rank, K)) / rank).astype(np.float16)
+    B = (rng.standard_normal((n_ad, rank, N)) * 0.05).astype(np.float16)
+    scale = (16.0 / rank * (1 + 0.25 * (np.arange(n_ad) % 8))).astype(np.float32)
+    rows = rng.integers(-1, n_ad, size=M).astype(np.int32)
+    rows[0], rows[1], rows[-1] = n_ad, -7, rows[M // 2]
+    dA, dB = dev(A), dev(B)
+    pa, pb = [torch.tensor([t[i].data_ptr() for i in range(n_ad)], dtype=torch.int64, device="cuda") for t in (dA, dB)]
+    none = int(rows[2]) if rows[2] >= 0 else 0
+    pa[none] = 0                                       # an adapter without matrices
+    pb[none] = 0
+    w = mb.mlora_weight_create(dev(qb), dev(sc), K, N, 64)
+    need = mb.mlora_linear_workspace_bytes(w, M, rank) - 7 * M * N * 4
+    ws = torch.full((need + 4096,), 255, dtype=torch.uint8, device="cuda")      # (what lies behind must stay as it is)
+    ws[:16640] = 0
+    y = torch.empty(M, N, dtype=torch.float32, device="cuda")
+    for _ in range(2):
+        mb.mlora_linear(w, dev(x), y, ws[:need], dev(rows), pa, pb, dev(scale), rank)
+    torch.cuda.synchronize()
+    rows = np.where((rows >= n_ad) | (rows == none), -1, np.maximum(rows, -1))
+    f = np.float64
+    want = ref.linear_lora(x.astype(f), ref.dequant(qb, sc, 64).astype(f), rows, list(A.astype(f)), list(B.astype(f)), scale.astype(f))
+    mb.mlora_weight_destroy(w)
+    compare(y.cpu().numpy(), want, f"M{M} adapters {n_ad}x{rank} K{K} N{N}")
+    assert bool((ws[need:] == 255).all())
+
+
 @pytest.mark.parametrize("count", [1, 7, 8, 9, 1023, 1025])
 def test_quantiser_tails(mb, count):
-    from oracle import ref
     x = np.random.default_rng(count).standard_normal((1, count)).astype(np.float16)
     for off in (0, 1):           # (an input that starts between 16-byte boundaries)
         buf = torch.zeros(count + 8, dtype=torch.float16, device="cuda")

@@ -133,10 +133,14 @@ struct GemmArgs {
   LoraArgs lora;
   // tcgen05 path only
   int late_wait;                  // the kernel ahead produces only the adapters' T: the activations are complete already
-  const unsigned long long* ssq_in;   // the rows of h still lack 1/rms: their sums of squares [M] (fixed point), or nullptr
+  // (sums of squares: ssq_add, row_down; the second part of each array lies ssq_hi entries on)
+  const unsigned long long* ssq_in;   // the rows of h still lack 1/rms: their sums of squares [M], or nullptr ...
+  const unsigned long long* ssq_in_prev;   // ... and those of the norm before
   float eps;
   unsigned long long* ssq_out;    // EPI_RESID: sums of squares of the new residual rows are added here (nullptr: not wanted)
-  __half* xg_out;                 // EPI_RESID: new residual x gain_next as fp16 (nullptr: not wanted)
+  const unsigned long long* ssq_out_prev;   // ... those of the norm before
+  size_t ssq_hi;
+  __half* xg_out;                 // EPI_RESID: new residual x gain_next (x row_down) as fp16 (nullptr: not wanted)
   const __half* gain_next;
   // EPI_QKV: row m = (stream m / T, node m % T) sits at position pos_base + suffix_len[stream] + depth[m]; its K/V go to row
   // suffix_len[stream] + node of the stream's segment
@@ -363,7 +367,7 @@ bool tensor_maps_available();
 cudaError_t launch_embed(const int32_t* tokens, const __half* embed, const __half* hidden_in, float* X, int M,
                          int d, int vocab, int* status, cudaStream_t st, const __half* forecast = nullptr,
                          int n_forecast = 0, const __half* gain = nullptr, __half* xg = nullptr,
-                         unsigned long long* ssq = nullptr);
+                         unsigned long long* ssq = nullptr, size_t ssq_hi = 0);
 cudaError_t launch_draft(const float* logits, int V, int n, int R, int m, int wmax, const int32_t* widths,
                          const int32_t* level, const int32_t* rank, const int32_t* forecast_of, const int32_t* acc_len,
                          const int32_t* acc_idx, const int32_t* next, int32_t* cand, int32_t* out_tokens, int* status,
@@ -507,6 +511,46 @@ __device__ __forceinline__ uint4 head_piece_f16(const float* __restrict__ head, 
 #pragma unroll
   for (int i = 0; i < 4; ++i) o[i] = __halves2half2(__float2half_rn(v[2 * i]), __float2half_rn(v[2 * i + 1]));
   return make_uint4(h2_as_u32(o[0]), h2_as_u32(o[1]), h2_as_u32(o[2]), h2_as_u32(o[3]));
+}
+
+// ---- rows of a pass that travel without their 1/rms (RMSNorm, Sec. 3.1, is linear up to that factor): fp16 x * gain, and the
+// row's sum of squares for whoever consumes it.  The sum is collected in 64-bit fixed point, so that it does not depend on the
+// order: contributions below 2^20 in units of 2^-32, larger ones in units of 1 in a second array `hi` entries on (2^-21 of
+// them), which keeps both the precision of small rows and any size that fp32 squares have.
+// Rows of a large residual are scaled down by a power of two on the way, so that x * gain stays inside fp16: by the second part of
+// their sum of squares at the norm BEFORE (the first norm: of its own), which all writers and readers of the row know.  That
+// is zero as long as no few features add up to 2^20 (|x| below 1024); from there on the row is divided by the power of two that
+// brings the rms of that part into [4, 16), if it is 16 or more.  What overflows is |x * gain| above 65504 times that power.
+// Two bits of the first part, whose sum stays below 2^62, say that there is a second part and that the row is scaled: a reader
+// of an ordinary row looks at one word.  (The decode kernels have their rows unscaled: the same there cost llama1b 0.3 to 3 %
+// in every arrangement tried.)  n = features of a row.
+constexpr unsigned long long SSQ_LARGE = 1ull << 63, SSQ_SCALED = 1ull << 62;
+__device__ __forceinline__ void ssq_red_add(unsigned long long* dst, unsigned long long v) {
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(dst), "l"(v) : "memory");
+}
+__device__ __forceinline__ bool ssq_is_large(float q) { return !(q < 1048576.f); }
+__device__ __forceinline__ void ssq_mark(unsigned long long* dst, unsigned long long bits) {
+  asm volatile("red.relaxed.gpu.global.or.b64 [%0], %1;" ::"l"(dst), "l"(bits) : "memory");
+}
+__device__ __forceinline__ void ssq_add(unsigned long long* dst, size_t hi, float q, bool scaled) {
+  const bool large = ssq_is_large(q);
+  if (large) ssq_red_add(dst + hi, (unsigned long long)__float2ll_rn(q));
+  else ssq_red_add(dst, (unsigned long long)__float2ll_rn(q * 4294967296.f));
+  if (large || scaled) ssq_mark(dst, (large ? SSQ_LARGE : 0ull) | (scaled ? SSQ_SCALED : 0ull));
+}
+__device__ __forceinline__ int row_shift(unsigned long long coarse, int n) {
+  const float ms = __ll2float_rn((long long)coarse) / (float)n;
+  return ms < 256.f ? 0 : (((__float_as_int(ms) >> 23) - 125) >> 1) - 4;   // half the exponent, rounded up, less four
+}
+// the factor of a row whose sum of squares at the norm before has the second part `coarse`
+__device__ __forceinline__ float row_down(unsigned long long coarse, int n) { return __int_as_float((127 - row_shift(coarse, n)) << 23); }
+// 1/rms from the sum of squares *s, the row's power of two (from the norm before: *prev) taken back
+__device__ __forceinline__ float norm_factor(const unsigned long long* s, const unsigned long long* prev, size_t hi, int n, float eps) {
+  const unsigned long long f = __ldcg(s);
+  if (f < SSQ_SCALED) return rsqrtf(__ll2float_rn((long long)f) * (1.f / 4294967296.f) / (float)n + eps);
+  const float ss = __ll2float_rn((long long)(f & (SSQ_SCALED - 1))) * (1.f / 4294967296.f) + __ll2float_rn((long long)__ldcg(s + hi));
+  const int up = f & SSQ_SCALED ? row_shift(__ldcg(prev + hi), n) : 0;
+  return rsqrtf(ss / (float)n + eps) * __int_as_float((127 + up) << 23);
 }
 
 __device__ __forceinline__ float warp_sum(float v) {

@@ -80,7 +80,7 @@ struct mlora_ctx {
   float *X = nullptr, *qkv = nullptr, *logits = nullptr, *T = nullptr, *partial = nullptr, *att_ws = nullptr;
   __half* q16 = nullptr;             // passes of many rows: rotated q, fp16 [Mmax][Nq]
   __half* h_ffn = nullptr;           // passes of many rows: residual rows times the gain of the norm ahead of gate/up (h: ahead of q,k,v)
-  unsigned long long* row_ssq = nullptr;   // ... and the residual rows' sums of squares, [2 L + 1][Mmax], fixed point
+  unsigned long long* row_ssq = nullptr;   // ... and the residual rows' sums of squares, two parts of [2 L + 1][Mmax]
   __half *h = nullptr, *attn16 = nullptr, *act16 = nullptr;
   size_t partial_floats = 0, att_ws_floats = 0;
   unsigned* counters = nullptr;
@@ -468,16 +468,16 @@ int forward_rows(mlora_ctx* c, PassIO& io) {
   const mlora_model_desc& d = c->d;
   cudaStream_t st = c->stream;
   const int M = io.n * io.T, dm = d.d_model, F = d.d_ffn;
-  const size_t ld_ssq = (size_t)c->Mmax;
-  CK(cudaMemsetAsync(c->row_ssq, 0, (size_t)(2 * c->L + 1) * ld_ssq * sizeof(unsigned long long), st));
+  const size_t ld_ssq = (size_t)c->Mmax, ssq_hi = (size_t)(2 * c->L + 1) * ld_ssq;
+  CK(cudaMemsetAsync(c->row_ssq, 0, 2 * ssq_hi * sizeof(unsigned long long), st));
   CK(run(c, MLORA_PROF_MISC, [&] { return launch_tree_prep(io.parent, io.n, io.T, c->anc, c->depth, c->status, st); }));
   CK(run(c, MLORA_PROF_MISC, [&] {
     return launch_embed(io.tokens, (const __half*)d.embed, io.hidden_in, c->X, M, dm, d.vocab, c->status, st, c->forecast,
-                        c->n_forecast, c->rms_attn[0], c->h, c->row_ssq);
+                        c->n_forecast, c->rms_attn[0], c->h, c->row_ssq, ssq_hi);
   }));
   // one projection group: the shrink of its input rows (if it has adapters), then the projection
   auto project = [&](GemmArgs& g, const PackedWeight& w, const __half* in, int l, int nseg, const int* projs, const int* widths) -> int {
-    g.w = w.data; g.K = w.K; g.N = w.N; g.G = w.G; g.h = in; g.M = M; g.eps = d.rms_eps;
+    g.w = w.data; g.K = w.K; g.N = w.N; g.G = w.G; g.h = in; g.M = M; g.eps = d.rms_eps; g.ssq_hi = ssq_hi;
     if (nseg > 0) g.lora = lora_args(c, io, l, nseg, projs, widths);
     if (g.lora.adapter_idx != nullptr) {
       ShrinkArgs s{};
@@ -505,7 +505,7 @@ int forward_rows(mlora_ctx* c, PassIO& io) {
       kv_destination(c, io, l, g.k_out, g.v_out, g.kv_stream_stride, g.kv_head_stride);
       g.cs_table = c->cs_table; g.suffix_len = io.suffix_len; g.depth = c->depth; g.hd = d.head_dim; g.pos_base = io.pos_base;
       g.rows_per_stream = io.T;
-      g.ssq_in = c->row_ssq + (size_t)(2 * l) * ld_ssq;
+      g.ssq_in = c->row_ssq + (size_t)(2 * l) * ld_ssq; g.ssq_in_prev = l > 0 ? g.ssq_in - ld_ssq : g.ssq_in;
       if ((rc = project(g, c->w_qkv[l], c->h, l, 3, projs, widths)) != MLORA_OK) return rc;
     }
     if ((rc = launch_attention_block(c, io, l)) != MLORA_OK) return rc;
@@ -514,7 +514,7 @@ int forward_rows(mlora_ctx* c, PassIO& io) {
       GemmArgs g{};
       prefetch(g, &c->w_gateup[l]);
       g.mode = MODE_PLAIN; g.epi = EPI_RESID; g.resid = c->X;
-      g.xg_out = c->h_ffn; g.gain_next = c->rms_ffn[l]; g.ssq_out = c->row_ssq + (size_t)(2 * l + 1) * ld_ssq;
+      g.xg_out = c->h_ffn; g.gain_next = c->rms_ffn[l]; g.ssq_out = c->row_ssq + (size_t)(2 * l + 1) * ld_ssq; g.ssq_out_prev = g.ssq_out - ld_ssq;
       if ((rc = project(g, c->w_o[l], c->attn16, l, 1, projs, widths)) != MLORA_OK) return rc;
     }
     {
@@ -522,7 +522,7 @@ int forward_rows(mlora_ctx* c, PassIO& io) {
       GemmArgs g{};
       prefetch(g, &c->w_down[l]);
       g.mode = MODE_GATEUP; g.epi = EPI_SWIGLU; g.out_f16 = c->act16;
-      g.ssq_in = c->row_ssq + (size_t)(2 * l + 1) * ld_ssq;
+      g.ssq_in = c->row_ssq + (size_t)(2 * l + 1) * ld_ssq; g.ssq_in_prev = g.ssq_in - ld_ssq;
       if ((rc = project(g, c->w_gateup[l], c->h_ffn, l, 2, projs, widths)) != MLORA_OK) return rc;
     }
     {
@@ -531,23 +531,27 @@ int forward_rows(mlora_ctx* c, PassIO& io) {
       prefetch(g, l + 1 < c->L ? &c->w_qkv[l + 1] : (io.logits != nullptr ? &c->w_lm : nullptr));
       g.mode = MODE_PLAIN; g.epi = EPI_RESID; g.resid = c->X;
       const __half* gain = l + 1 < c->L ? c->rms_attn[l + 1] : (const __half*)d.rms_final;
-      if (gain != nullptr) { g.xg_out = c->h; g.gain_next = gain; g.ssq_out = c->row_ssq + (size_t)(2 * l + 2) * ld_ssq; }
+      if (gain != nullptr) { g.xg_out = c->h; g.gain_next = gain; g.ssq_out = c->row_ssq + (size_t)(2 * l + 2) * ld_ssq; g.ssq_out_prev = g.ssq_out - ld_ssq; }
       if ((rc = project(g, c->w_down[l], c->act16, l, 1, projs, widths)) != MLORA_OK) return rc;
     }
   }
   if (d.vocab > 0 && io.logits != nullptr) {
     const unsigned long long* ssq = c->row_ssq + (size_t)(2 * c->L) * ld_ssq;
     if (io.last_row_logits) {
-      // one row: the decode path's lm_head
+      // one row: normalised from the residual itself, then the decode path's lm_head (whose rows carry no power of two)
+      ShrinkArgs n{};
+      n.x_f32 = c->X + (size_t)(M - 1) * dm; n.gain = (const __half*)d.rms_final; n.eps = d.rms_eps; n.h_out = c->h; n.M = 1; n.K = dm;
+      n.pdl = 1;
+      CK(run(c, MLORA_PROF_SHRINK, [&] { return launch_shrink(n, st); }));
       LeanArgs a{};
-      a.M = 1; a.eps = d.rms_eps; a.logits = io.logits; a.ssq = const_cast<unsigned long long*>(ssq) + (M - 1);
+      a.M = 1; a.eps = d.rms_eps; a.logits = io.logits;
       StepPhase ph{};
       ph.kind = SK_GEMM; ph.w = c->w_lm.data; ph.K = dm; ph.N = d.vocab; ph.G = c->w_lm.G; ph.mode = MODE_PLAIN; ph.epi = EPI_F32;
-      ph.in16 = c->h + (size_t)(M - 1) * dm; ph.norm_in = 0; ph.ldo = d.vocab; ph.ssq_out = -1;
+      ph.in16 = c->h; ph.norm_in = -1; ph.ldo = d.vocab; ph.ssq_out = -1;
       CK(run(c, MLORA_PROF_GEMM, [&] { return launch_lean_gemm(a, ph, st); }));
     } else {
       GemmArgs g{};
-      g.mode = MODE_PLAIN; g.epi = EPI_F32; g.out_f32 = io.logits; g.ldo = d.vocab; g.ssq_in = ssq;
+      g.mode = MODE_PLAIN; g.epi = EPI_F32; g.out_f32 = io.logits; g.ldo = d.vocab; g.ssq_in = ssq; g.ssq_in_prev = ssq - ld_ssq;
       if ((rc = project(g, c->w_lm, c->h, 0, 0, nullptr, nullptr)) != MLORA_OK) return rc;
     }
   }
@@ -873,7 +877,7 @@ int mlora_create(const mlora_model_desc* desc, mlora_ctx** out) {
   CKC(cudaMalloc(&c->qkv, Mm * c->Nqkv * sizeof(float)));
   CKC(cudaMalloc(&c->h, Mm * maxK * sizeof(__half)));
   CKC(cudaMalloc(&c->h_ffn, Mm * dm * sizeof(__half)));
-  CKC(cudaMalloc(&c->row_ssq, (size_t)(2 * L + 1) * Mm * sizeof(unsigned long long)));
+  CKC(cudaMalloc(&c->row_ssq, (size_t)2 * (2 * L + 1) * Mm * sizeof(unsigned long long)));
   CKC(cudaMalloc(&c->q16, Mm * Nq * sizeof(__half)));
   CKC(cudaMalloc(&c->attn16, Mm * Nq * sizeof(__half)));
   CKC(cudaMalloc(&c->act16, Mm * F * sizeof(__half)));

@@ -9,11 +9,11 @@ namespace mlora {
 // ----------------------------------------------------------------------------- embedding / hidden input
 // An id in [vocab, vocab + n_forecast) stands for a forecast row (Sec. 3.5: forecast embeddings ride along with the
 // tokens of a DS2D pass): its input is the forecast embedding of that index.  xg != nullptr: also the row times the gain
-// of the RMSNorm ahead of the first projection (fp16) and its sum of squares (fixed point).
+// of the RMSNorm ahead of the first projection (fp16, large rows scaled down) and its sum of squares.
 __global__ void embed_kernel(const int32_t* __restrict__ tokens, const __half* __restrict__ embed,
                              const __half* __restrict__ hidden_in, float* __restrict__ X, int d, int vocab,
                              const __half* __restrict__ forecast, int n_forecast, int* __restrict__ status,
-                             const __half* __restrict__ gain, __half* __restrict__ xg, unsigned long long* __restrict__ ssq) {
+                             const __half* __restrict__ gain, __half* __restrict__ xg, unsigned long long* __restrict__ ssq, size_t ssq_hi) {
   __shared__ float s_part[8];
   const int m = blockIdx.x;
   const __half* src;
@@ -46,17 +46,21 @@ __global__ void embed_kernel(const int32_t* __restrict__ tokens, const __half* _
   sq = warp_sum(sq);
   if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = sq;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    float tot = 0.f;
-    for (int w = 0; w < (int)blockDim.x / 32; ++w) tot += s_part[w];
-    ssq[m] = (unsigned long long)__float2ll_rn(tot * 4294967296.f);
-  }
+  float tot = 0.f;
+  for (int w = 0; w < (int)blockDim.x / 32; ++w) tot += s_part[w];
+  const float down = ssq_is_large(tot) ? row_down((unsigned long long)__float2ll_rn(tot), d) : 1.f;
+  if (threadIdx.x == 0) ssq_add(ssq + m, ssq_hi, tot, down != 1.f);
+  if (down != 1.f)
+    for (int k = threadIdx.x * 2; k < d; k += blockDim.x * 2) {
+      const float2 v = __half22float2(*reinterpret_cast<const __half2*>(src + k)), g = __half22float2(*reinterpret_cast<const __half2*>(gain + k));
+      *reinterpret_cast<__half2*>(xg + (size_t)m * d + k) = __floats2half2_rn(v.x * g.x * down, v.y * g.y * down);
+    }
 }
 
 cudaError_t launch_embed(const int32_t* tokens, const __half* embed, const __half* hidden_in, float* X, int M, int d,
                          int vocab, int* status, cudaStream_t st, const __half* forecast, int n_forecast,
-                         const __half* gain, __half* xg, unsigned long long* ssq) {
-  embed_kernel<<<M, 256, 0, st>>>(tokens, embed, hidden_in, X, d, vocab, forecast, forecast ? n_forecast : 0, status, gain, xg, ssq);
+                         const __half* gain, __half* xg, unsigned long long* ssq, size_t ssq_hi) {
+  embed_kernel<<<M, 256, 0, st>>>(tokens, embed, hidden_in, X, d, vocab, forecast, forecast ? n_forecast : 0, status, gain, xg, ssq, ssq_hi);
   return cudaGetLastError();
 }
 

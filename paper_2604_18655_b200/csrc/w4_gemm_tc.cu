@@ -17,8 +17,8 @@
 // Few output features and many SMs: a cluster of S CTAs splits K, each CTA ends with NR / S rows: the others push their
 // accumulators into its shared memory (distributed shared memory, reused activation tiles) and it adds them in rank order
 // -- no partial sums in global memory, bit-reproducible.
-// RMSNorm: the producer of the residual writes x * gain (fp16) and the rows' sums of squares (fixed point, order
-// independent); this kernel scales its finished sums by 1/rms.
+// RMSNorm: the producer of the residual writes x * gain (fp16, large rows scaled down: row_down) and the rows' sums of squares
+// (fixed point, order independent); this kernel scales its finished sums by 1/rms.
 // Every mbarrier wait is bounded; a wait that runs out sets the status word and the CTA winds down (it still waits,
 // bounded, for its MMAs and copies, takes its cluster barriers, and frees its tensor memory).
 #include <cuda.h>
@@ -31,7 +31,6 @@ namespace mlora {
 constexpr int TC_BM = 128;                 // output features per CTA (UMMA M)
 constexpr int TC_BK = 64;                  // input features per step: one 128-byte swizzle row of fp16
 constexpr int TC_WSLOT = 1024 + 64;        // ring slot of a warp: two tiles of nibbles, two scale entries
-constexpr float TC_FIX = 4294967296.f, TC_UNFIX = 1.f / 4294967296.f;   // fixed point of the rows' sums of squares
 
 // GR = groups of four dequantising warps: two where two CTAs share an SM (up to 128 rows), four where one has it alone.
 // Weight stages in tensor memory (32 columns each, behind the NR accumulator columns), activation tiles, ring depth in
@@ -59,8 +58,8 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
   unsigned char* const wring = base + (size_t)NB * B_BYTES;
   __shared__ __align__(8) uint64_t b_full[NB], b_empty[NB], a_full[NA], a_empty[NA], done_bar, acc_free;
   __shared__ uint32_t tmem_base_s;
-  __shared__ float s_inv[CW];
-  __shared__ unsigned long long s_ssq[CW];
+  __shared__ float s_inv[CW];                         // the factor of the finished sums; EPI_RESID: of the new fp16 rows
+  __shared__ unsigned long long s_ssq[2][CW];
   __shared__ int s_pos[CW];                           // EPI_QKV: the rows' positions ...
   __shared__ size_t s_dst[CW];                        // ... and their places in the cache
 
@@ -450,10 +449,13 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
     const int row0 = m0 + rank * CW;                       // rows this CTA finishes: row0 .. row0 + CW - 1
     if (tid < CW) {
       float inv = 1.f;
-      if (p.ssq_in != nullptr && row0 + tid < p.M)
-        inv = rsqrtf(__ll2float_rn((long long)__ldcg(p.ssq_in + row0 + tid)) * TC_UNFIX / (float)p.K + p.eps);
+      if (EPI == EPI_RESID) {
+        if (p.xg_out != nullptr && row0 + tid < p.M) inv = row_down(__ldcg(p.ssq_out_prev + p.ssq_hi + row0 + tid), p.N);
+        s_ssq[0][tid] = s_ssq[1][tid] = 0ull;
+      } else if (p.ssq_in != nullptr && row0 + tid < p.M) {
+        inv = norm_factor(p.ssq_in + row0 + tid, p.ssq_in_prev + row0 + tid, p.ssq_hi, p.K, p.eps);
+      }
       s_inv[tid] = inv;
-      s_ssq[tid] = 0ull;
       s_pos[tid] = 0;
       if (EPI == EPI_QKV && row0 + tid < p.M) {
         const int m = row0 + tid, st = stream_of(m), cached = p.suffix_len[st];
@@ -512,7 +514,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       } else {
         tc_ld_32x32b_x16(tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)c0, v);
       }
-      if (p.ssq_in != nullptr) {
+      if (EPI != EPI_RESID && p.ssq_in != nullptr) {
 #pragma unroll
         for (int j = 0; j < CH; ++j) v[j] *= s_inv[c0 + j];
       }
@@ -567,7 +569,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
           if (n_ok && m < p.M) {
             xn[j] = x_old[j] + v[j];
             p.resid[(size_t)m * p.N + n] = xn[j];
-            if (p.xg_out != nullptr) p.xg_out[(size_t)m * p.N + n] = __float2half_rn(xn[j] * gain);
+            if (p.xg_out != nullptr) p.xg_out[(size_t)m * p.N + n] = __float2half_rn(xn[j] * gain * s_inv[c0 + j]);
           }
         }
         if (c0 + CH < c_lo + HC) prefetch_resid(c0 + CH);
@@ -596,7 +598,10 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
             }
           }
           constexpr int DUP = 32 / CH;                     // lanes that hold the same row's sum
-          if ((lane & (DUP - 1)) == 0) atomicAdd(&s_ssq[c0 + id], (unsigned long long)__float2ll_rn(q[0] * TC_FIX));
+          if ((lane & (DUP - 1)) == 0) {
+            const bool large = ssq_is_large(q[0]);
+            atomicAdd(&s_ssq[large][c0 + id], (unsigned long long)__float2ll_rn(large ? q[0] : q[0] * 4294967296.f));
+          }
         }
       }
     }
@@ -605,7 +610,12 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
     __syncwarp();
     if (lane == 0) tc_arrive(tc_smem_u32(&acc_free));
     asm volatile("bar.sync 1, %0;" ::"n"(TC_WARPS * 32) : "memory");
-    if (p.ssq_out != nullptr && tid < CW && row0 + tid < p.M) atomicAdd(p.ssq_out + row0 + tid, s_ssq[tid]);
+    if (EPI == EPI_RESID && p.ssq_out != nullptr && tid < CW && row0 + tid < p.M) {
+      atomicAdd(p.ssq_out + row0 + tid, s_ssq[0][tid]);
+      const unsigned long long more = s_ssq[1][tid], bits = (more != 0ull ? SSQ_LARGE : 0ull) | (s_inv[tid] != 1.f ? SSQ_SCALED : 0ull);
+      if (more != 0ull) atomicAdd(p.ssq_out + p.ssq_hi + row0 + tid, more);
+      if (bits != 0ull) ssq_mark(p.ssq_out + row0 + tid, bits);
+    }
     if (!more) break;
     }
   }

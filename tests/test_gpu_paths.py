@@ -193,6 +193,51 @@ def test_passes_with_more_query_heads_a_group_than_a_block_has_rows(GpuModel):
     gm.close()
 
 
+@pytest.mark.parametrize("rms,channel,gain,decode_path", [
+    (3000., None, 8., 1),       # rows whose x * gain leaves fp16 everywhere, and whose squares add up to more than 2^31
+    (40., 60000., 1.5, 1),      # one massive channel
+    (45., None, 1., 0), (47., None, 1., 0),     # on either side of where rows start to be scaled (a sum of 2^20 over 512 features)
+])
+def test_large_residual_rows(GpuModel, rms, channel, gain, decode_path):
+    """A pass's residual rows travel as x * gain without their 1/rms: rows far beyond what fp16 holds give what normalised rows
+    give, in prefill (one row's logits), tree passes and decode steps of nine streams.  (Decode steps of few streams on the
+    path that normalises its rows first: the other one's bound is documented.)"""
+    from paper_2604_18655_b200 import binding as mb
+    cfg = gen.ModelCfg("large", 3, 512, 4, 2, 64, 192, 304, 64, 4, gen.configs.ALL7, 3, 9, 40, b_std=0.05)
+    m = gen.make_model(cfg, 0)
+    m.embed = (m.embed.astype(np.float32) * (rms / cfg.w_std)).astype(np.float16)
+    if channel:
+        m.embed[:, 5] = channel
+    for g in m.rms_attn + m.rms_ffn + [m.rms_final]:
+        g *= np.float16(gain)
+    orc, gm = ref.OracleModel.from_synth(m), GpuModel(m, max_suffix=40, max_tree=6)
+    mb.mlora_debug_set(gm.ctx, 6, decode_path)
+    for a in range(3):
+        A, B = gen.make_adapter(cfg, a, 0)
+        orc.set_adapter(a, A, B, cfg.alpha)
+        gm.set_adapter(a, A, B, cfg.alpha)
+    ids = gen.make_prompt_ids(cfg, 0)
+    compare(gm.prefill(ids), orc.prefill_shared(ids, n_streams=9), "prefill logits")
+    for l in range(3):
+        _, pk, pv = gm.export_kv(l, -1, 0, cfg.prompt_len)
+        compare(pk, orc.prefix_k[l], f"prefix K of layer {l}")
+        compare(pv, orc.prefix_v[l], f"prefix V of layer {l}")
+    ad = [0, 1, -1, 2, 0, 1, 2, -1, 0]
+    par = np.stack([np.array([-1, 0, 0, 1, 1, 2], dtype=np.int32)] * 9)
+    tree = np.random.default_rng(3).integers(0, cfg.vocab, size=(9, 6), dtype=np.int32)
+    got = gm.verify(ad, tree, par)
+    want = orc.verify_tree(ad, par, tree, follow_argmax=np.argmax(got["logits"], axis=1).reshape(9, 6))
+    compare(got["logits"], want["logits"], "verify logits")
+    toks = np.arange(3, 12, dtype=np.int32)
+    _, logits = gm.decode(ad, toks)
+    compare(logits, orc.decode_step(ad, tokens=toks)["logits"], "decode logits, nine streams")
+    nxt, logits = gm.decode(ad[:5], toks[:5])
+    compare(logits, orc.decode_step(ad[:5], tokens=toks[:5])["logits"], "decode logits, five streams")
+    only, _ = gm.decode(ad[:5], toks[:5], want_logits=False)
+    check_argmax(only, orc.decode_step(ad[:5], tokens=toks[:5])["logits"], "greedy tokens")
+    gm.close()
+
+
 # ------------------------------------------------------------------ decode
 @pytest.mark.parametrize("d_model,d_ffn,hd,n_q,n_kv,vocab,rank,n,P", [
     (3072, 4096, 128, 24, 8, 9600, 32, 8, 70),     # single-wave variants, pointer table, lm_head of K = 3072

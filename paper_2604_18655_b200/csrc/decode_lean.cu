@@ -713,7 +713,9 @@ cudaError_t launch_lean_embed(const LeanArgs& a, const StepPhase& ph, const int3
 // The variants of lean_gemm_kernel (NTILE, WARPS, PF, XB, OCC).  A grid that does not fit the SMs at once costs a whole
 // CTA's life more (llama3b gate/up, 512 CTAs at three an SM: 24.5 us, the last ones starting at 11; 12.9 at four), but the
 // registers of a fourth CTA are paid with loads in flight (llama1b gate/up, 352 CTAs: 9.1 us at three, 9.7 at four), so the
-// dense variants are taken only where they save a wave.  Single tiles in more than three CTAs an SM: 8 rows of 2048 x 8192
+// dense pair variant is taken only where it saves a wave (a step of one layer of 2048 with 8 streams: d_ffn 9472, four pairs an SM,
+// 57.3 -> 53.3 us; 11264, two waves either way, 57.4 and 57.3, with 4096 79.9 -> 81.9; 16384, three waves to two, 67.6 -> 63.5;
+// 22528, four to three, 79.9 -> 73.7).  Single tiles in more than three CTAs an SM: 8 rows of 2048 x 8192
 // without adapters 6.2 us at three, 4.9 at four; 4096 x 14336 with adapters 19.1 -> 18.4.
 #define LN_ONE 1, 8, 4, 4, 3
 #define LN_ONE_DENSE 1, 8, 4, 2, 4
@@ -771,7 +773,8 @@ static cudaError_t launch_lean_gemm_variant(const LeanArgs& a, const StepPhase& 
     LM_LAUNCH(8, 2)
   }
   if (mode == MODE_GATEUP) {
-    if (tiles / 2 > 3 * sms && tiles / 2 <= 4 * sms) LN_LAUNCH(LN_PAIR_DENSE);
+    const int pairs = tiles / 2;
+    if ((pairs + 3 * sms - 1) / (3 * sms) > (pairs + 4 * sms - 1) / (4 * sms)) LN_LAUNCH(LN_PAIR_DENSE);
     LN_LAUNCH(LN_PAIR);
   }
   if (wide && tiles > sms) LN_LAUNCH(LN_WIDE_DENSE);

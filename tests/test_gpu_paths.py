@@ -245,6 +245,7 @@ def test_large_residual_rows(GpuModel, rms, channel, gain, decode_path):
     (512, 8192, 64, 8, 8, 304, 16, 5, 33),         # down projection of K = 8192 with few columns
     (512, 1408, 64, 8, 4, 304, 64, 8, 2101),       # streaming attention + merge with the o projection's shrink, rank 64
     (256, 512, 128, 4, 1, 304, 8, 2, 2048),
+    (128, 14336, 64, 2, 1, 304, 8, 3, 9),          # gate/up in more than four CTAs an SM: the dense variant again
 ])
 def test_decode_variants(GpuModel, d_model, d_ffn, hd, n_q, n_kv, vocab, rank, n, P):
     cfg = gen.ModelCfg("decode", 2, d_model, n_q, n_kv, hd, d_ffn, vocab, 64, rank, gen.configs.ALL7, 3, n, P)

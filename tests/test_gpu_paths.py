@@ -89,6 +89,71 @@ def test_projection_with_many_adapters(mb, M, n_ad, rank, K, N):
     assert bool((ws[need:] == 255).all())
 
 
+@pytest.mark.parametrize("rows", [(8, 3, 8, 1), (40, 200, 9, 40), (64, 12, 300, 64), (8, 40, 5, 200)])
+def test_calls_that_follow_one_another_on_one_workspace(mb, rows):
+    """Calls chained by programmatic launches, nothing waited for in between: other rows, other adapters (few, many, none) and
+    other inputs each time on one workspace, every call's result in fp16 the input of the next but one."""
+    K = 512
+    rng = np.random.default_rng(sum(rows))
+    stream = torch.cuda.Stream()
+    sets = [None]
+    for n_ad, rank in ((4, 16), (70, 64)):
+        A = (rng.standard_normal((n_ad, rank, K)) / rank).astype(np.float16)
+        B = (rng.standard_normal((n_ad, rank, K)) * 0.05).astype(np.float16)
+        dA, dB = dev(A), dev(B)
+        ptr = [torch.tensor([t[i].data_ptr() for i in range(n_ad)], dtype=torch.int64, device="cuda") for t in (dA, dB)]
+        sets.append((A, B, rank, (dA, dB), ptr, torch.full((n_ad,), 16.0 / rank, device="cuda")))
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        ws, Wd = [], []
+        for i in range(2):
+            qb, sc = gen.quantize_int4(rng.standard_normal((K, K)).astype(np.float32) * 0.04, 64)
+            ws.append(mb.mlora_weight_create(dev(qb), dev(sc), K, K, 64))
+            Wd.append(ref.dequant(qb, sc, 64).astype(np.float64))
+        work = torch.zeros(max(mb.mlora_linear_workspace_bytes(ws[0], m, 64) for m in rows), dtype=torch.uint8, device="cuda")
+        plan, src = [], [dev(rng.standard_normal((max(rows), K)).astype(np.float16)) for _ in range(2)]
+        for i in range(10):
+            M, st = rows[i % 4], sets[(i + 1) % 3]
+            idx = rng.integers(-1, len(st[0]), size=M).astype(np.int32) if st else None
+            plan.append((M, st, idx, dev(idx) if st else None, torch.empty(M, K, device="cuda"), torch.empty(max(rows), K, dtype=torch.float16, device="cuda")))
+        stream.synchronize()
+        ins = []
+        for i, (M, st, idx, d_idx, y, h) in enumerate(plan):
+            x = src[i] if i < 2 else plan[i - 2][5]
+            ins.append(x)
+            mb.mlora_linear(ws[i % 2], x[:M], y, work, *((d_idx, *st[4], st[5], st[2]) if st else ()))
+            for j in (i - 1, i) if i % 2 else ():          # (two calls straight behind one another)
+                plan[j][5].copy_(src[j % 2])
+                plan[j][5][:plan[j][0]].copy_(plan[j][4])
+        stream.synchronize()
+        for i, (M, st, idx, _, y, _) in enumerate(plan):
+            x = ins[i][:M].double().cpu().numpy()
+            lora = (idx, list(st[0].astype(np.float64)), list(st[1].astype(np.float64)), st[5].double().cpu().numpy()) if st else ()
+            compare(y.cpu().numpy(), ref.linear_lora(x, Wd[i % 2], *lora), f"call {i}, {M} rows")
+        mb.mlora_linear_status(ws[0], work)
+        for w in ws:
+            mb.mlora_weight_destroy(w)
+
+
+def test_quantised_calls_that_follow_one_another(mb):
+    """Quantiser and INT8 projection in a chain over the same buffers, nothing waited for in between."""
+    K, N, stream = 512, 256, torch.cuda.Stream()
+    rng = np.random.default_rng(4)
+    qb, sc = gen.quantize_int4_per_channel(rng.standard_normal((K, N)).astype(np.float32) * 0.02)
+    xs = [rng.standard_normal((M, K)).astype(np.float16) for M in (8, 64, 1, 17, 8)]
+    dq, ds, dx, ys = dev(qb), dev(sc), [dev(x) for x in xs], [torch.empty(len(x), N, device="cuda") for x in xs]
+    qx = torch.empty(64, K, dtype=torch.int8, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        for x, y in zip(dx, ys):
+            mb.mlora_quantize_act_int8(x, 0.03, qx[:len(x)])
+            mb.mlora_linear_w4a8(dq, ds, qx[:len(x)], 0.03, y)
+        stream.synchronize()
+    for x, y in zip(xs, ys):
+        want = ref.linear_w4a8(ref.quantize_act_int8(x, 0.03), 0.03, qb, sc)
+        assert np.array_equal(y.cpu().numpy().view(np.uint32), want.view(np.uint32))
+
+
 @pytest.mark.parametrize("count", [1, 7, 8, 9, 1023, 1025])
 def test_quantiser_tails(mb, count):
     x = np.random.default_rng(count).standard_normal((1, count)).astype(np.float16)

@@ -200,12 +200,14 @@ cudaError_t launch_shrink_rows(const ShrinkArgs& a, cudaStream_t st) {
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   // Small grids: start beside the projection that is still running, whose SMs have the largest shared-memory share
-  // (with another share they would have to drain first; llama1b verify 2.64 -> 2.52 ms).  Larger grids only take room from
-  // the projection behind (llama3b, 192 CTAs: 7.82 -> 8.01 ms).
+  // (with another share they would have to drain first).  Larger grids only take room from the projection behind, the sooner the
+  // more rows it has.  Milliseconds of two tree passes with no grid, those up to 48 CTAs and those up to 96 let in: llama1b
+  // 128 rows 2.65 / 2.54 / 2.54, 240 rows 3.35 / 3.17 / 3.17, 512 rows 4.67 / 4.67 / 4.82; llama3b 128 rows of rank 32 6.47 / 6.36 /
+  // 6.02, 192 rows 7.18 / 7.36 / 7.28 (on the wrong side), 256 rows of rank 16 6.69 / 6.81 / 6.82 (as well), of rank 32 7.25 / 7.25 / 7.42.
   attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
   attr[1].val.sharedMemCarveout = 100;
   cfg.attrs = attr;
-  cfg.numAttrs = a.pdl ? ((long long)cfg.gridDim.x * cfg.gridDim.y <= 96 ? 2 : 1) : 0;
+  cfg.numAttrs = a.pdl ? ((long long)cfg.gridDim.x * cfg.gridDim.y <= (a.M <= 128 ? 96 : 48) ? 2 : 1) : 0;
   return cudaLaunchKernelEx(&cfg, shrink_mma_kernel, a, tps);
 }
 

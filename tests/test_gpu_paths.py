@@ -29,6 +29,7 @@ def test_projection_row_tiles(mb, M):
     (320, 4096, 64, 700),        # K of an odd number of steps, more tiles than CTAs: each stays for further ones
     (192, 9600, 64, 180),        # the same with the 192-row tile, fewer steps than weight stages
     (192, 9600, 64, 90),         # and the 96-row one
+    (2048, 3072, 128, 96), (2048, 3072, 128, 192),   # clusters of four would not all fit at once: split in two
 ])
 def test_projection_splits_and_persistent_tiles(mb, K, N, G, M):
     for n_ad, rank in ((0, 0), (3, 8)):

@@ -21,6 +21,11 @@
  *     and N output features, nibbles uint8 [K][N/2] where byte [k][j] holds column 2j in its low and
  *     column 2j+1 in its high nibble, stored nibble = q + 8 with q in [-8,7]; scales fp16 [K/G][N].
  *     Dequantised weight = fp16_round_to_nearest_even(q * scale)  (one fp16 multiply).
+ *   - Range of the residual: it is fp32, but its rows reach the projections as fp16.  Passes of 9 rows and more (prefill, trees,
+ *     many streams) take x * gain up to 65504, or 65504 / 16 times the rms that a row with features of 1024 and more had at the
+ *     norm before, whichever is larger.  Decode steps of up to 8 streams: x * gain up to 65504, and squares of a row that add up
+ *     to less than 2^31.  Beyond it a row becomes inf or NaN.  Key 6 = 1 of mlora_debug_set normalises the rows first (no limit,
+ *     slower).
  *   - LoRA tensors: A fp16 [r][K] and B fp16 [r][N] (both row-major); the projection computes
  *     y = x W + (alpha/r) * (x A^T) B, i.e. Eq. 1-4 with the low-rank factors A^T (K x r) and B (r x N).
  */
@@ -250,7 +255,9 @@ size_t mlora_linear_workspace_bytes(const mlora_weight* w, int32_t M, int32_t ra
  * x dev fp16 [M][K]; row_adapter dev int32 [M] (-1 = base) or NULL for no LoRA; A, B: DEV arrays of
  * n_adapters device pointers (fp16 [rank][K], fp16 [rank][N]); scale dev fp32 [n_adapters] (= alpha/r);
  * y dev fp32 [M][N]; workspace dev, zero-filled before first use (the call leaves it zeroed where it matters).
- * x, y, workspace and every A[a], B[a] must be 16-byte aligned (the kernels use 128-bit loads and bulk copies).
+ * x, y, workspace and every A[a], B[a] must be 16-byte aligned (the kernels use 128-bit loads and bulk copies).  An adapter has
+ * both matrices or neither (null pointers: base).  From 9 rows on with few adapters T = scale (x A^T) is held as two fp16
+ * numbers: beyond 65504 it becomes inf, and below it is good to 2^-25 or 2^-22 of itself, whichever is larger.
  * Errors: ARG (null or misaligned pointer), CAPACITY (workspace too small), UNSUPPORTED (M > 4096).  A bounded wait
  * that runs out on the device is reported by mlora_linear_status. */
 int mlora_linear(mlora_weight* w, const void* x, int32_t M, const int32_t* row_adapter, const void* const* A,
@@ -304,7 +311,8 @@ size_t mlora_attention_workspace_bytes(int32_t n_streams, int32_t n_nodes, int32
  * prefix_k/v dev fp16 [n_kv_heads][prefix_len][head_dim]; own_k/v dev fp16 [n_streams][n_kv_heads][own_capacity][head_dim]
  * holding suffix_len[s] cached rows followed by the n_nodes tree rows; suffix_len dev int32 [n_streams];
  * suffix_bound host upper bound of all suffix_len; tree_parent dev int32 [n_streams][n_nodes];
- * out dev fp16 [rows][n_q_heads][head_dim].  status dev int32 [1] receives MLORA_ERR_ARG for a bad tree. */
+ * out dev fp16 [rows][n_q_heads][head_dim].  q and the K/V buffers 16-byte aligned; out and the workspace may start anywhere.
+ * status dev int32 [1] receives MLORA_ERR_ARG for a bad tree. */
 int mlora_attention(const void* q, const void* prefix_k, const void* prefix_v, int32_t prefix_len,
                     const void* own_k, const void* own_v, int32_t own_capacity, const int32_t* suffix_len,
                     int32_t suffix_bound, const int32_t* tree_parent, int32_t n_streams, int32_t n_nodes,

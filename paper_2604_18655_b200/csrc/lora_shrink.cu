@@ -218,8 +218,10 @@ cudaError_t launch_shrink_rows(const ShrinkArgs& a, cudaStream_t st) {
 constexpr int SG_BLOCKS = 2;                 // 64-feature blocks of a warp per CTA: K share = 16 warps x 2 x 64 at most
 constexpr int SG_MAX_ROWS = 4096;
 // TEXT: T goes into the matrix that the projection reads; else to fp32 T, and rows without an adapter are not looked at.
+// (fp32 T: two CTAs an SM asked for, else the compiler takes 70 registers and one fits; 256 rows of 14336 x 4096 with 64 adapters of
+// rank 64 96 -> 91 us, of 4096 x 4096 45.6 -> 41.4.  TEXT has 62 by itself; asking for two moved it to 64 and some calls by 1.5 %.)
 template <int S, bool TEXT>
-__global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32) shrink_gather_kernel(const ShrinkArgs p) {
+__global__ void __launch_bounds__(SHRINK_MMA_WARPS * 32, TEXT ? 0 : 2) shrink_gather_kernel(const ShrinkArgs p) {
   __shared__ float red[SHRINK_MMA_WARPS][32][4];
   __shared__ float part[S][128];             // first CTA of a cluster: the CTAs' sums of a group of 16 rows
   __shared__ short rows[SG_MAX_ROWS];

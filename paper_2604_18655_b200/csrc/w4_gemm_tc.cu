@@ -705,10 +705,11 @@ bool gemm_tc_eligible(const GemmArgs& a) {
 
 // Rows per CTA and K split, by a model of the time in microseconds, fitted to measurements of all candidates at projections
 // of 2048 x 2048 .. 14336 x 4096 with 32 .. 2000 rows: the time of a step with one or two CTAs on an SM, set-up and
-// epilogue, what a further wave costs (less where the CTA stays), and the exchange of a split.  Clusters of four and eight CTAs do
-// not fill the machine: 33 and 15 of them on 148 SMs with one CTA each (cudaOccupancyMaxActiveClusters).  Against the best
-// candidate at nine projections and 9 .. 2000 rows: 1.9 % more on average, 30 % at worst (2048 x 2048, 512 rows); as if clusters
-// filled it 4.3 % and 68 %.  The expand's steps are left out: few where it is done inside.
+// epilogue, what a further wave costs (less where the CTA stays), and the exchange of a split.  Clusters of four CTAs do not
+// fill the machine: 33 of them on 148 SMs with one CTA each (cudaOccupancyMaxActiveClusters).  (Of eight 15, but their splits are so
+// fine that the rest of a wave costs little, and adapters gain from them: 14336 x 4096, 32 rows, 8 adapters of rank 16 24.4 us in
+// eight, 30.4 in four.)  Against the best candidate without adapters at nine projections and 9 .. 2000 rows: 1.9 % more on average,
+// 30 % at worst (2048 x 2048, 512 rows); as if clusters of four filled it 4.3 % and 68 %.  The expand's steps are left out.
 static void tc_plan(const GemmArgs& a, int sm_count, int& nr, int& split) {
   static const int sizes[6] = {32, 64, 96, 128, 192, 256};
   static const double step1[6] = {0.227, 0.242, 0.264, 0.286, 0.303, 0.320}, step2[6] = {0.393, 0.429, 0.484, 0.538, 0.0, 0.0};
@@ -719,7 +720,7 @@ static void tc_plan(const GemmArgs& a, int sm_count, int& nr, int& split) {
     if (ri > 0 && a.M <= sizes[ri - 1]) break;
     for (int S = 1; S <= max_split; S *= 2) {
       if (S > 1 && KT / S < 4) break;
-      const int sms = S == 4 ? sm_count - 16 : (S == 8 ? sm_count - 28 : sm_count);
+      const int sms = S == 4 ? sm_count - 16 : sm_count;
       const long long ctas = (long long)slabs * ((a.M + R - 1) / R) * S, per_wave = (long long)sms * (R > 128 ? 1 : 2);
       const long long full = ctas / per_wave, rest = ctas % per_wave;
       const double steps = (KT + S - 1) / S, f = R / 256.0;

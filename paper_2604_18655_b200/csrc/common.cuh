@@ -522,7 +522,7 @@ __device__ __forceinline__ uint4 head_piece_f16(const float* __restrict__ head, 
 // is zero as long as no few features add up to 2^20 (|x| below 1024); from there on the row is divided by the power of two that
 // brings the rms of that part into [4, 16), if it is 16 or more.  What overflows is |x * gain| above 65504 times that power.
 // Two bits of the first part, whose sum stays below 2^62, say that there is a second part and that the row is scaled: a reader
-// of an ordinary row looks at one word.  (The decode kernels have their rows unscaled: the same there cost llama1b 0.3 to 3 %
+// of an ordinary row looks at one word.  (The decode kernels have their rows unscaled: the same there cost llama1b 0.3 to 7 %
 // in every arrangement tried.)  n = features of a row.
 constexpr unsigned long long SSQ_LARGE = 1ull << 63, SSQ_SCALED = 1ull << 62;
 __device__ __forceinline__ void ssq_red_add(unsigned long long* dst, unsigned long long v) {

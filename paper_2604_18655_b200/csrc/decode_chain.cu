@@ -668,13 +668,8 @@ __global__ void __launch_bounds__(CH_THREADS, 1) decode_chain_kernel(const Chain
                     const uint32_t sw = *reinterpret_cast<const uint32_t*>(ssc + ((ktl + q) >> gshift) * 32);
                     const uint4 b01 = *reinterpret_cast<const uint4*>(hbase + q * TILE_K);
                     const uint4 b23 = *reinterpret_cast<const uint4*>(hbase + q * TILE_K + 8);
-                    __half2 s_lo, s_hi;
-                    split_scales(sw, s_lo, s_hi);
                     uint32_t af[4][4];
-                    dequant8(wv.x, s_lo, s_hi, af[0]);
-                    dequant8(wv.y, s_lo, s_hi, af[1]);
-                    dequant8(wv.z, s_lo, s_hi, af[2]);
-                    dequant8(wv.w, s_lo, s_hi, af[3]);
+                    dequant_tile(wv, sw, af);
                     mma_16816(acc0, af[0], b01.x, b01.y);
                     mma_16816(acc1, af[1], b01.z, b01.w);
                     mma_16816(acc0, af[2], b23.x, b23.y);

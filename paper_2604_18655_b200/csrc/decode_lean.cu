@@ -239,17 +239,10 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
       if (kb + ib + i < kt1) {
 #pragma unroll
         for (int u = 0; u < NTILE; ++u) {
-          __half2 s_lo, s_hi;
-          split_scales(sv[ib + i][u], s_lo, s_hi);
-          uint32_t af[4][4];
-          dequant8(wv[ib + i][u].x, s_lo, s_hi, af[0]);
-          dequant8(wv[ib + i][u].y, s_lo, s_hi, af[1]);
-          dequant8(wv[ib + i][u].z, s_lo, s_hi, af[2]);
-          dequant8(wv[ib + i][u].w, s_lo, s_hi, af[3]);
-          mma_16816(acc[u], af[0], x0[i].x, x0[i].y);
-          mma_16816(acc[u], af[1], x0[i].z, x0[i].w);
-          mma_16816(acc[u], af[2], x1[i].x, x1[i].y);
-          mma_16816(acc[u], af[3], x1[i].z, x1[i].w);
+          dequant_tile_warp(wv[ib + i][u], sv[ib + i][u], [&](int j, const uint32_t (&af)[4]) {
+            const uint4& x = j < 2 ? x0[i] : x1[i];
+            mma_16816(acc[u], af, j & 1 ? x.z : x.x, j & 1 ? x.w : x.y);
+          });
         }
       }
     }
@@ -469,17 +462,10 @@ __global__ void __launch_bounds__(WARPS * 32, 2) lean_lmhead_kernel(const LeanAr
       if (kt0 + i < kt1) {
         const uint4 wv = wring[((size_t)stage * LM_PF + i) * THREADS + threadIdx.x];
         const uint32_t sv = sring[((size_t)stage * LM_PF + i) * THREADS + threadIdx.x];
-        __half2 s_lo, s_hi;
-        split_scales(sv, s_lo, s_hi);
-        uint32_t af[4][4];
-        dequant8(wv.x, s_lo, s_hi, af[0]);
-        dequant8(wv.y, s_lo, s_hi, af[1]);
-        dequant8(wv.z, s_lo, s_hi, af[2]);
-        dequant8(wv.w, s_lo, s_hi, af[3]);
-        mma_16816(acc, af[0], x0[i].x, x0[i].y);
-        mma_16816(acc, af[1], x0[i].z, x0[i].w);
-        mma_16816(acc, af[2], x1[i].x, x1[i].y);
-        mma_16816(acc, af[3], x1[i].z, x1[i].w);
+        dequant_tile_warp(wv, sv, [&](int j, const uint32_t (&af)[4]) {
+          const uint4& x = j < 2 ? x0[i] : x1[i];
+          mma_16816(acc, af, j & 1 ? x.z : x.x, j & 1 ? x.w : x.y);
+        });
       }
     }
     issue(stage, tile + LM_DEPTH * (int)gridDim.x);          // refills the slots just read (this thread's own)

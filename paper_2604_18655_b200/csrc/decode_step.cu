@@ -269,17 +269,12 @@ __device__ __forceinline__ void gemm_tiles(const GemmLoop& q, const WaitCtx& wc,
           if (ok && itl < kc) {
             const uint4 wv = *reinterpret_cast<const uint4*>(sb + itl * 512 + lane * 16);
             const uint32_t sw = *reinterpret_cast<const uint32_t*>(sb + kc * 512 + g * 4 + (itl >> q.gshift) * 32);
-            __half2 s_lo, s_hi;
-            split_scales(sw, s_lo, s_hi);
-            uint32_t af[4];
-            dequant8(wv.x, s_lo, s_hi, af);
-            mma_16816(acc0, af, bfr[qi][0].x, bfr[qi][0].y);
-            dequant8(wv.y, s_lo, s_hi, af);
-            mma_16816(acc1, af, bfr[qi][0].z, bfr[qi][0].w);
-            dequant8(wv.z, s_lo, s_hi, af);
-            mma_16816(acc0, af, bfr[qi][1].x, bfr[qi][1].y);
-            dequant8(wv.w, s_lo, s_hi, af);
-            mma_16816(acc1, af, bfr[qi][1].z, bfr[qi][1].w);
+            uint32_t af[4][4];
+            dequant_tile(wv, sw, af);
+            mma_16816(acc0, af[0], bfr[qi][0].x, bfr[qi][0].y);
+            mma_16816(acc1, af[1], bfr[qi][0].z, bfr[qi][0].w);
+            mma_16816(acc0, af[2], bfr[qi][1].x, bfr[qi][1].y);
+            mma_16816(acc1, af[3], bfr[qi][1].z, bfr[qi][1].w);
           }
           __syncwarp();
           // one arrival per item; the last item of a ragged chunk also arrives for the items the chunk lacks

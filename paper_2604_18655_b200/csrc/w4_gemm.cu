@@ -32,7 +32,7 @@ __global__ void repack_kernel(const uint8_t* __restrict__ qw, const __half* __re
         const int k = kt * TILE_K + 16 * t + 4 * j + 2 * (a >> 1) + hi;
         const uint8_t byte = qw[(size_t)k * (N / 2) + (n >> 1)];
         const uint32_t u = (n & 1) ? (byte >> 4) : (byte & 0xF);
-        wd |= u << (4 * nib);
+        wd |= ((u << (4 * a + 2) | u >> (14 - 4 * a)) & 0xFFFFu) << (16 * hi);
       }
       words[j] = wd;
     }
@@ -87,13 +87,11 @@ __global__ void dequant_kernel(const unsigned char* __restrict__ w, const WLayou
     const unsigned char* unit = w + (size_t)pt * L.unit_bytes;
     const uint4 wv = ldg_stream(reinterpret_cast<const uint4*>(unit + wl_tile_off(L, kt)) + lane);
     const uint32_t sw = ldg_nc_u32(reinterpret_cast<const uint32_t*>(unit + wl_scale_off(L, kt)) + g);
-    __half2 s_lo, s_hi;
-    split_scales(sw, s_lo, s_hi);
-    const uint32_t words[4] = {wv.x, wv.y, wv.z, wv.w};
+    uint32_t frag[4][4];
+    dequant_tile(wv, sw, frag);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      uint32_t a[4];
-      dequant8(words[j], s_lo, s_hi, a);
+      const uint32_t (&a)[4] = frag[j];
       const int k = kt * TILE_K + 16 * t + 4 * j;
       const int n = nt * TILE_N + g;
       const __half2 a0 = u32_as_h2(a[0]), a1 = u32_as_h2(a[1]), a2 = u32_as_h2(a[2]), a3 = u32_as_h2(a[3]);
@@ -194,18 +192,14 @@ __global__ void __launch_bounds__(GEMM_THREADS) w4_gemm_kernel(const GemmArgs p,
       if (k0 + i < nk) {             // uniform across the CTA
         if (active) {
           const uint4 w = wr[i];
-          __half2 s_lo, s_hi;
-          split_scales(sr[i], s_lo, s_hi);
+          const uint32_t sw = sr[i];
           const int nxt = k0 + i + GEMM_PF;
           if (nxt < nk) {
             wr[i] = w_at(kt_begin + nxt);
             sr[i] = s_at(kt_begin + nxt);
           }
           uint32_t a[4][4];
-          dequant8(w.x, s_lo, s_hi, a[0]);
-          dequant8(w.y, s_lo, s_hi, a[1]);
-          dequant8(w.z, s_lo, s_hi, a[2]);
-          dequant8(w.w, s_lo, s_hi, a[3]);
+          dequant_tile(w, sw, a);
           const __half* hrow = hs + kl0 + i * TILE_K + 16 * t;
 #pragma unroll
           for (int mt = 0; mt < MT; ++mt) {

@@ -56,6 +56,31 @@ def test_dequant_bit_exact_random_weights(mb, K, N, G):
     assert np.array_equal(out.cpu().numpy().view(np.uint16), ref.dequant(qb, sc, G).view(np.uint16))
 
 
+@pytest.mark.parametrize("M,K,N", [(8, 512, 1040), (8, 512, 9600), (5, 4096, 64), (40, 512, 1040), (200, 192, 144)])
+def test_projection_unpacks_any_scale(mb, M, K, N):
+    """The unpacking inside the projections (few rows, the looping kernel for many columns, the tensor-core one): rows with a single
+    1 pick out weights, so the result is the dequantised weight itself, bit for bit.  Scales on both sides of the limits of
+    the fused way (2^-14, 2^-6), of both signs, subnormal, zero; most tiles without any such scale, some with one."""
+    rng, G = np.random.default_rng(M + N), 64
+    u = rng.integers(0, 16, size=(K, N)).astype(np.uint8)
+    sc = np.exp(rng.uniform(np.log(2.0 ** -13.9), np.log(2.0 ** -6.1), size=(K // G, N))).astype(np.float16)
+    edge = np.array([2.0 ** -14, np.nextafter(np.float16(2.0 ** -14), np.float16(0)), 2.0 ** -6, np.nextafter(np.float16(2.0 ** -6), np.float16(0)),
+                     -0.003, 0.0, 3e-6, 0.25, 7.0, 1000.0], dtype=np.float16)
+    odd = rng.random((K // G, N)) < 0.02
+    sc[odd] = rng.choice(edge, size=int(odd.sum()))
+    qb = gen.pack_nibbles(u)
+    w = mb.mlora_weight_create(dev(qb), dev(sc), K, N, G)
+    ws = torch.zeros(mb.mlora_linear_workspace_bytes(w, M, 1), dtype=torch.uint8, device="cuda")
+    k = rng.integers(0, K, size=M)
+    x = np.zeros((M, K), dtype=np.float16)
+    x[np.arange(M), k] = 1
+    y = torch.empty(M, N, device="cuda")
+    mb.mlora_linear(w, dev(x), y, ws)
+    torch.cuda.synchronize()
+    mb.mlora_weight_destroy(w)
+    assert np.array_equal(y.cpu().numpy(), ref.dequant(qb, sc, G)[k].astype(np.float32))
+
+
 # ------------------------------------------------------------------ fused GEMM + LoRA
 def run_linear(mb, K, N, G, M, n_ad, rank, seed, with_base_rows=True):
     rng = np.random.default_rng(seed)

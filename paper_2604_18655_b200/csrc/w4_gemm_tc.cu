@@ -32,11 +32,12 @@ constexpr int TC_BM = 128;                 // output features per CTA (UMMA M)
 constexpr int TC_BK = 64;                  // input features per step: one 128-byte swizzle row of fp16
 constexpr int TC_WSLOT = 1024 + 64;        // ring slot of a warp: two tiles of nibbles, two scale entries
 
-// GR = groups of four dequantising warps: two where two CTAs share an SM (up to 128 rows), four where one has it alone.
+// GR = groups of four dequantising warps: two where two CTAs share an SM, four where one has it alone (beyond 128 rows, and
+// smaller tiles whose grid leaves every CTA an SM: launch_gemm_tc).
 // Weight stages in tensor memory (32 columns each, behind the NR accumulator columns), activation tiles, ring depth in
 // visits; the accumulator and the stages fill 256 or 512 columns.
-template <int NR> struct TcCfg {
-  static constexpr int GR = NR > 128 ? 4 : 2, OCC = GR == 2 ? 2 : 1, COLS = GR == 2 ? 256 : 512;
+template <int NR, int GRP> struct TcCfg {
+  static constexpr int GR = GRP, OCC = GR == 2 ? 2 : 1, COLS = NR > 128 ? 512 : 256;
   static constexpr int NA = (COLS - NR) / 32 < 8 ? (COLS - NR) / 32 : 8;
   static constexpr int NB = NR == 32 ? 8 : (NR <= 96 ? 6 : 4);
   static constexpr int WD = 4;
@@ -44,11 +45,11 @@ template <int NR> struct TcCfg {
   static constexpr size_t SMEM = (size_t)NB * NR * TC_BK * 2 + (size_t)WD * GR * 4 * TC_WSLOT + 1024;
 };
 
-template <int NR, int S, int EPI>
-__global__ void __launch_bounds__(TcCfg<NR>::THREADS, TcCfg<NR>::OCC)
+template <int NR, int S, int EPI, int GRP>
+__global__ void __launch_bounds__(TcCfg<NR, GRP>::THREADS, TcCfg<NR, GRP>::OCC)
 w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_constant__ CUtensorMap act_map,
                   const __grid_constant__ CUtensorMap text_map) {
-  using C = TcCfg<NR>;
+  using C = TcCfg<NR, GRP>;
   constexpr int NA = C::NA, NB = C::NB, WD = C::WD, GR = C::GR, TC_WARPS = GR * 4;
   constexpr uint32_t B_BYTES = NR * TC_BK * 2;
   constexpr int CW = NR / S;                          // rows (accumulator columns) this CTA finishes
@@ -466,6 +467,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
     }
     constexpr int HC = CW / GR;                            // columns of a warp
     constexpr int CH = HC < 16 ? HC : 16;                  // columns handled at a time
+    static_assert(HC % CH == 0 && CH >= 2 && (S == 1 || NR % (GR * 16) == 0), "a warp's columns: whole chunks, pairs of rows, whole loads");
     const int c_lo = half * HC;
     // (The epilogue is bound by the instructions it issues, 25 to 47 an output by way of an address and a bound for each: pointers
     // that step, one bound a chunk.  llama1b, two passes of 128 rows 2.49 -> 2.45 ms, llama3b, of 256 rows 7.67 -> 7.47, prompt of 100 on llama1b
@@ -688,7 +690,7 @@ static cudaError_t encode_row_map(const __half* base, int ld, int M, int nrows, 
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int NR, int S, int EPI>
+template <int NR, int S, int EPI, int GRP>
 static cudaError_t tc_launch(const GemmArgs& a, int sm_count, int* status, cudaStream_t st) {
   CUtensorMap map, tmap;
   cudaError_t e = encode_row_map(a.h, a.K, a.M, NR, &map);
@@ -699,9 +701,9 @@ static cudaError_t tc_launch(const GemmArgs& a, int sm_count, int* status, cudaS
   cudaLaunchConfig_t cfg{};
   // one CTA (or cluster) a tile; CTAs that have their K to themselves stay and take further tiles
   const int tiles = (a.N + TC_BM - 1) / TC_BM * ((a.M + NR - 1) / NR);
-  if (S == 1 && tiles > sm_count * TcCfg<NR>::OCC) cfg.gridDim = dim3(1, (unsigned)(sm_count * TcCfg<NR>::OCC));
+  if (S == 1 && tiles > sm_count * TcCfg<NR, GRP>::OCC) cfg.gridDim = dim3(1, (unsigned)(sm_count * TcCfg<NR, GRP>::OCC));
   else cfg.gridDim = dim3(S, (unsigned)((a.N + TC_BM - 1) / TC_BM), (unsigned)((a.M + NR - 1) / NR));
-  cfg.blockDim = dim3(TcCfg<NR>::THREADS); cfg.dynamicSmemBytes = TcCfg<NR>::SMEM; cfg.stream = st;
+  cfg.blockDim = dim3(TcCfg<NR, GRP>::THREADS); cfg.dynamicSmemBytes = TcCfg<NR, GRP>::SMEM; cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -709,18 +711,21 @@ static cudaError_t tc_launch(const GemmArgs& a, int sm_count, int* status, cudaS
   attr[1].val.clusterDim.x = S; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = S > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, w4_gemm_tc_kernel<NR, S, EPI>, a, status, map, tmap);
+  return cudaLaunchKernelEx(&cfg, w4_gemm_tc_kernel<NR, S, EPI, GRP>, a, status, map, tmap);
 }
 
 #define TC_FOR_EACH(X) \
-  X(32, 1) X(32, 2) X(32, 4) X(32, 8) X(64, 1) X(64, 2) X(64, 4) X(64, 8) \
-  X(96, 1) X(192, 1) X(128, 1) X(128, 2) X(128, 4) X(128, 8) X(256, 1) X(256, 2) X(256, 4) X(256, 8)
+  X(32, 1, 2) X(32, 2, 2) X(32, 4, 2) X(32, 8, 2) X(64, 1, 2) X(64, 2, 2) X(64, 4, 2) X(64, 8, 2) \
+  X(96, 1, 2) X(128, 1, 2) X(128, 2, 2) X(128, 4, 2) X(128, 8, 2) \
+  X(64, 1, 4) X(64, 2, 4) X(64, 4, 4) X(64, 8, 4) \
+  X(128, 1, 4) X(128, 2, 4) X(128, 4, 4) X(128, 8, 4) \
+  X(192, 1, 4) X(256, 1, 4) X(256, 2, 4) X(256, 4, 4) X(256, 8, 4)
 cudaError_t init_gemm_tc() {
   cudaError_t e;
-#define TC_ATTR1(NR, S, EPI) \
-  if ((e = full_carveout(w4_gemm_tc_kernel<NR, S, EPI>)) != cudaSuccess) return e; \
-  if ((e = cudaFuncSetAttribute(w4_gemm_tc_kernel<NR, S, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<NR>::SMEM)) != cudaSuccess) return e;
-#define TC_ATTR(NR, S) TC_ATTR1(NR, S, EPI_F32) TC_ATTR1(NR, S, EPI_RESID) TC_ATTR1(NR, S, EPI_SWIGLU) TC_ATTR1(NR, S, EPI_QKV)
+#define TC_ATTR1(NR, S, EPI, GRP) \
+  if ((e = full_carveout(w4_gemm_tc_kernel<NR, S, EPI, GRP>)) != cudaSuccess) return e; \
+  if ((e = cudaFuncSetAttribute(w4_gemm_tc_kernel<NR, S, EPI, GRP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TcCfg<NR, GRP>::SMEM)) != cudaSuccess) return e;
+#define TC_ATTR(NR, S, GRP) TC_ATTR1(NR, S, EPI_F32, GRP) TC_ATTR1(NR, S, EPI_RESID, GRP) TC_ATTR1(NR, S, EPI_SWIGLU, GRP) TC_ATTR1(NR, S, EPI_QKV, GRP)
   TC_FOR_EACH(TC_ATTR)
 #undef TC_ATTR
 #undef TC_ATTR1
@@ -771,10 +776,15 @@ cudaError_t launch_gemm_tc(const GemmArgs& args, int sm_count, int* status, cuda
   a.stream_magic = T > 1 ? 0xffffffffu / T + 1u : 0u;      // exact for m, T below 65536
   int nr = 32, split = 1;
   tc_plan(a, sm_count, nr, split);
-#define TC_CASE(NR, S) \
-  if (nr == NR && split == S) \
-    return a.epi == EPI_F32 ? tc_launch<NR, S, EPI_F32>(a, sm_count, status, st) : a.epi == EPI_RESID ? tc_launch<NR, S, EPI_RESID>(a, sm_count, status, st) \
-         : a.epi == EPI_SWIGLU ? tc_launch<NR, S, EPI_SWIGLU>(a, sm_count, status, st) : tc_launch<NR, S, EPI_QKV>(a, sm_count, status, st);
+  const long long ctas = (long long)((a.N + TC_BM - 1) / TC_BM) * ((a.M + nr - 1) / nr) * split;
+  // Four dequantising groups where a CTA has an SM for itself: up to 128 rows it is the unpacking that bounds, two groups take 1080
+  // cycles for a step of 64 features each while the MMAs take 255 (128 rows).  llama3b, prompt of 300 3.74 -> 2.97 ms.  Not with
+  // adapters: their shrink kernel would no longer start beside the projection ahead (llama1b, two passes of 240 rows 3.02 -> 3.15 ms).
+  const int grp = nr > 128 || ((nr == 64 || nr == 128) && a.lora.adapter_idx == nullptr && ctas <= sm_count) ? 4 : 2;
+#define TC_CASE(NR, S, GRP) \
+  if (nr == NR && split == S && grp == GRP) \
+    return a.epi == EPI_F32 ? tc_launch<NR, S, EPI_F32, GRP>(a, sm_count, status, st) : a.epi == EPI_RESID ? tc_launch<NR, S, EPI_RESID, GRP>(a, sm_count, status, st) \
+         : a.epi == EPI_SWIGLU ? tc_launch<NR, S, EPI_SWIGLU, GRP>(a, sm_count, status, st) : tc_launch<NR, S, EPI_QKV, GRP>(a, sm_count, status, st);
   TC_FOR_EACH(TC_CASE)
 #undef TC_CASE
   return cudaErrorInvalidValue;

@@ -37,6 +37,14 @@ def test_projection_splits_and_persistent_tiles(mb, K, N, G, M):
         compare(got, want, f"projection K{K} N{N} M{M} adapters {n_ad}")
 
 
+@pytest.mark.parametrize("K,N,M", [(192, 1040, 40), (320, 1040, 64), (64, 16, 128), (2048, 272, 65), (832, 1040, 128), (4096, 400, 100)])
+def test_projection_with_four_unpacking_groups(mb, K, N, M):
+    """Tiles of 64 and 128 rows whose grid leaves every CTA an SM: fewer steps than groups, steps that the groups share
+    unevenly, K splits down to a pair of rows a warp."""
+    got, want = run_linear(mb, K, N, 64, M, 0, 0, seed=K + N + M)
+    compare(got, want, f"four groups K{K} N{N} M{M}")
+
+
 @pytest.mark.parametrize("M,n_ad,rank,K", [(9, 1, 1, 256), (17, 40, 12, 1024), (300, 2, 64, 8192), (64, 64, 16, 2112)])
 def test_shrink_of_rows_with_their_own_adapters(mb, M, n_ad, rank, K):
     """Adapters without a row, with one, with more than the 16 of a group; ranks off the tile of eight; K shares beyond what

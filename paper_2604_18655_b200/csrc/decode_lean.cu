@@ -129,9 +129,12 @@ __device__ __forceinline__ void ln_stamp(const LeanArgs& a, int slot) {
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// PF k-tiles' weights in flight per warp, the input rows of XB of them loaded together, OCC CTAs on an SM
+// PF k-tiles' weights in flight per warp, the input rows of XB of them loaded together, OCC CTAs on an SM.
+// Registers: what OCC CTAs leave each other, and 80 where a CTA of 16 warps has the SM to itself: CTAs of the kernels ahead and
+// behind then fit beside it (96 registers: llama1b, one stream 414 us, 405 with 80; llama3b, eight streams 13.63 -> 13.41 ms).
+constexpr int ln_registers(int warps, int occ) { return occ == 1 ? 80 : 65536 / (warps * 32 * occ) / 8 * 8; }
 template <int NTILE, int WARPS, int PF, int XB, int OCC, bool TRACE>
-__global__ void __launch_bounds__(WARPS * 32, OCC)
+__global__ void __launch_bounds__(WARPS * 32) __maxnreg__(ln_registers(WARPS, OCC))
 lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   constexpr int THREADS = WARPS * 32;
   __shared__ float red[WARPS][NTILE][32][4];

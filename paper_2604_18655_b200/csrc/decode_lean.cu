@@ -276,7 +276,11 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
 
-  // ---- one thread per (tile, row, column): sum of the warps' parts in warp order, LoRA expand, norm factor
+  // ---- one thread per (tile, row, column): sum of the warps' parts in warp order, LoRA expand, norm factor.  With one tile the
+  // same thread goes on with its sum (through shared memory and one more barrier: llama1b 15.25 ms, 15.09 so); shared memory is for
+  // the row maxima and for the other tile of a gate / up pair.
+  const bool maxima = ph.epi == EPI_F32 && ph.out_f32 == nullptr && a.amax != nullptr;
+  float y_own = 0.f;
   for (int o = threadIdx.x; o < NTILE * 128; o += THREADS) {
     const int u = o >> 7, m = (o >> 4) & 7, c = o & 15;
     // accumulator layout of m16n8k16: lane (g,t) holds (out g, row 2t), (g, 2t+1), (g+8, 2t), (g+8, 2t+1)
@@ -295,12 +299,13 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
       }
       y *= s_inv[m];
     }
-    s_y[u][m][c] = y;
+    if (u == 0) y_own = y;
+    if (NTILE == 2 || maxima) s_y[u][m][c] = y;
   }
-  __syncthreads();
+  if (NTILE == 2 || maxima) __syncthreads();
 
   const int n0 = tile0 * TILE_N;                                            // first physical column (NTILE = 1)
-  if (ph.epi == EPI_F32 && ph.out_f32 == nullptr && a.amax != nullptr) {
+  if (maxima) {
     // lm_head without a logits destination: the row argmax (Sec. 3.5: greedy tokens; lowest column on ties) is all that
     // is wanted.  Key = order-preserving image of the value (NaN lowest) over the complemented column: the CTA's best
     // per row goes to a global maximum -- tried only when it beats what is there already.
@@ -324,9 +329,14 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   }
   if (ph.epi == EPI_F32) {
     float* out = ph.out_f32 != nullptr ? ph.out_f32 : a.logits;
-    for (int o = threadIdx.x; o < NTILE * 128; o += THREADS) {
-      const int u = o >> 7, m = (o >> 4) & 7, c = o & 15;
-      if (m < M) out[(size_t)m * ph.ldo + (tile0 + u) * TILE_N + c] = s_y[u][m][c];
+    if (NTILE == 1) {
+      const int m = threadIdx.x >> 4, c = threadIdx.x & 15;
+      if (threadIdx.x < 128 && m < M) out[(size_t)m * ph.ldo + tile0 * TILE_N + c] = y_own;
+    } else {
+      for (int o = threadIdx.x; o < NTILE * 128; o += THREADS) {
+        const int u = o >> 7, m = (o >> 4) & 7, c = o & 15;
+        if (m < M) out[(size_t)m * ph.ldo + (tile0 + u) * TILE_N + c] = s_y[u][m][c];
+      }
     }
     ln_stamp<TRACE>(a, 3);
     return;
@@ -338,7 +348,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
       float xn = 0.f;
       __half hv = __float2half_rn(0.f);
       if (m < M) {
-        xn = x_old + s_y[0][m][c];
+        xn = x_old + (NTILE == 1 ? y_own : s_y[0][m][c]);
         a.X[(size_t)m * ph.N + n0 + c] = xn;
         if (ph.gain_next != nullptr) {
           hv = __float2half_rn(xn * gain_nx);
@@ -366,7 +376,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
       const int m = threadIdx.x >> 4, c = threadIdx.x & 15;
       __half hv = __float2half_rn(0.f);
       if (m < M) {
-        const float gt = s_y[0][m][c], up = s_y[NTILE - 1][m][c];
+        const float gt = y_own, up = s_y[NTILE - 1][m][c];
         hv = __float2half_rn(gt / (1.f + __expf(-gt)) * up);
         ph.out16[(size_t)m * F + f0 + c] = hv;
       }

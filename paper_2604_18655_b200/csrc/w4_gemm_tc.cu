@@ -739,16 +739,30 @@ bool gemm_tc_eligible(const GemmArgs& a) {
   return reinterpret_cast<uintptr_t>(a.h) % 16 == 0 && tensor_map_encoder() != nullptr;   // TMA needs both
 }
 
+// Four dequantising groups (GR) where a CTA has an SM for itself: up to 128 rows it is the unpacking that bounds, two groups take 540
+// cycles for a step of 64 features while the MMAs take 255 (128 rows).  llama3b, prompt of 300 3.74 -> 2.97 ms.  Not with
+// adapters: their shrink kernel would no longer start beside the projection ahead (llama1b, two passes of 240 rows 3.02 -> 3.15 ms).
+static bool tc_four_groups(const GemmArgs& a, int nr, long long ctas, int sm_count) {
+  return nr > 128 || ((nr == 64 || nr == 128) && a.lora.adapter_idx == nullptr && ctas <= sm_count);
+}
+
 // Rows per CTA and K split, by a model of the time in microseconds, fitted to measurements of all candidates at projections
-// of 2048 x 2048 .. 14336 x 4096 with 32 .. 2000 rows: the time of a step with one or two CTAs on an SM, set-up and
-// epilogue, what a further wave costs (less where the CTA stays), and the exchange of a split.  Clusters of four CTAs do not
-// fill the machine: 33 of them on 148 SMs with one CTA each (cudaOccupancyMaxActiveClusters).  (Of eight 15, but their splits are so
-// fine that the rest of a wave costs little, and adapters gain from them: 14336 x 4096, 32 rows, 8 adapters of rank 16 24.4 us in
-// eight, 30.4 in four.)  Against the best candidate without adapters at nine projections and 9 .. 2000 rows: 1.9 % more on average,
-// 30 % at worst (2048 x 2048, 512 rows); as if clusters of four filled it 4.3 % and 68 %.  The expand's steps are left out.
+// of 2048 x 2048 .. 14336 x 4096 with 16 .. 2000 rows: the time of a step with one or two CTAs on an SM (or one with four groups),
+// set-up and epilogue, what a further wave costs (less where the CTA stays), and the exchange of a split.  Clusters of four CTAs do
+// not fill the machine: 33 of them on 148 SMs with one CTA each (cudaOccupancyMaxActiveClusters).  (Of eight 15, but their splits are
+// so fine that the rest of a wave costs little, and adapters gain from them: 14336 x 4096, 32 rows, 8 adapters of rank 16 24.4 us in
+// eight, 30.4 in four.)  Without adapters, against the best candidate at ten projections and 16 .. 2000 rows: 0.4 % more on average,
+// 14 % at worst (2048 x 2048, 128 rows); the constants from before the four groups and the shorter epilogues 1.7 % and 19 %
+// (prompts of 100 and 512 on llama1b 0.776 -> 0.764 and 1.553 -> 1.526 ms).  Those stay with adapters, whose expand (left out of the
+// model) and shrink beside the projection ahead change the order: llama3b, two passes of 256 rows 7.43 ms, 8.04 with the others.
+struct TcCosts { double step1[6], step2[6], step4[6], fixed, tail, tail4, exchange, exchange4, eight, wave1, wave1_f, wave, wave_f; };
 static void tc_plan(const GemmArgs& a, int sm_count, int& nr, int& split) {
   static const int sizes[6] = {32, 64, 96, 128, 192, 256};
-  static const double step1[6] = {0.227, 0.242, 0.264, 0.286, 0.303, 0.320}, step2[6] = {0.393, 0.429, 0.484, 0.538, 0.0, 0.0};
+  static const TcCosts plain = {{0.227, 0.242, 0.228, 0.286, 0.303, 0.320}, {0.393, 0.399, 0.484, 0.602, 0.0, 0.0}, {0.0, 0.274, 0.0, 0.244, 0.303, 0.320},
+                                4.37, 5.86, 5.15, 4.86, 2.67, 1.41, 1.4, 7.04, 4.86, 5.71};
+  static const TcCosts lora = {{0.227, 0.242, 0.264, 0.286, 0.303, 0.320}, {0.393, 0.429, 0.484, 0.538, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0, 0.303, 0.320},
+                               3.34, 3.36, 3.36, 2.52, 2.52, 1.6, 1.4, 5.1, 4.8, 7.8};
+  const TcCosts& t = a.lora.adapter_idx == nullptr ? plain : lora;
   const int slabs = (a.N + TC_BM - 1) / TC_BM, KT = a.K / TILE_K;
   double best = 1e30;
   for (int ri = 0; ri < 6; ++ri) {
@@ -759,11 +773,12 @@ static void tc_plan(const GemmArgs& a, int sm_count, int& nr, int& split) {
       const int sms = S == 4 ? sm_count - 16 : sm_count;
       const long long ctas = (long long)slabs * ((a.M + R - 1) / R) * S, per_wave = (long long)sms * (R > 128 ? 1 : 2);
       const long long full = ctas / per_wave, rest = ctas % per_wave;
-      const double steps = (KT + S - 1) / S, f = R / 256.0;
-      const double full_t = R > 128 ? step1[ri] : step2[ri], rest_t = rest == 0 ? 0.0 : (rest > sms ? step2[ri] : step1[ri]);
+      const bool four = tc_four_groups(a, R, ctas, sm_count);
+      const double steps = (KT + S - 1) / S, f = R / 256.0, one = four ? t.step4[ri] : t.step1[ri];
+      const double full_t = R > 128 ? one : t.step2[ri], rest_t = rest == 0 ? 0.0 : (rest > sms ? t.step2[ri] : one);
       const double more = (double)full + (rest > 0 ? 1 : 0) - 1.0;
-      const double cost = steps * (full * full_t + rest_t) + 3.34 + 3.36 * f + (S > 1 ? 2.52 * f : 0.0) + (S == 8 ? 1.6 : 0.0) +
-                          more * (S == 1 ? 1.4 + 5.1 * f : 4.8 + 7.8 * f);
+      const double cost = steps * (full * full_t + rest_t) + t.fixed + (four ? t.tail4 : t.tail) * f + (S > 1 ? (four ? t.exchange4 : t.exchange) * f : 0.0) +
+                          (S == 8 ? t.eight : 0.0) + more * (S == 1 ? t.wave1 + t.wave1_f * f : t.wave + t.wave_f * f);
       if (cost < best) { best = cost; nr = R; split = S; }
     }
   }
@@ -777,10 +792,7 @@ cudaError_t launch_gemm_tc(const GemmArgs& args, int sm_count, int* status, cuda
   int nr = 32, split = 1;
   tc_plan(a, sm_count, nr, split);
   const long long ctas = (long long)((a.N + TC_BM - 1) / TC_BM) * ((a.M + nr - 1) / nr) * split;
-  // Four dequantising groups where a CTA has an SM for itself: up to 128 rows it is the unpacking that bounds, two groups take 1080
-  // cycles for a step of 64 features each while the MMAs take 255 (128 rows).  llama3b, prompt of 300 3.74 -> 2.97 ms.  Not with
-  // adapters: their shrink kernel would no longer start beside the projection ahead (llama1b, two passes of 240 rows 3.02 -> 3.15 ms).
-  const int grp = nr > 128 || ((nr == 64 || nr == 128) && a.lora.adapter_idx == nullptr && ctas <= sm_count) ? 4 : 2;
+  const int grp = tc_four_groups(a, nr, ctas, sm_count) ? 4 : 2;
 #define TC_CASE(NR, S, GRP) \
   if (nr == NR && split == S && grp == GRP) \
     return a.epi == EPI_F32 ? tc_launch<NR, S, EPI_F32, GRP>(a, sm_count, status, st) : a.epi == EPI_RESID ? tc_launch<NR, S, EPI_RESID, GRP>(a, sm_count, status, st) \

@@ -32,9 +32,9 @@ __global__ void repack_kernel(const uint8_t* __restrict__ qw, const __half* __re
         const int k = kt * TILE_K + 16 * t + 4 * j + 2 * (a >> 1) + hi;
         const uint8_t byte = qw[(size_t)k * (N / 2) + (n >> 1)];
         const uint32_t u = (n & 1) ? (byte >> 4) : (byte & 0xF);
-        wd |= ((u << (4 * a + 2) | u >> (14 - 4 * a)) & 0xFFFFu) << (16 * hi);
+        wd |= u << (4 * nib);
       }
-      words[j] = wd;
+      words[j] = ((wd << 2) & 0xFFFCFFFCu) | ((wd >> 14) & 0x00030003u);   // each half word two bits up, round itself
     }
     const int pt = tile_off + nt * tile_stride;
     unsigned char* unit = w + (size_t)pt * L.unit_bytes;

@@ -473,6 +473,48 @@ __global__ void attn_merge_kernel(const AttnArgs p) {
   merge_row(p, hq / g_heads, m * g_heads + hq % g_heads, m, hq, lane);
 }
 
+// The same for passes of many rows and few chunks (at most MERGE_SLOTS, no shrink to do): a quarter of a row's features a lane,
+// 16 bytes a load, every lane with all the row's weights, so that nothing is exchanged; blocks by kv head, so that rows lie
+// side by side in the scratch.  Bound by the partials from L2.  (A warp a row with 8-byte loads at 64 features and the weights exchanged:
+// two tree passes of llama1b, 8 x 64 rows 4.54 ms, 4.34 so; 240 rows 3.04, 2.95; llama3b, 256 rows 7.47, 7.35.)
+constexpr int MERGE_SLOTS = 8;
+template <int HD>
+__global__ void __launch_bounds__(256) attn_merge_rows_kernel(const AttnArgs p) {
+  constexpr int LANES = HD / 4;
+  const int g_heads = p.Hq / p.Hkv, R_all = p.n * p.T * g_heads, kh = blockIdx.y, c = (threadIdx.x & (LANES - 1)) * 4;
+  const int v = blockIdx.x * (256 / LANES) + threadIdx.x / LANES, m = v / g_heads, slots = p.n_prefix_chunks + p.n_own_chunks;
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
+  if (v >= R_all) return;
+  int n_valid = slots;
+  if (p.n_own_chunks > 1) n_valid = p.n_prefix_chunks + min(p.n_own_chunks, (p.suffix_len[m / p.T] + p.T + p.own_chunk - 1) / p.own_chunk);
+  const size_t base = ((size_t)kh * R_all + v) * slots;
+  const float2* const ml_at = reinterpret_cast<const float2*>(p.part_ml) + base;
+  const float* const po_at = p.part_o + base * HD + c;
+  float2 ml[MERGE_SLOTS];
+  float4 po[MERGE_SLOTS];
+#pragma unroll
+  for (int i = 0; i < MERGE_SLOTS; ++i) ml[i] = i < n_valid ? __ldcg(ml_at + i) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+  for (int i = 0; i < MERGE_SLOTS; ++i) {                  // (volatile: all of them on their way, not each behind the maximum)
+    po[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < n_valid) asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(po[i].x), "=f"(po[i].y), "=f"(po[i].z), "=f"(po[i].w) : "l"(po_at + i * HD) : "memory");
+  }
+  float mmax = -INFINITY, L = 0.f;
+#pragma unroll
+  for (int i = 0; i < MERGE_SLOTS; ++i) mmax = fmaxf(mmax, ml[i].x);
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int i = 0; i < MERGE_SLOTS; ++i) {                  // fixed order: chunk 0, 1, ...
+    const float w = ml[i].x == -INFINITY ? 0.f : exp2f(ml[i].x - mmax);
+    L = fmaf(w, ml[i].y, L);
+    acc.x = fmaf(w, po[i].x, acc.x); acc.y = fmaf(w, po[i].y, acc.y);
+    acc.z = fmaf(w, po[i].z, acc.z); acc.w = fmaf(w, po[i].w, acc.w);
+  }
+  const float inv = 1.f / L;
+  *reinterpret_cast<uint2*>(p.out + ((size_t)m * p.Hq + kh * g_heads + (v - m * g_heads)) * HD + c) =
+      make_uint2(h2_as_u32(__floats2half2_rn(acc.x * inv, acc.y * inv)), h2_as_u32(__floats2half2_rn(acc.z * inv, acc.w * inv)));
+}
+
 // ----------------------------------------------------------------------------- single-pass decode attention
 // One decode row per stream (T = 1) and a short context: a cluster of two CTAs per (kv head, stream) does the whole
 // softmax (the CTAs take alternate tiles and the second hands its result to the first through distributed shared
@@ -1292,6 +1334,8 @@ static cudaError_t launch_attn_hd(const AttnArgs& a, cudaStream_t st) {
 cudaError_t init_attention() {
   cudaError_t e;
   if ((e = full_carveout(attn_merge_kernel)) != cudaSuccess) return e;
+  if ((e = full_carveout(attn_merge_rows_kernel<64>)) != cudaSuccess) return e;
+  if ((e = full_carveout(attn_merge_rows_kernel<128>)) != cudaSuccess) return e;
   e = cudaFuncSetAttribute(attn_partial_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)((ATT_ROWS + 4 * ATT_KEYS) * (64 + 8) * sizeof(__half)));
   if (e != cudaSuccess) return e;
@@ -1403,6 +1447,13 @@ cudaError_t launch_attention_merge(const AttnArgs& a, cudaStream_t st) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = a.pdl ? 1 : 0;
+  // (whole pieces of the scratch and of the output, at most MERGE_SLOTS chunks, enough rows for all SMs)
+  const bool aligned = ((reinterpret_cast<uintptr_t>(a.part_o) & 15) | (reinterpret_cast<uintptr_t>(a.part_ml) & 7) | (reinterpret_cast<uintptr_t>(a.out) & 7)) == 0;
+  if ((a.hd == 64 || a.hd == 128) && a.o_tacc == nullptr && aligned && warps > 512 && a.n_prefix_chunks + a.n_own_chunks <= MERGE_SLOTS) {
+    const int rows = 256 / (a.hd / 4), R_all = a.n * a.T * (a.Hq / a.Hkv);
+    cfg.gridDim = dim3((unsigned)((R_all + rows - 1) / rows), (unsigned)a.Hkv); cfg.blockDim = dim3(256);
+    return a.hd == 64 ? cudaLaunchKernelEx(&cfg, attn_merge_rows_kernel<64>, a) : cudaLaunchKernelEx(&cfg, attn_merge_rows_kernel<128>, a);
+  }
   return cudaLaunchKernelEx(&cfg, attn_merge_kernel, a);
 }
 

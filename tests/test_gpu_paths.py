@@ -221,6 +221,19 @@ def test_tree_attention_edges(mb, n, T, Hq, Hkv, hd, P, suf, branch):
     compare(got, want, f"tree attention n{n} T{T} {Hq}q/{Hkv}kv hd{hd} P{P}")
 
 
+@pytest.mark.parametrize("n,T,Hq,Hkv,hd,P,suf,branch,out_off", [
+    (5, 13, 12, 4, 64, 200, [0, 1, 60, 130, 7], (3, 3), 0),       # rows of a kv head that fill no whole block
+    (3, 30, 32, 8, 64, 512, [0, 640, 9], (4, 4, 2), 0),           # own segments in chunks, one stream without keys in most of them
+    (2, 40, 24, 8, 128, 1000, [300, 2], (4, 4, 2), 0),
+    (9, 16, 8, 1, 128, 0, [5] * 9, (4, 2, 2), 0),                 # no prefix: one chunk a row
+    (2, 40, 24, 8, 64, 3000, [900, 2], (4, 4, 2), 0),             # more chunks than the kernel for few takes
+    (3, 30, 32, 8, 64, 512, [0, 40, 9], (4, 4, 2), 2),            # an output that does not start on 8 bytes
+])
+def test_merge_of_many_rows(mb, n, T, Hq, Hkv, hd, P, suf, branch, out_off):
+    got, want = run_attention(mb, n, T, Hq, Hkv, hd, P, suf, branch, seed=n + T + P, out_off=out_off)
+    compare(got, want, f"merge n{n} T{T} {Hq}q/{Hkv}kv hd{hd} P{P} out + {out_off}")
+
+
 @pytest.mark.parametrize("hd", [64, 128])
 @pytest.mark.parametrize("n,T,P,suf,branch", [(3, 1, 2100, [0, 40, 90], ()), (2, 16, 130, [3, 64], (4, 2, 2))])
 @pytest.mark.parametrize("out_off,ws_off", [(1, 8), (2, 0), (3, 4)])

@@ -266,7 +266,7 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
     // (matrix j = the eight rows' pieces) hands lane (g, t) word t of them: features 16j + 4t .. + 3, the order in which
     // the fragment store below lays k16 slice j down
     const uint32_t dpos = (uint32_t)((lane & 3) * 128 + (lane >> 2) * 16);
-    // The loop is bound by the instructions it issues (about 150 a visit, 104 of them the unpacking of 64 weights a lane),
+    // The loop is bound by the instructions it issues (about 130 a visit, 72 of them the unpacking of 64 weights a lane),
     // so the fetch keeps running pointers: k-tile f_r of its chunk, the tile's bytes, the chunk's scale entries
     int f_left = 0, f_r = 0, f_c = 0;                       // fetches still to issue in this tile
     const unsigned char *f_w = nullptr, *f_s = nullptr;

@@ -453,79 +453,77 @@ __device__ __forceinline__ uint32_t h2_as_u32(__half2 h) { return *reinterpret_c
 __device__ __forceinline__ __half2 u32_as_h2(uint32_t u) { return *reinterpret_cast<__half2*>(&u); }
 
 // Eight INT4 weights -> four fp16x2 registers in m16n8k16 A-fragment order, each the single correctly-rounded fp16 product
-// (u - 8) * scale of the stored nibble u.
+// (u - 8) * scale of the stored nibble u, in one of three ways.  The kernels that unpack are bound by the instructions they issue.
 //
-// The usual way, for scales in [2^-14, 2^-6): a nibble where it lies in a word is the mantissa of a subnormal, u 2^-22 or
-// u 2^-18, and one fused multiply-add with scale 2^22 (2^18) and -8 scale, all of them exact, gives the product with its one
-// rounding: a mask and a multiply-add a pair, one byte swap a word.  The kernels that unpack are bound by the instructions
-// they issue; 13 a word by way of the integers (below) took 203 cycles a step of four warps (64 weights a lane), these 9 139.
-// llama1b, eight streams, 33 steps 16.03 -> 15.70 ms, llama3b, 9 steps 14.37 -> 14.02 ms; 8 rows of 4096 x 14336 19.0 -> 18.0 us;
-// llama1b, two tree passes of 128 rows 2.53 -> 2.49 ms, a prompt of 512 1.605 -> 1.565 ms.
-__device__ __forceinline__ bool w4_scales_usual(uint32_t sw, uint32_t sw2 = 0x20002000u) {
-  return (((sw - 0x04000400u) | (sw2 - 0x04000400u)) & 0xE000E000u) == 0u;
-}
-struct W4Scales { __half2 s_lo, s_hi, c_lo, c_hi; };
-__device__ __forceinline__ W4Scales w4_scales(uint32_t sw) {
-  const uint32_t s = sw + 0x48005800u, c = sw + 0x8C008C00u;   // exponents + 18 | + 22; + 3 and the sign
-  return W4Scales{u32_as_h2(__byte_perm(s, s, 0x1010)), u32_as_h2(__byte_perm(s, s, 0x3232)),
-                  u32_as_h2(__byte_perm(c, c, 0x1010)), u32_as_h2(__byte_perm(c, c, 0x3232))};
-}
-__device__ __forceinline__ void dequant8(uint32_t w, const W4Scales& f, uint32_t (&a)[4]) {
+// 0, scales in [2^-14, 2^-6): a nibble where it lies in a word is the mantissa of a subnormal, u 2^-22 or u 2^-18, and one fused
+// multiply-add with scale 2^22 (2^18) and -8 scale, all of them exact, gives the product with its one rounding: a mask and a
+// multiply-add a pair, one byte swap a word.  9 instructions a word: 139 cycles a step of four warps (64 weights a lane), way 2 203.
+// 1, scales in [2^-14, 2^-2): all nibbles moved to where they are u 2^-18.  11 instructions.  (Groups that hold a |w| of 0.11 and more:
+// llama1b, weights of standard deviation 0.05, eight streams, 33 steps 15.92 ms with way 2 in its place, 15.27 so; one stream 434 and
+// 419 us.)
+// 2, any scale: the nibble in the mantissa of 1024.0 (giving 1024 + 4u or 1024 + 64u, as it lies), q = u - 8 exactly by one fused
+// multiply-add, then the product.  13 instructions.
+__device__ __forceinline__ uint32_t w4_odd(uint32_t sw) { return (sw - 0x04000400u) & 0xE000E000u; }   // 0: way 0 for both scales
+__device__ __forceinline__ uint32_t w4_odd_wide(uint32_t sw) { return (sw | (sw + 0x4C004C00u) | (sw - 0x04000400u)) & 0x80008000u; }   // 0: way 1
+template <int WAY> struct W4Scales {
+  __half2 s_lo, s_hi, c_lo, c_hi;                           // way 2: the scales; else scale 2^22 (2^18) | 2^18 and -8 scale
+  __device__ __forceinline__ explicit W4Scales(uint32_t sw) {
+    const uint32_t s = WAY == 0 ? sw + 0x48005800u : (WAY == 1 ? sw + 0x48004800u : sw), c = sw + 0x8C008C00u;   // (exponents + 18, + 22; + 3, sign)
+    s_lo = u32_as_h2(__byte_perm(s, s, 0x1010)); s_hi = u32_as_h2(__byte_perm(s, s, 0x3232));
+    if (WAY != 2) { c_lo = u32_as_h2(__byte_perm(c, c, 0x1010)); c_hi = u32_as_h2(__byte_perm(c, c, 0x3232)); }
+  }
+};
+template <int WAY>
+__device__ __forceinline__ void dequant8(uint32_t w, const W4Scales<WAY>& f, uint32_t (&a)[4]) {
   const uint32_t x = __byte_perm(w, w, 0x2301);
-  a[0] = h2_as_u32(__hfma2(u32_as_h2(w & 0x003C003Cu), f.s_lo, f.c_lo));
-  a[1] = h2_as_u32(__hfma2(u32_as_h2(w & 0x03C003C0u), f.s_hi, f.c_hi));
-  a[2] = h2_as_u32(__hfma2(u32_as_h2(x & 0x003C003Cu), f.s_lo, f.c_lo));
-  a[3] = h2_as_u32(__hfma2(u32_as_h2(x & 0x03C003C0u), f.s_hi, f.c_hi));
-}
-// Any scale: the nibble in the mantissa of 1024.0 (giving 1024+u, or 1024+16u for the nibbles one hex digit up), q = u - 8
-// exactly by one subtract / fused multiply-add, then the product.  (Not inlined: it must not cost the usual way registers.)
-static __device__ __noinline__ uint4 dequant8_any(uint32_t wr, uint32_t sw) {
-  const uint32_t w = ((wr >> 2) & 0x3FFF3FFFu) | ((wr & 0x00030003u) << 14);   // (stored two bits up, round its half)
-  const uint32_t MAGIC = 0x64006400u;                       // (1024.0, 1024.0)
-  const __half2 k1032 = u32_as_h2(0x64086408u);             // 1032.0
-  const __half2 k16th = u32_as_h2(0x2C002C00u);             // 1/16
-  const __half2 km72 = u32_as_h2(0xD480D480u);              // -72.0
-  const __half2 s_lo = u32_as_h2(__byte_perm(sw, sw, 0x1010)), s_hi = u32_as_h2(__byte_perm(sw, sw, 0x3232));
-  const uint32_t w8 = w >> 8;
-  const __half2 x0 = u32_as_h2((w & 0x000F000Fu) | MAGIC);
-  const __half2 x1 = u32_as_h2((w & 0x00F000F0u) | MAGIC);
-  const __half2 x2 = u32_as_h2((w8 & 0x000F000Fu) | MAGIC);
-  const __half2 x3 = u32_as_h2((w8 & 0x00F000F0u) | MAGIC);
-  return make_uint4(h2_as_u32(__hmul2(__hsub2(x0, k1032), s_lo)), h2_as_u32(__hmul2(__hfma2(x1, k16th, km72), s_hi)),
-                    h2_as_u32(__hmul2(__hsub2(x2, k1032), s_lo)), h2_as_u32(__hmul2(__hfma2(x3, k16th, km72), s_hi)));
-}
-__device__ __forceinline__ void dequant8(uint32_t w, uint32_t sw, uint32_t (&a)[4]) {
-  const uint4 v = dequant8_any(w, sw);
-  a[0] = v.x; a[1] = v.y; a[2] = v.z; a[3] = v.w;
+  if constexpr (WAY == 2) {
+    const uint32_t MAGIC = 0x64006400u;                     // (1024.0, 1024.0)
+    const __half2 k4th = u32_as_h2(0x34003400u), km264 = u32_as_h2(0xDC20DC20u);   // 1/4, -264.0
+    const __half2 k64th = u32_as_h2(0x24002400u), km24 = u32_as_h2(0xCE00CE00u);   // 1/64, -24.0
+    a[0] = h2_as_u32(__hmul2(__hfma2(u32_as_h2((w & 0x003C003Cu) | MAGIC), k4th, km264), f.s_lo));
+    a[1] = h2_as_u32(__hmul2(__hfma2(u32_as_h2((w & 0x03C003C0u) | MAGIC), k64th, km24), f.s_hi));
+    a[2] = h2_as_u32(__hmul2(__hfma2(u32_as_h2((x & 0x003C003Cu) | MAGIC), k4th, km264), f.s_lo));
+    a[3] = h2_as_u32(__hmul2(__hfma2(u32_as_h2((x & 0x03C003C0u) | MAGIC), k64th, km24), f.s_hi));
+  } else {
+    constexpr int UP = WAY == 1 ? 4 : 0;
+    constexpr uint32_t LOW = 0x003C003Cu << UP;
+    a[0] = h2_as_u32(__hfma2(u32_as_h2((w << UP) & LOW), f.s_lo, f.c_lo));
+    a[1] = h2_as_u32(__hfma2(u32_as_h2(w & 0x03C003C0u), f.s_hi, f.c_hi));
+    a[2] = h2_as_u32(__hfma2(u32_as_h2((x << UP) & LOW), f.s_lo, f.c_lo));
+    a[3] = h2_as_u32(__hfma2(u32_as_h2(x & 0x03C003C0u), f.s_hi, f.c_hi));
+  }
 }
 // a lane's share of a tile (lanes may go different ways: nothing that needs the whole warp happens inside)
-__device__ __forceinline__ void dequant_tile(const uint4& w, uint32_t sw, uint32_t (&a)[4][4]) {
-  if (w4_scales_usual(sw)) {
-    const W4Scales f = w4_scales(sw);
+__device__ __forceinline__ void dequant_tile_lane(const uint4& w, uint32_t sw, uint32_t (&a)[4][4]) {
+  if (w4_odd(sw) == 0u) {
+    const W4Scales<0> f(sw);
     dequant8(w.x, f, a[0]); dequant8(w.y, f, a[1]); dequant8(w.z, f, a[2]); dequant8(w.w, f, a[3]);
   } else {
-    dequant8(w.x, sw, a[0]); dequant8(w.y, sw, a[1]); dequant8(w.z, sw, a[2]); dequant8(w.w, sw, a[3]);
+    const W4Scales<2> f(sw);
+    dequant8(w.x, f, a[0]); dequant8(w.y, f, a[1]); dequant8(w.z, f, a[2]); dequant8(w.w, f, a[3]);
   }
 }
-// The same by a whole warp (all lanes call it): one lane's unusual scale sends it the other way as one, so that every word can
-// go straight to `use(j, fragment)`, a tensor-core step.  (Four fragments held until the lanes meet again cost the decode
-// kernels spills: llama1b, one stream 424 -> 460 us.)
-template <class F>
-__device__ __forceinline__ void dequant_tile_warp(const uint4& w, uint32_t sw, F&& use) {
+// The same, every word straight to `use(j, fragment)`, a tensor-core step.
+template <int WAY, class F>
+__device__ __forceinline__ void dequant_tile(const uint4& w, uint32_t sw, F&& use) {
+  const W4Scales<WAY> f(sw);
   uint32_t a[4];
-  if (__all_sync(0xffffffffu, w4_scales_usual(sw))) {
-    const W4Scales f = w4_scales(sw);
-    dequant8(w.x, f, a); use(0, a);
-    dequant8(w.y, f, a); use(1, a);
-    dequant8(w.z, f, a); use(2, a);
-    dequant8(w.w, f, a); use(3, a);
-  } else {
-    dequant8(w.x, sw, a); use(0, a);
-    dequant8(w.y, sw, a); use(1, a);
-    dequant8(w.z, sw, a); use(2, a);
-    dequant8(w.w, sw, a); use(3, a);
-  }
+  dequant8(w.x, f, a); use(0, a);
+  dequant8(w.y, f, a); use(1, a);
+  dequant8(w.z, f, a); use(2, a);
+  dequant8(w.w, f, a); use(3, a);
 }
+// Several tiles of a warp the same way: body(way) with a lane's odd and odd_wide of all their scales together.  All lanes call it; one
+// lane's scale sends the whole warp another way, so no branch that lanes take differently stands around the tensor-core steps.  Each
+// way in one piece: a vote and two ways tile by tile had the warp fetch what it jumps over (llama1b, one stream 401 -> 420 us).
+template <int WAY> struct W4Way { static constexpr int value = WAY; };
+template <class O, class W, class F>
+__device__ __forceinline__ void dequant_ways(O&& odd, W&& odd_wide, F&& body) {
+  if (__all_sync(0xffffffffu, odd() == 0u)) body(W4Way<0>{});
+  else if (__all_sync(0xffffffffu, odd_wide() == 0u)) body(W4Way<1>{});
+  else body(W4Way<2>{});
+}
+
 // physical column of a fused projection -> (segment, logical column)
 __device__ __forceinline__ void map_col(int mode, int c, int n0, int n1, int& seg, int& col) {
   if (mode == MODE_PLAIN) { seg = 0; col = c; }

@@ -669,7 +669,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) decode_chain_kernel(const Chain
                     const uint4 b01 = *reinterpret_cast<const uint4*>(hbase + q * TILE_K);
                     const uint4 b23 = *reinterpret_cast<const uint4*>(hbase + q * TILE_K + 8);
                     uint32_t af[4][4];
-                    dequant_tile(wv, sw, af);
+                    dequant_tile_lane(wv, sw, af);
                     mma_16816(acc0, af[0], b01.x, b01.y);
                     mma_16816(acc1, af[1], b01.z, b01.w);
                     mma_16816(acc0, af[2], b23.x, b23.y);

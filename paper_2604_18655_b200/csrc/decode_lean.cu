@@ -249,18 +249,28 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   for (int kb = kt0; kb < kt1; kb += PF) {
 #pragma unroll
    for (int ib = 0; ib < PF; ib += XB) {
+    auto any_of = [&](auto odd) {
+      uint32_t v = 0;
 #pragma unroll
-    for (int i = 0; i < XB; ++i) {
-      if (kb + ib + i < kt1) {
+      for (int i = 0; i < XB; ++i)
 #pragma unroll
-        for (int u = 0; u < NTILE; ++u) {
-          dequant_tile_warp(wv[ib + i][u], sv[ib + i][u], [&](int j, const uint32_t (&af)[4]) {
-            const uint4& x = j < 2 ? x0[i] : x1[i];
-            mma_16816(acc[u], af, j & 1 ? x.z : x.x, j & 1 ? x.w : x.y);
-          });
+        for (int u = 0; u < NTILE; ++u)
+          if (kb + ib + i < kt1) v |= odd(sv[ib + i][u]);
+      return v;
+    };
+    dequant_ways([&] { return any_of(w4_odd); }, [&] { return any_of(w4_odd_wide); }, [&](auto way) {
+#pragma unroll
+      for (int i = 0; i < XB; ++i) {
+        if (kb + ib + i < kt1) {
+#pragma unroll
+          for (int u = 0; u < NTILE; ++u)
+            dequant_tile<decltype(way)::value>(wv[ib + i][u], sv[ib + i][u], [&](int j, const uint32_t (&af)[4]) {
+              const uint4& x = j < 2 ? x0[i] : x1[i];
+              mma_16816(acc[u], af, j & 1 ? x.z : x.x, j & 1 ? x.w : x.y);
+            });
         }
       }
-    }
+    });
     if (kb + ib + XB < kt1) load_x(kb + ib + XB);
    }
     if (kb + PF < kt1) load_weights(kb + PF);
@@ -482,17 +492,27 @@ __global__ void __launch_bounds__(WARPS * 32, 2) lean_lmhead_kernel(const LeanAr
   for (; tile < L.NT; tile += gridDim.x) {
     asm volatile("cp.async.wait_group %0;" ::"n"(LM_DEPTH - 1) : "memory");   // this thread's pieces of the oldest tile are there
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    uint32_t sv[LM_PF];
 #pragma unroll
-    for (int i = 0; i < LM_PF; ++i) {
-      if (kt0 + i < kt1) {
-        const uint4 wv = wring[((size_t)stage * LM_PF + i) * THREADS + threadIdx.x];
-        const uint32_t sv = sring[((size_t)stage * LM_PF + i) * THREADS + threadIdx.x];
-        dequant_tile_warp(wv, sv, [&](int j, const uint32_t (&af)[4]) {
-          const uint4& x = j < 2 ? x0[i] : x1[i];
-          mma_16816(acc, af, j & 1 ? x.z : x.x, j & 1 ? x.w : x.y);
-        });
+    for (int i = 0; i < LM_PF; ++i) sv[i] = kt0 + i < kt1 ? sring[((size_t)stage * LM_PF + i) * THREADS + threadIdx.x] : 0x20002000u;   // (2^-7: no odd one)
+    auto any_of = [&](auto odd) {
+      uint32_t v = 0;
+#pragma unroll
+      for (int i = 0; i < LM_PF; ++i) v |= odd(sv[i]);
+      return v;
+    };
+    dequant_ways([&] { return any_of(w4_odd); }, [&] { return any_of(w4_odd_wide); }, [&](auto way) {
+#pragma unroll
+      for (int i = 0; i < LM_PF; ++i) {
+        if (kt0 + i < kt1) {
+          const uint4 wv = wring[((size_t)stage * LM_PF + i) * THREADS + threadIdx.x];
+          dequant_tile<decltype(way)::value>(wv, sv[i], [&](int j, const uint32_t (&af)[4]) {
+            const uint4& x = j < 2 ? x0[i] : x1[i];
+            mma_16816(acc, af, j & 1 ? x.z : x.x, j & 1 ? x.w : x.y);
+          });
+        }
       }
-    }
+    });
     issue(stage, tile + LM_DEPTH * (int)gridDim.x);          // refills the slots just read (this thread's own)
     stage = stage + 1 == LM_DEPTH ? 0 : stage + 1;
     *reinterpret_cast<float4*>(red[par][warp][lane]) = make_float4(acc[0], acc[1], acc[2], acc[3]);

@@ -270,7 +270,7 @@ __device__ __forceinline__ void gemm_tiles(const GemmLoop& q, const WaitCtx& wc,
             const uint4 wv = *reinterpret_cast<const uint4*>(sb + itl * 512 + lane * 16);
             const uint32_t sw = *reinterpret_cast<const uint32_t*>(sb + kc * 512 + g * 4 + (itl >> q.gshift) * 32);
             uint32_t af[4][4];
-            dequant_tile(wv, sw, af);
+            dequant_tile_lane(wv, sw, af);
             mma_16816(acc0, af[0], bfr[qi][0].x, bfr[qi][0].y);
             mma_16816(acc1, af[1], bfr[qi][0].z, bfr[qi][0].w);
             mma_16816(acc0, af[2], bfr[qi][1].x, bfr[qi][1].y);

@@ -88,7 +88,7 @@ __global__ void dequant_kernel(const unsigned char* __restrict__ w, const WLayou
     const uint4 wv = ldg_stream(reinterpret_cast<const uint4*>(unit + wl_tile_off(L, kt)) + lane);
     const uint32_t sw = ldg_nc_u32(reinterpret_cast<const uint32_t*>(unit + wl_scale_off(L, kt)) + g);
     uint32_t frag[4][4];
-    dequant_tile(wv, sw, frag);
+    dequant_tile_lane(wv, sw, frag);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const uint32_t (&a)[4] = frag[j];
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) w4_gemm_kernel(const GemmArgs p,
             sr[i] = s_at(kt_begin + nxt);
           }
           uint32_t a[4][4];
-          dequant_tile(w, sw, a);
+          dequant_tile_lane(w, sw, a);
           const __half* hrow = hs + kl0 + i * TILE_K + 16 * t;
 #pragma unroll
           for (int mt = 0; mt < MT; ++mt) {

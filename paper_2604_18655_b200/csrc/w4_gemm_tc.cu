@@ -361,21 +361,20 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       slot = slot + TC_WSLOT == ring_end ? ring0 : slot + TC_WSLOT;
       uint32_t r0[16], r1[16];
       {
-        auto unpack = [](const uint32_t (&w)[4], auto&& one, uint32_t (&r)[16]) {
+        auto unpack = [](const uint32_t (&w)[4], const auto& f, uint32_t (&r)[16]) {
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             uint32_t a[4];
-            one(w[j], a);
+            dequant8(w[j], f, a);
             r[4 * j] = a[0]; r[4 * j + 1] = a[2]; r[4 * j + 2] = a[1]; r[4 * j + 3] = a[3];
           }
         };
-        if (__all_sync(0xffffffffu, w4_scales_usual(sc0, sc1))) {
-          const W4Scales f0 = w4_scales(sc0), f1 = w4_scales(sc1);
-          unpack(w0, [&](uint32_t w, uint32_t (&a)[4]) { dequant8(w, f0, a); }, r0);
-          unpack(w1, [&](uint32_t w, uint32_t (&a)[4]) { dequant8(w, f1, a); }, r1);
+        if (__all_sync(0xffffffffu, (w4_odd(sc0) | w4_odd(sc1)) == 0u)) {
+          unpack(w0, W4Scales<0>(sc0), r0);
+          unpack(w1, W4Scales<0>(sc1), r1);
         } else {
-          unpack(w0, [&](uint32_t w, uint32_t (&a)[4]) { dequant8(w, sc0, a); }, r0);
-          unpack(w1, [&](uint32_t w, uint32_t (&a)[4]) { dequant8(w, sc1, a); }, r1);
+          unpack(w0, W4Scales<2>(sc0), r0);
+          unpack(w1, W4Scales<2>(sc1), r1);
         }
       }
       stage_free(a_free);

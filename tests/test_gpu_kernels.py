@@ -81,6 +81,29 @@ def test_projection_unpacks_any_scale(mb, M, K, N):
     assert np.array_equal(y.cpu().numpy(), ref.dequant(qb, sc, G)[k].astype(np.float32))
 
 
+@pytest.mark.parametrize("lo,hi", [(-9, -2.1), (-14, 4)])
+@pytest.mark.parametrize("M,K,N", [(8, 512, 1040), (1, 576, 7168), (8, 3072, 9600), (3, 4160, 64), (40, 512, 1040)])
+def test_projection_unpacks_larger_scales(mb, M, K, N, lo, hi):
+    """Scales beyond 2^-6: k-tiles whose scales all lie below 2^-2 but for a few, and k-tiles of every kind of scale; bit for bit."""
+    rng = np.random.default_rng(M + K)
+    u = rng.integers(0, 16, size=(K, N)).astype(np.uint8)
+    sc = np.exp2(rng.uniform(lo, hi, size=(K // 64, N))).astype(np.float16)
+    edge = np.array([2.0 ** -2, np.nextafter(np.float16(2.0 ** -2), np.float16(0)), 2.0 ** -15, -0.1, 0.0, 4000.0], dtype=np.float16)
+    odd = rng.random((K // 64, N)) < 0.002
+    sc[odd] = rng.choice(edge, size=int(odd.sum()))
+    qb = gen.pack_nibbles(u)
+    w = mb.mlora_weight_create(dev(qb), dev(sc), K, N, 64)
+    ws = torch.zeros(mb.mlora_linear_workspace_bytes(w, M, 1), dtype=torch.uint8, device="cuda")
+    k = rng.integers(0, K, size=M)
+    x = np.zeros((M, K), dtype=np.float16)
+    x[np.arange(M), k] = 1
+    y = torch.empty(M, N, device="cuda")
+    mb.mlora_linear(w, dev(x), y, ws)
+    torch.cuda.synchronize()
+    mb.mlora_weight_destroy(w)
+    assert np.array_equal(y.cpu().numpy(), ref.dequant(qb, sc, 64)[k].astype(np.float32))
+
+
 # ------------------------------------------------------------------ fused GEMM + LoRA
 def run_linear(mb, K, N, G, M, n_ad, rank, seed, with_base_rows=True):
     rng = np.random.default_rng(seed)

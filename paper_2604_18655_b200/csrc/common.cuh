@@ -493,17 +493,7 @@ __device__ __forceinline__ void dequant8(uint32_t w, const W4Scales<WAY>& f, uin
     a[3] = h2_as_u32(__hfma2(u32_as_h2(x & 0x03C003C0u), f.s_hi, f.c_hi));
   }
 }
-// a lane's share of a tile (lanes may go different ways: nothing that needs the whole warp happens inside)
-__device__ __forceinline__ void dequant_tile_lane(const uint4& w, uint32_t sw, uint32_t (&a)[4][4]) {
-  if (w4_odd(sw) == 0u) {
-    const W4Scales<0> f(sw);
-    dequant8(w.x, f, a[0]); dequant8(w.y, f, a[1]); dequant8(w.z, f, a[2]); dequant8(w.w, f, a[3]);
-  } else {
-    const W4Scales<2> f(sw);
-    dequant8(w.x, f, a[0]); dequant8(w.y, f, a[1]); dequant8(w.z, f, a[2]); dequant8(w.w, f, a[3]);
-  }
-}
-// The same, every word straight to `use(j, fragment)`, a tensor-core step.
+// A lane's share of a tile, every word straight to `use(j, fragment)`, a tensor-core step.
 template <int WAY, class F>
 __device__ __forceinline__ void dequant_tile(const uint4& w, uint32_t sw, F&& use) {
   const W4Scales<WAY> f(sw);

@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) decode_chain_kernel(const Chain
             const int kc = (c == L.nchunks - 1) ? L.kc_last : CHUNK_KT;
             const int items_here = (kc + CH_ITEM_KT - 1) / CH_ITEM_KT;
             const int it_end = min(it_hi, (c + 1) * CH_ITEMS_PER_CHUNK);
-            const bool ok = wait_mbar(smem_u32(full_bar + st), par, wc, 3, p);
+            const bool ok = __all_sync(0xffffffffu, wait_mbar(smem_u32(full_bar + st), par, wc, 3, p));   // one answer a warp: mma inside
             const unsigned char* sb = ring + (size_t)st * CH_STAGE_BYTES;
             const unsigned char* ssc = sb + kc * 512 + g * 4;
             const uint32_t ebar = smem_u32(empty_bar + st);
@@ -661,21 +661,25 @@ __global__ void __launch_bounds__(CH_THREADS, 1) decode_chain_kernel(const Chain
               const int ktl = itl * CH_ITEM_KT;                           // its first k-tile inside the chunk
               if (ok) {
                 const __half* hbase = hrow + (size_t)(c * CHUNK_KT + ktl) * TILE_K;
+                uint32_t sw[CH_ITEM_KT];
 #pragma unroll
-                for (int q = 0; q < CH_ITEM_KT; ++q) {
-                  if (ktl + q < kc) {
-                    const uint4 wv = *reinterpret_cast<const uint4*>(sb + (ktl + q) * 512 + lane * 16);
-                    const uint32_t sw = *reinterpret_cast<const uint32_t*>(ssc + ((ktl + q) >> gshift) * 32);
-                    const uint4 b01 = *reinterpret_cast<const uint4*>(hbase + q * TILE_K);
-                    const uint4 b23 = *reinterpret_cast<const uint4*>(hbase + q * TILE_K + 8);
-                    uint32_t af[4][4];
-                    dequant_tile_lane(wv, sw, af);
-                    mma_16816(acc0, af[0], b01.x, b01.y);
-                    mma_16816(acc1, af[1], b01.z, b01.w);
-                    mma_16816(acc0, af[2], b23.x, b23.y);
-                    mma_16816(acc1, af[3], b23.z, b23.w);
+                for (int q = 0; q < CH_ITEM_KT; ++q)
+                  sw[q] = ktl + q < kc ? *reinterpret_cast<const uint32_t*>(ssc + ((ktl + q) >> gshift) * 32) : 0x20002000u;   // (2^-7: no odd one)
+                static_assert(CH_ITEM_KT == 2, "the scales of an item");
+                dequant_ways([&] { return w4_odd(sw[0]) | w4_odd(sw[1]); }, [&] { return w4_odd_wide(sw[0]) | w4_odd_wide(sw[1]); }, [&](auto way) {
+#pragma unroll
+                  for (int q = 0; q < CH_ITEM_KT; ++q) {
+                    if (ktl + q < kc) {
+                      const uint4 wv = *reinterpret_cast<const uint4*>(sb + (ktl + q) * 512 + lane * 16);
+                      const uint4 b01 = *reinterpret_cast<const uint4*>(hbase + q * TILE_K);
+                      const uint4 b23 = *reinterpret_cast<const uint4*>(hbase + q * TILE_K + 8);
+                      dequant_tile<decltype(way)::value>(wv, sw[q], [&](int j, const uint32_t (&af)[4]) {
+                        const uint4& b = j < 2 ? b01 : b23;
+                        mma_16816(j & 1 ? acc1 : acc0, af, j & 1 ? b.z : b.x, j & 1 ? b.w : b.y);
+                      });
+                    }
                   }
-                }
+                });
               }
               __syncwarp();
               // one arrival per item; the last item of a ragged chunk also arrives for the items the chunk lacks

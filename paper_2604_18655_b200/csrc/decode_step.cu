@@ -262,19 +262,18 @@ __device__ __forceinline__ void gemm_tiles(const GemmLoop& q, const WaitCtx& wc,
             uint32_t par = par_t;
             if (st >= q.nstages) { st -= q.nstages; par ^= 1u; }
             kc = (c == q.nchunks - 1) ? q.kc_last : CHUNK_KT;
-            ok = wait_mbar(smem_u32(q.full_bar + st), par, wc, 3, q.phase);
+            ok = __all_sync(0xffffffffu, wait_mbar(smem_u32(q.full_bar + st), par, wc, 3, q.phase));   // one answer a warp: mma inside
             sb = q.ring + (size_t)st * DS_STAGE_BYTES;
             if (q.tr != nullptr && tl == 0 && pass == 0 && qi == 0) q.tr[8] = clock64();
           }
           if (ok && itl < kc) {
             const uint4 wv = *reinterpret_cast<const uint4*>(sb + itl * 512 + lane * 16);
             const uint32_t sw = *reinterpret_cast<const uint32_t*>(sb + kc * 512 + g * 4 + (itl >> q.gshift) * 32);
-            uint32_t af[4][4];
-            dequant_tile_lane(wv, sw, af);
-            mma_16816(acc0, af[0], bfr[qi][0].x, bfr[qi][0].y);
-            mma_16816(acc1, af[1], bfr[qi][0].z, bfr[qi][0].w);
-            mma_16816(acc0, af[2], bfr[qi][1].x, bfr[qi][1].y);
-            mma_16816(acc1, af[3], bfr[qi][1].z, bfr[qi][1].w);
+            // (way 2 for any scale: a vote and two ways a tile took the same time, and the kernel is bound by its instructions' fetch)
+            dequant_tile<2>(wv, sw, [&](int j, const uint32_t (&af)[4]) {
+              const uint4& b = bfr[qi][j >> 1];
+              mma_16816(j & 1 ? acc1 : acc0, af, j & 1 ? b.z : b.x, j & 1 ? b.w : b.y);
+            });
           }
           __syncwarp();
           // one arrival per item; the last item of a ragged chunk also arrives for the items the chunk lacks

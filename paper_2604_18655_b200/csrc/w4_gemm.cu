@@ -87,23 +87,21 @@ __global__ void dequant_kernel(const unsigned char* __restrict__ w, const WLayou
     const unsigned char* unit = w + (size_t)pt * L.unit_bytes;
     const uint4 wv = ldg_stream(reinterpret_cast<const uint4*>(unit + wl_tile_off(L, kt)) + lane);
     const uint32_t sw = ldg_nc_u32(reinterpret_cast<const uint32_t*>(unit + wl_scale_off(L, kt)) + g);
-    uint32_t frag[4][4];
-    dequant_tile_lane(wv, sw, frag);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t (&a)[4] = frag[j];
-      const int k = kt * TILE_K + 16 * t + 4 * j;
-      const int n = nt * TILE_N + g;
-      const __half2 a0 = u32_as_h2(a[0]), a1 = u32_as_h2(a[1]), a2 = u32_as_h2(a[2]), a3 = u32_as_h2(a[3]);
-      out[(size_t)(k + 0) * N + n] = __low2half(a0);
-      out[(size_t)(k + 1) * N + n] = __high2half(a0);
-      out[(size_t)(k + 0) * N + n + 8] = __low2half(a1);
-      out[(size_t)(k + 1) * N + n + 8] = __high2half(a1);
-      out[(size_t)(k + 2) * N + n] = __low2half(a2);
-      out[(size_t)(k + 3) * N + n] = __high2half(a2);
-      out[(size_t)(k + 2) * N + n + 8] = __low2half(a3);
-      out[(size_t)(k + 3) * N + n + 8] = __high2half(a3);
-    }
+    dequant_ways([&] { return w4_odd(sw); }, [&] { return w4_odd_wide(sw); }, [&](auto way) {
+      dequant_tile<decltype(way)::value>(wv, sw, [&](int j, const uint32_t (&a)[4]) {
+        const int k = kt * TILE_K + 16 * t + 4 * j;
+        const int n = nt * TILE_N + g;
+        const __half2 a0 = u32_as_h2(a[0]), a1 = u32_as_h2(a[1]), a2 = u32_as_h2(a[2]), a3 = u32_as_h2(a[3]);
+        out[(size_t)(k + 0) * N + n] = __low2half(a0);
+        out[(size_t)(k + 1) * N + n] = __high2half(a0);
+        out[(size_t)(k + 0) * N + n + 8] = __low2half(a1);
+        out[(size_t)(k + 1) * N + n + 8] = __high2half(a1);
+        out[(size_t)(k + 2) * N + n] = __low2half(a2);
+        out[(size_t)(k + 3) * N + n] = __high2half(a2);
+        out[(size_t)(k + 2) * N + n + 8] = __low2half(a3);
+        out[(size_t)(k + 3) * N + n + 8] = __high2half(a3);
+      });
+    });
   }
 }
 
@@ -199,7 +197,8 @@ __global__ void __launch_bounds__(GEMM_THREADS) w4_gemm_kernel(const GemmArgs p,
             sr[i] = s_at(kt_begin + nxt);
           }
           uint32_t a[4][4];
-          dequant_tile_lane(w, sw, a);
+          // (way 2 for any scale: a way for each batch of tiles made no difference, 8 tree rows of llama1b 1.78 ms either way)
+          dequant_tile<2>(w, sw, [&](int j, const uint32_t (&f)[4]) { a[j][0] = f[0]; a[j][1] = f[1]; a[j][2] = f[2]; a[j][3] = f[3]; });
           const __half* hrow = hs + kl0 + i * TILE_K + 16 * t;
 #pragma unroll
           for (int mt = 0; mt < MT; ++mt) {

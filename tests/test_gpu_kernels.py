@@ -104,6 +104,30 @@ def test_projection_unpacks_larger_scales(mb, M, K, N, lo, hi):
     assert np.array_equal(y.cpu().numpy(), ref.dequant(qb, sc, 64)[k].astype(np.float32))
 
 
+@pytest.mark.parametrize("call,M,K,N", [("linear", 8, 16448, 48), ("noalloc", 8, 1088, 2400), ("noalloc", 3, 4096, 48)])
+def test_projection_unpacks_tiles_of_mixed_scales(mb, call, M, K, N):
+    """The split-K kernel for few rows (here a K beyond the others' limits) and the persistent one: most tiles hold lanes with scales
+    on both sides of 2^-6, some of one side only; bit for bit."""
+    rng = np.random.default_rng(M + K + N)
+    u = rng.integers(0, 16, size=(K, N)).astype(np.uint8)
+    sc = np.exp2(rng.uniform(-8, -4, size=(K // 64, N))).astype(np.float16)
+    sc[::3] = np.exp2(rng.uniform(-8, -6.1, size=sc[::3].shape)).astype(np.float16)
+    sc[1::9] = np.exp2(rng.uniform(-5.9, 2, size=sc[1::9].shape)).astype(np.float16)
+    qb = gen.pack_nibbles(u)
+    w = mb.mlora_weight_create(dev(qb), dev(sc), K, N, 64)
+    k = rng.integers(0, K, size=M)
+    x = np.zeros((M, K), dtype=np.float16)
+    x[np.arange(M), k] = 1
+    y = torch.empty(M, N, device="cuda")
+    if call == "linear":
+        mb.mlora_linear(w, dev(x), y, torch.zeros(mb.mlora_linear_workspace_bytes(w, M, 1), dtype=torch.uint8, device="cuda"))
+    else:
+        mb.mlora_linear_noalloc(w, dev(x), y)
+    torch.cuda.synchronize()
+    mb.mlora_weight_destroy(w)
+    assert np.array_equal(y.cpu().numpy(), ref.dequant(qb, sc, 64)[k].astype(np.float32))
+
+
 # ------------------------------------------------------------------ fused GEMM + LoRA
 def run_linear(mb, K, N, G, M, n_ad, rank, seed, with_base_rows=True):
     rng = np.random.default_rng(seed)

@@ -91,6 +91,30 @@ def test_prefill_ragged_causal_chunks(GpuModel):
 
 
 @pytest.mark.parametrize("step_path", STEP_PATHS)
+def test_scales_on_both_sides_of_the_unpacks_limit(GpuModel, step_path):
+    """Weights of standard deviation 0.045 in groups of 64: the lanes of most tiles hold scales (max / 7) below and above 2^-6.  A
+    prefill, decode steps on every path, a tree pass of six rows (the projection for few rows)."""
+    cfg = TINYV.small(w_std=0.045)
+    sc = gen.make_model(cfg, 0).scales[0]
+    assert 0.2 < np.mean(np.asarray(sc, dtype=np.float32) < 2.0 ** -6) < 0.8
+    m, orc, gm = make_pair(GpuModel, cfg, max_suffix=16, max_tree=3, step_path=step_path)
+    ids = gen.make_prompt_ids(cfg, 0)
+    compare(gm.prefill(ids), orc.prefill_shared(ids, n_streams=3), "prefill logits")
+    toks = np.array([3, 50], dtype=np.int32)
+    for step in range(2):
+        nxt, logits = gm.decode([0, -1], toks)
+        compare(logits, orc.decode_step([0, -1], tokens=toks)["logits"], f"decode logits, step {step}")
+        toks = nxt
+    parent = np.array([[-1, 0, 1]] * 2, dtype=np.int32)
+    tree = np.array([[5, 6, 7], [8, 9, 10]], dtype=np.int32)
+    got = gm.verify([0, -1], tree, parent)
+    want = orc.verify_tree([0, -1], parent, tree, follow_argmax=np.argmax(got["logits"], axis=1).reshape(2, 3))
+    compare(got["logits"], want["logits"], "verify logits")
+    compare_kv(gm, orc, cfg, 2)
+    gm.close()
+
+
+@pytest.mark.parametrize("step_path", STEP_PATHS)
 def test_prefill_logits_and_follow_mode_decode(GpuModel, step_path):
     cfg = TINYV
     m, orc, gm = make_pair(GpuModel, cfg, max_suffix=32, step_path=step_path)

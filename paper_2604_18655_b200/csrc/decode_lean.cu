@@ -132,9 +132,11 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // PF k-tiles' weights in flight per warp, the input rows of XB of them loaded together, OCC CTAs on an SM.
 // Registers: what OCC CTAs leave each other, and 80 where a CTA of 16 warps has the SM to itself: CTAs of the kernels ahead and
 // behind then fit beside it (96 registers: llama1b, one stream 414 us, 405 with 80; llama3b, eight streams 13.63 -> 13.41 ms).
-constexpr int ln_registers(int warps, int occ) { return occ == 1 ? 80 : 65536 / (warps * 32 * occ) / 8 * 8; }
+// (the limit is stated as CTAs of up to 768 threads: 65536 registers leave those 80 each.  __maxnreg__ must not stand beside
+// __launch_bounds__.)
+constexpr int ln_max_threads(int warps, int occ) { return occ == 1 ? 768 : warps * 32; }
 template <int NTILE, int WARPS, int PF, int XB, int OCC, bool TRACE>
-__global__ void __launch_bounds__(WARPS * 32) __maxnreg__(ln_registers(WARPS, OCC))
+__global__ void __launch_bounds__(ln_max_threads(WARPS, OCC), OCC)
 lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   constexpr int THREADS = WARPS * 32;
   __shared__ float red[WARPS][NTILE][32][4];

@@ -131,7 +131,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 
 // PF k-tiles' weights in flight per warp, the input rows of XB of them loaded together, OCC CTAs on an SM.
 // Registers: what OCC CTAs leave each other, and 80 where a CTA of 16 warps has the SM to itself: CTAs of the kernels ahead and
-// behind then fit beside it (96 registers: llama1b, one stream 414 us, 405 with 80; llama3b, eight streams 13.63 -> 13.41 ms).
+// behind then fit beside it (96 registers: llama1b, one stream 414 us, 405 with 80; llama3b, eight streams 13.63 -> 13.41 ms).  No
+// variant spills: the epilogues that a variant never takes are left out of it (llama1b, one stream 399 -> 395 us).
 // (the limit is stated as CTAs of up to 768 threads: 65536 registers leave those 80 each.  __maxnreg__ must not stand beside
 // __launch_bounds__.)
 constexpr int ln_max_threads(int warps, int occ) { return occ == 1 ? 768 : warps * 32; }
@@ -159,11 +160,9 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   int seg[NTILE], col[NTILE];                                              // projection and first column of each tile
 #pragma unroll
   for (int u = 0; u < NTILE; ++u) map_col(ph.mode, (tile0 + u) * TILE_N, ph.seg_n0, ph.seg_n1, seg[u], col[u]);
-  const int n_out0 = ph.epi == EPI_SWIGLU ? (tile0 >> 1) * TILE_N : tile0 * TILE_N;   // first column the CTA produces
+  const int n_out0 = NTILE == 2 ? (tile0 >> 1) * TILE_N : tile0 * TILE_N;   // first column the CTA produces
   const int kt0 = (L.KT * warp) / WARPS, kt1 = (L.KT * (warp + 1)) / WARPS;
-  const unsigned char* unit[NTILE];
-#pragma unroll
-  for (int u = 0; u < NTILE; ++u) unit[u] = ph.w + (size_t)(tile0 + u) * L.unit_bytes;
+  const unsigned char* const unit = ph.w + (size_t)tile0 * L.unit_bytes;   // (a pair's tiles lie one behind the other)
   uint4 wv[PF][NTILE];
   uint32_t sv[PF][NTILE];
   // (offsets of a k-tile and its scales in 32 bits without a division: the general helpers' 64-bit ones were a quarter of the
@@ -180,8 +179,8 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
         const uint32_t s_off = chunk + ((int)c == L.nchunks - 1 ? L.kc_last : CHUNK_KT) * 512u + ((r * TILE_K) >> gsh) * 32u + g * 4u;
 #pragma unroll
         for (int u = 0; u < NTILE; ++u) {
-          wv[i][u] = ln_ldg_stream(unit[u] + w_off);
-          sv[i][u] = __ldg(reinterpret_cast<const uint32_t*>(unit[u] + s_off));
+          wv[i][u] = ln_ldg_stream(unit + (w_off + u * (uint32_t)L.unit_bytes));
+          sv[i][u] = __ldg(reinterpret_cast<const uint32_t*>(unit + (s_off + u * (uint32_t)L.unit_bytes)));
         }
       }
     }
@@ -202,7 +201,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   ln_stamp<TRACE>(a, 1);
   // ---- what earlier kernels produced: the old residual, norm factors, T of this group, the input rows
   float x_old = 0.f, gain_nx = 1.f;
-  if (ph.epi == EPI_RESID && threadIdx.x < 128 && (threadIdx.x >> 4) < M) {
+  if (NTILE == 1 && ph.epi == EPI_RESID && threadIdx.x < 128 && (threadIdx.x >> 4) < M) {
     x_old = __ldcg(a.X + (size_t)(threadIdx.x >> 4) * ph.N + n_out0 + (threadIdx.x & 15));
     if (ph.gain_next != nullptr) gain_nx = __half2float(__ldg(ph.gain_next + n_out0 + (threadIdx.x & 15)));
   }
@@ -291,7 +290,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
   // ---- one thread per (tile, row, column): sum of the warps' parts in warp order, LoRA expand, norm factor.  With one tile the
   // same thread goes on with its sum (through shared memory and one more barrier: llama1b 15.25 ms, 15.09 so); shared memory is for
   // the row maxima and for the other tile of a gate / up pair.
-  const bool maxima = ph.epi == EPI_F32 && ph.out_f32 == nullptr && a.amax != nullptr;
+  const bool maxima = NTILE == 1 && ph.epi == EPI_F32 && ph.out_f32 == nullptr && a.amax != nullptr;
   float y_own = 0.f;
   for (int o = threadIdx.x; o < NTILE * 128; o += THREADS) {
     const int u = o >> 7, m = (o >> 4) & 7, c = o & 15;
@@ -339,28 +338,21 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
     ln_stamp<TRACE>(a, 3);
     return;
   }
-  if (ph.epi == EPI_F32) {
+  if (NTILE == 1 && ph.epi == EPI_F32) {
     float* out = ph.out_f32 != nullptr ? ph.out_f32 : a.logits;
-    if (NTILE == 1) {
-      const int m = threadIdx.x >> 4, c = threadIdx.x & 15;
-      if (threadIdx.x < 128 && m < M) out[(size_t)m * ph.ldo + tile0 * TILE_N + c] = y_own;
-    } else {
-      for (int o = threadIdx.x; o < NTILE * 128; o += THREADS) {
-        const int u = o >> 7, m = (o >> 4) & 7, c = o & 15;
-        if (m < M) out[(size_t)m * ph.ldo + (tile0 + u) * TILE_N + c] = s_y[u][m][c];
-      }
-    }
+    const int m = threadIdx.x >> 4, c = threadIdx.x & 15;
+    if (threadIdx.x < 128 && m < M) out[(size_t)m * ph.ldo + tile0 * TILE_N + c] = y_own;
     ln_stamp<TRACE>(a, 3);
     return;
   }
-  if (ph.epi == EPI_RESID) {
+  if (NTILE == 1 && ph.epi == EPI_RESID) {
     // new residual; x * gain for the norm that follows; the rows' sums of squares; the next group's partial shrink
     if (threadIdx.x < 128) {
       const int m = threadIdx.x >> 4, c = threadIdx.x & 15;
       float xn = 0.f;
       __half hv = __float2half_rn(0.f);
       if (m < M) {
-        xn = x_old + (NTILE == 1 ? y_own : s_y[0][m][c]);
+        xn = x_old + y_own;
         a.X[(size_t)m * ph.N + n0 + c] = xn;
         if (ph.gain_next != nullptr) {
           hv = __float2half_rn(xn * gain_nx);
@@ -381,7 +373,7 @@ lean_gemm_kernel(const LeanArgs a, const __grid_constant__ StepPhase ph) {
     ln_stamp<TRACE>(a, 3);
     return;
   }
-  // EPI_SWIGLU: tile0 is the gate tile, tile0 + 1 the up tile of 16 features
+  // EPI_SWIGLU (pairs have this epilogue only, single tiles the others): tile0 is the gate tile, tile0 + 1 the up tile of 16 features
   if (NTILE == 2) {
     const int f0 = (tile0 >> 1) * TILE_N, F = ph.N / 2;
     if (threadIdx.x < 128) {

@@ -269,7 +269,7 @@ __device__ __forceinline__ void gemm_tiles(const GemmLoop& q, const WaitCtx& wc,
           if (ok && itl < kc) {
             const uint4 wv = *reinterpret_cast<const uint4*>(sb + itl * 512 + lane * 16);
             const uint32_t sw = *reinterpret_cast<const uint32_t*>(sb + kc * 512 + g * 4 + (itl >> q.gshift) * 32);
-            // (way 2 for any scale: a vote and two ways a tile took the same time, and the kernel is bound by its instructions' fetch)
+            // (way 2 for any scale: with a vote and two ways a tile 32 steps of llama1b took 31.26 ms, 31.13 so)
             dequant_tile<2>(wv, sw, [&](int j, const uint32_t (&af)[4]) {
               const uint4& b = bfr[qi][j >> 1];
               mma_16816(j & 1 ? acc1 : acc0, af, j & 1 ? b.z : b.x, j & 1 ? b.w : b.y);

@@ -465,7 +465,9 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
       }
     }
     constexpr int HC = CW / GR;                            // columns of a warp
-    constexpr int CH = HC < 16 ? HC : 16;                  // columns handled at a time
+    // columns handled at a time: 8 where the next tile's state is held beside the chunk's old rows or table entries (with 16 these
+    // kernels spilled; llama3b, prompt of 1999 13.95 ms, 13.64 so, llama1b, of 512 1.530 and 1.509 ms)
+    constexpr int CH_MAX = S == 1 && (EPI == EPI_RESID || EPI == EPI_QKV) ? 8 : 16, CH = HC < CH_MAX ? HC : CH_MAX;
     static_assert(HC % CH == 0 && CH >= 2 && (S == 1 || NR % (GR * 16) == 0), "a warp's columns: whole chunks, pairs of rows, whole loads");
     const int c_lo = half * HC;
     // (The epilogue is bound by the instructions it issues, 25 to 47 an output by way of an address and a bound for each: pointers
@@ -535,7 +537,8 @@ w4_gemm_tc_kernel(const __grid_constant__ GemmArgs p, int* status, const __grid_
 #pragma unroll
           for (int j = 0; j < CH; ++j) v[j] += xch[(size_t)(q * CW + c0 + j) * TC_BM + lq * 32 + lane];
       } else {
-        tc_ld_32x32b_x16(tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)c0, v);
+        if constexpr (CH == 8) tc_ld_32x32b_x8(tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)c0, v);
+        else tc_ld_32x32b_x16(tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)c0, v);
       }
       float inv[CH];
       if (EPI == EPI_RESID || p.ssq_in != nullptr) {

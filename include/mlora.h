@@ -289,6 +289,11 @@ int mlora_linear_noalloc(mlora_weight* w, const void* x, int32_t M, const int32_
  * kernel's barrier words, so that the next call starts afresh.  Allocates nothing.  Errors: ARG, CUDA, TIMEOUT. */
 int mlora_linear_status(mlora_weight* w, void* workspace);
 
+/* Diagnostics, on the host alone: how the tensor-core projection (from 9 rows on) runs M rows of a K x N matrix on a GPU of sm_count
+ * SMs, called (call = 0) in a pass, (1) with adapters inside it, (2) by mlora_linear without adapters: out[0] rows of a tile, out[1] CTAs
+ * that split K, out[2] groups of unpacking warps.  Errors: ARG. */
+int mlora_debug_gemm_plan(int32_t M, int32_t K, int32_t N, int32_t call, int32_t sm_count, int32_t* out);
+
 /* ---- the paper's own precision regime, single projection (Sec. 3.3 "LLM Quantization": activations quantised per
  * tensor to Int8, weights per channel to Int4) ----
  * mlora_quantize_act_int8: out[i] = clip(round_half_even(x[i] / scale), -127, 127) with the division in float32.

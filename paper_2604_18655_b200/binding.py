@@ -80,6 +80,7 @@ _SIGS = {
     "mlora_linear_noalloc": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
                                        C.c_int32, C.c_int32, C.c_void_p]),
     "mlora_linear_status": (C.c_int, [C.c_void_p, C.c_void_p]),
+    "mlora_debug_gemm_plan": (C.c_int, [C.c_int32] * 5 + [C.POINTER(C.c_int32)]),
     "mlora_attention_workspace_bytes": (C.c_size_t, [C.c_int32] * 7),
     "mlora_attention": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p, C.c_int32,
                                   C.c_void_p, C.c_int32, C.c_void_p, C.c_int32, C.c_int32, C.c_int32, C.c_int32,
@@ -337,6 +338,13 @@ def mlora_linear_noalloc(w, x, y, row_adapter=None, A_ptrs=None, B_ptrs=None, sc
 def mlora_linear_status(w, workspace=None):
     """Raises MloraError if a bounded wait ran out in an mlora_linear / mlora_linear_noalloc call (None: the latter)."""
     _check(lib().mlora_linear_status(w, _ptr(workspace)))
+
+
+def mlora_debug_gemm_plan(M, K, N, call=2, sm_count=148):
+    """(rows of a tile, CTAs that split K, groups of unpacking warps) of the tensor-core projection; needs no GPU"""
+    out = (C.c_int32 * 3)()
+    _check(lib().mlora_debug_gemm_plan(M, K, N, call, sm_count, out))
+    return tuple(out)
 
 
 def mlora_attention_workspace_bytes(n, T, Hq, Hkv, hd, P, own_capacity):

@@ -118,6 +118,9 @@ __host__ __device__ inline int text_width(int slots, int rows_per_slot, int rank
 }
 __host__ __device__ inline int text_mask(int slots, int rank, int ke) { return (long long)slots * rank > ke ? ke - 1 : -1; }
 
+// how a tensor-core projection is called, which decides its plan: in a pass (or ahead of an expand of its own), with adapters inside, or
+// by itself with neither
+enum TcCall { TC_PASS = 0, TC_LORA = 1, TC_ALONE = 2 };
 struct GemmArgs {
   const unsigned char* w;         // packed weights (chunked fragment-major layout)
   int K, N, G;                    // N = physical (fused) width
@@ -134,6 +137,7 @@ struct GemmArgs {
   LoraArgs lora;
   // tcgen05 path only
   int late_wait;                  // the kernel ahead produces only the adapters' T: the activations are complete already
+  int call;                       // TC_PASS or TC_ALONE
   // (sums of squares: ssq_add, row_down; the second part of each array lies ssq_hi entries on)
   const unsigned long long* ssq_in;   // the rows of h still lack 1/rms: their sums of squares [M], or nullptr ...
   const unsigned long long* ssq_in_prev;   // ... and those of the norm before
@@ -357,6 +361,8 @@ constexpr int TC_MIN_ROWS = 9;
 cudaError_t init_gemm_tc();
 bool gemm_tc_eligible(const GemmArgs& a);
 cudaError_t launch_gemm_tc(const GemmArgs& a, int sm_count, int* status, cudaStream_t st);
+struct TcPlan { int rows, split, groups; };       // rows of a tile, CTAs that split K, groups of unpacking warps
+TcPlan tc_plan(int M, int K, int N, TcCall call, int sm_count);
 constexpr int SHRINK_MAX_K = 48 * 1024;   // launch_shrink: a row as fp16 in shared memory
 cudaError_t launch_shrink(const ShrinkArgs& a, cudaStream_t st);
 // T of a pass whose rows are grouped by stream (rows_per_stream each), from fp16 rows, on mma.sync

@@ -1773,6 +1773,7 @@ int mlora_linear(mlora_weight* w, const void* x, int32_t M, const int32_t* row_a
   g.partial = (float*)(ws + fixed); g.partial_capacity = (workspace_bytes - fixed) / sizeof(float);
   g.counters = (unsigned*)(ws + LIN_SYNC_BYTES);
   if (!lora) {
+    g.call = TC_ALONE;
     if (gemm_tc_eligible(g)) CK(launch_gemm_tc(g, w->sm_count, (int*)(ws + 32), w->stream));
     else CK(launch_gemm(g, w->stream));
     return MLORA_OK;
@@ -1876,6 +1877,13 @@ int mlora_linear_noalloc(mlora_weight* w, const void* x, int32_t M, const int32_
   a.status = (int*)(ws + 32);
   a.nstages = stages; a.kmax = w->w.K;
   CK(launch_chain(a, w->sm_count, w->stream));
+  return MLORA_OK;
+}
+
+int mlora_debug_gemm_plan(int32_t M, int32_t K, int32_t N, int32_t call, int32_t sm_count, int32_t* out) {
+  if (!out || M <= 0 || K <= 0 || N <= 0 || K % 64 || N % 16 || call < TC_PASS || call > TC_ALONE || sm_count <= 28) return fail(MLORA_ERR_ARG, "bad size");
+  const TcPlan p = tc_plan(M, K, N, (TcCall)call, sm_count);
+  out[0] = p.rows; out[1] = p.split; out[2] = p.groups;
   return MLORA_OK;
 }
 

@@ -741,49 +741,64 @@ bool gemm_tc_eligible(const GemmArgs& a) {
   return reinterpret_cast<uintptr_t>(a.h) % 16 == 0 && tensor_map_encoder() != nullptr;   // TMA needs both
 }
 
-// Four dequantising groups (GR) where a CTA has an SM for itself: up to 128 rows it is the unpacking that bounds, two groups take 540
-// cycles for a step of 64 features while the MMAs take 255 (128 rows).  llama3b, prompt of 300 3.74 -> 2.97 ms.  Not with
-// adapters: their shrink kernel would no longer start beside the projection ahead (llama1b, two passes of 240 rows 3.02 -> 3.15 ms).
-static bool tc_four_groups(const GemmArgs& a, int nr, long long ctas, int sm_count) {
-  return nr > 128 || ((nr == 64 || nr == 128) && a.lora.adapter_idx == nullptr && ctas <= sm_count);
+// CTAs that run at once with one on an SM: clusters do not fill the machine, 33 of four CTAs and 15 of eight on 148 SMs
+// (cudaOccupancyMaxActiveClusters).
+static int tc_resident(int split, int sm_count) { return sm_count - (split == 4 ? 16 : (split == 8 ? 28 : 0)); }
+
+// Four dequantising groups (GR) where a CTA has an SM for itself: in a pass (the weights are in L2, asked for by the projection
+// ahead) it is the unpacking that bounds up to 128 rows, two groups take 540 cycles for a step of 64 features while the MMAs take 255
+// (128 rows).  llama3b, prompt of 300 3.64 -> 3.05 ms, llama1b 1.33 -> 1.17.  Not with adapters: their shrink kernel would no
+// longer start beside the projection ahead (llama1b, two passes of 240 rows 3.02 -> 3.15 ms).  Not in a call of its own, whose weights
+// come from HBM: over the best candidate with two it gained at most 2 % (21 projections, 9 .. 2000 rows), and the next call's CTAs find no room.
+// Not where a cluster would have to wait for a second wave (8192 x 2048, 64 rows in clusters of eight: 16.7 us, 10.1 with two groups).
+static bool tc_four_groups(TcCall call, int nr, int split, long long ctas, int sm_count) {
+  return nr > 128 || ((nr == 64 || nr == 128) && call == TC_PASS && ctas <= tc_resident(split, sm_count));
 }
 
-// Rows per CTA and K split, by a model of the time in microseconds, fitted to measurements of all candidates at projections
-// of 2048 x 2048 .. 14336 x 4096 with 16 .. 2000 rows: the time of a step with one or two CTAs on an SM (or one with four groups),
-// set-up and epilogue, what a further wave costs (less where the CTA stays), and the exchange of a split.  Clusters of four CTAs do
-// not fill the machine: 33 of them on 148 SMs with one CTA each (cudaOccupancyMaxActiveClusters).  (Of eight 15, but their splits are
-// so fine that the rest of a wave costs little, and adapters gain from them: 14336 x 4096, 32 rows, 8 adapters of rank 16 24.4 us in
-// eight, 30.4 in four.)  Without adapters, against the best candidate at ten projections and 16 .. 2000 rows: 0.4 % more on average,
-// 14 % at worst (2048 x 2048, 128 rows); the constants from before the four groups and the shorter epilogues 1.7 % and 19 %
-// (prompts of 100 and 512 on llama1b 0.776 -> 0.764 and 1.553 -> 1.526 ms).  Those stay with adapters, whose expand (left out of the
-// model) and shrink beside the projection ahead change the order: llama3b, two passes of 256 rows 7.43 ms, 8.04 with the others.
+// Rows per CTA and K split, by a model of the time in microseconds: that of a step of 64 features with one or two CTAs on an SM (or
+// one with four groups), set-up and epilogue, what a further wave costs (less where the CTA stays), and the exchange of a split.
+// pass: fitted to all candidates of ten projections of 2048 x 2048 .. 14336 x 4096 with 16 .. 2000 rows, four groups among them (prompts of
+// 100 and 512 on llama1b 0.776 -> 0.764 and 1.553 -> 1.526 ms against the constants of lora).
+// alone: fitted to all candidates with two groups at half of 462 pairs of a projection (512 x 512 .. 14336 x 4096) and a row count (9 ..
+// 2000), steps' times held to rise with the rows.  Against the best candidate 0.3 % more on average on the fitted half, 0.6 % on the
+// other, 14 % at worst; calls of their own with the constants of pass 9.4 %, and 92 % at worst.
+// lora: the expand (left out of the model) and the shrink beside the projection ahead change the order; these are the constants with
+// which llama3b's tree passes were fastest (two of 256 rows 7.43 ms, 8.04 with those of pass).  Splits in eight gain there even where
+// the rest of them waits (14336 x 4096, 32 rows, 8 adapters of rank 16 24.4 us, 30.4 in four).
 struct TcCosts { double step1[6], step2[6], step4[6], fixed, tail, tail4, exchange, exchange4, eight, wave1, wave1_f, wave, wave_f; };
-static void tc_plan(const GemmArgs& a, int sm_count, int& nr, int& split) {
+TcPlan tc_plan(int M, int K, int N, TcCall call, int sm_count) {
   static const int sizes[6] = {32, 64, 96, 128, 192, 256};
-  static const TcCosts plain = {{0.227, 0.242, 0.228, 0.286, 0.303, 0.320}, {0.393, 0.399, 0.484, 0.602, 0.0, 0.0}, {0.0, 0.274, 0.0, 0.244, 0.303, 0.320},
-                                4.37, 5.86, 5.15, 4.86, 2.67, 1.41, 1.4, 7.04, 4.86, 5.71};
-  static const TcCosts lora = {{0.227, 0.242, 0.264, 0.286, 0.303, 0.320}, {0.393, 0.429, 0.484, 0.538, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0, 0.303, 0.320},
-                               3.34, 3.36, 3.36, 2.52, 2.52, 1.6, 1.4, 5.1, 4.8, 7.8};
-  const TcCosts& t = a.lora.adapter_idx == nullptr ? plain : lora;
-  const int slabs = (a.N + TC_BM - 1) / TC_BM, KT = a.K / TILE_K;
+  static const TcCosts costs[3] = {
+      {{0.227, 0.242, 0.228, 0.286, 0.303, 0.320}, {0.393, 0.399, 0.484, 0.602, 0.0, 0.0}, {0.0, 0.274, 0.0, 0.244, 0.303, 0.320},
+       4.37, 5.86, 5.15, 4.86, 2.67, 1.41, 1.4, 7.04, 4.86, 5.71},
+      {{0.227, 0.242, 0.264, 0.286, 0.303, 0.320}, {0.393, 0.429, 0.484, 0.538, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0, 0.303, 0.320},
+       3.34, 3.36, 3.36, 2.52, 2.52, 1.6, 1.4, 5.1, 4.8, 7.8},
+      {{0.1957, 0.2, 0.2147, 0.2147, 0.2829, 0.3241}, {0.4481, 0.4481, 0.4997, 0.526, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0, 0.2829, 0.3241},
+       2.11, 4.07, 3.08, 1.87, 2.33, 0.13, 0.78, 3.82, 0.0, 9.61}};
+  static const int below[6] = {0, 32, 64, 64, 128, 128};   // alone: tiles that some smaller one with the same splits leaves without use
+  const TcCosts& t = costs[call];
+  const int slabs = (N + TC_BM - 1) / TC_BM, KT = K / TILE_K;
   double best = 1e30;
+  TcPlan plan{32, 1, 2};
   for (int ri = 0; ri < 6; ++ri) {
     const int R = sizes[ri], max_split = R == 96 || R == 192 ? 1 : 8;
-    if (ri > 0 && a.M <= sizes[ri - 1]) break;
+    if (ri > 0 && M <= (call == TC_ALONE ? below[ri] : sizes[ri - 1])) break;
     for (int S = 1; S <= max_split; S *= 2) {
       if (S > 1 && KT / S < 4) break;
-      const int sms = S == 4 ? sm_count - 16 : sm_count;
-      const long long ctas = (long long)slabs * ((a.M + R - 1) / R) * S, per_wave = (long long)sms * (R > 128 ? 1 : 2);
+      // (not counted with so few rows that the weights bound: 14336 x 2048, 32 rows 13.5 us in eight, 14.6 in four)
+      const int sms = S < 8 || (call == TC_ALONE && M > 32) ? tc_resident(S, sm_count) : sm_count;
+      const long long ctas = (long long)slabs * ((M + R - 1) / R) * S, per_wave = (long long)sms * (R > 128 ? 1 : 2);
       const long long full = ctas / per_wave, rest = ctas % per_wave;
-      const bool four = tc_four_groups(a, R, ctas, sm_count);
+      const bool four = tc_four_groups(call, R, S, ctas, sm_count);
       const double steps = (KT + S - 1) / S, f = R / 256.0, one = four ? t.step4[ri] : t.step1[ri];
       const double full_t = R > 128 ? one : t.step2[ri], rest_t = rest == 0 ? 0.0 : (rest > sms ? t.step2[ri] : one);
       const double more = (double)full + (rest > 0 ? 1 : 0) - 1.0;
       const double cost = steps * (full * full_t + rest_t) + t.fixed + (four ? t.tail4 : t.tail) * f + (S > 1 ? (four ? t.exchange4 : t.exchange) * f : 0.0) +
                           (S == 8 ? t.eight : 0.0) + more * (S == 1 ? t.wave1 + t.wave1_f * f : t.wave + t.wave_f * f);
-      if (cost < best) { best = cost; nr = R; split = S; }
+      if (cost < best) { best = cost; plan = TcPlan{R, S, four ? 4 : 2}; }
     }
   }
+  return plan;
 }
 
 // `status` may be nullptr
@@ -791,12 +806,9 @@ cudaError_t launch_gemm_tc(const GemmArgs& args, int sm_count, int* status, cuda
   GemmArgs a = args;
   const unsigned T = (unsigned)(a.epi == EPI_QKV ? a.rows_per_stream : (a.lora.adapter_idx != nullptr ? a.lora.rows_per_stream : 1));
   a.stream_magic = T > 1 ? 0xffffffffu / T + 1u : 0u;      // exact for m, T below 65536
-  int nr = 32, split = 1;
-  tc_plan(a, sm_count, nr, split);
-  const long long ctas = (long long)((a.N + TC_BM - 1) / TC_BM) * ((a.M + nr - 1) / nr) * split;
-  const int grp = tc_four_groups(a, nr, ctas, sm_count) ? 4 : 2;
+  const TcPlan plan = tc_plan(a.M, a.K, a.N, a.lora.adapter_idx != nullptr ? TC_LORA : (TcCall)a.call, sm_count);
 #define TC_CASE(NR, S, GRP) \
-  if (nr == NR && split == S && grp == GRP) \
+  if (plan.rows == NR && plan.split == S && plan.groups == GRP) \
     return a.epi == EPI_F32 ? tc_launch<NR, S, EPI_F32, GRP>(a, sm_count, status, st) : a.epi == EPI_RESID ? tc_launch<NR, S, EPI_RESID, GRP>(a, sm_count, status, st) \
          : a.epi == EPI_SWIGLU ? tc_launch<NR, S, EPI_SWIGLU, GRP>(a, sm_count, status, st) : tc_launch<NR, S, EPI_QKV, GRP>(a, sm_count, status, st);
   TC_FOR_EACH(TC_CASE)

@@ -62,3 +62,23 @@ def test_unsupported_rope_style_is_refused_on_the_host(libpath):
     out = ctypes.c_void_p()
     assert L.mlora_create(ctypes.byref(d), ctypes.byref(out)) == -6
     assert b"rope_style" in L.mlora_last_error(None)
+
+
+def test_projection_plan_waits_for_no_second_wave_of_clusters(libpath):
+    """Host side of the tensor-core projection: four unpacking groups (one CTA an SM) only where all clusters run at once (15 of eight CTAs,
+    33 of four on 148 SMs), never in a call of its own or with adapters; every tile has a use."""
+    from paper_2604_18655_b200 import binding as mb
+    resident, seen = {1: 148, 2: 148, 4: 132, 8: 120}, set()
+    for K in (64, 512, 1408, 2048, 4096, 6144, 8192, 14336):
+        for N in (16, 512, 1024, 1152, 2048, 2176, 2304, 3072, 4096, 11264, 14336):
+            for M in (9, 33, 40, 64, 65, 100, 128, 129, 200, 256, 300, 700, 1999):
+                for call in (0, 1, 2):
+                    rows, split, groups = mb.mlora_debug_gemm_plan(M, K, N, call)
+                    seen.add(rows)
+                    ctas = -(-N // 128) * -(-M // rows) * split
+                    if rows <= 128 and groups == 4:
+                        assert call == 0 and ctas <= resident[split], (M, K, N, rows, split)
+    assert seen == {32, 64, 96, 128, 192, 256}
+    assert mb.mlora_debug_gemm_plan(64, 8192, 2048, 0)[2] == 2      # 16 clusters of eight
+    with pytest.raises(mb.MloraError):
+        mb.mlora_debug_gemm_plan(64, 100, 2048, 0)

@@ -27,8 +27,9 @@ def test_projection_row_tiles(mb, M):
     (4096, 256, 128, 40),        # few columns: the widest split of K
     (14336, 128, 128, 250),      # the longest K in two row blocks
     (320, 4096, 64, 700),        # K of an odd number of steps, more tiles than CTAs: each stays for further ones
-    (192, 9600, 64, 180),        # the same with the 192-row tile, fewer steps than weight stages
-    (192, 9600, 64, 90),         # and the 96-row one
+    (192, 9600, 64, 180),        # the same with fewer steps than weight stages
+    (192, 9600, 64, 90),
+    (64, 15376, 64, 280),        # the 96-row tile, again more tiles than CTAs
     (2048, 3072, 128, 96), (2048, 3072, 128, 192),   # clusters of four would not all fit at once: split in two
 ])
 def test_projection_splits_and_persistent_tiles(mb, K, N, G, M):
@@ -38,11 +39,39 @@ def test_projection_splits_and_persistent_tiles(mb, K, N, G, M):
 
 
 @pytest.mark.parametrize("K,N,M", [(192, 1040, 40), (320, 1040, 64), (64, 16, 128), (2048, 272, 65), (832, 1040, 128), (4096, 400, 100)])
-def test_projection_with_four_unpacking_groups(mb, K, N, M):
-    """Tiles of 64 and 128 rows whose grid leaves every CTA an SM: fewer steps than groups, steps that the groups share
-    unevenly, K splits down to a pair of rows a warp."""
+def test_projection_of_few_columns(mb, K, N, M):
+    """Fewer steps than pairs of unpacking groups, K splits down to a pair of rows a warp."""
     got, want = run_linear(mb, K, N, 64, M, 0, 0, seed=K + N + M)
+    compare(got, want, f"few columns K{K} N{N} M{M}")
+
+
+@pytest.mark.parametrize("K,N,M,plan", [
+    (320, 4112, 200, (64, 1, 4)), (832, 4112, 250, (64, 1, 4)), (1088, 4112, 65, (64, 2, 4)), (2048, 2064, 33, (64, 4, 4)),
+    (2048, 528, 200, (64, 4, 4)), (8192, 528, 100, (64, 8, 4)), (8192, 272, 250, (64, 8, 4)), (2048, 4112, 200, (128, 2, 4)),
+    (3136, 4112, 100, (128, 4, 4)), (8192, 528, 250, (128, 8, 4)),
+])
+def test_projection_with_four_unpacking_groups(mb, K, N, M, plan):
+    """Tiles of 64 and 128 rows whose grid leaves every CTA an SM (the projection ahead of an expand of its own): steps that the groups
+    share unevenly, K splits down to a pair of rows a warp."""
+    assert mb.mlora_debug_gemm_plan(M, K, N, 0) == plan
+    got, want = run_linear(mb, K, N, 64, M, 70, 16, seed=K + N + M)
     compare(got, want, f"four groups K{K} N{N} M{M}")
+
+
+@pytest.mark.parametrize("P", [100, 200])
+def test_prefill_with_four_unpacking_groups(GpuModel, P):
+    """The other epilogues with four groups: q,k,v, o, gate/up and down of one layer of 2048."""
+    from paper_2604_18655_b200 import binding as mb
+    cfg = gen.ModelCfg("four", 1, 2048, 32, 8, 64, 5632, 0, 128, 4, gen.configs.ALL7, 1, 1, P)
+    shapes = ((2048, 3072), (2048, 2048), (2048, 11264), (5632, 2048))
+    assert sum(mb.mlora_debug_gemm_plan(P, K, N, 0)[2] == 4 for K, N in shapes) == 4
+    _, orc, gm = make_pair(GpuModel, cfg, max_suffix=2)
+    x = gen.make_hidden(cfg, P, 0, 0)
+    compare(gm.prefill_h(x), orc.prefill_shared(hidden=x), f"prefill of {P}")
+    _, pk, pv = gm.export_kv(0, -1, 0, P)
+    compare(pk, orc.prefix_k[0], "prefix K")
+    compare(pv, orc.prefix_v[0], "prefix V")
+    gm.close()
 
 
 @pytest.mark.parametrize("M,n_ad,rank,K", [(9, 1, 1, 256), (17, 40, 12, 1024), (300, 2, 64, 8192), (64, 64, 16, 2112)])
